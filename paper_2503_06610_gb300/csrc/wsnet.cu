@@ -15,12 +15,12 @@
 //
 // Convolutions run on the tensor cores as implicit GEMMs (BF16 inputs, FP32
 // accumulators):
-//   forward       M = voxels (128 per CTA), N = cout, K = 27 taps x cin, on the
+//   forward       M = voxels (128 per step), N = cout, K = 27 taps x cin, on the
 //                 5th-generation tensor cores (tcgen05.mma, accumulator in TMEM)
 //   data grad     M = voxels, N = cin, K = 27 taps x cout (transposed weights),
-//                 mma.sync.m16n8k16
-//   weight grad   M = cout, N = cin, K = voxels (per tap; shared-memory tiles,
-//                 FP32 atomics across voxel chunks), mma.sync.m16n8k16
+//                 the same kernel
+//   weight grad   M = cout, N = cin, K = voxels (all taps from one shared-memory
+//                 halo tile, FP32 atomics across blocks), mma.sync.m16n8k16
 #include <stdint.h>
 #include <string.h>
 
@@ -66,19 +66,9 @@ __device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], const 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__device__ __forceinline__ uint32_t ld_pair(const bf16* p) { return __ldg(reinterpret_cast<const unsigned int*>(p)); }
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
-
-__device__ __forceinline__ uint32_t pack_raw(bf16 lo, bf16 hi)
-{
-    __nv_bfloat162 v;
-    v.x = lo;
-    v.y = hi;
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
@@ -86,84 +76,55 @@ struct Dims {
     int nx, ny, nz, nvox, batch;
 };
 
-// Voxel v split into (batch, x, y, z) once, and shifted by (dx, dy, dz):
-// periodic in x, y; -1 outside in z (a kernel shifts one voxel by up to 27
-// taps).
-struct VoxCoord {
-    int b, x, y, z;  // b < 0: no voxel
-};
-__device__ __forceinline__ VoxCoord vox_coord(const Dims& d, int v)
-{
-    VoxCoord c{-1, 0, 0, 0};
-    if (v < 0 || v >= d.nvox * d.batch) return c;
-    c.b = v / d.nvox;
-    const int r = v - c.b * d.nvox;
-    c.x = r % d.nx;
-    const int t = r / d.nx;
-    c.y = t % d.ny;
-    c.z = t / d.ny;
-    return c;
-}
-__device__ __forceinline__ int shifted(const Dims& d, const VoxCoord& c, int dx, int dy, int dz)
-{
-    const int zs = c.z + dz;
-    if (c.b < 0 || zs < 0 || zs >= d.nz) return -1;
-    int xs = c.x + dx, ys = c.y + dy;
-    xs = xs < 0 ? xs + d.nx : (xs >= d.nx ? xs - d.nx : xs);
-    ys = ys < 0 ? ys + d.ny : (ys >= d.ny ? ys - d.ny : ys);
-    return c.b * d.nvox + xs + d.nx * (ys + d.ny * zs);
-}
+// ------------------------------------------------------------------ convolution on tcgen05: forward and data gradient
+//
+// One CTA (four warps) computes 8 x 16 output voxels of a z plane x NB output
+// channels per step and walks up a chunk of planes; each plane is the implicit
+// GEMM D[128][NB] = sum over the 27 taps of A_t[128][K] W_t^T.  Planes of the
+// input with a one-voxel halo in x and y (10 x 18 voxels) sit in a ring of four
+// shared-memory slots in the tensor core's no-swizzle K-major layout, 16-byte
+// channel groups of consecutive voxels next to each other: the eight voxels of
+// an x run are a core matrix, so the A operand of *every* tap is the same plane
+// read from a shifted start address (LBO = one channel-group plane, SBO = one
+// row of ten voxels), and a plane is copied once instead of once per tap.
+// (Copying each tap's rows took 339 us for a 16 -> 16 layer of 8 x 64 x 64 x 32
+// voxels, bound by the copies and a barrier per three taps.)  The weights of all
+// taps stay in shared memory for the CTA's life.  One thread issues a plane's 27
+// K/16 MMAs (kind::f16, BF16 x BF16 -> FP32, M = 128, N = NB, K = 16) into one of
+// two TMEM accumulators and commits them to its mbarrier; the copies of the plane
+// after next and the epilogue of the plane before run meanwhile.  Every mbarrier
+// wait is bounded: on expiry the kernel raises a.status, skips the epilogue,
+// waits for its copies and frees its TMEM.
+//
+// Forward: input = the layer's sources, D + bias, ReLU, BF16 rows.  Data gradient
+// (Flip): input = the pre-activation gradient, taps mirrored, transposed weights,
+// FP32 rows overwritten in dst1 (channels below n1) or added to dst2.
 
-// ------------------------------------------------------------------ convolution: forward
-
-struct ConvFwd {
+struct ConvTc {
     const bf16* src1;
     int c1;
-    const bf16* src2;  // concatenated after src1 (may be null, c2 = 0)
+    const bf16* src2;  // concatenated after src1 (c2 = 0: none)
     int c2;
-    const bf16* w;     // [27][cout][cin]
-    const float* bias; // [cout]
-    bf16* dst;         // [vox][cout]
+    int up1;           // src1 is held at half the resolution and read nearest (upsampling)
+    const bf16* w;     // [27][n][c1 + c2]
+    int n;             // output channels; blockIdx.y takes NB of them
     Dims d;
-    int relu;
-    int* status;       // set to 1 when a bounded wait of the tensor-core kernel expires
-    int tps;           // taps per shared-memory stage of the tensor-core kernel (1..9)
+    int zc;            // planes per chunk
+    const float* bias; // forward: [n]
+    bf16* out;         // forward: [vox][n]
+    float* dst1;       // data gradient: [vox][n1], overwritten
+    int n1;
+    float* dst2;       // data gradient: [vox][n - n1], accumulated
+    int* status;       // set to 1 when a bounded wait expires
 };
-
-// ------------------------------------------------------------------ convolution: forward on tcgen05
-//
-// One CTA (four warps) computes 128 output voxels x COUT channels, the
-// implicit GEMM D[128][COUT] = sum over the 27 taps of A_t[128][cin] W_t^T,
-// A_t the cin input channels of the tap-shifted voxels.  Per tap, A_t and W_t
-// are copied into shared memory with 16-byte cp.async (zero rows where the tap
-// leaves the volume in z) in the tensor core's no-swizzle K-major layout:
-// core matrices of 8 rows x 16 bytes, adjacent core matrices along K 128 bytes
-// apart (LBO), along M / N cin/8 x 128 bytes apart (SBO).  A stage holds tps
-// consecutive taps (tc_taps_per_stage: as many as fit in 14 KB, 1 to 9);
-// one thread issues their cin/16 MMAs each (tcgen05.mma kind::f16, BF16 x
-// BF16 -> FP32, M = 128, N = COUT, K = 16) into a TMEM accumulator and commits
-// them to the stage's mbarrier; two stages let the copies of the next taps
-// overlap the MMAs of these.  The epilogue reads each warp's 32 accumulator rows with
-// tcgen05.ld, adds the bias, applies the ReLU and stores BF16 rows.  Every
-// mbarrier wait is bounded: on expiry the kernel raises a.status, skips the
-// epilogue, waits for its copies and frees its TMEM.
 
 constexpr int kTcM = 128;
 constexpr int kTcThreads = 128;
-constexpr int kTcMaxCin = 96;
-constexpr int kTcMaxCout = 64;
-// A stage holds as many taps as fit in kTcStageBytes (at least one, at most 9:
-// one dz plane of the stencil), so that thin layers commit a K of several
-// taps per barrier round trip while several CTAs still fit on an SM.
-constexpr size_t kTcStageBytes = 14 * 1024;
-constexpr size_t kTcWidestTap = (size_t)(kTcM + kTcMaxCout) * kTcMaxCin * sizeof(bf16);
-constexpr size_t kTcSmem = 2 * (kTcWidestTap > kTcStageBytes ? kTcWidestTap : kTcStageBytes) + 64;
-inline int tc_taps_per_stage(int cin, int cout)
-{
-    const size_t tap = (size_t)(kTcM + cout) * cin * sizeof(bf16);
-    const int t = (int)(kTcStageBytes / tap);
-    return t < 1 ? 1 : (t > 9 ? 9 : t);
-}
+constexpr int kTcX = 8, kTcY = 16;                                // output voxels of a plane step
+constexpr int kTcHX = kTcX + 2, kTcHY = kTcY + 2, kTcHalo = kTcHX * kTcHY;
+constexpr int kTcRing = 4;
+inline size_t tc_smem(int K, int NB) { return (size_t)K * 2 * (kTcRing * kTcHalo + 27 * NB) + 64; }
+constexpr size_t kTcMaxSmem = 227 * 1024;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
@@ -218,24 +179,29 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <int COUT>
-__global__ void __launch_bounds__(kTcThreads) conv_fwd_tc_kernel(const ConvFwd a)
+template <int NB, bool Flip>
+__global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
 {
-    extern __shared__ __align__(128) unsigned char tc_smem[];
-    const int cin = a.c1 + a.c2;
-    const int kb = cin / 8;                        // 16-byte core-matrix columns along K
-    const uint32_t sbo_a = (uint32_t)kb * 128u;    // between 8-row groups
-    const uint32_t a_bytes = kTcM * cin * 2, b_bytes = COUT * cin * 2;
-    const int tps = a.tps;                              // taps per stage
-    const uint32_t tap_bytes = a_bytes + b_bytes, stage_bytes = (uint32_t)tps * tap_bytes;
-    const int stages = (27 + tps - 1) / tps;
-    const uint32_t smem0 = smem_u32(tc_smem);  // stage s starts at smem0 + s stage_bytes
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem + 2 * stage_bytes);
+    extern __shared__ __align__(128) unsigned char tc_smem_raw[];
+    const int K = a.c1 + a.c2, kb = K / 8;  // 16-byte channel groups
+    constexpr uint32_t kGroup = kTcHalo * 16;              // one channel group of a plane
+    const uint32_t plane_bytes = (uint32_t)kb * kGroup;
+    const uint32_t tap_bytes = (uint32_t)NB * K * 2;
+    const uint32_t ring = smem_u32(tc_smem_raw), wbase = ring + kTcRing * plane_bytes;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem_raw + kTcRing * plane_bytes + 27 * tap_bytes);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
-    constexpr uint32_t kCols = COUT < 32 ? 32 : COUT;
+    constexpr uint32_t kCols = 2 * NB;  // two accumulators: 32 or 64 columns
+    static_assert(NB == 16 || NB == 32, "TMEM columns are allocated in powers of two, at least 32");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int total = a.d.nvox * a.d.batch;
-    const int v0 = blockIdx.x * kTcM;
+    const Dims d = a.d;
+    const int tx = (d.nx + kTcX - 1) / kTcX, ty = (d.ny + kTcY - 1) / kTcY, tz = (d.nz + a.zc - 1) / a.zc;
+    int blk = blockIdx.x;
+    const int x0 = (blk % tx) * kTcX;
+    blk /= tx;
+    const int y0 = (blk % ty) * kTcY;
+    blk /= ty;
+    const int z0 = (blk % tz) * a.zc, z1 = min(z0 + a.zc, d.nz), batch = blk / tz;
+    const int n0 = blockIdx.y * NB;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
@@ -248,111 +214,138 @@ __global__ void __launch_bounds__(kTcThreads) conv_fwd_tc_kernel(const ConvFwd a
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&bars[1])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+
+    // a thread copies one channel group of every vstep-th voxel of a plane
+    const int cq = tid % kb, vfirst = tid / kb, vstep = kTcThreads / kb;
+    const bool loader = vfirst < vstep;
+    const bool from1 = cq * 8 < a.c1;
+    const bool up = from1 && a.up1;
+    const bf16* lsrc = from1 ? a.src1 + cq * 8 : a.src2 + (cq * 8 - a.c1);
+    const int lc = from1 ? a.c1 : a.c2;
+    auto load_plane = [&](int z) {  // zero beyond the volume in z
+        if (loader) {
+            const bool zin = z >= 0 && z < d.nz;
+            const uint32_t dst = ring + (uint32_t)(z & (kTcRing - 1)) * plane_bytes + (uint32_t)cq * kGroup;
+            for (int v = vfirst; v < kTcHalo; v += vstep) {
+                const int hy = v / kTcHX, hx = v - hy * kTcHX;
+                int x = x0 - 1 + hx, y = y0 - 1 + hy;
+                x = x < 0 ? x + d.nx : (x >= d.nx ? x - d.nx : x);
+                y = y < 0 ? y + d.ny : (y >= d.ny ? y - d.ny : y);
+                const bool ok = zin && x < d.nx && y < d.ny;  // beyond a ragged tile's halo: unused, zero
+                const int s = up ? batch * (d.nvox >> 3) + (x >> 1) + (d.nx >> 1) * ((y >> 1) + (d.ny >> 1) * (z >> 1))
+                                 : batch * d.nvox + x + d.nx * (y + d.ny * z);
+                cp_async16(dst + (uint32_t)v * 16u, ok ? lsrc + (size_t)s * lc : lsrc, ok);
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    for (int i = tid; i < 27 * NB * kb; i += kTcThreads) {
+        const int q = i % kb, r = i / kb, n = r % NB, t = r / NB;
+        cp_async16(wbase + (uint32_t)t * tap_bytes + (uint32_t)(n >> 3) * (uint32_t)(kb * 128) + (uint32_t)q * 128u +
+                       (uint32_t)(n & 7) * 16u,
+                   a.w + ((size_t)t * a.n + n0 + n) * K + q * 8, true);
+    }
+    for (int z = z0 - 1; z <= z0 + 1; ++z) load_plane(z);
+
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
-    // Thread tid stages A row tid (voxel v0 + tid) for every tap: its
-    // coordinates are split once here, and a tap only shifts and wraps them.
-    static_assert(kTcM == kTcThreads, "one A row per thread");
-    const VoxCoord row = vox_coord(a.d, v0 + tid);
-    const uint32_t arow = (uint32_t)(tid >> 3) * sbo_a + (uint32_t)(tid & 7) * 16u;
-
-    // copies of tap t into slot tt of stage s: the A rows (voxels) and the W_t rows (output channels)
-    auto load_tap = [&](int t, int s, int tt) {
-        const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-        const uint32_t sa = (smem0 + (uint32_t)s * stage_bytes) + (uint32_t)tt * tap_bytes, sb = sa + a_bytes;
-        {
-            const int sv = shifted(a.d, row, dx, dy, dz);  // -1 beyond the plates (zero fill)
-            const bf16* s1 = sv >= 0 ? a.src1 + (size_t)sv * a.c1 : a.src1;
-            const bf16* s2 = sv >= 0 ? a.src2 + (size_t)sv * a.c2 : a.src1;
-            for (int q = 0; q < kb; ++q) {
-                const int c = q * 8;
-                cp_async16(sa + arow + (uint32_t)q * 128u, c < a.c1 ? s1 + c : s2 + (c - a.c1), sv >= 0);
-            }
-        }
-        const bf16* w = a.w + (size_t)t * COUT * cin;
-        for (int i = tid; i < COUT * kb; i += kTcThreads) {
-            const int n = i / kb, q = i - n * kb;
-            cp_async16(sb + (uint32_t)(n >> 3) * sbo_a + (uint32_t)q * 128u + (uint32_t)(n & 7) * 16u,
-                       w + (size_t)n * cin + q * 8, true);
-        }
-    };
-    // stage g: taps g tps .. g tps + tps - 1, one commit group
-    auto load_stage = [&](int g, int s) {
-        for (int tt = 0; tt < tps; ++tt) {
-            const int t = g * tps + tt;
-            if (t < 27) load_tap(t, s, tt);
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    };
-
-    constexpr uint32_t idesc = umma_idesc_bf16(kTcM, COUT);
-    bool ok = true;
-    load_stage(0, 0);
-    for (int g = 0; g < stages; ++g) {
-        const int s = g & 1;
-        if (g + 1 < stages) {
-            if (g >= 1) ok = ok && mbar_wait(smem_u32(&bars[s ^ 1]), ((g - 1) >> 1) & 1);  // MMAs of stage g - 1
-            if (ok) load_stage(g + 1, s ^ 1);
-            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        }
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the copies, to the tensor core's view
-        ok = __syncthreads_and(ok) != 0;  // every thread takes the same branch
-        if (!ok) break;
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            for (int tt = 0; tt < tps && g * tps + tt < 27; ++tt) {
-                const uint32_t sa = (smem0 + (uint32_t)s * stage_bytes) + (uint32_t)tt * tap_bytes, sb = sa + a_bytes;
-                for (int j = 0; j < cin / 16; ++j) {
-                    const uint64_t ad = umma_desc(sa + 256u * j, 128u, sbo_a);
-                    const uint64_t bd = umma_desc(sb + 256u * j, 128u, sbo_a);
-                    const uint32_t acc = (g > 0 || tt > 0 || j > 0) ? 1u : 0u;
-                    asm volatile(
-                        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                        : "memory");
-                }
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                             smem_u32(&bars[s]))
-                         : "memory");
-        }
-    }
-    // the commit of the last stage covers every MMA
-    if (ok) ok = mbar_wait(smem_u32(&bars[(stages - 1) & 1]), ((stages - 1) >> 1) & 1);
-    ok = __syncthreads_and(ok) != 0;
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (ok) {
-        const int r = warp * 32 + lane;
-        const int v = v0 + r;
+    constexpr uint32_t idesc = umma_idesc_bf16(kTcM, NB);
+    // row r of the accumulator is voxel (x0 + r % 8, y0 + r / 8) of the plane
+    const int row = warp * 32 + lane;
+    const int vx = x0 + (row & 7), vy = y0 + (row >> 3);
+    const bool inside = vx < d.nx && vy < d.ny;
+    auto epilogue = [&](int z) {
+        const uint32_t acc0 = tmem + (uint32_t)(((z - z0) & 1) * NB) + ((uint32_t)(warp * 32) << 16);
+        const size_t v = (size_t)batch * d.nvox + vx + (size_t)d.nx * (vy + (size_t)d.ny * z);
 #pragma unroll
-        for (int c0 = 0; c0 < COUT; c0 += 16) {
+        for (int c0 = 0; c0 < NB; c0 += 16) {
             float acc[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, acc);
-            if (v < total) {
+            tmem_ld16(acc0 + (uint32_t)c0, acc);
+            if (!inside) continue;
+            if constexpr (!Flip) {
                 uint32_t packed[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    float x0 = acc[2 * i] + a.bias[c0 + 2 * i], x1 = acc[2 * i + 1] + a.bias[c0 + 2 * i + 1];
-                    if (a.relu) {
-                        x0 = fmaxf(x0, 0.f);
-                        x1 = fmaxf(x1, 0.f);
-                    }
-                    packed[i] = pack_bf16(x0, x1);
+                    const float b0 = __ldg(a.bias + n0 + c0 + 2 * i), b1 = __ldg(a.bias + n0 + c0 + 2 * i + 1);
+                    packed[i] = pack_bf16(fmaxf(acc[2 * i] + b0, 0.f), fmaxf(acc[2 * i + 1] + b1, 0.f));
                 }
-                uint4* dst = reinterpret_cast<uint4*>(a.dst + (size_t)v * COUT + c0);
+                uint4* dst = reinterpret_cast<uint4*>(a.out + v * a.n + n0 + c0);
                 dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                 dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+            } else if (n0 + c0 < a.n1) {
+                float4* dst = reinterpret_cast<float4*>(a.dst1 + v * a.n1 + n0 + c0);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dst[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+            } else {
+                float4* dst = reinterpret_cast<float4*>(a.dst2 + v * (a.n - a.n1) + (n0 + c0 - a.n1));
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float4 o = dst[i];
+                    o.x += acc[4 * i];
+                    o.y += acc[4 * i + 1];
+                    o.z += acc[4 * i + 2];
+                    o.w += acc[4 * i + 3];
+                    dst[i] = o;
+                }
             }
         }
-    } else if (tid == 0) {
-        atomicExch(a.status, 1);
+    };
+
+    bool ok = true;
+    for (int z = z0; z < z1; ++z) {
+        const int k = z - z0;
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the copies, to the tensor core's view
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");  // the epilogue's TMEM reads
+        ok = __syncthreads_and(ok) != 0;
+        if (!ok) break;
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint64_t ad0 = umma_desc(0, kGroup, kTcHX * 16), bd0 = umma_desc(0, 128u, (uint32_t)kb * 128u);
+            const uint32_t acc0 = tmem + (uint32_t)((k & 1) * NB);
+            uint32_t acc = 0;
+            for (int dz = 0; dz < 3; ++dz) {
+                const int zp = Flip ? z + 1 - dz : z - 1 + dz;
+                const uint32_t pa = (ring + (uint32_t)(zp & (kTcRing - 1)) * plane_bytes) >> 4;
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+                    const int off = Flip ? (2 - q / 3) * kTcHX + (2 - q % 3) : (q / 3) * kTcHX + q % 3;
+                    const uint32_t wa = (wbase + (uint32_t)(dz * 9 + q) * tap_bytes) >> 4;
+                    for (int j = 0; j < kb / 2; ++j) {
+                        const uint64_t ad = ad0 | (uint64_t)(pa + off + (uint32_t)j * (2 * kGroup >> 4));
+                        const uint64_t bd = bd0 | (uint64_t)(wa + (uint32_t)j * 16u);
+                        asm volatile(
+                            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc0),
+                            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                            : "memory");
+                        acc = 1;
+                    }
+                }
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                             smem_u32(&bars[k & 1]))
+                         : "memory");
+        }
+        __syncwarp();
+        // the MMAs of plane z - 1 are done: their lowest input plane's slot takes plane z + 2
+        if (k > 0) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[(k - 1) & 1]), ((k - 1) >> 1) & 1)) != 0;
+        if (ok && z + 1 < z1) load_plane(z + 2);
+        if (ok && k > 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            epilogue(z - 1);
+        }
     }
+    if (ok) {
+        const int k = z1 - 1 - z0;
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[k & 1]), (k >> 1) & 1)) != 0;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        if (ok) epilogue(z1 - 1);
+    }
+    if (!ok && lane == 0) atomicExch(a.status, 1);
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -361,71 +354,35 @@ __global__ void __launch_bounds__(kTcThreads) conv_fwd_tc_kernel(const ConvFwd a
     }
 }
 
-// ------------------------------------------------------------------ convolution: data gradient
-
-struct ConvBwdData {
-    const bf16* gp;     // [vox][cout] gradient of the pre-activation (ReLU mask applied), BF16
-    const bf16* wt;     // [27][cin][cout] transposed weights
-    float* dst1;        // [vox][c1] gradient of source 1 (overwritten)
-    int c1;
-    float* dst2;        // [vox][c2] gradient of source 2 (accumulated)
-    int c2;
-    int cout;
-    Dims d;
-};
-
-template <int CIN>
-__global__ void __launch_bounds__(128) conv_bwd_data_kernel(const ConvBwdData a)
+// Launch over every plane tile of the level.  NB = 32 where two such weight
+// sets fit an SM (K <= 32), else 16: more CTAs on the coarse levels, whose wide
+// layers have few voxels.  A chunk is at most 8 planes (two of its ten input
+// planes are read twice), fewer when the level has too few tiles for four CTAs
+// per SM.
+template <bool Flip>
+cudaError_t launch_conv_tc(ConvTc a, cudaStream_t st)
 {
-    const int lane = threadIdx.x & 31;
-    const int g = lane >> 2, t = lane & 3;
-    const int tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int total = a.d.nvox * a.d.batch;
-    const int v0 = tile * 16;
-    if (v0 >= total) return;
-    const int vA = v0 + g, vB = v0 + g + 8;
-    const VoxCoord cA = vox_coord(a.d, vA), cB = vox_coord(a.d, vB);
-    const int cout = a.cout;
-    float acc[CIN / 8][4];
-#pragma unroll
-    for (int j = 0; j < CIN / 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-    for (int tap = 0; tap < 27; ++tap) {
-        const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-        // the output voxel that reads v through this tap sits at v - offset
-        const int sA = shifted(a.d, cA, -dx, -dy, -dz);
-        const int sB = shifted(a.d, cB, -dx, -dy, -dz);
-        const bf16* wt = a.wt + (size_t)tap * CIN * cout;
-        for (int c = 0; c < cout; c += 16) {
-            uint32_t fa[4];
-            const int cols[4] = {c + 2 * t, c + 2 * t, c + 8 + 2 * t, c + 8 + 2 * t};
-            const int src[4] = {sA, sB, sA, sB};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) fa[q] = src[q] >= 0 ? ld_pair(a.gp + (size_t)src[q] * cout + cols[q]) : 0u;
-#pragma unroll
-            for (int j = 0; j < CIN / 8; ++j) {
-                const bf16* wr = wt + (size_t)(j * 8 + g) * cout + c;
-                const uint32_t fb[2] = {ld_pair(wr + 2 * t), ld_pair(wr + 8 + 2 * t)};
-                mma16816(acc[j], fa, fb);
-            }
-        }
+    static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<16, Flip>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kTcMaxSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(conv_tc_kernel<32, Flip>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcMaxSmem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
     }
-#pragma unroll
-    for (int j = 0; j < CIN / 8; ++j) {
-        const int ci = j * 8 + 2 * t;
-        const float r[4] = {acc[j][0], acc[j][1], acc[j][2], acc[j][3]};
-        const int vv[2] = {vA, vB};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            for (int e = 0; e < 2; ++e) {
-                const int cc = ci + e;
-                const float val = r[2 * h + e];
-                if (cc < a.c1)
-                    a.dst1[(size_t)vv[h] * a.c1 + cc] = val;
-                else
-                    a.dst2[(size_t)vv[h] * a.c2 + (cc - a.c1)] += val;
-            }
-        }
-    }
+    const int K = a.c1 + a.c2;
+    const int NB = a.n % 32 == 0 && K <= 32 ? 32 : 16;
+    if (K % 16 || a.n % 16 || a.c1 % 8 || tc_smem(K, NB) > kTcMaxSmem) return cudaErrorInvalidValue;
+    const int cols = ((a.d.nx + kTcX - 1) / kTcX) * ((a.d.ny + kTcY - 1) / kTcY) * a.d.batch;
+    const int zc = (int)((int64_t)cols * a.d.nz * (a.n / NB) / (4 * 152));
+    a.zc = std::min(std::max(zc, 1), std::min(8, a.d.nz));
+    const dim3 grid(cols * ((a.d.nz + a.zc - 1) / a.zc), a.n / NB);
+    if (NB == 32)
+        conv_tc_kernel<32, Flip><<<grid, kTcThreads, tc_smem(K, NB), st>>>(a);
+    else
+        conv_tc_kernel<16, Flip><<<grid, kTcThreads, tc_smem(K, NB), st>>>(a);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ convolution: weight gradient
@@ -437,90 +394,154 @@ struct ConvBwdW {
     const bf16* src2;   // [vox][c2]
     int c2;
     int cout;
+    int up1;            // src1 is held at half the resolution and read nearest (upsampling)
     float* gw;          // [27][cout][cin] (accumulated)
     Dims d;
-    int chunk;          // voxels per block
+    int tiles;          // voxel tiles of the level
 };
 
-constexpr int kWChunkSub = 32;  // voxels staged per shared-memory round
+// A block owns 16 output x 16 input channels (blockIdx.y) of all 27 taps and
+// walks 8 x 8 x 4 voxel tiles (blockIdx.x, grid stride).  A tile's gradient rows
+// and its activation rows with a one-voxel halo are copied into shared memory
+// once (cp.async, the next tile in flight) and serve all 27 taps: reading the
+// activations again for every tap made this 2291 us for a 16 -> 16 layer of
+// 8 x 64 x 64 x 32 voxels.  Warp w takes the nine taps of dz = w % 3 - 1 and half
+// w / 3 of the tile's voxels: per 16 voxels (two x runs of eight) one transposed
+// ldmatrix of the gradient is multiplied with nine of the shifted activations;
+// the 9 x 16 x 16 sums stay in registers (72 a thread) until the block's last
+// tile.  Rows are 32 bytes; their two 16-byte halves are swapped on every other
+// group of four voxels of a run, so that the eight rows of an ldmatrix hit
+// distinct banks at any x shift.
+constexpr int kWTx = 8, kWTy = 8, kWTz = 4, kWVox = kWTx * kWTy * kWTz;
+constexpr int kWHx = kWTx + 2, kWHy = kWTy + 2, kWHz = kWTz + 2, kWHalo = kWHx * kWHy * kWHz;
+constexpr int kWThreads = 192;
+constexpr int kWStage = (kWVox + kWHalo) * 32;  // bytes: gradient rows, then activation rows
+constexpr int kWSmem = 2 * kWStage;
+constexpr int kWBlocksPerSM = 3;
 
-// grid = (voxel chunks, 27 taps); 8 warps share the (cout/16) x (cin/8) tiles.
-__global__ void __launch_bounds__(256) conv_bwd_w_kernel(const ConvBwdW a)
+__device__ __forceinline__ void ldm_x4_trans(uint32_t addr, uint32_t r[4])
 {
-    extern __shared__ unsigned char smem_raw[];
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+__global__ void __launch_bounds__(kWThreads, kWBlocksPerSM) conv_bwd_w_kernel(const ConvBwdW a)
+{
+    extern __shared__ __align__(128) unsigned char w_smem[];
+    const uint32_t smem0 = smem_u32(w_smem);
     const int cin = a.c1 + a.c2;
-    const int cout = a.cout;
-    bf16* Gs = reinterpret_cast<bf16*>(smem_raw);  // [kWChunkSub][cout]
-    bf16* Xs = Gs + kWChunkSub * cout;              // [kWChunkSub][cin]
-    __shared__ int srow[kWChunkSub];                // tap-shifted source voxel of each staged row
-    const int tap = blockIdx.y;
-    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-    const int total = a.d.nvox * a.d.batch;
-    const int vbeg = blockIdx.x * a.chunk;
-    const int vend = min(vbeg + a.chunk, total);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    const int mt = cout / 16, nt = cin / 8, tiles = mt * nt;
-    constexpr int kMaxTiles = 6;  // per warp: up to 48 tiles / 8 warps (cout 64 x cin 96 -> 4 x 12)
-    float acc[kMaxTiles][4];
+    const int nci = cin / 16;
+    const int co0 = ((int)blockIdx.y / nci) * 16, ci0 = ((int)blockIdx.y % nci) * 16;
+    const bool first = ci0 < a.c1;
+    const bf16* xs = first ? a.src1 + ci0 : a.src2 + (ci0 - a.c1);
+    const int xc = first ? a.c1 : a.c2;
+    const bool up = first && a.up1;
+    const Dims d = a.d;
+    const int tx = (d.nx + kWTx - 1) / kWTx, ty = (d.ny + kWTy - 1) / kWTy, tz = (d.nz + kWTz - 1) / kWTz;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+    // copies of one tile into stage s; rows outside the volume (and the
+    // gradient of voxels beyond a ragged tile's end) are zero
+    auto load_tile = [&](int t, int s) {
+        const int x0 = (t % tx) * kWTx;
+        int r = t / tx;
+        const int y0 = (r % ty) * kWTy;
+        r /= ty;
+        const int z0 = (r % tz) * kWTz, batch = r / tz, vb = batch * d.nvox;
+        const uint32_t G = smem0 + (uint32_t)s * kWStage, X = G + kWVox * 32;
+        for (int i = tid; i < kWVox * 2; i += kWThreads) {
+            const int c = i & 1, v = i >> 1;
+            const int x = x0 + v % kWTx, y = y0 + (v / kWTx) % kWTy, z = z0 + v / (kWTx * kWTy);
+            const bool ok = x < d.nx && y < d.ny && z < d.nz;
+            const bf16* src = ok ? a.gp + (size_t)(vb + x + d.nx * (y + d.ny * z)) * a.cout + co0 + 8 * c : a.gp;
+            cp_async16(G + v * 32 + ((c ^ ((v >> 2) & 1)) << 4), src, ok);
+        }
+        for (int i = tid; i < kWHalo * 2; i += kWThreads) {
+            const int c = i & 1, v = i >> 1;
+            const int hx = v % kWHx, hy = (v / kWHx) % kWHy, hz = v / (kWHx * kWHy);
+            int x = x0 - 1 + hx, y = y0 - 1 + hy;
+            const int z = z0 - 1 + hz;
+            x = x < 0 ? x + d.nx : (x >= d.nx ? x - d.nx : x);
+            y = y < 0 ? y + d.ny : (y >= d.ny ? y - d.ny : y);
+            const bool ok = x < d.nx && y < d.ny && z >= 0 && z < d.nz;
+            const int sv = up ? batch * (d.nvox >> 3) + (x >> 1) + (d.nx >> 1) * ((y >> 1) + (d.ny >> 1) * (z >> 1))
+                              : vb + x + d.nx * (y + d.ny * z);
+            const bf16* src = ok ? xs + (size_t)sv * xc + 8 * c : xs;
+            cp_async16(X + v * 32 + ((c ^ ((hx >> 2) & 1)) << 4), src, ok);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+
+    const int dz = warp % 3, half = warp / 3;
+    const int mi = lane >> 3, r8 = lane & 7;
+    // A[co][v] = G[v][co]: matrices (v 0-7, co 0-7), (v 0-7, co 8-15), (v 8-15, co 0-7), (v 8-15, co 8-15)
+    const uint32_t laneA = (uint32_t)(((mi >> 1) * 8 + r8) * 32 + (((mi & 1) ^ ((r8 >> 2) & 1)) << 4));
+    // B[v][ci] = X[v + tap][ci]: (v 0-7, ci 0-7), (v 8-15, ci 0-7), (v 0-7, ci 8-15), (v 8-15, ci 8-15)
+    uint32_t laneB[3];
 #pragma unroll
-    for (int k = 0; k < kMaxTiles; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.f;
-    for (int s0 = vbeg; s0 < vend; s0 += kWChunkSub) {
-        __syncthreads();
-        if (threadIdx.x < kWChunkSub) {
-            const int v = s0 + threadIdx.x;
-            srow[threadIdx.x] = v < vend ? shifted(a.d, vox_coord(a.d, v), dx, dy, dz) : -1;
-        }
-        // 16-byte groups of 8 channels (cout, c1 and c2 are multiples of 8)
-        const int cg = cout >> 3;
-        for (int e = threadIdx.x; e < kWChunkSub * cg; e += blockDim.x) {
-            const int r = e / cg, q = e - r * cg;
-            const int v = s0 + r;
-            uint4 gv = make_uint4(0u, 0u, 0u, 0u);
-            if (v < vend) gv = __ldg(reinterpret_cast<const uint4*>(a.gp + (size_t)v * cout) + q);
-            reinterpret_cast<uint4*>(Gs)[e] = gv;
-        }
-        __syncthreads();  // srow
-        const int ig = cin >> 3, ig1 = a.c1 >> 3;
-        for (int e = threadIdx.x; e < kWChunkSub * ig; e += blockDim.x) {
-            const int r = e / ig, q = e - r * ig;
-            const int sv = srow[r];
-            uint4 xv = make_uint4(0u, 0u, 0u, 0u);
-            if (sv >= 0)
-                xv = q < ig1 ? __ldg(reinterpret_cast<const uint4*>(a.src1 + (size_t)sv * a.c1) + q)
-                             : __ldg(reinterpret_cast<const uint4*>(a.src2 + (size_t)sv * a.c2) + (q - ig1));
-            reinterpret_cast<uint4*>(Xs)[e] = xv;
-        }
-        __syncthreads();
-        for (int kk = 0; kk < kWChunkSub; kk += 16) {
+    for (int dx = 0; dx < 3; ++dx)
+        laneB[dx] = (uint32_t)((mi & 1) * (kWHx * 32) + (r8 + dx) * 32 + (((mi >> 1) ^ (((r8 + dx) >> 2) & 1)) << 4));
+    float acc[9][2][4];
 #pragma unroll
-            for (int q = 0; q < kMaxTiles; ++q) {
-                const int tile = warp + 8 * q;
-                if (tile >= tiles) break;
-                const int m0 = (tile / nt) * 16, n0 = (tile % nt) * 8;
-                // A[co][v] = G[v][co]; B[v][ci] = X[v][ci]
-                uint32_t fa[4], fb[2];
-                fa[0] = pack_raw(Gs[(kk + 2 * t) * cout + m0 + g], Gs[(kk + 2 * t + 1) * cout + m0 + g]);
-                fa[1] = pack_raw(Gs[(kk + 2 * t) * cout + m0 + g + 8], Gs[(kk + 2 * t + 1) * cout + m0 + g + 8]);
-                fa[2] = pack_raw(Gs[(kk + 8 + 2 * t) * cout + m0 + g], Gs[(kk + 9 + 2 * t) * cout + m0 + g]);
-                fa[3] = pack_raw(Gs[(kk + 8 + 2 * t) * cout + m0 + g + 8], Gs[(kk + 9 + 2 * t) * cout + m0 + g + 8]);
-                fb[0] = pack_raw(Xs[(kk + 2 * t) * cin + n0 + g], Xs[(kk + 2 * t + 1) * cin + n0 + g]);
-                fb[1] = pack_raw(Xs[(kk + 8 + 2 * t) * cin + n0 + g], Xs[(kk + 9 + 2 * t) * cin + n0 + g]);
-                mma16816(acc[q], fa, fb);
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) acc[q][h][0] = acc[q][h][1] = acc[q][h][2] = acc[q][h][3] = 0.f;
+
+    int t = blockIdx.x;
+    if (t < a.tiles) load_tile(t, 0);
+    for (int s = 0; t < a.tiles; t += gridDim.x, s ^= 1) {
+        if (t + (int)gridDim.x < a.tiles) {
+            load_tile(t + gridDim.x, s ^ 1);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        }
+        __syncthreads();
+        const uint32_t G = smem0 + (uint32_t)s * kWStage, X = G + kWVox * 32;
+#pragma unroll 2
+        for (int k = 0; k < 8; ++k) {  // 16 voxels: rows y = 2 j, 2 j + 1 of layer z
+            const int z = 2 * half + (k >> 2), j = k & 3;
+            uint32_t fa[4];
+            ldm_x4_trans(G + laneA + (uint32_t)((z * kWTy + 2 * j) * kWTx * 32), fa);
+            const uint32_t xb = X + (uint32_t)(((z + dz) * kWHy + 2 * j) * (kWHx * 32));
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                uint32_t fb[4];
+                ldm_x4_trans(xb + laneB[q % 3] + (uint32_t)(q / 3) * (kWHx * 32), fb);
+                mma16816(acc[q][0], fa, fb);
+                mma16816(acc[q][1], fa, fb + 2);
             }
         }
+        __syncthreads();
     }
-    float* gw = a.gw + (size_t)tap * cout * cin;
+
+    // the two voxel halves meet in shared memory, then one add per value and block
+    float* red = reinterpret_cast<float*>(w_smem) + (size_t)dz * 72 * 32 + lane;
+    if (half == 1) {
 #pragma unroll
-    for (int q = 0; q < kMaxTiles; ++q) {
-        const int tile = warp + 8 * q;
-        if (tile >= tiles) break;
-        const int m0 = (tile / nt) * 16, n0 = (tile % nt) * 8;
-        atomicAdd(&gw[(size_t)(m0 + g) * cin + n0 + 2 * t], acc[q][0]);
-        atomicAdd(&gw[(size_t)(m0 + g) * cin + n0 + 2 * t + 1], acc[q][1]);
-        atomicAdd(&gw[(size_t)(m0 + g + 8) * cin + n0 + 2 * t], acc[q][2]);
-        atomicAdd(&gw[(size_t)(m0 + g + 8) * cin + n0 + 2 * t + 1], acc[q][3]);
+        for (int q = 0; q < 9; ++q)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) red[(q * 8 + i) * 32] = acc[q][i >> 2][i & 3];
     }
+    __syncthreads();
+    if (half == 1) return;
+    const int g = lane >> 2, c2 = 2 * (lane & 3);
+    const bool vec = (reinterpret_cast<uintptr_t>(a.gw) & 7) == 0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {  // i: n half (4), row half (2)
+            const float v0 = acc[q][i >> 2][i & 3] + red[(q * 8 + i) * 32];
+            const float v1 = acc[q][i >> 2][(i & 3) + 1] + red[(q * 8 + i + 1) * 32];
+            float* dst = a.gw + (size_t)((dz * 9 + q) * a.cout + co0 + g + ((i & 2) ? 8 : 0)) * cin + ci0 + (i >> 2) * 8 + c2;
+            if (vec) {
+                atomicAdd(reinterpret_cast<float2*>(dst), make_float2(v0, v1));
+            } else {
+                atomicAdd(dst, v0);
+                atomicAdd(dst + 1, v1);
+            }
+        }
 }
 
 // Gradient of the pre-activation, once per layer: gp = BF16(gout masked by
@@ -603,22 +624,6 @@ __global__ void pool_bwd_kernel(const float* __restrict__ gdst, float* __restric
         const int x = r % fine.nx, y = (r / fine.nx) % fine.ny, z = r / (fine.nx * fine.ny);
         const size_t cv = (size_t)b * (fine.nvox / 8) + x / 2 + cx * (y / 2 + cy * (z / 2));
         gsrc[i] += 0.125f * gdst[cv * C + c];
-    }
-}
-
-// dst (fine) = src (coarse) nearest
-__global__ void up_fwd_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, Dims fine, int C)
-{
-    const int cx = fine.nx / 2, cy = fine.ny / 2;
-    const int64_t total = (int64_t)fine.nvox * fine.batch * C;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const int64_t v = i / C;
-        const int b = (int)(v / fine.nvox);
-        const int r = (int)(v - (int64_t)b * fine.nvox);
-        const int x = r % fine.nx, y = (r / fine.nx) % fine.ny, z = r / (fine.nx * fine.ny);
-        const size_t cv = (size_t)b * (fine.nvox / 8) + x / 2 + cx * (y / 2 + cy * (z / 2));
-        dst[i] = src[cv * C + c];
     }
 }
 
@@ -789,7 +794,7 @@ struct nh_unet {
     size_t ws_bytes = 0;
     size_t need = 0;
     // offsets into the workspace
-    size_t wbf, wt[kLayers], x, act[kLayers], pool_[3], up_[3], grad_a, grad_b, grad_skip[3], gd1, gprep, status;
+    size_t wbf, wt[kLayers], x, act[kLayers], pool_[3], grad_a, grad_b, grad_skip[3], gd1, gprep, status;
     std::string err;
 };
 
@@ -820,11 +825,9 @@ void plan(nh_unet* u)
     const int level_of[kLayers] = {0, 0, 1, 1, 2, 2, 3, 3, 2, 2, 1, 1, 0, 0};
     for (int l = 0; l < kLayers; ++l)
         u->act[l] = take((size_t)u->lv[level_of[l]].nvox * u->batch * kConv[l].cout * sizeof(bf16));
-    // pooled inputs of levels 1..3 and upsampled inputs of decoder levels 2..0
+    // pooled inputs of levels 1..3
     const int pool_c[3] = {16, 16, 32};
     for (int k = 0; k < 3; ++k) u->pool_[k] = take((size_t)u->lv[k + 1].nvox * u->batch * pool_c[k] * sizeof(bf16));
-    const int up_c[3] = {64, 32, 16};
-    for (int k = 0; k < 3; ++k) u->up_[k] = take((size_t)u->lv[2 - k].nvox * u->batch * up_c[k] * sizeof(bf16));
     // gradient scratch: two ping-pong buffers large enough for any [vox][96] level-0..3 tensor,
     // three skip-gradient buffers (e1, e2, e3) and the head-input gradient
     size_t gmax = 0;
@@ -848,49 +851,30 @@ T* P(nh_unet* u, size_t off)
     return reinterpret_cast<T*>(u->ws + off);
 }
 
-cudaError_t conv_fwd(nh_unet* u, int l, int level, const bf16* s1, int c1, const bf16* s2, int c2,
+// Forward conv layer l; up1: source 1 is the coarser level's output, read upsampled.
+cudaError_t conv_fwd(nh_unet* u, int l, int level, const bf16* s1, int c1, const bf16* s2, int c2, bool up1,
                      const float* params, cudaStream_t st)
 {
-    ConvFwd a;
+    ConvTc a{};
     a.src1 = s1;
     a.c1 = c1;
     a.src2 = s2;
     a.c2 = c2;
+    a.up1 = up1;
     a.w = P<bf16>(u, u->wbf) + layer_offset(l);
+    a.n = kConv[l].cout;
     a.bias = params + layer_offset(l) + 27LL * kConv[l].cin * kConv[l].cout;
-    a.dst = P<bf16>(u, u->act[l]);
+    a.out = P<bf16>(u, u->act[l]);
     a.d = u->lv[level];
-    a.relu = 1;
     a.status = P<int>(u, u->status);
-    static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(conv_fwd_tc_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTcSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv_fwd_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv_fwd_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    const int cin = c1 + c2;
-    if (cin % 16 || cin > kTcMaxCin || kConv[l].cout > kTcMaxCout) return cudaErrorInvalidValue;
-    const int blocks = (a.d.nvox * a.d.batch + kTcM - 1) / kTcM;
-    a.tps = tc_taps_per_stage(cin, kConv[l].cout);
-    const size_t smem = 2 * (size_t)a.tps * (kTcM + kConv[l].cout) * cin * sizeof(bf16) + 64;
-    switch (kConv[l].cout) {
-    case 16: conv_fwd_tc_kernel<16><<<blocks, kTcThreads, smem, st>>>(a); break;
-    case 32: conv_fwd_tc_kernel<32><<<blocks, kTcThreads, smem, st>>>(a); break;
-    default: conv_fwd_tc_kernel<64><<<blocks, kTcThreads, smem, st>>>(a); break;
-    }
-    return cudaGetLastError();
+    return launch_conv_tc<false>(a, st);
 }
 
 // Backward of conv layer l: gout (FP32 [vox][cout]) -> data gradient into
 // dst1 (c1 channels, overwritten) and dst2 (c2, accumulated); weight and bias
 // gradients accumulated into grad.
 cudaError_t conv_bwd(nh_unet* u, int l, int level, const float* gout, const bf16* s1, int c1, const bf16* s2, int c2,
-                     float* dst1, float* dst2, float* grad, bool need_data, cudaStream_t st)
+                     bool up1, float* dst1, float* dst2, float* grad, bool need_data, cudaStream_t st)
 {
     const Dims d = u->lv[level];
     const int total = d.nvox * d.batch;
@@ -908,32 +892,33 @@ cudaError_t conv_bwd(nh_unet* u, int l, int level, const float* gout, const bf16
     w.src2 = s2;
     w.c2 = c2;
     w.cout = cout;
+    w.up1 = up1;
     w.gw = grad + layer_offset(l);
     w.d = d;
-    w.chunk = 1024;
-    dim3 grid((total + w.chunk - 1) / w.chunk, 27);
-    const size_t smem = (size_t)kWChunkSub * (cin + cout) * sizeof(bf16);
-    conv_bwd_w_kernel<<<grid, 256, smem, st>>>(w);
+    w.tiles = ((d.nx + kWTx - 1) / kWTx) * ((d.ny + kWTy - 1) / kWTy) * ((d.nz + kWTz - 1) / kWTz) * d.batch;
+    static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
+    if (!attr_set) {
+        e = cudaFuncSetAttribute(conv_bwd_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    // one wave of resident blocks over the channel pairs; each walks its share of the tiles
+    const int pairs = (cin / 16) * (cout / 16);
+    dim3 grid(std::min(w.tiles, std::max(1, kWBlocksPerSM * 152 / pairs)), pairs);
+    conv_bwd_w_kernel<<<grid, kWThreads, kWSmem, st>>>(w);
     e = cudaGetLastError();
     if (e != cudaSuccess || !need_data) return e;
-    ConvBwdData b;
-    b.gp = gp;
-    b.wt = P<bf16>(u, u->wt[l]);
-    b.dst1 = dst1;
-    b.c1 = c1;
-    b.dst2 = dst2;
-    b.c2 = c2;
-    b.cout = cout;
+    ConvTc b{};
+    b.src1 = gp;
+    b.c1 = cout;
+    b.w = P<bf16>(u, u->wt[l]);
+    b.n = cin;
     b.d = d;
-    const int blocks = (total / 16 + 3) / 4;
-    switch (cin) {
-    case 16: conv_bwd_data_kernel<16><<<blocks, 128, 0, st>>>(b); break;
-    case 32: conv_bwd_data_kernel<32><<<blocks, 128, 0, st>>>(b); break;
-    case 48: conv_bwd_data_kernel<48><<<blocks, 128, 0, st>>>(b); break;
-    case 64: conv_bwd_data_kernel<64><<<blocks, 128, 0, st>>>(b); break;
-    default: conv_bwd_data_kernel<96><<<blocks, 128, 0, st>>>(b); break;
-    }
-    return cudaGetLastError();
+    b.dst1 = dst1;
+    b.n1 = c1;
+    b.dst2 = dst2;
+    b.status = P<int>(u, u->status);
+    return launch_conv_tc<true>(b, st);
 }
 
 }  // namespace
@@ -1028,27 +1013,23 @@ int nh_unet_forward(nh_unet* u, const float* params, const float* n_ansatz, cons
     UNET_CUDA(u, cudaGetLastError());
     auto act = [&](int l) { return P<bf16>(u, u->act[l]); };
     auto pool = [&](int k) { return P<bf16>(u, u->pool_[k]); };
-    auto upb = [&](int k) { return P<bf16>(u, u->up_[k]); };
-    UNET_CUDA(u, conv_fwd(u, ENC1A, 0, P<bf16>(u, u->x), 16, nullptr, 0, params, st));
-    UNET_CUDA(u, conv_fwd(u, ENC1B, 0, act(ENC1A), 16, nullptr, 0, params, st));
+    UNET_CUDA(u, conv_fwd(u, ENC1A, 0, P<bf16>(u, u->x), 16, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, ENC1B, 0, act(ENC1A), 16, nullptr, 0, false, params, st));
     pool_fwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 16), 256, 0, st>>>(act(ENC1B), pool(0), u->lv[0], 16);
-    UNET_CUDA(u, conv_fwd(u, ENC2A, 1, pool(0), 16, nullptr, 0, params, st));
-    UNET_CUDA(u, conv_fwd(u, ENC2B, 1, act(ENC2A), 16, nullptr, 0, params, st));
+    UNET_CUDA(u, conv_fwd(u, ENC2A, 1, pool(0), 16, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, ENC2B, 1, act(ENC2A), 16, nullptr, 0, false, params, st));
     pool_fwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 16), 256, 0, st>>>(act(ENC2B), pool(1), u->lv[1], 16);
-    UNET_CUDA(u, conv_fwd(u, ENC3A, 2, pool(1), 16, nullptr, 0, params, st));
-    UNET_CUDA(u, conv_fwd(u, ENC3B, 2, act(ENC3A), 32, nullptr, 0, params, st));
+    UNET_CUDA(u, conv_fwd(u, ENC3A, 2, pool(1), 16, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, ENC3B, 2, act(ENC3A), 32, nullptr, 0, false, params, st));
     pool_fwd_kernel<<<grid_for((int64_t)u->lv[3].nvox * u->batch * 32), 256, 0, st>>>(act(ENC3B), pool(2), u->lv[2], 32);
-    UNET_CUDA(u, conv_fwd(u, BOTA, 3, pool(2), 32, nullptr, 0, params, st));
-    UNET_CUDA(u, conv_fwd(u, BOTB, 3, act(BOTA), 64, nullptr, 0, params, st));
-    up_fwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 64), 256, 0, st>>>(act(BOTB), upb(0), u->lv[2], 64);
-    UNET_CUDA(u, conv_fwd(u, DEC3A, 2, upb(0), 64, act(ENC3B), 32, params, st));
-    UNET_CUDA(u, conv_fwd(u, DEC3B, 2, act(DEC3A), 32, nullptr, 0, params, st));
-    up_fwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 32), 256, 0, st>>>(act(DEC3B), upb(1), u->lv[1], 32);
-    UNET_CUDA(u, conv_fwd(u, DEC2A, 1, upb(1), 32, act(ENC2B), 16, params, st));
-    UNET_CUDA(u, conv_fwd(u, DEC2B, 1, act(DEC2A), 16, nullptr, 0, params, st));
-    up_fwd_kernel<<<grid_for((int64_t)u->lv[0].nvox * u->batch * 16), 256, 0, st>>>(act(DEC2B), upb(2), u->lv[0], 16);
-    UNET_CUDA(u, conv_fwd(u, DEC1A, 0, upb(2), 16, act(ENC1B), 16, params, st));
-    UNET_CUDA(u, conv_fwd(u, DEC1B, 0, act(DEC1A), 16, nullptr, 0, params, st));
+    UNET_CUDA(u, conv_fwd(u, BOTA, 3, pool(2), 32, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, BOTB, 3, act(BOTA), 64, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, DEC3A, 2, act(BOTB), 64, act(ENC3B), 32, true, params, st));
+    UNET_CUDA(u, conv_fwd(u, DEC3B, 2, act(DEC3A), 32, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, DEC2A, 1, act(DEC3B), 32, act(ENC2B), 16, true, params, st));
+    UNET_CUDA(u, conv_fwd(u, DEC2B, 1, act(DEC2A), 16, nullptr, 0, false, params, st));
+    UNET_CUDA(u, conv_fwd(u, DEC1A, 0, act(DEC2B), 16, act(ENC1B), 16, true, params, st));
+    UNET_CUDA(u, conv_fwd(u, DEC1B, 0, act(DEC1A), 16, nullptr, 0, false, params, st));
     head_kernel<<<grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st>>>(act(DEC1B), n_ansatz, params + head_offset(), n_out,
                                                                         nullptr, nullptr, nullptr, nullptr, d0);
     UNET_CUDA(u, cudaGetLastError());
@@ -1066,7 +1047,6 @@ int nh_unet_backward(nh_unet* u, const float* params, const float* n_ansatz, con
     UNET_CUDA(u, cudaMemsetAsync(loss, 0, sizeof(float), st));
     auto act = [&](int l) { return P<bf16>(u, u->act[l]); };
     auto pool = [&](int k) { return P<bf16>(u, u->pool_[k]); };
-    auto upb = [&](int k) { return P<bf16>(u, u->up_[k]); };
     float* ga = P<float>(u, u->grad_a);
     float* gb = P<float>(u, u->grad_b);
     float* gskip[3] = {P<float>(u, u->grad_skip[0]), P<float>(u, u->grad_skip[1]), P<float>(u, u->grad_skip[2])};
@@ -1075,41 +1055,41 @@ int nh_unet_backward(nh_unet* u, const float* params, const float* n_ansatz, con
         act(DEC1B), n_ansatz, params + head_offset(), nullptr, target, gd1, grad + head_offset(), loss, d0);
     UNET_CUDA(u, cudaGetLastError());
     // decoder level 0: dec1b <- gd1, dec1a <- ga  (sources [up2 | e1])
-    UNET_CUDA(u, conv_bwd(u, DEC1B, 0, gd1, act(DEC1A), 16, nullptr, 0, ga, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, DEC1B, 0, gd1, act(DEC1A), 16, nullptr, 0, false, ga, nullptr, grad, true, st));
     UNET_CUDA(u, cudaMemsetAsync(gskip[0], 0, (size_t)d0.nvox * d0.batch * 16 * sizeof(float), st));
-    UNET_CUDA(u, conv_bwd(u, DEC1A, 0, ga, upb(2), 16, act(ENC1B), 16, gb, gskip[0], grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, DEC1A, 0, ga, act(DEC2B), 16, act(ENC1B), 16, true, gb, gskip[0], grad, true, st));
     up_bwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 16), 256, 0, st>>>(gb, ga, u->lv[0], 16);  // -> g(dec2b)
     UNET_CUDA(u, cudaGetLastError());
     // decoder level 1
-    UNET_CUDA(u, conv_bwd(u, DEC2B, 1, ga, act(DEC2A), 16, nullptr, 0, gb, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, DEC2B, 1, ga, act(DEC2A), 16, nullptr, 0, false, gb, nullptr, grad, true, st));
     UNET_CUDA(u, cudaMemsetAsync(gskip[1], 0, (size_t)u->lv[1].nvox * u->batch * 16 * sizeof(float), st));
-    UNET_CUDA(u, conv_bwd(u, DEC2A, 1, gb, upb(1), 32, act(ENC2B), 16, ga, gskip[1], grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, DEC2A, 1, gb, act(DEC3B), 32, act(ENC2B), 16, true, ga, gskip[1], grad, true, st));
     up_bwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 32), 256, 0, st>>>(ga, gb, u->lv[1], 32);  // -> g(dec3b)
     UNET_CUDA(u, cudaGetLastError());
     // decoder level 2
-    UNET_CUDA(u, conv_bwd(u, DEC3B, 2, gb, act(DEC3A), 32, nullptr, 0, ga, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, DEC3B, 2, gb, act(DEC3A), 32, nullptr, 0, false, ga, nullptr, grad, true, st));
     UNET_CUDA(u, cudaMemsetAsync(gskip[2], 0, (size_t)u->lv[2].nvox * u->batch * 32 * sizeof(float), st));
-    UNET_CUDA(u, conv_bwd(u, DEC3A, 2, ga, upb(0), 64, act(ENC3B), 32, gb, gskip[2], grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, DEC3A, 2, ga, act(BOTB), 64, act(ENC3B), 32, true, gb, gskip[2], grad, true, st));
     up_bwd_kernel<<<grid_for((int64_t)u->lv[3].nvox * u->batch * 64), 256, 0, st>>>(gb, ga, u->lv[2], 64);  // -> g(botb)
     UNET_CUDA(u, cudaGetLastError());
     // bottleneck
-    UNET_CUDA(u, conv_bwd(u, BOTB, 3, ga, act(BOTA), 64, nullptr, 0, gb, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, BOTA, 3, gb, pool(2), 32, nullptr, 0, ga, nullptr, grad, true, st));   // ga = g(pool2 out)
+    UNET_CUDA(u, conv_bwd(u, BOTB, 3, ga, act(BOTA), 64, nullptr, 0, false, gb, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, BOTA, 3, gb, pool(2), 32, nullptr, 0, false, ga, nullptr, grad, true, st));   // ga = g(pool2 out)
     pool_bwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 32), 256, 0, st>>>(ga, gskip[2], u->lv[2], 32);
     UNET_CUDA(u, cudaGetLastError());
     // encoder level 2 (e3 gradient complete in gskip[2])
-    UNET_CUDA(u, conv_bwd(u, ENC3B, 2, gskip[2], act(ENC3A), 32, nullptr, 0, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, ENC3A, 2, ga, pool(1), 16, nullptr, 0, gb, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, ENC3B, 2, gskip[2], act(ENC3A), 32, nullptr, 0, false, ga, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, ENC3A, 2, ga, pool(1), 16, nullptr, 0, false, gb, nullptr, grad, true, st));
     pool_bwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 16), 256, 0, st>>>(gb, gskip[1], u->lv[1], 16);
     UNET_CUDA(u, cudaGetLastError());
     // encoder level 1
-    UNET_CUDA(u, conv_bwd(u, ENC2B, 1, gskip[1], act(ENC2A), 16, nullptr, 0, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, ENC2A, 1, ga, pool(0), 16, nullptr, 0, gb, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, ENC2B, 1, gskip[1], act(ENC2A), 16, nullptr, 0, false, ga, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, ENC2A, 1, ga, pool(0), 16, nullptr, 0, false, gb, nullptr, grad, true, st));
     pool_bwd_kernel<<<grid_for((int64_t)d0.nvox * d0.batch * 16), 256, 0, st>>>(gb, gskip[0], u->lv[0], 16);
     UNET_CUDA(u, cudaGetLastError());
     // encoder level 0 (the input needs no gradient)
-    UNET_CUDA(u, conv_bwd(u, ENC1B, 0, gskip[0], act(ENC1A), 16, nullptr, 0, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, ENC1A, 0, ga, P<bf16>(u, u->x), 16, nullptr, 0, nullptr, nullptr, grad, false, st));
+    UNET_CUDA(u, conv_bwd(u, ENC1B, 0, gskip[0], act(ENC1A), 16, nullptr, 0, false, ga, nullptr, grad, true, st));
+    UNET_CUDA(u, conv_bwd(u, ENC1A, 0, ga, P<bf16>(u, u->x), 16, nullptr, 0, false, nullptr, nullptr, grad, false, st));
     return NH_OK;
 }
 

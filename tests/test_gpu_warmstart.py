@@ -307,3 +307,20 @@ def test_trained_network_saves_relaxation_steps(env):
     # accumulation); 0.75 leaves room for that and still asks for a clear gain
     assert res["median_rms_prediction_vs_relaxed"] < 0.75 * res["median_rms_ansatz_vs_relaxed"]
     assert res["step_ratio"] < 0.98
+
+
+@pytest.mark.parametrize("B,dims", [(3, (16, 48, 32)), (2, (40, 32, 32)), (4, (72, 16, 16)), (8, (16, 32, 8)),
+                                    (1, (24, 128, 16))])
+def test_convolution_tiles_at_ragged_sizes(env, B, dims):
+    """Level sizes that fill, split and leave unfinished the convolutions' plane
+    tiles (8 x 16), their chunks of planes and the weight gradient's 8 x 8 x 4
+    tiles, down to a coarsest level of 2 x 2 x 1: same oracle and bounds as
+    test_gradients_match_bf16_storage_oracle."""
+    torch, nh, ws, U = env
+    flat, n_ans, target, scal = _problem(B=B, nx=dims[0], ny=dims[1], nz=dims[2], seed=4, smooth_target=True)
+    loss_e, grad_e, npred_e = _oracle(U, flat, n_ans, target, scal, dims, bf16_storage=True)
+    loss, g, npred = _gpu_loss_grad(torch, nh, flat, n_ans, scal, target, dims)
+    rows = _per_layer(U, g, grad_e)
+    assert abs(loss - loss_e) / loss_e < 1e-3
+    assert np.linalg.norm(npred - npred_e) / np.linalg.norm(npred_e - n_ans) < 1e-2
+    assert all(w < 3e-2 and b < 3e-2 for _, w, b in rows), rows
