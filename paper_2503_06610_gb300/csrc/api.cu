@@ -552,22 +552,7 @@ int enqueue_fd(nh_ctx* c, cudaStream_t st)
     return enqueue_force_only<Real>(c, st, true);
 }
 
-template <typename Real>
-int enqueue_predict_correct(nh_ctx* c, cudaStream_t st)
-{
-    auto a = fd_chan<Real>(c);
-    if (c->fd_fused) {
-        int r = timed(c, NH_KCLASS_FD_PREDICT, st, [&] { return launch_fd_fused_a<Real>(a, a.n, a.nP, st); },
-                      "fd_fused");
-        if (r) return r;
-        return cudaMemcpyAsync(a.n, a.nP, 3 * (size_t)c->N * sizeof(Real), cudaMemcpyDeviceToDevice, st) == cudaSuccess
-                   ? NH_OK
-                   : fail(c, NH_ECUDA, "copy of the relaxed director");
-    }
-    return enqueue_predict_correct_sites<Real>(c, a, st);
-}
-
-// Relaxation with the fused kernel, alternating n -> nP -> n; an odd count
+// Relaxation with the fused kernel at rest, alternating n -> nP -> n; an odd count
 // ends with one copy back into n.
 template <typename Real>
 int relax_fused(nh_ctx* c, int64_t steps, cudaStream_t st)
@@ -576,8 +561,8 @@ int relax_fused(nh_ctx* c, int64_t steps, cudaStream_t st)
     for (int64_t k = 0; k < steps; ++k) {
         const bool even = (k & 1) == 0;
         int r = timed(c, NH_KCLASS_FD_PREDICT, st,
-                      [&] { return even ? launch_fd_fused_a<Real>(a, a.n, a.nP, st) : launch_fd_fused_a<Real>(a, a.nP, a.n, st); },
-                      "fd_fused");
+                      [&] { return even ? launch_relax<Real>(a, a.n, a.nP, st) : launch_relax<Real>(a, a.nP, a.n, st); },
+                      "relax");
         if (r) return r;
     }
     if (steps & 1) NH_CUDA(c, cudaMemcpyAsync(a.n, a.nP, 3 * (size_t)c->N * sizeof(Real), cudaMemcpyDeviceToDevice, st));
@@ -953,11 +938,10 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
         fused = fused && c->fd_fused;
         frank3 = frank3 || c->p.frank3;
     }
-    if (fused) {
-        // stages == 4: full FD update (A: n -> nP, B: nP -> F and n); stages == 2: one relaxation step (A, copy back)
+    if (fused) {  // full FD update (A: n -> nP, B: nP -> F and n)
         const int fstages[2] = {0, 1};
         const int classes[2] = {NH_KCLASS_FD_PREDICT, NH_KCLASS_STRESS};
-        for (int k = 0; k < (stages == 4 ? 2 : 1); ++k) {
+        for (int k = 0; k < 2; ++k) {
             for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
                 batch.count = std::min(kMaxBatch, n - g0);
                 for (int j = 0; j < batch.count; ++j) batch.ch[j] = fd_chan<Real>(b->ctxs[g0 + j]);
@@ -967,12 +951,6 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
                 if (r) return r;
             }
         }
-        if (stages != 4)
-            for (nh_ctx* c : b->ctxs) {
-                cudaError_t e = cudaMemcpyAsync(c->ws + c->L.n, c->ws + c->L.nP, 3 * (size_t)c->N * sizeof(Real),
-                                                cudaMemcpyDeviceToDevice, st);
-                if (e != cudaSuccess) return fail(c0, NH_ECUDA, "copy of the relaxed director");
-            }
         return NH_OK;
     }
     // per-site stages: predict, correct, stress, force; with the three-constant energy each of the
@@ -991,6 +969,43 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
                 if (r) return r;
             }
         }
+    }
+    return NH_OK;
+}
+
+// Batched relaxation: with the fused kernels the steps alternate n -> nP -> n
+// and one launch per group clears u and brings an odd count's result back into
+// n; otherwise u is cleared first and the per-site stages run in place.
+template <typename Real>
+int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
+{
+    nh_ctx* c0 = b->ctxs[0];
+    const int n = (int)b->ctxs.size();
+    static thread_local FDBatch<Real> batch;
+    bool fused = true;
+    for (nh_ctx* c : b->ctxs) fused = fused && c->fd_fused;
+    if (!fused) {
+        for (nh_ctx* c : b->ctxs)
+            if (cudaMemsetAsync(c->ws + c->L.u, 0, 3 * (size_t)c->N * sizeof(Real), st) != cudaSuccess)
+                return fail(c0, NH_ECUDA, "clearing u");
+        for (int64_t k = 0; k < steps; ++k) {
+            int r = batch_fd_typed<Real>(b, st, 2);
+            if (r) return r;
+        }
+        return NH_OK;
+    }
+    const int grid = 8 * c0->sm_count;
+    for (int g0 = 0; g0 < n; g0 += kMaxBatch) {  // channels are independent: group by group
+        batch.count = std::min(kMaxBatch, n - g0);
+        for (int j = 0; j < batch.count; ++j) batch.ch[j] = fd_chan<Real>(b->ctxs[g0 + j]);
+        for (int64_t k = 0; k < steps; ++k) {
+            int r = timed(c0, NH_KCLASS_FD_PREDICT, st,
+                          [&] { return launch_fd_fused_batch(batch, (k & 1) ? 3 : 2, grid, st); }, "relax_batch");
+            if (r) return r;
+        }
+        cudaError_t e = launch_relax_end(batch, (steps & 1) != 0, st);
+        if (e != cudaSuccess) return cuda_fail(c0, e, "relax_end");
+        c0->launches += 1;
     }
     return NH_OK;
 }
@@ -1680,8 +1695,8 @@ int nh_relax(nh_ctx* c, int64_t n_fd_steps, void* stream)
         r = c->p.precision == NH_FP64 ? relax_fused<double>(c, n_fd_steps, st) : relax_fused<float>(c, n_fd_steps, st);
     } else {
         for (int64_t k = 0; k < n_fd_steps && r == NH_OK; ++k)
-            r = c->p.precision == NH_FP64 ? enqueue_predict_correct<double>(c, st)
-                                          : enqueue_predict_correct<float>(c, st);
+            r = c->p.precision == NH_FP64 ? enqueue_predict_correct_sites<double>(c, fd_chan<double>(c), st)
+                                          : enqueue_predict_correct_sites<float>(c, fd_chan<float>(c), st);
     }
     close_segment(c);
     return r;
@@ -1698,11 +1713,9 @@ int nh_batch_relax(nh_ctx* const* ctxs, int count, int64_t n_fd_steps, void* str
     for (nh_ctx* c : plan->ctxs) {
         c->lbp_step = -1;  // u is cleared
         c->bdp_step = -1;
-        cudaError_t e = cudaMemsetAsync(c->ws + c->L.u, 0, 3 * (size_t)c->N * real_size(c->p), st);
-        if (e != cudaSuccess) return fail(nullptr, NH_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
     }
-    for (int64_t k = 0; k < n_fd_steps && r == NH_OK; ++k)
-        r = c0->p.precision == NH_FP64 ? batch_fd_typed<double>(plan, st, 2) : batch_fd_typed<float>(plan, st, 2);
+    r = c0->p.precision == NH_FP64 ? batch_relax_typed<double>(plan, n_fd_steps, st)
+                                   : batch_relax_typed<float>(plan, n_fd_steps, st);
     close_segment(c0);
     if (r) return fail(nullptr, r, "batch relax: " + c0->err);
     return NH_OK;

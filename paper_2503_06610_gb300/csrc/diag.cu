@@ -613,11 +613,13 @@ __global__ void director_change_kernel(const Real* __restrict__ n, Real* __restr
             d2 += d * d;
             snap[(size_t)a * N + s] = v;
         }
-        m = fmax(m, sqrt(d2));
+        m = fmax(m, d2);
     }
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     __shared__ double wm[8];
-    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+    // one square root per warp, not per site (monotonic and correctly rounded: the
+    // same maximum); the FP64 pipe is 1/64 of FP32's rate
+    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = sqrt(m);
     __syncthreads();
     if (threadIdx.x == 0) {
         double b = 0.0;

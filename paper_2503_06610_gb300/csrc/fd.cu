@@ -1013,6 +1013,273 @@ __device__ void fused_a_tile(const FDChan<Real>& c, const Real* __restrict__ nin
     }
 }
 
+// Relaxation tile: kernel A for a fluid at rest (u = 0 everywhere), the step of
+// nh_relax and nh_batch_relax.  The flow terms of the rate vanish, so only n is
+// staged (a ring of four planes, one __syncthreads per layer: the plane that is
+// overwritten was last read a layer earlier), and what a thread reads of its
+// own column -- n and n^P one layer below and above -- stays in its registers,
+// which leaves four of a rate's seven points to shared memory.  Bit-identical to
+// kernel A at u = 0, whose extra terms add exact zeros.  Bound by shared-memory
+// bandwidth and issue; 4.2 M sites, FP32: RELAX_US us a step, kernel A 112 us.
+constexpr int kHaloPts = kP2 - kTX * kTY;  // points of a 2-halo plane beyond the tile's own
+template <typename Real>
+__host__ __device__ constexpr int relax_pt() { return sizeof(Real) == 4 ? 4 : 3; }  // Reals per staged point (float4, or three planes)
+template <typename Real>
+size_t relax_smem() { return (size_t)(4 * kP2 + 2 * kP1) * relax_pt<Real>() * sizeof(Real) + (4 * kP2 + 15) / 16 * 16; }
+
+template <int Points>
+__device__ __forceinline__ void ldn(const float* slot, int i, float v[3]) { ld3(slot, i, v); }
+template <int Points>
+__device__ __forceinline__ void ldn(const double* slot, int i, double v[3])
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v[a] = slot[a * Points + i];
+}
+template <int Points>
+__device__ __forceinline__ void stn(float* slot, int i, const float v[3]) { st3(slot, i, v); }
+template <int Points>
+__device__ __forceinline__ void stn(double* slot, int i, const double v[3])
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) slot[a * Points + i] = v[a];
+}
+
+// Rate at rest, dn/dt = h / gamma1, in the operation order of director_rate.
+template <typename Real>
+__device__ __forceinline__ void rest_rate(const Real nn[7][3], const FDPar<Real>& p, Real rate[3], int side)
+{
+    const Real* n = nn[0];
+    const Real ce[3] = {(nn[3][2] - nn[4][2]) - (nn[5][1] - nn[6][1]), (nn[5][0] - nn[6][0]) - (nn[1][2] - nn[2][2]),
+                        (nn[1][1] - nn[2][1]) - (nn[3][0] - nn[4][0])};
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const Real S = ((nn[1][m] + nn[2][m]) + (nn[3][m] + nn[4][m])) + (nn[5][m] + nn[6][m]);
+        rate[m] = fma(-p.kqg, ce[m], p.kg * (S - Real(6) * n[m]));
+    }
+    rate[2] = fma(p.w0g, n[2], rate[2]);
+    if (side != 0) {
+        const Real sk = Real(side) * p.kqg;
+        rate[0] = fma(-sk, n[1], rate[0]);
+        rate[1] = fma(sk, n[0], rate[1]);
+    }
+}
+
+template <typename Real>
+__device__ __forceinline__ void rest_predict(const Real n[3], const Real r[3], const FDPar<Real>& p, Real np[3])
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) np[a] = n[a] + p.dt * r[a];
+    if (p.renorm_p) {
+        const Real inv = Real(1) / sqrt(np[0] * np[0] + np[1] * np[1] + np[2] * np[2]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) np[a] *= inv;
+    }
+}
+
+template <typename Real, bool Solid>
+__device__ void relax_tile(const FDChan<Real>& c, const Real* __restrict__ nin, Real* __restrict__ nout, int tile)
+{
+    extern __shared__ __align__(16) unsigned char smem_fd[];
+    constexpr int kPt = relax_pt<Real>();
+    Real* in = reinterpret_cast<Real*>(smem_fd);  // 4 slots: n of plane p in slot p & 3
+    Real* pr = in + 4 * kPt * kP2;                // 2 slots: n^P of plane p in slot p & 1
+    unsigned char* mk = reinterpret_cast<unsigned char*>(pr + 2 * kPt * kP1);  // 4 slots: obstacle masks
+    const Geom& g = c.g;
+    const int ntx = (g.nx + kTX - 1) / kTX, nty = (g.ny + kTY - 1) / kTY;
+    const int tx_t = tile % ntx, ty_t = (tile / ntx) % nty, zc = tile / (ntx * nty);
+    const int x0 = tx_t * kTX, y0 = ty_t * kTY;
+    const int zch = fused_zchunk(c);
+    const int zb = zc * zch, ze = min(zb + zch, g.nz);
+    const int tx = threadIdx.x % kTX, ty = threadIdx.x / kTX;
+    const bool active = x0 + tx < g.nx && y0 + ty < g.ny;
+    const int N = g.N;
+    const int i1 = (tx + 1) + kHX1 * (ty + 1), i2 = (tx + 2) + kHX2 * (ty + 2);
+    // a thread loads its own point and, below kHaloPts, one point of the halo:
+    // two rows below, two above, two columns on each side
+    int h2 = -1;
+    if (threadIdx.x < kHaloPts) {
+        int hx, hy;
+        if (threadIdx.x < 4 * kHX2) {
+            const int r = threadIdx.x / kHX2;
+            hx = threadIdx.x - r * kHX2;
+            hy = r < 2 ? r : kTY + r;
+        } else {
+            const int j = threadIdx.x - 4 * kHX2;
+            hy = 2 + (j >> 2);
+            hx = (j & 3) < 2 ? (j & 3) : kTX + (j & 3);
+        }
+        h2 = hx + kHX2 * hy;
+    }
+    const int off_own = wrapm(x0 + tx, g.nx) + g.nx * wrapm(y0 + ty, g.ny);
+    const int off_halo = h2 < 0 ? 0 : wrapm(x0 - 2 + h2 % kHX2, g.nx) + g.nx * wrapm(y0 - 2 + h2 / kHX2, g.ny);
+    const HaloPoint hp = halo_point();
+    const bool homeo = g.anchoring == NH_ANCHOR_HOMEOTROPIC;
+    const int plane = g.nx * g.ny;
+    auto IN = [&](int p) { return in + (p & 3) * (kPt * kP2); };
+    auto PR = [&](int p) { return pr + (p & 1) * (kPt * kP1); };
+
+    // n of plane p at the own and the halo point (ghost planes: z_hat or the adjacent layer)
+    auto fetch = [&](int p, Real vo[3], Real vh[3], unsigned char& so, unsigned char& sh) {
+        const bool ghost = is_ghost_plane(g, p);
+        so = sh = 0;
+        if (ghost && homeo) {
+            vo[0] = vo[1] = vh[0] = vh[1] = Real(0);
+            vo[2] = vh[2] = Real(1);
+            return;
+        }
+        const int zz = g.walls ? (p < 0 ? 0 : (p >= g.nz ? g.nz - 1 : p)) : wrapm(p, g.nz);
+        const Real* __restrict__ src = nin + (size_t)plane * zz;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) vo[a] = src[a * N + off_own];
+        if (h2 >= 0) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) vh[a] = src[a * N + off_halo];
+        }
+        if (Solid && c.solid != nullptr && !ghost) {
+            so = c.solid[(size_t)plane * zz + off_own];
+            if (h2 >= 0) sh = c.solid[(size_t)plane * zz + off_halo];
+        }
+    };
+    auto commit = [&](int p, const Real vo[3], const Real vh[3], unsigned char so, unsigned char sh) {
+        stn<kP2>(IN(p), i2, vo);
+        if (h2 >= 0) stn<kP2>(IN(p), h2, vh);
+        if (Solid) {
+            mk[(p & 3) * kP2 + i2] = so;
+            if (h2 >= 0) mk[(p & 3) * kP2 + h2] = sh;
+        }
+    };
+    auto held = [&](int p, int i) { return Solid && mk[(p & 3) * kP2 + i] != 0; };
+    // rate and prediction at the own point of plane p from n of planes p - 1, p, p + 1
+    auto predict_own = [&](int p, const Real lo[3], const Real mid[3], const Real hi[3], Real r[3], Real np[3]) {
+        Real nn[7][3];
+        const Real* s = IN(p);
+        ldn<kP2>(s, i2 + 1, nn[1]);
+        ldn<kP2>(s, i2 - 1, nn[2]);
+        ldn<kP2>(s, i2 + kHX2, nn[3]);
+        ldn<kP2>(s, i2 - kHX2, nn[4]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            nn[0][a] = mid[a];
+            nn[5][a] = hi[a];
+            nn[6][a] = lo[a];
+        }
+        rest_rate(nn, c.p, r, free_plate_side(g, p));
+        if (held(p, i2)) r[0] = r[1] = r[2] = Real(0);
+        rest_predict(mid, r, c.p, np);
+        if (held(p, i2)) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) np[a] = mid[a];
+        }
+    };
+    auto predict_halo = [&](int p) {
+        if (!hp.has) return;
+        Real nn[7][3], r[3], np[3];
+        const Real* s = IN(p);
+        ldn<kP2>(s, hp.i2, nn[0]);
+        if (held(p, hp.i2)) {
+            stn<kP1>(PR(p), hp.i1, nn[0]);
+            return;
+        }
+        ldn<kP2>(s, hp.i2 + 1, nn[1]);
+        ldn<kP2>(s, hp.i2 - 1, nn[2]);
+        ldn<kP2>(s, hp.i2 + kHX2, nn[3]);
+        ldn<kP2>(s, hp.i2 - kHX2, nn[4]);
+        ldn<kP2>(IN(p + 1), hp.i2, nn[5]);
+        ldn<kP2>(IN(p - 1), hp.i2, nn[6]);
+        rest_rate(nn, c.p, r, free_plate_side(g, p));
+        rest_predict(nn[0], r, c.p, np);
+        stn<kP1>(PR(p), hp.i1, np);
+    };
+
+    Real vo[3], vh[3], na[3], nb[3], nc[3];  // own n of planes z, z + 1, z + 2 in na, nb, nc
+    unsigned char so, sh;
+    {   // planes zb - 2 .. zb + 1 in flight together
+        Real wo[3][3], wh[3][3];
+        unsigned char to[3], th[3];
+        fetch(zb - 2, wo[0], wh[0], to[0], th[0]);
+        fetch(zb - 1, wo[1], wh[1], to[1], th[1]);
+        fetch(zb, wo[2], wh[2], to[2], th[2]);
+        fetch(zb + 1, vo, vh, so, sh);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) commit(zb - 2 + k, wo[k], wh[k], to[k], th[k]);
+        commit(zb + 1, vo, vh, so, sh);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            na[a] = wo[2][a];
+            nb[a] = vo[a];
+            nc[a] = wo[0][a];  // plane zb - 2, for the predictor of plane zb - 1
+            vh[a] = wo[1][a];
+        }
+    }
+    Real plo[3], pmid[3], phi[3], rcur[3], rnext[3];  // own n^P of planes z - 1, z, z + 1; rates of z, z + 1
+    __syncthreads();
+    {
+        Real nm1[3], r[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) nm1[a] = vh[a];
+        fetch(zb + 2, vo, vh, so, sh);  // in flight during the first predictor planes
+        predict_own(zb - 1, nc, nm1, na, r, plo);
+        predict_own(zb, nm1, na, nb, rcur, pmid);
+        stn<kP1>(PR(zb), i1, pmid);
+        predict_halo(zb);
+    }
+    __syncthreads();  // plane zb - 2 is no longer read: its slot takes plane zb + 2
+    commit(zb + 2, vo, vh, so, sh);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) nc[a] = vo[a];
+    for (int z = zb; z < ze; ++z) {
+        __syncthreads();  // plane z + 2 staged, n^P of plane z complete
+        const bool more = z + 1 < ze;
+        if (more) fetch(z + 3, vo, vh, so, sh);
+        const bool glo = is_ghost_plane(g, z - 1), ghi = is_ghost_plane(g, z + 1);
+        if (!ghi) {
+            predict_own(z + 1, na, nb, nc, rnext, phi);
+            if (more) {
+                stn<kP1>(PR(z + 1), i1, phi);
+                predict_halo(z + 1);
+            }
+        }
+        // corrector; n^P beyond a plate: z_hat, or the adjacent layer's
+        Real nn[7][3], r[3];
+        const Real* s = PR(z);
+        ldn<kP1>(s, i1 + 1, nn[1]);
+        ldn<kP1>(s, i1 - 1, nn[2]);
+        ldn<kP1>(s, i1 + kHX1, nn[3]);
+        ldn<kP1>(s, i1 - kHX1, nn[4]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            nn[0][a] = pmid[a];
+            nn[5][a] = ghi ? (homeo ? Real(a == 2 ? 1 : 0) : pmid[a]) : phi[a];
+            nn[6][a] = glo ? (homeo ? Real(a == 2 ? 1 : 0) : pmid[a]) : plo[a];
+        }
+        rest_rate(nn, c.p, r, free_plate_side(g, z));
+        Real nw[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) nw[a] = na[a] + c.p.dt * Real(0.5) * (rcur[a] + r[a]);
+        Real inv = Real(1) / sqrt(nw[0] * nw[0] + nw[1] * nw[1] + nw[2] * nw[2]);
+        if (held(z, i2)) {  // obstacle: the director is held
+#pragma unroll
+            for (int a = 0; a < 3; ++a) nw[a] = na[a];
+            inv = Real(1);
+        }
+        if (active) {
+            const int site = (x0 + tx) + g.nx * (y0 + ty) + plane * z;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) nout[a * N + site] = nw[a] * inv;
+        }
+        if (more) commit(z + 3, vo, vh, so, sh);  // slot of plane z - 1, last read a layer ago
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            plo[a] = pmid[a];
+            pmid[a] = phi[a];
+            rcur[a] = rnext[a];
+            na[a] = nb[a];
+            nb[a] = nc[a];
+            nc[a] = vo[a];
+        }
+    }
+}
+
 // Kernel B tile: stress on plane p from planes p - 1, p, p + 1 of the 3-slot
 // input ring.  The divergence at a tile point needs sigma_ax at its x
 // neighbours and sigma_ay at its y neighbours in the same plane (into slot:
@@ -1209,6 +1476,12 @@ __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 4 : 2) fuse
     fused_a_tile<Real, Solid>(c, nin, nout, blockIdx.x);
 }
 
+template <typename Real, bool Solid>
+__global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 4 : 2) relax_kernel(const FDChan<Real> c, const Real* nin, Real* nout)
+{
+    relax_tile<Real, Solid>(c, nin, nout, blockIdx.x);
+}
+
 // Fused B at three blocks per SM (up to 85 registers): 101 us against 116 us
 // at four blocks of 64 registers on the 256x256x64 channel, FP32.
 template <typename Real, bool Solid>
@@ -1228,9 +1501,10 @@ __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 3 : 2)
 
 // Batched fused kernels: a persistent grid walks the (channel, tile) work
 // list; stage 0 = kernel A (n -> nP), 1 = kernel B (nP -> F, copy into n),
-// 2 = kernel A (nP -> n), for relaxations that alternate the two buffers.
+// 2 = relaxation step (n -> nP), 3 = relaxation step (nP -> n): relaxations
+// alternate the two buffers.
 template <typename Real, int Stage, bool Solid>
-__global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 3 : 2) fused_batch_kernel(const FDBatch<Real> b)
+__global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? (Stage >= 2 ? 4 : 3) : 2) fused_batch_kernel(const FDBatch<Real> b)
 {
     const int total = b.prefix[b.count];
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
@@ -1248,8 +1522,23 @@ __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 3 : 2) fuse
         else if (Stage == 1)
             fused_b_tile<Real, Solid>(c, c.nP, c.n, t - b.prefix[lo]);
         else
-            fused_a_tile<Real, Solid>(c, c.nP, c.n, t - b.prefix[lo]);
+            relax_tile<Real, Solid>(c, Stage == 2 ? c.n : c.nP, Stage == 2 ? c.nP : c.n, t - b.prefix[lo]);
         __syncthreads();
+    }
+}
+
+// End of a batched relaxation: u = 0 in every channel and, when an odd number of
+// steps left the director in nP, its copy back into n.
+template <typename Real>
+__global__ void __launch_bounds__(256) relax_end_kernel(const FDBatch<Real> b, bool copy)
+{
+    for (int k = blockIdx.y; k < b.count; k += gridDim.y) {
+        const FDChan<Real>& c = b.ch[k];
+        Real* u = const_cast<Real*>(c.u);
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * c.g.N; i += gridDim.x * blockDim.x) {
+            u[i] = Real(0);
+            if (copy) c.n[i] = c.nP[i];
+        }
     }
 }
 
@@ -1265,7 +1554,7 @@ cudaError_t prepare_fused()
 {
     static bool done = false;  // the attribute is per function; setting it twice is harmless
     if (done) return cudaSuccess;
-    const int a = (int)fused_a_smem<Real>(), b = (int)fused_b_smem<Real>();
+    const int a = (int)fused_a_smem<Real>(), b = (int)fused_b_smem<Real>(), r = (int)relax_smem<Real>();
     const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(fused_a_kernel<Real, false>, attr, a);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_a_kernel<Real, true>, attr, a);
@@ -1276,8 +1565,12 @@ cudaError_t prepare_fused()
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 0, true>, attr, a);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 1, false>, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 1, true>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, false>, attr, a);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, true>, attr, a);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, false>, attr, r);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, true>, attr, r);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 3, false>, attr, r);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 3, true>, attr, r);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(relax_kernel<Real, false>, attr, r);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(relax_kernel<Real, true>, attr, r);
     if (e == cudaSuccess) done = true;
     return e;
 }
@@ -1355,6 +1648,26 @@ cudaError_t launch_fd_fused_a(const FDChan<Real>& c, const Real* nin, Real* nout
 }
 
 template <typename Real>
+cudaError_t launch_relax(const FDChan<Real>& c, const Real* nin, Real* nout, cudaStream_t st)
+{
+    cudaError_t e = prepare_fused<Real>();
+    if (e != cudaSuccess) return e;
+    if (c.solid != nullptr)
+        relax_kernel<Real, true><<<fused_tiles(c), kFusedThreads, relax_smem<Real>(), st>>>(c, nin, nout);
+    else
+        relax_kernel<Real, false><<<fused_tiles(c), kFusedThreads, relax_smem<Real>(), st>>>(c, nin, nout);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t launch_relax_end(const FDBatch<Real>& b, bool copy, cudaStream_t st)
+{
+    if (b.count < 1 || b.count > kMaxBatch) return cudaErrorInvalidValue;
+    relax_end_kernel<Real><<<dim3(64, b.count), 256, 0, st>>>(b, copy);
+    return cudaGetLastError();
+}
+
+template <typename Real>
 cudaError_t launch_fd_fused_b(const FDChan<Real>& c, const Real* nin, Real* ncopy, cudaStream_t st, const BDiag* diag)
 {
     cudaError_t e = prepare_fused<Real>();
@@ -1391,20 +1704,22 @@ cudaError_t launch_fd_fused_batch(FDBatch<Real>& b, int stage, int grid, cudaStr
         b.prefix[k + 1] = b.prefix[k] + fused_tiles(b.ch[k]);
     }
     const int blocks = grid < b.prefix[b.count] ? grid : b.prefix[b.count];
-    const size_t smem = stage == 1 ? fused_b_smem<Real>() : fused_a_smem<Real>();
+    const size_t smem = stage == 1 ? fused_b_smem<Real>() : (stage == 0 ? fused_a_smem<Real>() : relax_smem<Real>());
     bool solid = false;
     for (int k = 0; k < b.count; ++k) solid = solid || b.ch[k].solid != nullptr;
     if (solid) {
         switch (stage) {
         case 0: fused_batch_kernel<Real, 0, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
         case 1: fused_batch_kernel<Real, 1, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        default: fused_batch_kernel<Real, 2, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
+        case 2: fused_batch_kernel<Real, 2, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
+        default: fused_batch_kernel<Real, 3, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
         }
     } else {
         switch (stage) {
         case 0: fused_batch_kernel<Real, 0, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
         case 1: fused_batch_kernel<Real, 1, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        default: fused_batch_kernel<Real, 2, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
+        case 2: fused_batch_kernel<Real, 2, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
+        default: fused_batch_kernel<Real, 3, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
         }
     }
     return cudaGetLastError();
@@ -1415,6 +1730,10 @@ template cudaError_t launch_fd_fused_a<float>(const FDChan<float>&, const float*
 template cudaError_t launch_fd_fused_b<double>(const FDChan<double>&, const double*, double*, cudaStream_t,
                                                 const BDiag*);
 template int fd_fused_tiles<double>(const FDChan<double>&);
+template cudaError_t launch_relax<double>(const FDChan<double>&, const double*, double*, cudaStream_t);
+template cudaError_t launch_relax<float>(const FDChan<float>&, const float*, float*, cudaStream_t);
+template cudaError_t launch_relax_end<double>(const FDBatch<double>&, bool, cudaStream_t);
+template cudaError_t launch_relax_end<float>(const FDBatch<float>&, bool, cudaStream_t);
 template cudaError_t launch_fd_fused_b<float>(const FDChan<float>&, const float*, float*, cudaStream_t, const BDiag*);
 template int fd_fused_tiles<float>(const FDChan<float>&);
 template cudaError_t launch_fd_fused_batch<double>(FDBatch<double>&, int, int, cudaStream_t);

@@ -229,12 +229,16 @@ cudaError_t launch_fd_batch(FDBatch<Real>& b, int stage, int grid, cudaStream_t 
 // Fused FD kernels (2.5D shared-memory tiles): A = predictor + corrector +
 // renormalisation (nin, u -> nout), B = stress + force (nin, u -> F; copies
 // nin into ncopy when ncopy is not null); batched stages 0 = A (n -> nP),
-// 1 = B (nP -> F, n), 2 = A (nP -> n).
+// 1 = B (nP -> F, n), 2 / 3 = relaxation step (A at u = 0, n -> nP / nP -> n).
 template <typename Real>
 cudaError_t launch_fd_fused_a(const FDChan<Real>& c, const Real* nin, Real* nout, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_fd_fused_b(const FDChan<Real>& c, const Real* nin, Real* ncopy, cudaStream_t s,
                               const BDiag* diag = nullptr);
+template <typename Real>
+cudaError_t launch_relax(const FDChan<Real>& c, const Real* nin, Real* nout, cudaStream_t s);  // A at u = 0 (u not read)
+template <typename Real>
+cudaError_t launch_relax_end(const FDBatch<Real>& b, bool copy, cudaStream_t s);  // u = 0; copy: n <- nP
 template <typename Real>
 int fd_fused_tiles(const FDChan<Real>& c);  // blocks of a single-channel fused launch
 template <typename Real>
