@@ -225,7 +225,7 @@ int nh_fd_update(nh_ctx* ctx, void* stream);
  * kernels (with the three-constant P stages when a channel has frank3); with
  * obstacles in any channel the LB sweep runs one site per thread.  Launch
  * counts and timing are recorded on ctxs[0]; the launch shape is ctxs[0]'s LB
- * variant (see nh_batch_autotune).  Asynchronous on stream (NULL = ctxs[0]'s
+ * variant if one was set (see nh_batch_autotune).  Asynchronous on stream (NULL = ctxs[0]'s
  * stream). */
 int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stream);
 
@@ -365,8 +365,9 @@ int nh_get_timing(nh_ctx* ctx, nh_timing* out);
 /* Kernel launches this context has issued (graph nodes counted per replay). */
 int64_t nh_launch_count(const nh_ctx* ctx);
 
-/* Select the launch shape of the fused LB kernel: 0 = two sites per thread,
- * 256 threads (default; needs even nx), 1 = one site per thread, 256 threads,
+/* Select the launch shape of the fused LB kernel (the default is chosen from
+ * the size and the store): 0 = two sites per thread,
+ * 256 threads (needs even nx), 1 = one site per thread, 256 threads,
  * 2 = two sites, 128 threads, 3 = one site, 128 threads, 4 = four sites,
  * 128 threads, 5 = four sites, 64 threads (4 and 5 need nx % 4 == 0),
  * 6 = 16-bit stores only (F16S, BF16S): whole x-rows of the 19 source planes
@@ -374,13 +375,14 @@ int64_t nh_launch_count(const nh_ctx* ctx);
  * while a block collides the current one, four sites per thread (needs
  * nx % 128 == 0 and nx <= 256; with obstacles it runs as variant 0).  All variants compute the same arithmetic
  * and give bit-identical results.  Batches use variants 0 .. 5 (a batch of
- * channels set to 6 runs variant 0).  NH_EINVAL if the variant does not fit
+ * channels set to 6 runs variant 2, or 1 with an odd nx among them).  NH_EINVAL if the variant does not fit
  * the domain.  Variant 6 bounds its waits on the copies: an expired wait is
  * reported by the next nh_diagnostics / nh_diagnostics_read as NH_ETIMEOUT
  * (that launch's populations are incomplete). */
 int nh_set_lb_variant(nh_ctx* ctx, int variant);
 
-/* Select the FD kernels: 1 = fused (default): one 2.5D shared-memory kernel
+/* Select the FD kernels (default: 1 in FP32, 0 in FP64, whose repeated
+ * evaluations on tile halos cost more than they save): 1 = fused: one 2.5D shared-memory kernel
  * for predictor + corrector + renormalisation and one for stress + force
  * (the stress never leaves the chip); 0 = one kernel per stage.  Same
  * arithmetic.  With the fused kernels the timing classes FD_PREDICT and

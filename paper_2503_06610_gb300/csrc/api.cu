@@ -217,7 +217,8 @@ struct nh_ctx {
     double tubes[NH_MAX_TUBES][2] = {};
     bool use_graphs = true;
     int lb_variant = 0;
-    int fd_fused = 1;  // 1: fused 2.5D FD kernels; 0: per-site kernels
+    bool lb_chosen = false;  // the launch shape was set or autotuned, not the default of lb_default_variant
+    int fd_variant = -1;     // 1: fused 2.5D FD kernels; 0: per-site kernels; -1: by precision (fd_fused)
     int sm_count = 152;
     int64_t epoch = 0;  // bumped whenever buffers or launch shapes change (invalidates batch plans)
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -253,6 +254,17 @@ struct nh_ctx {
 };
 
 namespace {
+
+// The FD kernels of an update.  By default FP32 runs the fused kernels and FP64
+// the per-site ones: the fused kernels evaluate the predictor and the stress
+// again on each tile's halo (about 2.3 evaluations a site at 96x96x32), which
+// saves memory traffic and launches in FP32, but FP64 is bound by the FP64 pipe
+// (1/64 of FP32's rate).  96x96x32, FP64: an FD update 506 us fused, 302 us per site.
+bool fd_fused(const nh_ctx* c) { return c->fd_variant >= 0 ? c->fd_variant == 1 : c->p.precision == NH_FP32; }
+// Relaxations run the kernel at rest unless the per-site kernels were asked
+// for: it has no flow terms, and reads a third (96x96x32, FP64: 104 us a step
+// against 154 us per site).
+bool relax_fused_ok(const nh_ctx* c) { return c->fd_variant != 0; }
 
 int fail(nh_ctx* c, int code, const std::string& msg)
 {
@@ -503,7 +515,7 @@ int enqueue_force_only(nh_ctx* c, cudaStream_t st, bool after_update = false)
 {
     auto a = fd_chan<Real>(c);
     a.p.n_rate = after_update && c->p.n_from_rate;
-    if (c->fd_fused)
+    if (fd_fused(c))
         return timed(c, NH_KCLASS_STRESS, st, [&] { return launch_fd_fused_b<Real>(a, a.n, nullptr, st); },
                      "stress_force");
     int r = NH_OK;
@@ -519,7 +531,7 @@ int enqueue_fd(nh_ctx* c, cudaStream_t st)
 {
     auto a = fd_chan<Real>(c);
     c->bdp_step = -1;
-    if (c->fd_fused) {
+    if (fd_fused(c)) {
         // predictor + corrector: n -> nP; stress + force from nP, which is copied back into n
         int r = timed(c, NH_KCLASS_FD_PREDICT, st, [&] { return launch_fd_fused_a<Real>(a, a.n, a.nP, st); },
                       "fd_fused");
@@ -856,14 +868,19 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
         if (!plan) return fail(nullptr, NH_ENOMEM, "host allocation of the batch plan failed");
         plan->ctxs = key;
         plan->epochs = epochs;
-        int v = c0->lb_variant;
-        bool ok = true;
-        for (nh_ctx* c : key) ok = ok && lb_variant_valid(v, c->p.nx);
-        if (!ok) {  // the row-staged variant (single channels only), or a shape some channel cannot take
-            v = 0;
-            for (nh_ctx* c : key)
-                if (!lb_variant_valid(0, c->p.nx)) v = 1;  // one site per thread fits every domain
-        }
+        // ctxs[0]'s shape if it was set and fits every channel (the row-staged one runs single channels only),
+        // else the default of the batch's channels taken as one domain
+        auto fits = [&](int v) {
+            bool ok = true;
+            for (nh_ctx* c : key) ok = ok && lb_variant_valid(v, c->p.nx);
+            return ok;
+        };
+        int64_t rows = 0;
+        for (nh_ctx* c : key) rows += (int64_t)c->p.ny * c->p.nz;
+        int v = c0->lb_chosen ? c0->lb_variant
+                              : lb_default_variant(c0->p.nx, (int)std::min<int64_t>(rows, 1 << 30), 1, (int)store_size(c0->p));
+        if (!fits(v)) v = 2;
+        if (!fits(v)) v = 1;  // one site per thread fits every domain
         plan->variant = v;
     }
     *out = plan;
@@ -935,7 +952,7 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
     // n_from_rate, nor a channel set to the per-site kernels)
     bool fused = true, frank3 = false;
     for (nh_ctx* c : b->ctxs) {
-        fused = fused && c->fd_fused;
+        fused = fused && fd_fused(c);
         frank3 = frank3 || c->p.frank3;
     }
     if (fused) {  // full FD update (A: n -> nP, B: nP -> F and n)
@@ -983,7 +1000,7 @@ int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
     const int n = (int)b->ctxs.size();
     static thread_local FDBatch<Real> batch;
     bool fused = true;
-    for (nh_ctx* c : b->ctxs) fused = fused && c->fd_fused;
+    for (nh_ctx* c : b->ctxs) fused = fused && relax_fused_ok(c);
     if (!fused) {
         for (nh_ctx* c : b->ctxs)
             if (cudaMemsetAsync(c->ws + c->L.u, 0, 3 * (size_t)c->N * sizeof(Real), st) != cudaSuccess)
@@ -1310,9 +1327,9 @@ int nh_create(const nh_params* p, void* cuda_stream, nh_ctx** out)
     if (!c) return fail(nullptr, NH_ENOMEM, "host allocation of the context failed");
     c->p = *p;
     c->N = p->nx * p->ny * p->nz;
-    c->lb_variant = lb_variant_valid(0, p->nx) ? 0 : 1;
+    c->lb_variant = lb_default_variant(p->nx, p->ny, p->nz, (int)store_size(*p));
     // the three-constant correction, the wide Laplacian and N from the rate run on the per-site FD kernels
-    if (p->frank3 || p->lap_wide || p->n_from_rate) c->fd_fused = 0;
+    if (p->frank3 || p->lap_wide || p->n_from_rate) c->fd_variant = 0;
     c->L = make_layout(*p);
     c->stream = static_cast<cudaStream_t>(cuda_stream);
     cudaError_t e = cudaGetDevice(&c->device);
@@ -1568,7 +1585,7 @@ int nh_step(nh_ctx* c, int64_t n_lb_steps, void* stream)
                 c->lbp_step = c->step;
                 c->lbp_blocks = lb_blocks(c->lb_variant, c->N);
                 c->bdp_step = -1;
-                if (c->fd_fused) {  // ... and its fused stress kernel left the director's partials
+                if (fd_fused(c)) {  // ... and its fused stress kernel left the director's partials
                     c->bdp_step = c->step;
                     c->bdp_blocks = c->p.precision == NH_FP64 ? fd_fused_tiles(fd_chan<double>(c))
                                                              : fd_fused_tiles(fd_chan<float>(c));
@@ -1691,7 +1708,7 @@ int nh_relax(nh_ctx* c, int64_t n_fd_steps, void* stream)
     c->lbp_step = -1;  // u is cleared
     c->bdp_step = -1;
     NH_CUDA(c, cudaMemsetAsync(c->ws + c->L.u, 0, 3 * (size_t)c->N * real_size(c->p), st));
-    if (c->fd_fused) {
+    if (relax_fused_ok(c)) {
         r = c->p.precision == NH_FP64 ? relax_fused<double>(c, n_fd_steps, st) : relax_fused<float>(c, n_fd_steps, st);
     } else {
         for (int64_t k = 0; k < n_fd_steps && r == NH_OK; ++k)
@@ -1928,6 +1945,7 @@ int nh_set_lb_variant(nh_ctx* c, int variant)
         return fail(c, NH_EINVAL, "LB variant not valid for this domain");
     if (variant != c->lb_variant) drop_graphs(c);
     c->lb_variant = variant;
+    c->lb_chosen = true;
     return NH_OK;
 }
 
@@ -1957,8 +1975,8 @@ int nh_set_fd_variant(nh_ctx* c, int fused)
     if (fused && c->p.frank3) return fail(c, NH_EINVAL, "the three-constant energy runs on the per-site FD kernels only");
     if (fused && (c->p.lap_wide || c->p.n_from_rate))
         return fail(c, NH_EINVAL, "lap_wide and n_from_rate run on the per-site FD kernels only");
-    if (fused != c->fd_fused) drop_graphs(c);
-    c->fd_fused = fused;
+    if ((fused != 0) != fd_fused(c)) drop_graphs(c);
+    c->fd_variant = fused;
     return NH_OK;
 }
 
@@ -2000,6 +2018,7 @@ int nh_autotune(nh_ctx* c, void* stream, int* chosen)
     c->free_events.push_back(e1);
     c->timing = saved_timing;
     c->lb_variant = best;
+    c->lb_chosen = true;
     if (best != saved_variant) drop_graphs(c);
     if (chosen) *chosen = best;
     return r;

@@ -1020,7 +1020,7 @@ __device__ void fused_a_tile(const FDChan<Real>& c, const Real* __restrict__ nin
 // own column -- n and n^P one layer below and above -- stays in its registers,
 // which leaves four of a rate's seven points to shared memory.  Bit-identical to
 // kernel A at u = 0, whose extra terms add exact zeros.  Bound by shared-memory
-// bandwidth and issue; 4.2 M sites, FP32: RELAX_US us a step, kernel A 112 us.
+// bandwidth and issue; 4.2 M sites, FP32: 57 us a step, kernel A 105 us.
 constexpr int kHaloPts = kP2 - kTX * kTY;  // points of a 2-halo plane beyond the tile's own
 template <typename Real>
 __host__ __device__ constexpr int relax_pt() { return sizeof(Real) == 4 ? 4 : 3; }  // Reals per staged point (float4, or three planes)

@@ -197,18 +197,6 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return fma(a, b, c); }
 
-// e . v for a lattice vector with components in {-1, 0, 1} (constants once the
-// direction loop is unrolled): sums and differences only.
-template <typename Real>
-__device__ __forceinline__ Real edot(int X, int Y, int Z, Real vx, Real vy, Real vz)
-{
-    Real r = Real(0);
-    if (X != 0) r = X > 0 ? vx : -vx;
-    if (Y != 0) r = (X != 0) ? (Y > 0 ? r + vy : r - vy) : (Y > 0 ? vy : -vy);
-    if (Z != 0) r = (X != 0 || Y != 0) ? (Z > 0 ? r + vz : r - vz) : (Z > 0 ? vz : -vz);
-    return r;
-}
-
 // Moments, equilibrium, Guo source and relaxation of one site s from its
 // streamed populations f (decoded values; raw 2^k-scaled ones for the 16-bit
 // stores, whose power-of-two factors inv_in and scale_out are folded in) and
@@ -222,22 +210,22 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
                                                 Real (&fo)[19], Real flx, Real fly, Real flz, float inv_in,
                                                 float scale_out, Real& psum, Real& pmax, int& pbad, float& amax)
 {
-    NH_D3Q19_TABLES
     constexpr bool kScaled = sizeof(Store) == 2;
     constexpr bool WriteMacro = Macro >= 1;
     constexpr bool Partials = Macro == 2;
     const int N = c.g.N;
     // 2. moments: pair sums and differences of (e_i, -e_i)
-    Real sum = f[0], mx = 0, my = 0, mz = 0;
+    Real d[9];
+    Real sum = f[0];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const int i = 2 * k + 1;
-        sum += f[i] + f[i + 1];
-        const Real d = f[i] - f[i + 1];
-        if (EX[i] != 0) mx += EX[i] > 0 ? d : -d;
-        if (EY[i] != 0) my += EY[i] > 0 ? d : -d;
-        if (EZ[i] != 0) mz += EZ[i] > 0 ? d : -d;
+        sum += f[2 * k + 1] + f[2 * k + 2];
+        d[k] = f[2 * k + 1] - f[2 * k + 2];
     }
+    // pairs: x, y, z, (x+y, x-y), (x+z, x-z), (y+z, y-z)
+    Real mx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+    Real my = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+    Real mz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
     if (kScaled) {  // raw populations: scale the sums once
         sum = mul_rn(sum, Real(inv_in));
         mx = mul_rn(mx, Real(inv_in));
@@ -245,7 +233,6 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
         mz = mul_rn(mz, Real(inv_in));
     }
     const Real rho = Shifted ? Real(1) + sum : sum;
-    const Real drho = Shifted ? sum : sum - Real(1);
     const Real Fx = fma_rn(rho, c.gx, flx);
     const Real Fy = fma_rn(rho, c.gy, fly);
     const Real Fz = fma_rn(rho, c.gz, flz);
@@ -270,40 +257,52 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
     //   f^eq = w rho [3 eu + 4.5 eu^2 - 1.5 u.u] + w (rho - 1 | rho)
     //   S    = w [3 eF + 9 eu eF - 3 u.F]
     //   f*   = (1 - omega) f + omega f^eq + (1 - omega/2) S
-    // with a 16-bit store the constants carry scale_out (and omc the raw
-    // input's inv_in), so fo[] leaves here already in encoded units
+    // With g = 1.5 omega rho u + 3 (1 - omega/2) F and h = g + 1.5 omega rho u the two sums are
+    //   omega f^eq + (1 - omega/2) S = w [3 (e.u)(e.g) + T + e.h],  T = omega (rho - 1 | rho) - u.g
+    // so a pair costs one even and one odd part from three projections: 150
+    // operations a site instead of 215.  FP64 LB is bound by the FP64 pipe and
+    // the 16-bit stores by issue (times in the launch variants' table).
+    // With a 16-bit store the constants carry scale_out (and omc the raw
+    // input's inv_in), so fo[] leaves here already in encoded units.
     const Real so = kScaled ? Real(scale_out) : Real(1);
     const Real omega = mul_rn(c.omega, so);
     const Real omc = mul_rn(Real(1) - c.omega, kScaled ? mul_rn(Real(inv_in), so) : Real(1));
-    const Real cS = mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so);
-    const Real u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
-    const Real uu15 = mul_rn(Real(1.5), u2);
-    const Real uF3 = mul_rn(Real(3), fma_rn(uz, Fz, fma_rn(uy, Fy, mul_rn(ux, Fx))));
-    const Real base = Shifted ? drho : rho;
-    // rest population (w = 1/3)
-    {
-        const Real w = Real(1) / Real(3);
-        const Real t = fma_rn(-rho, uu15, base);
-        fo[0] = fma_rn(omc, f[0], fma_rn(mul_rn(omega, w), t, -mul_rn(mul_rn(cS, w), uF3)));
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int i = 2 * k + 1;
-        const Real w = i < 7 ? Real(1) / Real(18) : Real(1) / Real(36);
-        const Real ow = mul_rn(omega, w);
-        const Real A = mul_rn(ow, rho);
-        const Real B = mul_rn(ow, base);
-        const Real C = mul_rn(cS, w);
-        const Real eu = edot(EX[i], EY[i], EZ[i], ux, uy, uz);
-        const Real eF = edot(EX[i], EY[i], EZ[i], Fx, Fy, Fz);
-        const Real X = fma_rn(mul_rn(Real(4.5), eu), eu, -uu15);
-        const Real Y = fma_rn(mul_rn(Real(9), eu), eF, -uF3);
-        const Real even = fma_rn(C, Y, fma_rn(A, X, B));
-        const Real odd = mul_rn(Real(3), fma_rn(A, eu, mul_rn(C, eF)));
-        fo[i] = fma_rn(omc, f[i], even) + odd;
-        fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
-    }
+    const Real cS3 = mul_rn(Real(3), mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so));
+    const Real a15 = mul_rn(mul_rn(Real(1.5), omega), rho);
+    const Real gx = fma_rn(a15, ux, mul_rn(cS3, Fx));
+    const Real gy = fma_rn(a15, uy, mul_rn(cS3, Fy));
+    const Real gz = fma_rn(a15, uz, mul_rn(cS3, Fz));
+    constexpr Real w36 = Real(1) / Real(36), w12 = Real(1) / Real(12);
+    const Real hx = mul_rn(w36, fma_rn(a15, ux, gx));
+    const Real hy = mul_rn(w36, fma_rn(a15, uy, gy));
+    const Real hz = mul_rn(w36, fma_rn(a15, uz, gz));
+    const Real vx = mul_rn(w12, ux), vy = mul_rn(w12, uy), vz = mul_rn(w12, uz);
+    const Real ug = fma_rn(uz, gz, fma_rn(uy, gy, mul_rn(ux, gx)));
+    const Real T = fma_rn(mul_rn(w36, omega), Shifted ? sum : rho, -mul_rn(w36, ug));
+    fo[0] = fma_rn(Real(12), T, mul_rn(omc, f[0]));
+    const Real omc_half = mul_rn(Real(0.5), omc);
+    // axis pair (w = 1/18: twice the 1/36 parts), diagonal pair
+    auto axis = [&](int i, Real v, Real g, Real h) {
+        const Real even = fma_rn(v, g, T);
+        fo[i] = mul_rn(Real(2), fma_rn(omc_half, f[i], even) + h);
+        fo[i + 1] = mul_rn(Real(2), fma_rn(omc_half, f[i + 1], even) - h);
+    };
+    auto diagonal = [&](int i, Real v, Real g, Real h) {
+        const Real even = fma_rn(v, g, T);
+        fo[i] = fma_rn(omc, f[i], even + h);
+        fo[i + 1] = fma_rn(omc, f[i + 1], even - h);
+    };
+    axis(1, vx, gx, hx);
+    axis(3, vy, gy, hy);
+    axis(5, vz, gz, hz);
+    diagonal(7, vx + vy, gx + gy, hx + hy);
+    diagonal(9, vx - vy, gx - gy, hx - hy);
+    diagonal(11, vx + vz, gx + gz, hx + hz);
+    diagonal(13, vx - vz, gx - gz, hx - hz);
+    diagonal(15, vy + vz, gy + gz, hy + hz);
+    diagonal(17, vy - vz, gy - gz, hy - hz);
     if (Partials) {  // the sums nh_diagnostics forms from the stored state, site by site
+        const Real u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
         Real fs = fo[0];
 #pragma unroll
         for (int i = 1; i < 19; ++i) fs += fo[i];
@@ -870,6 +869,28 @@ bool lb_variant_valid_for(int variant, int nx, int store_bytes)
 {
     if (variant == kLBRowsVariant) return lb_rows_valid(nx, store_bytes);
     return lb_variant_valid(variant, nx);
+}
+
+// The default shape of a channel (microseconds of 16 LB steps and an FD update,
+// two sites x 256 | one x 256 | two x 128 | one x 128 | four x 128 | rows):
+//   FP32 32x32x16: 62 | 50 | 51 | 45 | 64, 96x96x32: 137 | 143 | 132 | 137 | 137,
+//   256x256x64: 1825 | 1818 | 1820 | 1821 | 1837 (at the HBM limit);
+//   F16S 64x64x32: 115 | 127 | 115 | 126 | 108, 180x140x50: 554 | 599 | 539 | 645 | 485,
+//   256x256x16: 439 | 496 | 427 | 519 | 385 | 363, 256x256x64: 1598 | 1716 | 1514 | 1875 | 1370 | 1265,
+//   128x128x32: 243 | 275 | 245 | 294 | 216 | 237.
+// So: small blocks of single sites while they do not fill the GPU (up to 2^15
+// sites), two sites x 128 otherwise; the 16-bit stores, bound by issue rather than
+// HBM, take the four-site shape from 10^5 sites, and the staged rows where a row
+// is 256 sites and every resident block gets a few of them.
+int lb_default_variant(int nx, int ny, int nz, int store_bytes)
+{
+    const double N = (double)nx * ny * nz;
+    if (store_bytes == 2) {
+        if (nx == kRowMaxNx && (double)ny * nz >= 4096.0) return kLBRowsVariant;
+        if (nx % 4 == 0 && N > 1e5) return 4;
+    }
+    if (N <= 32768.0) return 3;
+    return nx % 2 == 0 ? 2 : 1;
 }
 
 int lb_blocks(int variant, int N)
