@@ -204,7 +204,7 @@ int nh_restore(nh_ctx* ctx, const double* n, const double* F, const double* u, c
  * collide-and-stream launch; after each step whose count s is a multiple of
  * dt_fd, the FD predictor-corrector on n with that step's u, then the LC
  * stress and force.  Asynchronous on stream (NULL = the context's stream).
- * Whole dt_fd blocks run from a CUDA graph unless timing is on. */
+ * Whole dt_fd blocks of at least 12 steps run from a CUDA graph unless timing is on. */
 int nh_step(nh_ctx* ctx, int64_t n_lb_steps, void* stream);
 
 /* Run one FD update now (predictor, corrector + renormalisation, stress,
@@ -215,7 +215,7 @@ int nh_fd_update(nh_ctx* ctx, void* stream);
  * by n_lb_steps each.  Every pass (LB sweep, FD predict, correct, stress,
  * force) is one persistent launch per group of up to 64 channels: the grid
  * walks a work list of (channel, tile) pairs, and the channel descriptors
- * travel as kernel parameters.  Whole dt_fd blocks are replayed from a CUDA
+ * travel as kernel parameters.  Whole dt_fd blocks (of at least 12 steps) are replayed from a CUDA
  * graph cached per list of contexts (dropped when a context is rebound,
  * re-tuned or destroyed).  All contexts must share precision, storage,
  * shifted and dt_fd, be on one device, have fields set and be at the same
@@ -394,7 +394,7 @@ int nh_set_fd_variant(nh_ctx* ctx, int fused);
  * fastest and return its index in *chosen (may be NULL).  Synchronises. */
 int nh_autotune(nh_ctx* ctx, void* stream, int* chosen);
 
-/* Use CUDA graphs for whole dt_fd blocks (default on). */
+/* Use CUDA graphs for whole dt_fd blocks of at least 12 steps (default on). */
 int nh_set_graphs(nh_ctx* ctx, int on);
 
 /* Diagnostics folded into the step (default on): every LB launch that

@@ -654,6 +654,14 @@ int capture_block(nh_ctx* c, int src)
     return NH_OK;
 }
 
+// Whether whole dt_fd blocks of a channel or batch run from a CUDA graph: from
+// twelve steps a block.  Shorter ones launch directly, which overlaps consecutive
+// blocks too, where each graph launch waits for the one before to end
+// (32x32x16, a block of one step: 17.2 us against 20.5 us, of eight: 29.8 / 31.0,
+// of sixteen: 44.7 / 43.5).
+constexpr int kGraphMinSteps = 12;
+bool use_block_graph(const nh_ctx* c) { return c->use_graphs && !c->timing && c->p.dt_fd >= kGraphMinSteps; }
+
 int check_ready(nh_ctx* c)
 {
     if (!c) return fail(nullptr, NH_EINVAL, "ctx is NULL");
@@ -1571,7 +1579,7 @@ int nh_step(nh_ctx* c, int64_t n_lb_steps, void* stream)
     const int dt = c->p.dt_fd;
     int64_t left = n_lb_steps;
     while (left > 0) {
-        if (c->use_graphs && !c->timing && c->step % dt == 0 && left >= dt) {
+        if (use_block_graph(c) && c->step % dt == 0 && left >= dt) {
             if (!c->graph[c->cur]) {
                 r = capture_block(c, c->cur);
                 if (r) return r;
@@ -1628,7 +1636,7 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
     const int dt = c0->p.dt_fd;
     int64_t left = n_lb_steps;
     while (left > 0) {
-        if (c0->use_graphs && !c0->timing && c0->step % dt == 0 && left >= dt) {
+        if (use_block_graph(c0) && c0->step % dt == 0 && left >= dt) {
             const int parity = c0->cur;
             if (!plan->graph[parity]) {
                 r = batch_capture(plan, parity);

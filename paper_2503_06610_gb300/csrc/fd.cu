@@ -558,6 +558,7 @@ __device__ __forceinline__ void fd_stage_site(const FDChan<Real>& c, int s)
 template <typename Real, int Stage>
 __global__ void __launch_bounds__(256) fd_kernel(const FDChan<Real> c)
 {
+    step_kernel_enter();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < c.g.N) fd_stage_site<Real, Stage>(c, s);
 }
@@ -566,6 +567,7 @@ __global__ void __launch_bounds__(256) fd_kernel(const FDChan<Real> c)
 template <typename Real, int Stage>
 __global__ void __launch_bounds__(256) fd_batch_kernel(const FDBatch<Real> b)
 {
+    step_kernel_enter();
     const int total = b.prefix[b.count];
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
         int lo = 0, hi = b.count - 1;
@@ -1473,12 +1475,14 @@ __device__ void fused_b_tile(const FDChan<Real>& c, const Real* __restrict__ nin
 template <typename Real, bool Solid>
 __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 4 : 2) fused_a_kernel(const FDChan<Real> c, const Real* nin, Real* nout)
 {
+    step_kernel_enter();
     fused_a_tile<Real, Solid>(c, nin, nout, blockIdx.x);
 }
 
 template <typename Real, bool Solid>
 __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 4 : 2) relax_kernel(const FDChan<Real> c, const Real* nin, Real* nout)
 {
+    step_kernel_enter();
     relax_tile<Real, Solid>(c, nin, nout, blockIdx.x);
 }
 
@@ -1487,6 +1491,7 @@ __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 4 : 2) rela
 template <typename Real, bool Solid>
 __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 3 : 2) fused_b_kernel(const FDChan<Real> c, const Real* nin, Real* ncopy)
 {
+    step_kernel_enter();
     fused_b_tile<Real, Solid>(c, nin, ncopy, blockIdx.x);
 }
 // The same with the diagnostics partials of the updated director (no obstacles).
@@ -1496,6 +1501,7 @@ template <typename Real>
 __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 3 : 2)
     fused_b_diag_kernel(const FDChan<Real> c, const Real* nin, Real* ncopy, const BDiag bd)
 {
+    step_kernel_enter();
     fused_b_tile<Real, false, true>(c, nin, ncopy, blockIdx.x, &bd);
 }
 
@@ -1506,6 +1512,7 @@ __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? 3 : 2)
 template <typename Real, int Stage, bool Solid>
 __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? (Stage >= 2 ? 4 : 3) : 2) fused_batch_kernel(const FDBatch<Real> b)
 {
+    step_kernel_enter();
     const int total = b.prefix[b.count];
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
         int lo = 0, hi = b.count - 1;
@@ -1532,6 +1539,7 @@ __global__ void __launch_bounds__(kFusedThreads, sizeof(Real) == 4 ? (Stage >= 2
 template <typename Real>
 __global__ void __launch_bounds__(256) relax_end_kernel(const FDBatch<Real> b, bool copy)
 {
+    step_kernel_enter();
     for (int k = blockIdx.y; k < b.count; k += gridDim.y) {
         const FDChan<Real>& c = b.ch[k];
         Real* u = const_cast<Real*>(c.u);
@@ -1587,12 +1595,12 @@ cudaError_t launch_fd_batch(FDBatch<Real>& b, int stage, int grid, cudaStream_t 
     for (int k = 0; k < b.count; ++k) b.prefix[k + 1] = b.prefix[k] + blocks_for(b.ch[k].g.N);
     const int blocks = grid < b.prefix[b.count] ? grid : b.prefix[b.count];
     switch (stage) {
-    case 0: fd_batch_kernel<Real, 0><<<blocks, 256, 0, st>>>(b); break;
-    case 1: fd_batch_kernel<Real, 1><<<blocks, 256, 0, st>>>(b); break;
-    case 2: fd_batch_kernel<Real, 2><<<blocks, 256, 0, st>>>(b); break;
-    case 3: fd_batch_kernel<Real, 3><<<blocks, 256, 0, st>>>(b); break;
-    case 4: fd_batch_kernel<Real, 4><<<blocks, 256, 0, st>>>(b); break;  // three-constant P stage from n
-    case 5: fd_batch_kernel<Real, 5><<<blocks, 256, 0, st>>>(b); break;  // ... and from n^P
+    case 0: launch_step_kernel(fd_batch_kernel<Real, 0>, blocks, 256, 0, st, b); break;
+    case 1: launch_step_kernel(fd_batch_kernel<Real, 1>, blocks, 256, 0, st, b); break;
+    case 2: launch_step_kernel(fd_batch_kernel<Real, 2>, blocks, 256, 0, st, b); break;
+    case 3: launch_step_kernel(fd_batch_kernel<Real, 3>, blocks, 256, 0, st, b); break;
+    case 4: launch_step_kernel(fd_batch_kernel<Real, 4>, blocks, 256, 0, st, b); break;  // three-constant P stage from n
+    case 5: launch_step_kernel(fd_batch_kernel<Real, 5>, blocks, 256, 0, st, b); break;  // ... and from n^P
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -1603,25 +1611,25 @@ template cudaError_t launch_fd_batch<float>(FDBatch<float>&, int, int, cudaStrea
 template <typename Real>
 cudaError_t launch_fd_predict(const FDChan<Real>& c, cudaStream_t st)
 {
-    fd_kernel<Real, 0><<<blocks_for(c.g.N), 256, 0, st>>>(c);
+    launch_step_kernel(fd_kernel<Real, 0>, blocks_for(c.g.N), 256, 0, st, c);
     return cudaGetLastError();
 }
 template <typename Real>
 cudaError_t launch_fd_correct(const FDChan<Real>& c, cudaStream_t st)
 {
-    fd_kernel<Real, 1><<<blocks_for(c.g.N), 256, 0, st>>>(c);
+    launch_step_kernel(fd_kernel<Real, 1>, blocks_for(c.g.N), 256, 0, st, c);
     return cudaGetLastError();
 }
 template <typename Real>
 cudaError_t launch_stress(const FDChan<Real>& c, cudaStream_t st)
 {
-    fd_kernel<Real, 2><<<blocks_for(c.g.N), 256, 0, st>>>(c);
+    launch_step_kernel(fd_kernel<Real, 2>, blocks_for(c.g.N), 256, 0, st, c);
     return cudaGetLastError();
 }
 template <typename Real>
 cudaError_t launch_force(const FDChan<Real>& c, cudaStream_t st)
 {
-    fd_kernel<Real, 3><<<blocks_for(c.g.N), 256, 0, st>>>(c);
+    launch_step_kernel(fd_kernel<Real, 3>, blocks_for(c.g.N), 256, 0, st, c);
     return cudaGetLastError();
 }
 template <typename Real>
@@ -1629,9 +1637,9 @@ cudaError_t launch_frank3_p(const FDChan<Real>& c, bool from_predictor, cudaStre
 {
     if (c.P3 == nullptr) return cudaErrorInvalidValue;
     if (from_predictor)
-        fd_kernel<Real, 5><<<blocks_for(c.g.N), 256, 0, st>>>(c);
+        launch_step_kernel(fd_kernel<Real, 5>, blocks_for(c.g.N), 256, 0, st, c);
     else
-        fd_kernel<Real, 4><<<blocks_for(c.g.N), 256, 0, st>>>(c);
+        launch_step_kernel(fd_kernel<Real, 4>, blocks_for(c.g.N), 256, 0, st, c);
     return cudaGetLastError();
 }
 
@@ -1641,9 +1649,9 @@ cudaError_t launch_fd_fused_a(const FDChan<Real>& c, const Real* nin, Real* nout
     cudaError_t e = prepare_fused<Real>();
     if (e != cudaSuccess) return e;
     if (c.solid != nullptr)
-        fused_a_kernel<Real, true><<<fused_tiles(c), kFusedThreads, fused_a_smem<Real>(), st>>>(c, nin, nout);
+        launch_step_kernel(fused_a_kernel<Real, true>, fused_tiles(c), kFusedThreads, fused_a_smem<Real>(), st, c, nin, nout);
     else
-        fused_a_kernel<Real, false><<<fused_tiles(c), kFusedThreads, fused_a_smem<Real>(), st>>>(c, nin, nout);
+        launch_step_kernel(fused_a_kernel<Real, false>, fused_tiles(c), kFusedThreads, fused_a_smem<Real>(), st, c, nin, nout);
     return cudaGetLastError();
 }
 
@@ -1653,9 +1661,9 @@ cudaError_t launch_relax(const FDChan<Real>& c, const Real* nin, Real* nout, cud
     cudaError_t e = prepare_fused<Real>();
     if (e != cudaSuccess) return e;
     if (c.solid != nullptr)
-        relax_kernel<Real, true><<<fused_tiles(c), kFusedThreads, relax_smem<Real>(), st>>>(c, nin, nout);
+        launch_step_kernel(relax_kernel<Real, true>, fused_tiles(c), kFusedThreads, relax_smem<Real>(), st, c, nin, nout);
     else
-        relax_kernel<Real, false><<<fused_tiles(c), kFusedThreads, relax_smem<Real>(), st>>>(c, nin, nout);
+        launch_step_kernel(relax_kernel<Real, false>, fused_tiles(c), kFusedThreads, relax_smem<Real>(), st, c, nin, nout);
     return cudaGetLastError();
 }
 
@@ -1663,7 +1671,7 @@ template <typename Real>
 cudaError_t launch_relax_end(const FDBatch<Real>& b, bool copy, cudaStream_t st)
 {
     if (b.count < 1 || b.count > kMaxBatch) return cudaErrorInvalidValue;
-    relax_end_kernel<Real><<<dim3(64, b.count), 256, 0, st>>>(b, copy);
+    launch_step_kernel(relax_end_kernel<Real>, dim3(64, b.count), 256, 0, st, b, copy);
     return cudaGetLastError();
 }
 
@@ -1674,11 +1682,11 @@ cudaError_t launch_fd_fused_b(const FDChan<Real>& c, const Real* nin, Real* ncop
     if (e != cudaSuccess) return e;
     if (diag != nullptr) {
         if (c.solid != nullptr || diag->n_tubes < 0 || diag->n_tubes > NH_MAX_TUBES) return cudaErrorInvalidValue;
-        fused_b_diag_kernel<Real><<<fused_tiles(c), kFusedThreads, fused_b_smem<Real>(), st>>>(c, nin, ncopy, *diag);
+        launch_step_kernel(fused_b_diag_kernel<Real>, fused_tiles(c), kFusedThreads, fused_b_smem<Real>(), st, c, nin, ncopy, *diag);
     } else if (c.solid != nullptr) {
-        fused_b_kernel<Real, true><<<fused_tiles(c), kFusedThreads, fused_b_smem<Real>(), st>>>(c, nin, ncopy);
+        launch_step_kernel(fused_b_kernel<Real, true>, fused_tiles(c), kFusedThreads, fused_b_smem<Real>(), st, c, nin, ncopy);
     } else {
-        fused_b_kernel<Real, false><<<fused_tiles(c), kFusedThreads, fused_b_smem<Real>(), st>>>(c, nin, ncopy);
+        launch_step_kernel(fused_b_kernel<Real, false>, fused_tiles(c), kFusedThreads, fused_b_smem<Real>(), st, c, nin, ncopy);
     }
     return cudaGetLastError();
 }
@@ -1709,17 +1717,17 @@ cudaError_t launch_fd_fused_batch(FDBatch<Real>& b, int stage, int grid, cudaStr
     for (int k = 0; k < b.count; ++k) solid = solid || b.ch[k].solid != nullptr;
     if (solid) {
         switch (stage) {
-        case 0: fused_batch_kernel<Real, 0, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        case 1: fused_batch_kernel<Real, 1, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        case 2: fused_batch_kernel<Real, 2, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        default: fused_batch_kernel<Real, 3, true><<<blocks, kFusedThreads, smem, st>>>(b); break;
+        case 0: launch_step_kernel(fused_batch_kernel<Real, 0, true>, blocks, kFusedThreads, smem, st, b); break;
+        case 1: launch_step_kernel(fused_batch_kernel<Real, 1, true>, blocks, kFusedThreads, smem, st, b); break;
+        case 2: launch_step_kernel(fused_batch_kernel<Real, 2, true>, blocks, kFusedThreads, smem, st, b); break;
+        default: launch_step_kernel(fused_batch_kernel<Real, 3, true>, blocks, kFusedThreads, smem, st, b); break;
         }
     } else {
         switch (stage) {
-        case 0: fused_batch_kernel<Real, 0, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        case 1: fused_batch_kernel<Real, 1, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        case 2: fused_batch_kernel<Real, 2, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
-        default: fused_batch_kernel<Real, 3, false><<<blocks, kFusedThreads, smem, st>>>(b); break;
+        case 0: launch_step_kernel(fused_batch_kernel<Real, 0, false>, blocks, kFusedThreads, smem, st, b); break;
+        case 1: launch_step_kernel(fused_batch_kernel<Real, 1, false>, blocks, kFusedThreads, smem, st, b); break;
+        case 2: launch_step_kernel(fused_batch_kernel<Real, 2, false>, blocks, kFusedThreads, smem, st, b); break;
+        default: launch_step_kernel(fused_batch_kernel<Real, 3, false>, blocks, kFusedThreads, smem, st, b); break;
         }
     }
     return cudaGetLastError();

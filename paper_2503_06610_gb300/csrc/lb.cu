@@ -541,6 +541,7 @@ __device__ __forceinline__ void lb_tile(const LBChan<Real, Store>& c, int tile, 
 template <typename Real, typename Store, bool Shifted, int Macro, int SPT, bool Solid = false>
 __global__ void __launch_bounds__(kLBThreads) lb_kernel(const LBChan<Real, Store> c)
 {
+    step_kernel_enter();
     lb_tile<Real, Store, Shifted, Macro, SPT, Solid, true>(c, blockIdx.x, gridDim.x);
 }
 
@@ -655,6 +656,7 @@ __device__ __forceinline__ void issue_row(const Store* fsrc, const Real* F, cons
 template <typename Real, typename Store, bool Shifted, int Macro>
 __global__ void __launch_bounds__(kRowMaxNx / kRowSPT, kRowMinBlocks) lb_rows_kernel(const LBChan<Real, Store> c)
 {
+    step_kernel_enter();
     static_assert(sizeof(Store) == 2 && Macro < 2, "row staging: 16-bit stores, no diagnostics partials");
     static_assert(kRowSPT == 4, "the staged rows are read as aligned 4-site chunks");
     static_assert(std::is_same<Real, float>::value, "16-bit stores compute in FP32");
@@ -825,8 +827,8 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
     if (resident <= 0) return cudaErrorNotReady;  // lb_rows_prepare was not run for this row length
     const int rows = c.g.ny * c.g.nz;
     const int blocks = rows < resident ? rows : resident;
-    lb_rows_kernel<Real, Store, Shifted, Macro>
-        <<<blocks, c.g.nx / kRowSPT, lb_rows_smem(c.g.nx, (int)sizeof(Store)), st>>>(c);
+    launch_step_kernel(lb_rows_kernel<Real, Store, Shifted, Macro>, blocks, c.g.nx / kRowSPT,
+                       lb_rows_smem(c.g.nx, (int)sizeof(Store)), st, c);
     return cudaGetLastError();
 }
 
@@ -835,6 +837,7 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
 template <typename Real, typename Store, bool Shifted, bool WriteMacro, int SPT, bool Solid = false>
 __global__ void __launch_bounds__(kLBThreads) lb_batch_kernel(const LBBatch<Real, Store> b)
 {
+    step_kernel_enter();
     const int total = b.prefix[b.count];
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
         int lo = 0, hi = b.count - 1;  // channel k with prefix[k] <= t < prefix[k+1]
@@ -909,7 +912,7 @@ cudaError_t launch_lb_spt(const LBChan<Real, Store>& c, int variant, cudaStream_
     }
     if (c.solid != nullptr) {  // obstacles: one site per thread, 256 threads
         if constexpr (Macro < 2)
-            lb_kernel<Real, Store, Shifted, Macro, 1, true><<<(c.g.N + 255) / 256, 256, 0, st>>>(c);
+            launch_step_kernel(lb_kernel<Real, Store, Shifted, Macro, 1, true>, (c.g.N + 255) / 256, 256, 0, st, c);
         else
             return cudaErrorInvalidValue;
         return cudaGetLastError();
@@ -917,11 +920,11 @@ cudaError_t launch_lb_spt(const LBChan<Real, Store>& c, int variant, cudaStream_
     const LBVariantShape v = kLBVariants[variant];
     const int blocks = lb_blocks(variant, c.g.N);
     if (v.spt == 4)
-        lb_kernel<Real, Store, Shifted, Macro, 4><<<blocks, v.threads, 0, st>>>(c);
+        launch_step_kernel(lb_kernel<Real, Store, Shifted, Macro, 4>, blocks, v.threads, 0, st, c);
     else if (v.spt == 2)
-        lb_kernel<Real, Store, Shifted, Macro, 2><<<blocks, v.threads, 0, st>>>(c);
+        launch_step_kernel(lb_kernel<Real, Store, Shifted, Macro, 2>, blocks, v.threads, 0, st, c);
     else
-        lb_kernel<Real, Store, Shifted, Macro, 1><<<blocks, v.threads, 0, st>>>(c);
+        launch_step_kernel(lb_kernel<Real, Store, Shifted, Macro, 1>, blocks, v.threads, 0, st, c);
     return cudaGetLastError();
 }
 
@@ -953,7 +956,7 @@ cudaError_t launch_lb_batch_spt(LBBatch<Real, Store>& b, int variant, int grid, 
         b.prefix[0] = 0;
         for (int k = 0; k < b.count; ++k) b.prefix[k + 1] = b.prefix[k] + (b.ch[k].g.N + 255) / 256;
         const int blocks = grid < b.prefix[b.count] ? grid : b.prefix[b.count];
-        lb_batch_kernel<Real, Store, Shifted, WriteMacro, 1, true><<<blocks, 256, 0, st>>>(b);
+        launch_step_kernel(lb_batch_kernel<Real, Store, Shifted, WriteMacro, 1, true>, blocks, 256, 0, st, b);
         return cudaGetLastError();
     }
     const LBVariantShape v = kLBVariants[variant];
@@ -964,11 +967,11 @@ cudaError_t launch_lb_batch_spt(LBBatch<Real, Store>& b, int variant, int grid, 
     }
     const int blocks = grid < b.prefix[b.count] ? grid : b.prefix[b.count];
     if (v.spt == 4)
-        lb_batch_kernel<Real, Store, Shifted, WriteMacro, 4><<<blocks, v.threads, 0, st>>>(b);
+        launch_step_kernel(lb_batch_kernel<Real, Store, Shifted, WriteMacro, 4>, blocks, v.threads, 0, st, b);
     else if (v.spt == 2)
-        lb_batch_kernel<Real, Store, Shifted, WriteMacro, 2><<<blocks, v.threads, 0, st>>>(b);
+        launch_step_kernel(lb_batch_kernel<Real, Store, Shifted, WriteMacro, 2>, blocks, v.threads, 0, st, b);
     else
-        lb_batch_kernel<Real, Store, Shifted, WriteMacro, 1><<<blocks, v.threads, 0, st>>>(b);
+        launch_step_kernel(lb_batch_kernel<Real, Store, Shifted, WriteMacro, 1>, blocks, v.threads, 0, st, b);
     return cudaGetLastError();
 }
 
