@@ -397,8 +397,8 @@ int nh_autotune(nh_ctx* ctx, void* stream, int* chosen);
 /* Use CUDA graphs for whole dt_fd blocks of at least 12 steps (default on). */
 int nh_set_graphs(nh_ctx* ctx, int on);
 
-/* Diagnostics folded into the step (default on): every LB launch that
- * writes u and rho (the steps that feed an FD update or end a call) also
+/* Diagnostics folded into the step (default on): the LB launch that ends a
+ * call also
  * leaves per-block FP64 sums of the stored populations, max |u| and the
  * non-finite count, so that nh_diagnostics of that state reads only the
  * director (the energy, |n| and the tube sums) instead of every population,
