@@ -210,7 +210,8 @@ struct nh_ctx {
     bool fields_set = false;
     bool has_solid = false;  // an obstacle mask is set (nh_set_solid)
     int64_t n_fluid = 0;     // fluid sites when has_solid
-    int cur = 0;
+    int cur = 0;    // population buffer that holds the current state
+    int phase = 0;  // LB steps since the fields were set, mod 2
     int64_t step = 0;
     std::string err;
     int n_tubes = 0;
@@ -224,6 +225,8 @@ struct nh_ctx {
     // whole dt_FD blocks by starting buffer, [1] with the diagnostics' sums
     cudaGraphExec_t graph[2][2] = {};
     int64_t graph_kernels[2][2] = {};
+    int graph_end[2][2] = {};     // buffer the block ends in
+    int graph_sums[2][2] = {};    // blocks of its LB sums
     int timing = 0;  // 0 off, 1 every kernel class, 2 the LB class only
     std::vector<TimedLaunch> pending;
     bool seg_open = false;
@@ -344,6 +347,8 @@ cudaEvent_t get_event(nh_ctx* c)
 
 // ------------------------------------------------------------ launch helpers
 
+Geom geom(const nh_ctx* c) { return Geom{c->p.nx, c->p.ny, c->p.nz, c->p.walls_z, c->p.anchoring, c->N}; }
+
 template <typename Real, typename Store>
 LBChan<Real, Store> lb_chan(nh_ctx* c, int src)
 {
@@ -359,7 +364,7 @@ LBChan<Real, Store> lb_chan(nh_ctx* c, int src)
     a.ctrl = c->at<unsigned>(c->L.absmax);
     a.part = nullptr;
     a.src = src;
-    a.g = Geom{c->p.nx, c->p.ny, c->p.nz, c->p.walls_z, c->p.anchoring, c->N};
+    a.g = geom(c);
     a.omega = Real(1.0 / c->p.tau);
     a.gx = Real(c->p.g[0]);
     a.gy = Real(c->p.g[1]);
@@ -379,7 +384,7 @@ FDChan<Real> fd_chan(nh_ctx* c)
     a.F = c->at<Real>(c->L.F);
     a.P3 = c->p.frank3 ? c->at<Real>(c->L.P3) : nullptr;
     a.solid = c->has_solid ? c->at<const unsigned char>(c->L.solid) : nullptr;
-    a.g = Geom{c->p.nx, c->p.ny, c->p.nz, c->p.walls_z, c->p.anchoring, c->N};
+    a.g = geom(c);
     const nh_params& p = c->p;
     a.p.K = Real(p.K);
     a.p.q0 = Real(p.q0);
@@ -492,6 +497,21 @@ int enqueue_lb(nh_ctx* c, int src, bool write_macro, cudaStream_t st, bool stale
         return timed(c, NH_KCLASS_LB, st, [&] { return launch_lb(a, sh, write_macro, c->lb_variant, st); }, "lb");
     }
     }
+}
+
+// Two LB steps in one launch: FP32 populations, no obstacles, large enough.
+bool pair_fits(const nh_ctx* c) { return c->p.storage == NH_STORE_F32 && !c->has_solid && lb_pair_valid(geom(c)); }
+bool pair_ok(const nh_ctx* c) { return lb_pair_pays(c->N) && pair_fits(c); }
+
+int enqueue_lb_pair(nh_ctx* c, bool write_macro, cudaStream_t st, bool sums)
+{
+    auto a = lb_chan<float, float>(c, c->cur);
+    if (write_macro && sums && fold_ok(c)) {
+        c->lbp_step = c->step + 2;
+        c->lbp_blocks = lb_pair_blocks(a.g);
+        a.part = c->at<double>(c->L.lbpart);
+    }
+    return timed(c, NH_KCLASS_LB, st, [&] { return launch_lb_pair(a, c->p.shifted != 0, write_macro, st); }, "lb_pair");
 }
 
 // Per-site predictor and corrector; with the three-constant energy each is
@@ -617,14 +637,36 @@ int enqueue_one_step(nh_ctx* c, bool last_of_call, cudaStream_t st, bool sums)
         r = enqueue_lb(c, c->cur, false, st, true);
         if (r) return r;
         c->cur ^= 1;
+        c->phase ^= 1;
         c->step = next;
         return NH_OK;
     }
     int r = enqueue_lb(c, c->cur, fd || last_of_call, st, false, sums);
     if (r) return r;
     c->cur ^= 1;
+    c->phase ^= 1;
     c->step = next;
     if (fd) return enqueue_fd_any(c, st);
+    return NH_OK;
+}
+
+// The next step, or the next two in one LB launch where no FD update falls
+// between them (nor, with paper_order, on the second); left: steps up to the
+// end of the call or block, ends_call: its last step ends the call.
+int enqueue_next(nh_ctx* c, int64_t left, bool ends_call, cudaStream_t st, bool sums, int64_t* done)
+{
+    const int dt = c->p.dt_fd;
+    const bool fd2 = (c->step + 2) % dt == 0;
+    if (left < 2 || (c->step + 1) % dt == 0 || (fd2 && c->p.paper_order) || !pair_ok(c)) {
+        *done = 1;
+        return enqueue_one_step(c, ends_call && left == 1, st, sums && left == 1);
+    }
+    *done = 2;
+    int r = enqueue_lb_pair(c, fd2 || (ends_call && left == 2), st, sums && left == 2);
+    if (r) return r;
+    c->cur ^= 1;
+    c->step += 2;
+    if (fd2) return enqueue_fd_any(c, st);
     return NH_OK;
 }
 
@@ -632,7 +674,7 @@ int enqueue_one_step(nh_ctx* c, bool last_of_call, cudaStream_t st, bool sums)
 // last step leaves the diagnostics' sums.
 int capture_block(nh_ctx* c, int src, bool sums)
 {
-    const int saved_cur = c->cur;
+    const int saved_cur = c->cur, saved_phase = c->phase;
     const int64_t saved_step = c->step;
     const int64_t saved_launches = c->launches;
     cudaStream_t cs = c->cap_stream;
@@ -641,11 +683,14 @@ int capture_block(nh_ctx* c, int src, bool sums)
     c->step = 0;
     c->lbp_step = -1;  // the captured steps decide by themselves (the caller sets it for the replayed block)
     int r = NH_OK;
-    for (int k = 0; k < c->p.dt_fd && r == NH_OK; ++k) r = enqueue_one_step(c, false, cs, sums);
+    for (int64_t left = c->p.dt_fd, done = 0; left > 0 && r == NH_OK; left -= done)
+        r = enqueue_next(c, left, false, cs, sums, &done);
+    const int end = c->cur;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     const int64_t kernels = c->launches - saved_launches;
     c->cur = saved_cur;
+    c->phase = saved_phase;
     c->step = saved_step;
     c->launches = saved_launches;
     if (r) {
@@ -659,6 +704,8 @@ int capture_block(nh_ctx* c, int src, bool sums)
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphInstantiate");
     c->graph[src][sums] = ex;
     c->graph_kernels[src][sums] = kernels;
+    c->graph_end[src][sums] = end;
+    c->graph_sums[src][sums] = c->lbp_blocks;
     return NH_OK;
 }
 
@@ -773,7 +820,7 @@ int enqueue_diag(nh_ctx* c, cudaStream_t st)
     a.rho = c->ws + c->L.rho;
     a.precision = c->p.precision;
     a.scale = c->at<const float>(c->L.scales) + c->cur;
-    a.g = Geom{c->p.nx, c->p.ny, c->p.nz, c->p.walls_z, c->p.anchoring, c->N};
+    a.g = geom(c);
     a.K = c->p.K;
     a.q0 = c->p.q0;
     a.W0 = c->p.W0;
@@ -816,6 +863,7 @@ struct BatchPlan {
     int variant = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     int64_t graph_kernels[2] = {0, 0};
+    int graph_end[2] = {0, 0};  // buffer a block that starts in buffer 0 / 1 ends in
 };
 
 std::mutex g_batch_mu;
@@ -862,7 +910,7 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
             return fail(nullptr, NH_EINVAL, "channel " + std::to_string(k) +
                                                 ": paper_order, lap_wide and n_from_rate are not supported in batches");
         if (c->device != c0->device) return fail(nullptr, NH_EINVAL, "channels must be on one device");
-        if (c->cur != c0->cur || c->step % c0->p.dt_fd != c0->step % c0->p.dt_fd)
+        if (c->phase != c0->phase || c->step % c0->p.dt_fd != c0->step % c0->p.dt_fd)
             return fail(nullptr, NH_EINVAL, "channels must be at the same step phase (step mod dt_fd, buffer parity)");
         for (int j = 0; j < k; ++j)
             if (ctxs[j] == c) return fail(nullptr, NH_EINVAL, "a context appears twice in the batch");
@@ -1043,18 +1091,46 @@ int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
     return NH_OK;
 }
 
-// One batched LB step (+ the batched FD update when the step count reaches a
-// multiple of dt_fd) for every channel of the plan.
-int batch_one_step(BatchPlan* b, bool last_of_call, cudaStream_t st)
+bool batch_pair_ok(const BatchPlan* b)
+{
+    double sites = 0;
+    for (const nh_ctx* c : b->ctxs) {
+        if (!pair_fits(c)) return false;
+        sites += c->N;
+    }
+    return lb_pair_pays(sites);
+}
+
+int batch_enqueue_lb_pair(BatchPlan* b, bool write_macro, cudaStream_t st)
 {
     nh_ctx* c0 = b->ctxs[0];
-    const int64_t next = c0->step + 1;
-    const bool fd = (next % c0->p.dt_fd) == 0;
-    int r = batch_enqueue_lb(b, fd || last_of_call, st);
+    const int n = (int)b->ctxs.size();
+    static thread_local LBBatch<float, float> batch;
+    for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
+        batch.count = std::min(kMaxBatch, n - g0);
+        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<float, float>(b->ctxs[g0 + k], b->ctxs[g0 + k]->cur);
+        int r = timed(c0, NH_KCLASS_LB, st,
+                      [&] { return launch_lb_pair_batch(batch, c0->p.shifted != 0, write_macro, st); }, "lb_pair_batch");
+        if (r) return r;
+    }
+    return NH_OK;
+}
+
+// The next batched LB step, or two in one launch (as enqueue_next), and the
+// batched FD update when the step count reaches a multiple of dt_fd, for every
+// channel of the plan; left: steps up to the end of the call or block.
+int batch_next(BatchPlan* b, int64_t left, bool ends_call, cudaStream_t st, int64_t* done)
+{
+    nh_ctx* c0 = b->ctxs[0];
+    const int dt = c0->p.dt_fd;
+    *done = left >= 2 && (c0->step + 1) % dt != 0 && batch_pair_ok(b) ? 2 : 1;
+    const bool fd = (c0->step + *done) % dt == 0, macro = fd || (ends_call && left == *done);
+    int r = *done == 2 ? batch_enqueue_lb_pair(b, macro, st) : batch_enqueue_lb(b, macro, st);
     if (r) return r;
     for (nh_ctx* c : b->ctxs) {
         c->cur ^= 1;
-        c->step += 1;
+        c->phase ^= *done & 1;
+        c->step += *done;
     }
     if (fd) return c0->p.precision == NH_FP64 ? batch_fd_typed<double>(b, st) : batch_fd_typed<float>(b, st);
     return NH_OK;
@@ -1063,10 +1139,11 @@ int batch_one_step(BatchPlan* b, bool last_of_call, cudaStream_t st)
 int batch_capture(BatchPlan* b, int parity)
 {
     nh_ctx* c0 = b->ctxs[0];
-    std::vector<int> cur;
+    std::vector<int> cur, phase;
     std::vector<int64_t> step;
     for (nh_ctx* c : b->ctxs) {
         cur.push_back(c->cur);
+        phase.push_back(c->phase);
         step.push_back(c->step);
         c->cur = parity;
         c->step = 0;
@@ -1076,7 +1153,9 @@ int batch_capture(BatchPlan* b, int parity)
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     int r = e == cudaSuccess ? NH_OK : cuda_fail(c0, e, "cudaStreamBeginCapture");
     if (r == NH_OK) {
-        for (int k = 0; k < c0->p.dt_fd && r == NH_OK; ++k) r = batch_one_step(b, false, cs);
+        for (int64_t left = c0->p.dt_fd, done = 0; left > 0 && r == NH_OK; left -= done)
+            r = batch_next(b, left, false, cs, &done);
+        b->graph_end[parity] = c0->cur;
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(cs, &g);
         if (r == NH_OK && e != cudaSuccess) r = cuda_fail(c0, e, "cudaStreamEndCapture");
@@ -1095,6 +1174,7 @@ int batch_capture(BatchPlan* b, int parity)
     c0->launches = saved_launches;
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
         b->ctxs[k]->cur = cur[k];
+        b->ctxs[k]->phase = phase[k];
         b->ctxs[k]->step = step[k];
     }
     return r;
@@ -1193,7 +1273,7 @@ int slab_validate(nh_ctx* const* slabs, int count)
         if (c->p.storage != NH_STORE_F64 && c->p.storage != NH_STORE_F32)
             return fail(nullptr, NH_EINVAL, "slabs exchange raw populations: F64 or F32 stores only");
         if (c->device != c0->device) return fail(nullptr, NH_EINVAL, "slabs must be on one device");
-        if (c->cur != c0->cur || c->step != c0->step)
+        if (c->phase != c0->phase || c->step != c0->step)
             return fail(nullptr, NH_EINVAL, "slabs must be at the same step and buffer parity");
         for (int j = 0; j < k; ++j)
             if (slabs[j] == c) return fail(nullptr, NH_EINVAL, "a context appears twice among the slabs");
@@ -1293,6 +1373,7 @@ int nh_slab_step(nh_ctx* const* slabs, int count, int64_t n_lb_steps, void* stre
         for (int k = 0; k < count; ++k) {
             if ((r = enqueue_lb(slabs[k], slabs[k]->cur, fd || last, st, false, last))) return fail(nullptr, r, slabs[k]->err);
             slabs[k]->cur ^= 1;
+            slabs[k]->phase ^= 1;
             slabs[k]->step = next;
         }
         if ((r = slab_copy(slabs, count, NH_HALO_POPULATIONS, nullptr, true, S, st))) return r;
@@ -1382,6 +1463,7 @@ int nh_bind_workspace(nh_ctx* c, void* dev_ptr, size_t bytes)
     c->bdp_step = -1;
     c->fields_set = false;
     c->cur = 0;
+    c->phase = 0;
     c->step = 0;
     return NH_OK;
 }
@@ -1414,6 +1496,7 @@ int nh_set_fields(nh_ctx* c, const double* n, const double* u, const double* rho
     NH_CUDA(c, cudaMemcpyAsync(c->ws + c->L.scales, ones, sizeof(ones), cudaMemcpyHostToDevice, st));
     NH_CUDA(c, cudaMemsetAsync(c->ws + c->L.absmax, 0, 4 * sizeof(float), st));
     c->cur = 0;
+    c->phase = 0;
     c->step = 0;
     if (c->p.precision == NH_FP64) {
         NH_CUDA(c, launch_load_fields<double>(dn, du, drho, c->at<double>(c->L.n), c->at<double>(c->L.u),
@@ -1597,12 +1680,14 @@ int nh_step(nh_ctx* c, int64_t n_lb_steps, void* stream)
             }
             NH_CUDA(c, cudaGraphLaunch(c->graph[c->cur][sums], st));
             c->launches += c->graph_kernels[c->cur][sums];
-            if (dt & 1) c->cur ^= 1;
+            const int sum_blocks = c->graph_sums[c->cur][sums];
+            c->cur = c->graph_end[c->cur][sums];
+            c->phase ^= dt & 1;
             c->step += dt;
             left -= dt;
             if (sums) {  // the block ends with a macro LB launch (an FD step)
                 c->lbp_step = c->step;
-                c->lbp_blocks = lb_blocks(c->lb_variant, c->N);
+                c->lbp_blocks = sum_blocks;
                 c->bdp_step = -1;
                 if (fd_fused(c)) {  // ... and its fused stress kernel left the director's partials
                     c->bdp_step = c->step;
@@ -1614,9 +1699,10 @@ int nh_step(nh_ctx* c, int64_t n_lb_steps, void* stream)
                 c->bdp_step = -1;
             }
         } else {
-            r = enqueue_one_step(c, left == 1, st, left == 1);
+            int64_t done = 1;
+            r = enqueue_next(c, left, true, st, true, &done);
             if (r) return r;
-            left -= 1;
+            left -= done;
         }
     }
     close_segment(c);
@@ -1647,7 +1733,10 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
     const int dt = c0->p.dt_fd;
     int64_t left = n_lb_steps;
     while (left > 0) {
-        if (use_block_graph(c0) && c0->step % dt == 0 && left >= dt) {
+        // (channels that stepped alone in pairs may sit in different buffers: direct launches then)
+        bool one_buffer = true;
+        for (nh_ctx* c : plan->ctxs) one_buffer = one_buffer && c->cur == c0->cur;
+        if (use_block_graph(c0) && one_buffer && c0->step % dt == 0 && left >= dt) {
             const int parity = c0->cur;
             if (!plan->graph[parity]) {
                 r = batch_capture(plan, parity);
@@ -1657,14 +1746,16 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
             if (e != cudaSuccess) return fail(nullptr, NH_ECUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
             c0->launches += plan->graph_kernels[parity];
             for (nh_ctx* c : plan->ctxs) {
-                if (dt & 1) c->cur ^= 1;
+                c->cur = plan->graph_end[parity];
+                c->phase ^= dt & 1;
                 c->step += dt;
             }
             left -= dt;
         } else {
-            r = batch_one_step(plan, left == 1, st);
+            int64_t done = 1;
+            r = batch_next(plan, left, true, st, &done);
             if (r) return fail(nullptr, r, "batch step: " + c0->err);
-            left -= 1;
+            left -= done;
         }
     }
     close_segment(c0);

@@ -20,6 +20,7 @@
 // leave per-block partial sums for the diagnostics (mass, max |u|, non-finite
 // count), so that the diagnostics of that state need not read the
 // populations, u and rho again.
+#include <algorithm>
 #include <type_traits>
 
 #include "nh_internal.cuh"
@@ -318,6 +319,35 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
     }
 }
 
+// The block's diagnostics partials: warp sums in the build's precision (FP64
+// arithmetic is scarce on GB300: a per-thread FP64 reduction would cost a third
+// of the launch), then FP64 across the block's warps in a fixed order.
+template <typename Real>
+__device__ __forceinline__ void lb_block_partials(Real m, Real mx, int bad, double* part, int tile, int ntiles)
+{
+    __shared__ double pred[32][3];
+    for (int o = 16; o > 0; o >>= 1) {
+        m += __shfl_xor_sync(0xffffffffu, m, o);
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    const int nb = __reduce_add_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0) {
+        pred[threadIdx.x >> 5][0] = (double)m;
+        pred[threadIdx.x >> 5][1] = (double)sqrt(mx);
+        pred[threadIdx.x >> 5][2] = (double)nb;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            v[0] += pred[w][0];
+            v[1] = fmax(v[1], pred[w][1]);
+            v[2] += pred[w][2];
+        }
+        for (int k = 0; k < 3; ++k) part[(size_t)k * ntiles + tile] = v[k];
+    }
+}
+
 // Macro: 0 = populations only; 1 = also u and rho; 2 = also the diagnostics'
 // block partials c.part[k * ntiles + tile] of k = 0: sum of the stored
 // post-collision populations, 1: max |u|, 2: sites with a non-finite u, rho
@@ -479,33 +509,7 @@ __device__ __forceinline__ void lb_tile(const LBChan<Real, Store>& c, int tile, 
             }
         }
     }
-    if constexpr (Partials) {
-        // block partials: warp sums in the build's precision (FP64 arithmetic is
-        // scarce on GB300: a per-thread FP64 reduction would cost a third of the
-        // launch), then FP64 across the block's warps in a fixed order
-        __shared__ double pred[kLBThreads / 32][3];
-        Real m = psum, mx = pmax;
-        for (int o = 16; o > 0; o >>= 1) {
-            m += __shfl_xor_sync(0xffffffffu, m, o);
-            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        }
-        const int nb = __reduce_add_sync(0xffffffffu, pbad);
-        if ((threadIdx.x & 31) == 0) {
-            pred[threadIdx.x >> 5][0] = (double)m;
-            pred[threadIdx.x >> 5][1] = (double)sqrt(mx);
-            pred[threadIdx.x >> 5][2] = (double)nb;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double v[3] = {0.0, 0.0, 0.0};
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                v[0] += pred[w][0];
-                v[1] = fmax(v[1], pred[w][1]);
-                v[2] += pred[w][2];
-            }
-            for (int k = 0; k < 3; ++k) c.part[(size_t)k * ntiles + tile] = v[k];
-        }
-    }
+    if constexpr (Partials) lb_block_partials(psum, pmax, pbad, c.part, tile, ntiles);
     if (kScaled) {
         // In-kernel scale controller: block max -> global running max; the last
         // block to finish records the scale of the buffer just written and sets
@@ -829,6 +833,320 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
     const int blocks = rows < resident ? rows : resident;
     launch_step_kernel(lb_rows_kernel<Real, Store, Shifted, Macro>, blocks, c.g.nx / kRowSPT,
                        lb_rows_smem(c.g.nx, (int)sizeof(Store)), st, c);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ FP32 stores: two steps in one pass
+//
+// At 164 bytes a site and step the FP32 sweep runs at the HBM limit, so a second
+// step has to come from on-chip data.  A block takes a tile of 32 x rows columns
+// (7 rows at most) and marches up its layers.  For every layer it computes the
+// first step on the tile and a ring of one site around it, straight from global
+// memory, and keeps the post-collision populations in shared memory; the second
+// step of the layer below then pulls from there and writes global memory: 82
+// bytes a site and step, at the price of repeating the first step on the ring
+// and on one layer at each end of a march.  Populations are kept only as long as
+// a pull can ask for them: the five that move up (e_z = +1) for three layers, the
+// nine with e_z = 0 for two, the five that move down for two (the second for the
+// bounce-back at the lower plate), 43 floats a point.  A thread's next layer is
+// loaded into registers while the second step runs.  Both steps call
+// lb_collide_site, and the force is the same in both (it changes only in FD
+// updates): bit-identical to two single steps.
+//
+// Bound by issue (110 M warp instructions a pass at 256x256x64, a quarter of them
+// 64-bit addresses) and by the two barriers a layer.  Two steps at 256x256x64:
+// 155 us, two single steps 200 us.  Seven rows leave 96 registers to each of two
+// blocks per SM, so that the prefetch does not spill; with eight rows (80
+// registers) it does (181 us), without it a layer waits for its loads (158 us).
+// All tiles march up together, so that what neighbours share is read from HBM
+// once: cutting the layers of all tiles evenly among the blocks read it three
+// times (246 us).  Staging the source rows by 16-byte cp.async (192 us) or by bulk
+// copies of 160 bytes (276 us), two sites a thread on the paired FP32
+// instructions (200 us: half the instructions, but too few warps) and a fourth
+// slot that saves a barrier (193 us) were slower.
+constexpr int kPairTX = 32, kPairTY = 7;
+constexpr int kPairHX = kPairTX + 2, kPairHY = kPairTY + 2, kPairPts = kPairHX * kPairHY;
+constexpr int kPairThreads = (kPairPts + 31) / 32 * 32;
+constexpr int kPairSmem = 43 * kPairPts * (int)sizeof(float);
+constexpr int kPairPerSM = 2;
+
+struct PairGrid {
+    int tx, ty, rows, zc, chunks;  // tiles in x and y, rows of a tile, layers per chunk, chunks
+};
+__host__ __device__ __forceinline__ int pair_blocks(const PairGrid& p) { return p.tx * p.ty * p.chunks; }
+
+__device__ __forceinline__ float ld_byte(const float* base, unsigned off)
+{
+    return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + off);
+}
+__device__ __forceinline__ void st_byte(float* base, unsigned off, float v)
+{
+    *reinterpret_cast<float*>(reinterpret_cast<char*>(base) + off) = v;
+}
+
+template <bool Shifted, int Macro>
+__device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, const PairGrid& pg, int tile, int ntiles)
+{
+    NH_D3Q19_TABLES
+    // index of direction i within its e_z group
+    constexpr int GI[19] = {0, 1, 2, 3, 4, 0, 0, 5, 6, 7, 8, 1, 1, 2, 2, 3, 3, 4, 4};
+    extern __shared__ float pair_smem[];
+    float* up = pair_smem;                  // 3 slots x 5: e_z = +1 of plane p in slot p mod 3
+    float* flat = up + 15 * kPairPts;       // 2 slots x 9: e_z = 0
+    float* down = flat + 18 * kPairPts;     // 2 slots x 5: e_z = -1
+    const Geom& g = c.g;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N;
+    const int t = tile / pg.tx, rows = pg.rows, nown = kPairTX * rows;
+    const int x0 = (tile - t * pg.tx) * kPairTX, y0 = (t % pg.ty) * rows;
+    const int zb = (t / pg.ty) * pg.zc, ze = min(zb + pg.zc, nz);
+    const int tid = threadIdx.x;
+    const bool own = tid < nown, point = tid < kPairHX * (rows + 2);
+    int hx, hy;  // the thread's point in the tile with its ring: own points first, then two rows, then two columns
+    if (own) {
+        hx = 1 + tid % kPairTX;
+        hy = 1 + tid / kPairTX;
+    } else {
+        const int e = tid - nown;
+        if (e < 2 * kPairHX) {
+            hy = e < kPairHX ? 0 : rows + 1;
+            hx = e < kPairHX ? e : e - kPairHX;
+        } else {
+            const int j = e - 2 * kPairHX;
+            hy = min(1 + (j >> 1), rows);
+            hx = (j & 1) ? kPairHX - 1 : 0;
+        }
+    }
+    const int i1 = hx + kPairHX * hy;
+    const bool active = own && x0 + hx - 1 < nx && y0 + hy - 1 < ny;
+    // wrapped coordinates of the point (a ragged tile's outer points repeat inner ones) and, in bytes, the
+    // x and row parts of its neighbours' places in a plane
+    const int x = (x0 + hx - 1 + nx) % nx, y = (y0 + hy - 1 + ny) % ny;
+    const unsigned bx[3] = {4u * (x == 0 ? nx - 1 : x - 1), 4u * x, 4u * (x == nx - 1 ? 0 : x + 1)};
+    const unsigned by[3] = {4u * nx * (y == 0 ? ny - 1 : y - 1), 4u * nx * y, 4u * nx * (y == ny - 1 ? 0 : y + 1)};
+    const unsigned here = bx[1] + by[1];
+    const int plane = nx * ny;
+
+    // the 19 populations that arrive at the point's site of layer p, and its force
+    auto pull = [&](int p, float (&f)[19], float (&F)[3]) {
+        if (p > 0 && p < nz - 1) {
+            const float* fz = c.fsrc + (size_t)plane * p;
+#pragma unroll
+            for (int i = 0; i < 19; ++i)
+                f[i] = ld_byte(fz, 4u * (unsigned)(i * N - EZ[i] * plane) + (bx[1 - EX[i]] + by[1 - EY[i]]));
+        } else {  // the lowest and the highest layer: plates, or periodic in z
+            const int z = g.walls ? p : wrap_p(p, nz);
+            const int zl = z == 0 ? nz - 1 : z - 1, zh = z == nz - 1 ? 0 : z + 1;
+            const bool bb_lo = g.walls && z == 0, bb_hi = g.walls && z == nz - 1;
+#pragma unroll
+            for (int i = 0; i < 19; ++i) {
+                const bool bb = (EZ[i] > 0 && bb_lo) || (EZ[i] < 0 && bb_hi);
+                const float* fz = c.fsrc + (size_t)(bb ? OPP[i] : i) * N +
+                                  (size_t)plane * (bb || EZ[i] == 0 ? z : (EZ[i] > 0 ? zl : zh));
+                f[i] = ld_byte(fz, bb ? here : bx[1 - EX[i]] + by[1 - EY[i]]);
+            }
+            p = z;
+        }
+        const float* Fz = c.F + (size_t)plane * p;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) F[a] = ld_byte(Fz, 4u * (unsigned)(a * N) + here);
+    };
+    auto exists = [&](int p) { return !g.walls || (p >= 0 && p < nz); };
+
+    float psum = 0.f, pmax = 0.f, none = 0.f;
+    int pbad = 0, inone = 0;
+    float f[19], F[3], Fz[3] = {0.f, 0.f, 0.f};  // Fz: the force at the own point one layer below
+    if (point && exists(zb - 1)) pull(zb - 1, f, F);
+    int su = 0;  // slot of plane p in `up`; planes p - 1, p - 2 precede it cyclically
+    for (int p = zb - 1; p <= ze; ++p) {
+        if (point && exists(p)) {
+            float fo[19];
+            lb_collide_site<float, float, Shifted, 0>(c, 0, f, fo, F[0], F[1], F[2], 1.f, 1.f, none, none, inone, none);
+            float* dst[3] = {down + (p & 1) * (5 * kPairPts) + i1, flat + (p & 1) * (9 * kPairPts) + i1,
+                             up + su * (5 * kPairPts) + i1};
+#pragma unroll
+            for (int i = 0; i < 19; ++i) dst[EZ[i] + 1][GI[i] * kPairPts] = fo[i];
+        }
+        const float Fn[3] = {F[0], F[1], F[2]};
+        if (point && p < ze && exists(p + 1)) pull(p + 1, f, F);  // in flight during the second step
+        __syncthreads();
+        const int z = p - 1;
+        const bool second = active && z >= zb;
+        float h[19];
+        if (second) {
+            const int s1 = su == 0 ? 2 : su - 1, s2 = s1 == 0 ? 2 : s1 - 1;  // slots of planes z, z - 1
+            const float* src[3] = {down + (p & 1) * (5 * kPairPts) + i1, flat + (z & 1) * (9 * kPairPts) + i1,
+                                   up + s2 * (5 * kPairPts) + i1};
+            if (!g.walls || (z > 0 && z < nz - 1)) {
+#pragma unroll
+                for (int i = 0; i < 19; ++i) h[i] = src[1 + EZ[i]][GI[i] * kPairPts - EX[i] - kPairHX * EY[i]];
+            } else {  // half-way bounce-back: the site's own opposite populations
+                const float* low = down + (z & 1) * (5 * kPairPts) + i1;
+                const float* high = up + s1 * (5 * kPairPts) + i1;
+#pragma unroll
+                for (int i = 0; i < 19; ++i) {
+                    const int back = GI[OPP[i]] * kPairPts;
+                    if (EZ[i] > 0 && z == 0)
+                        h[i] = low[back];
+                    else if (EZ[i] < 0 && z == nz - 1)
+                        h[i] = high[back];
+                    else
+                        h[i] = src[1 + EZ[i]][GI[i] * kPairPts - EX[i] - kPairHX * EY[i]];
+                }
+            }
+        }
+        __syncthreads();  // the slots of planes p - 2 (up) and p - 1 (the others) may be overwritten
+        if (second) {
+            float ho[19];
+            lb_collide_site<float, float, Shifted, Macro>(c, (int)(here >> 2) + plane * z, h, ho, Fz[0], Fz[1], Fz[2], 1.f,
+                                                          1.f, psum, pmax, pbad, none);
+            float* fz = c.fdst + (size_t)plane * z;
+#pragma unroll
+            for (int i = 0; i < 19; ++i) st_byte(fz, 4u * (unsigned)(i * N) + here, ho[i]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Fz[a] = Fn[a];
+        su = su == 2 ? 0 : su + 1;
+    }
+    if constexpr (Macro == 2) lb_block_partials(psum, pmax, pbad, c.part, tile, ntiles);
+}
+
+template <bool Shifted, int Macro>
+__global__ void __launch_bounds__(kPairThreads, kPairPerSM) lb_pair_kernel(const LBChan<float, float> c, const PairGrid pg)
+{
+    step_kernel_enter();
+    lb_pair_tile<Shifted, Macro>(c, pg, blockIdx.x, gridDim.x);
+}
+
+// Batch: one tile of one channel per block.
+struct PairGridBatch {
+    PairGrid pg[kMaxBatch];
+};
+template <bool Shifted, int Macro>
+__global__ void __launch_bounds__(kPairThreads, kPairPerSM) lb_pair_batch_kernel(const LBBatch<float, float> b, const PairGridBatch pb)
+{
+    step_kernel_enter();
+    const int t = blockIdx.x;
+    int lo = 0, hi = b.count - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (b.prefix[mid] <= t)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    lb_pair_tile<Shifted, Macro>(b.ch[lo], pb.pg[lo], t - b.prefix[lo], b.prefix[lo + 1] - b.prefix[lo]);
+}
+
+// Rows of a tile and layers per chunk: the blocks run in waves of two per SM, and
+// a block takes (layers + 2) x (points of a layer); the split with the least sum
+// (256x256x64: 296 blocks of 7 rows and 64 layers).
+PairGrid pair_split(const Geom& g, int rows, int chunks)
+{
+    PairGrid p{(g.nx + kPairTX - 1) / kPairTX, (g.ny + rows - 1) / rows, rows, (g.nz + chunks - 1) / chunks, 0};
+    p.chunks = (g.nz + p.zc - 1) / p.zc;
+    return p;
+}
+PairGrid pair_grid(const Geom& g)
+{
+    constexpr int kSlots = kPairPerSM * 152;
+    PairGrid best = pair_split(g, kPairTY, 1);
+    long long cost = -1;
+    for (int rows = kPairTY; rows >= 4; --rows)
+        for (int n = 1; n <= g.nz && n <= 64; ++n) {
+            const PairGrid p = pair_split(g, rows, n);
+            const long long w = (long long)((pair_blocks(p) + kSlots - 1) / kSlots) * (p.zc + 2) * (rows + 2);
+            if (cost < 0 || w < cost) {
+                cost = w;
+                best = p;
+            }
+        }
+    return best;
+}
+
+// From 7.5e5 sites, where the two population buffers no longer stay in L2 (16 LB
+// steps and an FD update, single steps | pairs, us: 128x128x32 195 | 218,
+// 160x128x32 275 | 288, 128x128x48 337 | 323, 256x256x12 343 | 315, 180x140x32 355 |
+// 355, 151x117x45 407 | 349, 256x256x64 1815 | 1446).
+constexpr double kPairMinSites = 7.5e5;
+bool lb_pair_pays(double sites) { return sites >= kPairMinSites; }
+// 32-bit byte offsets within the populations; no more blocks than the diagnostics' partials have room for
+bool lb_pair_valid(const Geom& g)
+{
+    return 19.0 * 4.0 * g.N < 4294967296.0 && pair_blocks(pair_grid(g)) <= (g.N + 127) / 128;
+}
+int lb_pair_blocks(const Geom& g) { return pair_blocks(pair_grid(g)); }
+
+namespace {
+
+template <bool Shifted, int Macro>
+cudaError_t pair_attr()
+{
+    cudaError_t e = cudaFuncSetAttribute(lb_pair_kernel<Shifted, Macro>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kPairSmem);
+    if constexpr (Macro < 2)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(lb_pair_batch_kernel<Shifted, Macro>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kPairSmem);
+    return e;
+}
+cudaError_t prepare_pair()
+{
+    static bool done = false;  // the attribute is per function; setting it twice is harmless
+    if (done) return cudaSuccess;
+    cudaError_t e = pair_attr<true, 0>();
+    if (e == cudaSuccess) e = pair_attr<true, 1>();
+    if (e == cudaSuccess) e = pair_attr<true, 2>();
+    if (e == cudaSuccess) e = pair_attr<false, 0>();
+    if (e == cudaSuccess) e = pair_attr<false, 1>();
+    if (e == cudaSuccess) e = pair_attr<false, 2>();
+    done = e == cudaSuccess;
+    return e;
+}
+
+template <bool Shifted>
+void launch_pair(const LBChan<float, float>& c, const PairGrid& pg, int macro, cudaStream_t st)
+{
+    const int blocks = pair_blocks(pg), threads = (kPairHX * (pg.rows + 2) + 31) / 32 * 32;
+    if (macro == 0)
+        launch_step_kernel(lb_pair_kernel<Shifted, 0>, blocks, threads, kPairSmem, st, c, pg);
+    else if (macro == 1)
+        launch_step_kernel(lb_pair_kernel<Shifted, 1>, blocks, threads, kPairSmem, st, c, pg);
+    else
+        launch_step_kernel(lb_pair_kernel<Shifted, 2>, blocks, threads, kPairSmem, st, c, pg);
+}
+
+}  // namespace
+
+cudaError_t launch_lb_pair(const LBChan<float, float>& c, bool shifted, bool write_macro, cudaStream_t st)
+{
+    if (c.solid != nullptr || c.Fu != nullptr || !lb_pair_valid(c.g)) return cudaErrorInvalidValue;
+    cudaError_t e = prepare_pair();
+    if (e != cudaSuccess) return e;
+    const int macro = write_macro ? (c.part != nullptr ? 2 : 1) : 0;
+    if (shifted)
+        launch_pair<true>(c, pair_grid(c.g), macro, st);
+    else
+        launch_pair<false>(c, pair_grid(c.g), macro, st);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, bool shifted, bool write_macro, cudaStream_t st)
+{
+    if (b.count < 1 || b.count > kMaxBatch) return cudaErrorInvalidValue;
+    cudaError_t e = prepare_pair();
+    if (e != cudaSuccess) return e;
+    PairGridBatch pb;
+    b.prefix[0] = 0;
+    for (int k = 0; k < b.count; ++k) {
+        if (b.ch[k].solid != nullptr || !lb_pair_valid(b.ch[k].g)) return cudaErrorInvalidValue;
+        pb.pg[k] = pair_split(b.ch[k].g, kPairTY, b.count >= 8 ? 1 : (b.ch[k].g.nz + 15) / 16);
+        b.prefix[k + 1] = b.prefix[k] + pair_blocks(pb.pg[k]);
+    }
+    auto go = [&](auto kernel) { launch_step_kernel(kernel, b.prefix[b.count], kPairThreads, kPairSmem, st, b, pb); };
+    if (shifted)
+        write_macro ? go(lb_pair_batch_kernel<true, 1>) : go(lb_pair_batch_kernel<true, 0>);
+    else
+        write_macro ? go(lb_pair_batch_kernel<false, 1>) : go(lb_pair_batch_kernel<false, 0>);
     return cudaGetLastError();
 }
 
