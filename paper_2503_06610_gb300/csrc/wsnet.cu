@@ -8,8 +8,8 @@
 // ansatz, n = normalise(n_ansatz + delta).  Convolutions are cross-correlations,
 // periodic in x and y and zero-padded in z.
 //
-// Layouts: activations are channels-last BF16 [batch][z][y][x][c]; activation
-// gradients are channels-last FP32.  Parameters are one flat FP32 vector, layer
+// Layouts: activations are channels-last BF16 [batch][z][y][x][c]; gradients of
+// pre-activations are channels-last BF16, of pooled and upsampled tensors FP32.  Parameters are one flat FP32 vector, layer
 // by layer W[tap][cout][cin] (tap = 9 kz + 3 ky + kx) then bias[cout]; the head
 // is W[3][16] then bias[3].
 //
@@ -97,8 +97,12 @@ struct Dims {
 // waits for its copies and frees its TMEM.
 //
 // Forward: input = the layer's sources, D + bias, ReLU, BF16 rows.  Data gradient
-// (Flip): input = the pre-activation gradient, taps mirrored, transposed weights,
-// FP32 rows overwritten in dst1 (channels below n1) or added to dst2.
+// (Flip): input = the pre-activation gradient, taps mirrored, transposed weights.
+// Where the source is another convolution's output (mask), the epilogue makes that
+// layer's pre-activation gradient at once -- masked by its ReLU, BF16 -- and its
+// bias gradient, which spares the FP32 gradient's way through memory (a separate
+// pass took 30 us a layer of 8 x 64 x 64 x 32 voxels); else FP32 rows go to dst1
+// (channels below n1) and dst2.
 
 struct ConvTc {
     const bf16* src1;
@@ -112,9 +116,12 @@ struct ConvTc {
     int zc;            // planes per chunk
     const float* bias; // forward: [n]
     bf16* out;         // forward: [vox][n]
-    float* dst1;       // data gradient: [vox][n1], overwritten
+    const bf16* mask;  // data gradient: the source's activations [vox][n], or null
+    bf16* gp;          // with mask: pre-activation gradient of the source's layer [vox][n]
+    float* gb;         // with mask: its bias gradient [n] (accumulated)
+    float* dst1;       // data gradient without mask: [vox][n1]
     int n1;
-    float* dst2;       // data gradient: [vox][n - n1], accumulated
+    float* dst2;       // data gradient without mask: [vox][n - n1]
     int* status;       // set to 1 when a bounded wait expires
 };
 
@@ -123,7 +130,7 @@ constexpr int kTcThreads = 128;
 constexpr int kTcX = 8, kTcY = 16;                                // output voxels of a plane step
 constexpr int kTcHX = kTcX + 2, kTcHY = kTcY + 2, kTcHalo = kTcHX * kTcHY;
 constexpr int kTcRing = 4;
-inline size_t tc_smem(int K, int NB) { return (size_t)K * 2 * (kTcRing * kTcHalo + 27 * NB) + 64; }
+inline size_t tc_smem(int K, int NB) { return (size_t)K * 2 * (kTcRing * kTcHalo + 27 * NB) + 64 + NB * sizeof(float); }
 constexpr size_t kTcMaxSmem = 227 * 1024;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -179,10 +186,35 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// g = 0 where the activation y (8 BF16 values) is not positive; and 8 FP32 values as BF16.
+__device__ __forceinline__ void relu_mask(float g[8], const uint4 y)
+{
+    const __nv_bfloat162* yh = reinterpret_cast<const __nv_bfloat162*>(&y);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!(__low2float(yh[k]) > 0.f)) g[2 * k] = 0.f;
+        if (!(__high2float(yh[k]) > 0.f)) g[2 * k + 1] = 0.f;
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float g[8])
+{
+    return make_uint4(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), pack_bf16(g[4], g[5]), pack_bf16(g[6], g[7]));
+}
+__device__ __forceinline__ void unpack8(const uint4 y, float v[8])
+{
+    const __nv_bfloat162* yh = reinterpret_cast<const __nv_bfloat162*>(&y);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[2 * k] = __low2float(yh[k]);
+        v[2 * k + 1] = __high2float(yh[k]);
+    }
+}
+
 template <int NB, bool Flip>
 __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
 {
     extern __shared__ __align__(128) unsigned char tc_smem_raw[];
+    nh::step_kernel_enter();
     const int K = a.c1 + a.c2, kb = K / 8;  // 16-byte channel groups
     constexpr uint32_t kGroup = kTcHalo * 16;              // one channel group of a plane
     const uint32_t plane_bytes = (uint32_t)kb * kGroup;
@@ -190,6 +222,8 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
     const uint32_t ring = smem_u32(tc_smem_raw), wbase = ring + kTcRing * plane_bytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem_raw + kTcRing * plane_bytes + 27 * tap_bytes);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
+    float* bshared = reinterpret_cast<float*>(bars + 8);  // bias gradient of the CTA's voxels (with mask)
+    if (Flip && threadIdx.x < NB) bshared[threadIdx.x] = 0.f;
     constexpr uint32_t kCols = 2 * NB;  // two accumulators: 32 or 64 columns
     static_assert(NB == 16 || NB == 32, "TMEM columns are allocated in powers of two, at least 32");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -257,6 +291,9 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
     const int row = warp * 32 + lane;
     const int vx = x0 + (row & 7), vy = y0 + (row >> 3);
     const bool inside = vx < d.nx && vy < d.ny;
+    float bsum[Flip ? NB : 1];  // bias gradient of this thread's voxels (with mask)
+#pragma unroll
+    for (int i = 0; i < (Flip ? NB : 1); ++i) bsum[i] = 0.f;
     auto epilogue = [&](int z) {
         const uint32_t acc0 = tmem + (uint32_t)(((z - z0) & 1) * NB) + ((uint32_t)(warp * 32) << 16);
         const size_t v = (size_t)batch * d.nvox + vx + (size_t)d.nx * (vy + (size_t)d.ny * z);
@@ -275,21 +312,23 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
                 uint4* dst = reinterpret_cast<uint4*>(a.out + v * a.n + n0 + c0);
                 dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                 dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-            } else if (n0 + c0 < a.n1) {
-                float4* dst = reinterpret_cast<float4*>(a.dst1 + v * a.n1 + n0 + c0);
+            } else if (a.mask != nullptr) {
+                const uint4* m = reinterpret_cast<const uint4*>(a.mask + v * a.n + n0 + c0);
+                uint4* dst = reinterpret_cast<uint4*>(a.gp + v * a.n + n0 + c0);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float* g = acc + 8 * h;
+                    relu_mask(g, __ldg(m + h));
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) bsum[c0 + 8 * h + i] += g[i];
+                    dst[h] = pack8(g);
+                }
+            } else {
+                const bool first = n0 + c0 < a.n1;
+                float4* dst = reinterpret_cast<float4*>(first ? a.dst1 + v * a.n1 + n0 + c0
+                                                              : a.dst2 + v * (a.n - a.n1) + (n0 + c0 - a.n1));
 #pragma unroll
                 for (int i = 0; i < 4; ++i) dst[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-            } else {
-                float4* dst = reinterpret_cast<float4*>(a.dst2 + v * (a.n - a.n1) + (n0 + c0 - a.n1));
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float4 o = dst[i];
-                    o.x += acc[4 * i];
-                    o.y += acc[4 * i + 1];
-                    o.z += acc[4 * i + 2];
-                    o.w += acc[4 * i + 3];
-                    dst[i] = o;
-                }
             }
         }
     };
@@ -346,9 +385,27 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
         if (ok) epilogue(z1 - 1);
     }
     if (!ok && lane == 0) atomicExch(a.status, 1);
+    if constexpr (Flip) {
+        if (a.mask != nullptr) {
+            // halve the channels a lane holds as the lanes that add to it double: after the steps lane l has the
+            // warp's sum of channel l mod NB (of NB 16, lanes l and l + 16 each half of it)
+#pragma unroll
+            for (int w = NB / 2; w > 0; w >>= 1) {
+                const bool high = (lane & w) != 0;
+#pragma unroll
+                for (int i = 0; i < w; ++i) {
+                    const float send = high ? bsum[i] : bsum[i + w], keep = high ? bsum[i + w] : bsum[i];
+                    bsum[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+                }
+            }
+            atomicAdd(&bshared[lane & (NB - 1)], bsum[0]);
+        }
+    }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
+    if constexpr (Flip)
+        if (a.mask != nullptr && tid < NB) atomicAdd(a.gb + n0 + tid, bshared[tid]);
     if (warp == 0) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
     }
@@ -356,9 +413,10 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
 
 // Launch over every plane tile of the level.  NB = 32 where two such weight
 // sets fit an SM (K <= 32), else 16: more CTAs on the coarse levels, whose wide
-// layers have few voxels.  A chunk is at most 8 planes (two of its ten input
-// planes are read twice), fewer when the level has too few tiles for four CTAs
-// per SM.
+// layers have few voxels.  Planes per chunk: the CTAs run in waves of as many as
+// an SM holds (shared memory, TMEM columns), and a chunk loads two planes beyond
+// its own; the split with the least waves x (planes + 2).  (8 planes of
+// 8 x 64 x 64 x 32 voxels made 1024 CTAs of which 912 are resident.)
 template <bool Flip>
 cudaError_t launch_conv_tc(ConvTc a, cudaStream_t st)
 {
@@ -375,13 +433,22 @@ cudaError_t launch_conv_tc(ConvTc a, cudaStream_t st)
     const int NB = a.n % 32 == 0 && K <= 32 ? 32 : 16;
     if (K % 16 || a.n % 16 || a.c1 % 8 || tc_smem(K, NB) > kTcMaxSmem) return cudaErrorInvalidValue;
     const int cols = ((a.d.nx + kTcX - 1) / kTcX) * ((a.d.ny + kTcY - 1) / kTcY) * a.d.batch;
-    const int zc = (int)((int64_t)cols * a.d.nz * (a.n / NB) / (4 * 152));
-    a.zc = std::min(std::max(zc, 1), std::min(8, a.d.nz));
+    const int resident = 152 * std::min((int)(kTcMaxSmem / (tc_smem(K, NB) + 1024)), 512 / (2 * NB));
+    int64_t best = -1;
+    for (int n = 1; n <= a.d.nz; ++n) {
+        const int zc = (a.d.nz + n - 1) / n;
+        const int64_t blocks = (int64_t)cols * ((a.d.nz + zc - 1) / zc) * (a.n / NB);
+        const int64_t cost = (blocks + resident - 1) / resident * (zc + 2);
+        if (best < 0 || cost < best) {
+            best = cost;
+            a.zc = zc;
+        }
+    }
     const dim3 grid(cols * ((a.d.nz + a.zc - 1) / a.zc), a.n / NB);
     if (NB == 32)
-        conv_tc_kernel<32, Flip><<<grid, kTcThreads, tc_smem(K, NB), st>>>(a);
+        nh::launch_step_kernel(conv_tc_kernel<32, Flip>, grid, kTcThreads, tc_smem(K, NB), st, a);
     else
-        conv_tc_kernel<16, Flip><<<grid, kTcThreads, tc_smem(K, NB), st>>>(a);
+        nh::launch_step_kernel(conv_tc_kernel<16, Flip>, grid, kTcThreads, tc_smem(K, NB), st, a);
     return cudaGetLastError();
 }
 
@@ -429,6 +496,7 @@ __device__ __forceinline__ void ldm_x4_trans(uint32_t addr, uint32_t r[4])
 __global__ void __launch_bounds__(kWThreads, kWBlocksPerSM) conv_bwd_w_kernel(const ConvBwdW a)
 {
     extern __shared__ __align__(128) unsigned char w_smem[];
+    nh::step_kernel_enter();
     const uint32_t smem0 = smem_u32(w_smem);
     const int cin = a.c1 + a.c2;
     const int nci = cin / 16;
@@ -544,107 +612,119 @@ __global__ void __launch_bounds__(kWThreads, kWBlocksPerSM) conv_bwd_w_kernel(co
         }
 }
 
-// Gradient of the pre-activation, once per layer: gp = BF16(gout masked by
-// the ReLU, out > 0), the operand of both convolution gradients; and the
-// bias gradient gb[co] += sum_v of the masked gout (FP32).  A thread takes
-// 8-channel groups of voxels (32-byte gout loads, 16-byte stores); the grid
-// stride is a multiple of cout/8, so a thread's group -- and its 8 bias
-// partials -- stay fixed; the block sums them in shared memory and adds
-// them to gb with one atomic per channel.
-__global__ void __launch_bounds__(256) grad_prep_kernel(const float* __restrict__ gout, const bf16* __restrict__ out,
-                                                        bf16* __restrict__ gp, float* gb, int cout, int total)
-{
-    __shared__ float bsum[64];
-    const int cg = cout >> 3;
-    for (int k = threadIdx.x; k < cout; k += blockDim.x) bsum[k] = 0.f;
-    __syncthreads();
-    const int64_t items = (int64_t)total * cg;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int q = (int)(i0 % cg);  // fixed: stride % cg == 0
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int64_t i = i0; i < items; i += stride) {
-        const float4 g0 = __ldg(reinterpret_cast<const float4*>(gout) + 2 * i);
-        const float4 g1 = __ldg(reinterpret_cast<const float4*>(gout) + 2 * i + 1);
-        const uint4 y = __ldg(reinterpret_cast<const uint4*>(out) + i);
-        const __nv_bfloat162* yh = reinterpret_cast<const __nv_bfloat162*>(&y);
-        float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (!(__low2float(yh[k]) > 0.f)) g[2 * k] = 0.f;
-            if (!(__high2float(yh[k]) > 0.f)) g[2 * k + 1] = 0.f;
-        }
-        uint4 o;
-        o.x = pack_bf16(g[0], g[1]);
-        o.y = pack_bf16(g[2], g[3]);
-        o.z = pack_bf16(g[4], g[5]);
-        o.w = pack_bf16(g[6], g[7]);
-        reinterpret_cast<uint4*>(gp)[i] = o;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += g[k];
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) atomicAdd(&bsum[q * 8 + k], acc[k]);
-    __syncthreads();
-    for (int k = threadIdx.x; k < cout; k += blockDim.x) atomicAdd(&gb[k], bsum[k]);
-}
-
 // ------------------------------------------------------------------ pooling / upsampling
+//
+// All of these move 8-channel groups (16 bytes of BF16, 32 of FP32): a thread per
+// group, so that a warp reads and writes whole lines.
 
 // dst (coarse) = mean of the 2x2x2 children in src (fine), channels-last, C channels
 __global__ void pool_fwd_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, Dims fine, int C)
 {
-    const int cx = fine.nx / 2, cy = fine.ny / 2, cz = fine.nz / 2, cvox = cx * cy * cz;
-    const int64_t total = (int64_t)cvox * fine.batch * C;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const int64_t v = i / C;
-        const int b = (int)(v / cvox);
-        const int r = (int)(v - (int64_t)b * cvox);
+    nh::step_kernel_enter();
+    const int cx = fine.nx / 2, cy = fine.ny / 2, cz = fine.nz / 2, cvox = cx * cy * cz, cg = C / 8;
+    const int total = cvox * fine.batch * cg;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const int v = i / cg, q = i - v * cg;
+        const int b = v / cvox, r = v - b * cvox;
         const int x = r % cx, y = (r / cx) % cy, z = r / (cx * cy);
-        float s = 0.f;
+        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int fx = 2 * x + (k & 1), fy = 2 * y + ((k >> 1) & 1), fz = 2 * z + (k >> 2);
-            s += __bfloat162float(src[((size_t)b * fine.nvox + fx + fine.nx * (fy + fine.ny * fz)) * C + c]);
+            float c[8];
+            unpack8(__ldg(reinterpret_cast<const uint4*>(src) + (size_t)(b * fine.nvox + fx + fine.nx * (fy + fine.ny * fz)) * cg + q), c);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s[j] += c[j];
         }
-        dst[(size_t)v * C + c] = __float2bfloat16_rn(0.125f * s);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] *= 0.125f;
+        reinterpret_cast<uint4*>(dst)[i] = pack8(s);
     }
 }
 
-// gsrc (fine) += gdst (coarse) / 8
-__global__ void pool_bwd_kernel(const float* __restrict__ gdst, float* __restrict__ gsrc, Dims fine, int C)
+// A pre-activation gradient from the gradient g of an activation group: masked
+// by the ReLU of act, BF16 into gp, and summed into the thread's bias sums.
+__device__ __forceinline__ void prep_group(float g[8], const bf16* act, bf16* gp, int64_t i, float bias[8])
 {
-    const int cx = fine.nx / 2, cy = fine.ny / 2;
-    const int64_t total = (int64_t)fine.nvox * fine.batch * C;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const int64_t v = i / C;
-        const int b = (int)(v / fine.nvox);
-        const int r = (int)(v - (int64_t)b * fine.nvox);
+    relu_mask(g, __ldg(reinterpret_cast<const uint4*>(act) + i));
+    reinterpret_cast<uint4*>(gp)[i] = pack8(g);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) bias[k] += g[k];
+}
+// The block's bias sums into gb: a thread's group q is fixed (the grid stride is
+// a multiple of C / 8, and so are a warp's 32 threads), so the lanes of a group
+// add by shuffles, the warps in shared memory, and the block with one atomic per
+// channel.
+__device__ __forceinline__ void bias_out(const float bias[8], int q, int C, float* gb)
+{
+    __shared__ float bsum[64];
+    for (int k = threadIdx.x; k < C; k += blockDim.x) bsum[k] = 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        float v = bias[k];
+        for (int o = 16; o >= C / 8; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) < C / 8) atomicAdd(&bsum[q * 8 + k], v);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < C; k += blockDim.x) atomicAdd(&gb[k], bsum[k]);
+}
+
+__device__ __forceinline__ void ld8(const float* p, int64_t i, float v[8])
+{
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p) + 2 * i), b = __ldg(reinterpret_cast<const float4*>(p) + 2 * i + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// Pre-activation gradient of the layer that a pooling and a skip connection read:
+// the skip's gradient plus an eighth of the pooled one's.
+__global__ void __launch_bounds__(256) pool_bwd_kernel(const float* __restrict__ gpool, const float* __restrict__ gskip,
+                                                       const bf16* __restrict__ act, bf16* __restrict__ gp, float* gb,
+                                                       Dims fine, int C)
+{
+    nh::step_kernel_enter();
+    const int cx = fine.nx / 2, cy = fine.ny / 2, cg = C / 8;
+    const int total = fine.nvox * fine.batch * cg, first = blockIdx.x * blockDim.x + threadIdx.x;
+    float bias[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int i = first; i < total; i += gridDim.x * blockDim.x) {
+        const int v = i / cg, q = i - v * cg;
+        const int b = v / fine.nvox, r = v - b * fine.nvox;
         const int x = r % fine.nx, y = (r / fine.nx) % fine.ny, z = r / (fine.nx * fine.ny);
-        const size_t cv = (size_t)b * (fine.nvox / 8) + x / 2 + cx * (y / 2 + cy * (z / 2));
-        gsrc[i] += 0.125f * gdst[cv * C + c];
+        const int64_t cv = (int64_t)b * (fine.nvox / 8) + x / 2 + cx * (y / 2 + cy * (z / 2));
+        float g[8], c[8];
+        ld8(gskip, i, g);
+        ld8(gpool, cv * cg + q, c);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) g[k] += 0.125f * c[k];
+        prep_group(g, act, gp, i, bias);
     }
+    bias_out(bias, first % cg, C, gb);
 }
 
-// gsrc (coarse) = sum of gdst over the 8 children (overwrites)
-__global__ void up_bwd_kernel(const float* __restrict__ gdst, float* __restrict__ gsrc, Dims fine, int C)
+// Pre-activation gradient of the layer that an upsampling reads: the sum over the 8 children.
+__global__ void __launch_bounds__(256) up_bwd_kernel(const float* __restrict__ gup, const bf16* __restrict__ act,
+                                                     bf16* __restrict__ gp, float* gb, Dims fine, int C)
 {
-    const int cx = fine.nx / 2, cy = fine.ny / 2, cz = fine.nz / 2, cvox = cx * cy * cz;
-    const int64_t total = (int64_t)cvox * fine.batch * C;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const int64_t v = i / C;
-        const int b = (int)(v / cvox);
-        const int r = (int)(v - (int64_t)b * cvox);
+    nh::step_kernel_enter();
+    const int cx = fine.nx / 2, cy = fine.ny / 2, cz = fine.nz / 2, cvox = cx * cy * cz, cg = C / 8;
+    const int total = cvox * fine.batch * cg, first = blockIdx.x * blockDim.x + threadIdx.x;
+    float bias[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int i = first; i < total; i += gridDim.x * blockDim.x) {
+        const int v = i / cg, q = i - v * cg;
+        const int b = v / cvox, r = v - b * cvox;
         const int x = r % cx, y = (r / cx) % cy, z = r / (cx * cy);
-        float s = 0.f;
+        float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int fx = 2 * x + (k & 1), fy = 2 * y + ((k >> 1) & 1), fz = 2 * z + (k >> 2);
-            s += gdst[((size_t)b * fine.nvox + fx + fine.nx * (fy + fine.ny * fz)) * C + c];
+            float c[8];
+            ld8(gup, (int64_t)(b * fine.nvox + fx + fine.nx * (fy + fine.ny * fz)) * cg + q, c);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) g[j] += c[j];
         }
-        gsrc[i] = s;
+        prep_group(g, act, gp, i, bias);
     }
+    bias_out(bias, first % cg, C, gb);
 }
 
 // ------------------------------------------------------------------ input, head, loss, optimiser
@@ -652,90 +732,112 @@ __global__ void up_bwd_kernel(const float* __restrict__ gdst, float* __restrict_
 // x[v][0..2] = n_ansatz, x[v][3] = q0 Lz / 2 pi, [4] = Lz / 32, [5] = W0 / 1e-3, rest 0.
 __global__ void input_kernel(const float* __restrict__ n, const float* __restrict__ scal, bf16* __restrict__ x, Dims d)
 {
+    nh::step_kernel_enter();
     const int total = d.nvox * d.batch;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < total; v += gridDim.x * blockDim.x) {
         const int b = v / d.nvox, r = v - b * d.nvox;
         const float* nb = n + (size_t)b * 3 * d.nvox;
-        float vals[kInCh];
-        for (int c = 0; c < kInCh; ++c) vals[c] = 0.f;
-        vals[0] = nb[r];
-        vals[1] = nb[d.nvox + r];
-        vals[2] = nb[2 * d.nvox + r];
         const float q0 = scal[3 * b], lz = scal[3 * b + 1], w0 = scal[3 * b + 2];
-        vals[3] = q0 * lz / 6.283185307179586f;
-        vals[4] = lz / 32.f;
-        vals[5] = w0 / 1e-3f;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(x + (size_t)v * kInCh);
-        for (int c = 0; c < kInCh; c += 2) dst[c / 2] = pack_bf16(vals[c], vals[c + 1]);
+        const float vals[8] = {nb[r], nb[d.nvox + r], nb[2 * d.nvox + r], q0 * lz / 6.283185307179586f, lz / 32.f,
+                               w0 / 1e-3f, 0.f, 0.f};
+        uint4* dst = reinterpret_cast<uint4*>(x + (size_t)v * kInCh);
+        dst[0] = pack8(vals);
+        dst[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
-// Head (1x1x1 conv 16 -> 3), residual on the ansatz, normalisation; optionally
-// the loss mean |n - target|^2 and the gradients of d1, W_head, b_head.
+// Head (1x1x1 conv 16 -> 3), residual on the ansatz, normalisation.  Train: the
+// loss mean |n - target|^2, the gradients of W_head and b_head, and the last
+// convolution's pre-activation gradient (ReLU mask of d1, BF16) and bias gradient.
+template <bool Train>
 __global__ void __launch_bounds__(256) head_kernel(const bf16* __restrict__ d1, const float* __restrict__ n_ans,
                                                    const float* __restrict__ params_head, float* __restrict__ n_out,
-                                                   const float* __restrict__ target, float* __restrict__ g_d1,
-                                                   float* __restrict__ g_head, float* __restrict__ loss, Dims d)
+                                                   const float* __restrict__ target, bf16* __restrict__ gp,
+                                                   float* __restrict__ gb, float* __restrict__ g_head,
+                                                   float* __restrict__ loss, Dims d)
 {
-    __shared__ float sh[kHeadOut * kHeadIn + kHeadOut];
-    __shared__ float red[kHeadOut * kHeadIn + kHeadOut + 1][8];
-    for (int k = threadIdx.x; k < kHeadOut * kHeadIn + kHeadOut; k += blockDim.x) sh[k] = params_head[k];
+    nh::step_kernel_enter();
+    constexpr int kW = kHeadOut * kHeadIn, kSums = kW + kHeadOut + 1 + kHeadIn;  // W, b, loss, bias of the last conv
+    __shared__ float sh[kW + kHeadOut];
+    __shared__ float red[kSums][8];
+    for (int k = threadIdx.x; k < kW + kHeadOut; k += blockDim.x) sh[k] = params_head[k];
     __syncthreads();
     const int total = d.nvox * d.batch;
     const float inv_total = 1.f / (float)total;
-    float gacc[kHeadOut * kHeadIn + kHeadOut + 1];
-    for (int k = 0; k < kHeadOut * kHeadIn + kHeadOut + 1; ++k) gacc[k] = 0.f;
+    float gacc[Train ? kSums : 1];
+#pragma unroll
+    for (int k = 0; k < (Train ? kSums : 1); ++k) gacc[k] = 0.f;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < total; v += gridDim.x * blockDim.x) {
         const int b = v / d.nvox, r = v - b * d.nvox;
+        const size_t o0 = (size_t)b * 3 * d.nvox + r;
         float h[kHeadIn];
-        for (int c = 0; c < kHeadIn; ++c) h[c] = __bfloat162float(d1[(size_t)v * kHeadIn + c]);
+        const uint4* row = reinterpret_cast<const uint4*>(d1 + (size_t)v * kHeadIn);
+        unpack8(__ldg(row), h);
+        unpack8(__ldg(row + 1), h + 8);
         float vv[3];
+#pragma unroll
         for (int o = 0; o < 3; ++o) {
-            float s = sh[kHeadOut * kHeadIn + o];
+            float s = sh[kW + o];
+#pragma unroll
             for (int c = 0; c < kHeadIn; ++c) s += sh[o * kHeadIn + c] * h[c];
-            vv[o] = n_ans[(size_t)b * 3 * d.nvox + o * d.nvox + r] + s;
+            vv[o] = n_ans[o0 + (size_t)o * d.nvox] + s;
         }
         const float len = sqrtf(vv[0] * vv[0] + vv[1] * vv[1] + vv[2] * vv[2]);
         const float nn[3] = {vv[0] / len, vv[1] / len, vv[2] / len};
         if (n_out)
-            for (int o = 0; o < 3; ++o) n_out[(size_t)b * 3 * d.nvox + o * d.nvox + r] = nn[o];
-        if (target) {
+#pragma unroll
+            for (int o = 0; o < 3; ++o) n_out[o0 + (size_t)o * d.nvox] = nn[o];
+        if constexpr (Train) {
             float gn[3], dot = 0.f, l = 0.f;
+#pragma unroll
             for (int o = 0; o < 3; ++o) {
-                const float diff = nn[o] - target[(size_t)b * 3 * d.nvox + o * d.nvox + r];
+                const float diff = nn[o] - target[o0 + (size_t)o * d.nvox];
                 l += diff * diff;
                 gn[o] = 2.f * diff * inv_total;
                 dot += gn[o] * nn[o];
             }
-            gacc[kHeadOut * kHeadIn + kHeadOut] += l * inv_total;
+            gacc[kW + kHeadOut] += l * inv_total;
             float gd[3];
+#pragma unroll
             for (int o = 0; o < 3; ++o) gd[o] = (gn[o] - dot * nn[o]) / len;  // d/dv of v/|v|
+            float g[kHeadIn];
+#pragma unroll
             for (int c = 0; c < kHeadIn; ++c) {
                 float s = 0.f;
+#pragma unroll
                 for (int o = 0; o < 3; ++o) {
                     s += sh[o * kHeadIn + c] * gd[o];
                     gacc[o * kHeadIn + c] += gd[o] * h[c];
                 }
-                g_d1[(size_t)v * kHeadIn + c] = s;
+                g[c] = h[c] > 0.f ? s : 0.f;
+                gacc[kW + kHeadOut + 1 + c] += g[c];
             }
-            for (int o = 0; o < 3; ++o) gacc[kHeadOut * kHeadIn + o] += gd[o];
+#pragma unroll
+            for (int o = 0; o < 3; ++o) gacc[kW + o] += gd[o];
+            uint4* dst = reinterpret_cast<uint4*>(gp + (size_t)v * kHeadIn);
+            dst[0] = pack8(g);
+            dst[1] = pack8(g + 8);
         }
     }
-    if (!target) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < kHeadOut * kHeadIn + kHeadOut + 1; ++k) {
-        float s = gacc[k];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) red[k][warp] = s;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < kHeadOut * kHeadIn + kHeadOut + 1; k += blockDim.x) {
-        float s = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[k][w];
-        if (k < kHeadOut * kHeadIn + kHeadOut)
-            atomicAdd(&g_head[k], s);
-        else
-            atomicAdd(loss, s);
+    if constexpr (Train) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+        for (int k = 0; k < kSums; ++k) {
+            float s = gacc[k];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) red[k][warp] = s;
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < kSums; k += blockDim.x) {
+            float s = 0.f;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[k][w];
+            if (k < kW + kHeadOut)
+                atomicAdd(&g_head[k], s);
+            else if (k == kW + kHeadOut)
+                atomicAdd(loss, s);
+            else
+                atomicAdd(&gb[k - (kW + kHeadOut + 1)], s);
+        }
     }
 }
 
@@ -745,21 +847,26 @@ __global__ void bf16_to_f32_kernel(const bf16* __restrict__ a, float* __restrict
         out[i] = __bfloat162float(a[i]);
 }
 
-__global__ void cast_params_kernel(const float* __restrict__ p, bf16* __restrict__ w, int64_t n)
+// BF16 copies of all parameters, and of the convolution weights transposed,
+// wt[l][tap][ci][co] = w[l][tap][co][ci], in one launch (one per layer took 45 us).
+struct ParamTable {
+    int begin[kLayers + 1];  // first parameter of each layer, and of the head
+    int cin[kLayers], cout[kLayers];
+    bf16* wt[kLayers];
+};
+__global__ void params_kernel(const float* __restrict__ p, bf16* __restrict__ w, const ParamTable t, int n)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        w[i] = __float2bfloat16_rn(p[i]);
-}
-
-// wt[tap][ci][co] = w[tap][co][ci]
-__global__ void transpose_kernel(const float* __restrict__ p, bf16* __restrict__ wt, int cin, int cout)
-{
-    const int n = 27 * cin * cout;
+    nh::step_kernel_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int tap = i / (cin * cout);
-        const int r = i - tap * cin * cout;
-        const int ci = r / cout, co = r - ci * cout;
-        wt[i] = __float2bfloat16_rn(p[(size_t)tap * cout * cin + (size_t)co * cin + ci]);
+        const bf16 v = __float2bfloat16_rn(p[i]);
+        w[i] = v;
+        int l = 0;
+        while (l < kLayers && i >= t.begin[l + 1]) ++l;
+        if (l == kLayers) continue;
+        const int k = i - t.begin[l], cc = t.cin[l] * t.cout[l];
+        if (k >= 27 * cc) continue;  // bias
+        const int tap = k / cc, r = k - tap * cc, co = r / t.cin[l], ci = r - co * t.cin[l];
+        t.wt[l][tap * cc + ci * t.cout[l] + co] = v;
     }
 }
 
@@ -767,6 +874,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
                             float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps, float c1,
                             float c2)
 {
+    nh::step_kernel_enter();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -794,7 +902,7 @@ struct nh_unet {
     size_t ws_bytes = 0;
     size_t need = 0;
     // offsets into the workspace
-    size_t wbf, wt[kLayers], x, act[kLayers], pool_[3], grad_a, grad_b, grad_skip[3], gd1, gprep, status;
+    size_t wbf, wt[kLayers], x, act[kLayers], pool_[3], grad, grad_skip[3], gp[2], status;
     std::string err;
 };
 
@@ -828,19 +936,12 @@ void plan(nh_unet* u)
     // pooled inputs of levels 1..3
     const int pool_c[3] = {16, 16, 32};
     for (int k = 0; k < 3; ++k) u->pool_[k] = take((size_t)u->lv[k + 1].nvox * u->batch * pool_c[k] * sizeof(bf16));
-    // gradient scratch: two ping-pong buffers large enough for any [vox][96] level-0..3 tensor,
-    // three skip-gradient buffers (e1, e2, e3) and the head-input gradient
-    size_t gmax = 0;
-    for (int k = 0; k < 4; ++k) gmax = std::max(gmax, (size_t)u->lv[k].nvox * u->batch * 96);
-    u->grad_a = take(gmax * sizeof(float));
-    u->grad_b = take(gmax * sizeof(float));
+    // FP32 gradient of a tensor that a pooling or an upsampling produced (at most 16 channels of level 0, 32 of
+    // level 1, 64 of level 2), the three skip gradients (e1, e2, e3), and two pre-activation gradients
+    u->grad = take(V0 * 16 * sizeof(float));
     const int skip_c[3] = {16, 16, 32};
     for (int k = 0; k < 3; ++k) u->grad_skip[k] = take((size_t)u->lv[k].nvox * u->batch * skip_c[k] * sizeof(float));
-    u->gd1 = take(V0 * kHeadIn * sizeof(float));
-    size_t gp_max = 0;  // BF16 pre-activation gradient of the largest layer output
-    for (int l = 0; l < kLayers; ++l)
-        gp_max = std::max(gp_max, (size_t)u->lv[level_of[l]].nvox * u->batch * kConv[l].cout);
-    u->gprep = take(gp_max * sizeof(bf16));
+    for (int k = 0; k < 2; ++k) u->gp[k] = take(V0 * 16 * sizeof(bf16));  // level 0 has the largest output
     u->status = take(sizeof(int));  // raised by an expired wait of the tensor-core convolution
     u->need = off;
 }
@@ -870,21 +971,15 @@ cudaError_t conv_fwd(nh_unet* u, int l, int level, const bf16* s1, int c1, const
     return launch_conv_tc<false>(a, st);
 }
 
-// Backward of conv layer l: gout (FP32 [vox][cout]) -> data gradient into
-// dst1 (c1 channels, overwritten) and dst2 (c2, accumulated); weight and bias
-// gradients accumulated into grad.
-cudaError_t conv_bwd(nh_unet* u, int l, int level, const float* gout, const bf16* s1, int c1, const bf16* s2, int c2,
-                     bool up1, float* dst1, float* dst2, float* grad, bool need_data, cudaStream_t st)
+// Backward of conv layer l from its pre-activation gradient gp: weight gradient
+// into grad, then the data gradient: of a single source that is layer `below`
+// its pre-activation gradient into gp_below (and its bias gradient into grad),
+// else (below < 0) FP32 into dst1 (c1 channels) and dst2 (c2); none with both null.
+cudaError_t conv_bwd(nh_unet* u, int l, int level, const bf16* gp, const bf16* s1, int c1, const bf16* s2, int c2, bool up1,
+                     int below, bf16* gp_below, float* dst1, float* dst2, float* grad, cudaStream_t st)
 {
     const Dims d = u->lv[level];
-    const int total = d.nvox * d.batch;
     const int cout = kConv[l].cout, cin = kConv[l].cin;
-    const bf16* out = P<bf16>(u, u->act[l]);
-    bf16* gp = P<bf16>(u, u->gprep);
-    grad_prep_kernel<<<std::min(4 * 152, grid_for(total * (cout / 8), 256)), 256, 0, st>>>(
-        gout, out, gp, grad + layer_offset(l) + 27LL * cin * cout, cout, total);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     ConvBwdW w;
     w.gp = gp;
     w.src1 = s1;
@@ -898,28 +993,36 @@ cudaError_t conv_bwd(nh_unet* u, int l, int level, const float* gout, const bf16
     w.tiles = ((d.nx + kWTx - 1) / kWTx) * ((d.ny + kWTy - 1) / kWTy) * ((d.nz + kWTz - 1) / kWTz) * d.batch;
     static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
     if (!attr_set) {
-        e = cudaFuncSetAttribute(conv_bwd_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
+        cudaError_t e = cudaFuncSetAttribute(conv_bwd_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     // one wave of resident blocks over the channel pairs; each walks its share of the tiles
     const int pairs = (cin / 16) * (cout / 16);
     dim3 grid(std::min(w.tiles, std::max(1, kWBlocksPerSM * 152 / pairs)), pairs);
-    conv_bwd_w_kernel<<<grid, kWThreads, kWSmem, st>>>(w);
-    e = cudaGetLastError();
-    if (e != cudaSuccess || !need_data) return e;
+    nh::launch_step_kernel(conv_bwd_w_kernel, grid, kWThreads, kWSmem, st, w);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || (gp_below == nullptr && dst1 == nullptr)) return e;
     ConvTc b{};
     b.src1 = gp;
     b.c1 = cout;
     b.w = P<bf16>(u, u->wt[l]);
     b.n = cin;
     b.d = d;
+    if (below >= 0) {
+        b.mask = P<bf16>(u, u->act[below]);
+        b.gp = gp_below;
+        b.gb = grad + layer_offset(below) + 27LL * kConv[below].cin * kConv[below].cout;
+    }
     b.dst1 = dst1;
     b.n1 = c1;
     b.dst2 = dst2;
     b.status = P<int>(u, u->status);
     return launch_conv_tc<true>(b, st);
 }
+
+// Grid of the group kernels: a stride that is a multiple of C / 8 (1, 2, 4 or 8).
+inline int group_grid(int64_t groups) { return (int)std::min<int64_t>(8 * 152, (groups + 255) / 256); }
 
 }  // namespace
 
@@ -992,14 +1095,17 @@ int nh_unet_set_params(nh_unet* u, const float* params, void* stream)
 {
     if (!u || !u->ws || !params) return unet_fail(u, NH_EINVAL, "unbound network or NULL params");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int64_t n = total_params();
-    cast_params_kernel<<<grid_for(n), 256, 0, st>>>(params, P<bf16>(u, u->wbf), n);
-    UNET_CUDA(u, cudaGetLastError());
+    const int n = (int)total_params();
+    ParamTable t;
     for (int l = 0; l < kLayers; ++l) {
-        transpose_kernel<<<grid_for(27LL * kConv[l].cin * kConv[l].cout), 256, 0, st>>>(
-            params + layer_offset(l), P<bf16>(u, u->wt[l]), kConv[l].cin, kConv[l].cout);
-        UNET_CUDA(u, cudaGetLastError());
+        t.begin[l] = (int)layer_offset(l);
+        t.cin[l] = kConv[l].cin;
+        t.cout[l] = kConv[l].cout;
+        t.wt[l] = P<bf16>(u, u->wt[l]);
     }
+    t.begin[kLayers] = (int)head_offset();
+    nh::launch_step_kernel(params_kernel, grid_for(n), 256, 0, st, params, P<bf16>(u, u->wbf), t, n);
+    UNET_CUDA(u, cudaGetLastError());
     return NH_OK;
 }
 
@@ -1009,19 +1115,23 @@ int nh_unet_forward(nh_unet* u, const float* params, const float* n_ansatz, cons
     if (!u || !u->ws || !params || !n_ansatz || !scalars) return unet_fail(u, NH_EINVAL, "NULL argument");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Dims d0 = u->lv[0];
-    input_kernel<<<grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st>>>(n_ansatz, scalars, P<bf16>(u, u->x), d0);
+    nh::launch_step_kernel(input_kernel, grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st, n_ansatz, scalars,
+                           P<bf16>(u, u->x), d0);
     UNET_CUDA(u, cudaGetLastError());
     auto act = [&](int l) { return P<bf16>(u, u->act[l]); };
     auto pool = [&](int k) { return P<bf16>(u, u->pool_[k]); };
     UNET_CUDA(u, conv_fwd(u, ENC1A, 0, P<bf16>(u, u->x), 16, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, ENC1B, 0, act(ENC1A), 16, nullptr, 0, false, params, st));
-    pool_fwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 16), 256, 0, st>>>(act(ENC1B), pool(0), u->lv[0], 16);
+    nh::launch_step_kernel(pool_fwd_kernel, group_grid((int64_t)u->lv[1].nvox * u->batch * 2), 256, 0, st, act(ENC1B), pool(0),
+                           u->lv[0], 16);
     UNET_CUDA(u, conv_fwd(u, ENC2A, 1, pool(0), 16, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, ENC2B, 1, act(ENC2A), 16, nullptr, 0, false, params, st));
-    pool_fwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 16), 256, 0, st>>>(act(ENC2B), pool(1), u->lv[1], 16);
+    nh::launch_step_kernel(pool_fwd_kernel, group_grid((int64_t)u->lv[2].nvox * u->batch * 2), 256, 0, st, act(ENC2B), pool(1),
+                           u->lv[1], 16);
     UNET_CUDA(u, conv_fwd(u, ENC3A, 2, pool(1), 16, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, ENC3B, 2, act(ENC3A), 32, nullptr, 0, false, params, st));
-    pool_fwd_kernel<<<grid_for((int64_t)u->lv[3].nvox * u->batch * 32), 256, 0, st>>>(act(ENC3B), pool(2), u->lv[2], 32);
+    nh::launch_step_kernel(pool_fwd_kernel, group_grid((int64_t)u->lv[3].nvox * u->batch * 4), 256, 0, st, act(ENC3B), pool(2),
+                           u->lv[2], 32);
     UNET_CUDA(u, conv_fwd(u, BOTA, 3, pool(2), 32, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, BOTB, 3, act(BOTA), 64, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, DEC3A, 2, act(BOTB), 64, act(ENC3B), 32, true, params, st));
@@ -1030,8 +1140,8 @@ int nh_unet_forward(nh_unet* u, const float* params, const float* n_ansatz, cons
     UNET_CUDA(u, conv_fwd(u, DEC2B, 1, act(DEC2A), 16, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, DEC1A, 0, act(DEC2B), 16, act(ENC1B), 16, true, params, st));
     UNET_CUDA(u, conv_fwd(u, DEC1B, 0, act(DEC1A), 16, nullptr, 0, false, params, st));
-    head_kernel<<<grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st>>>(act(DEC1B), n_ansatz, params + head_offset(), n_out,
-                                                                        nullptr, nullptr, nullptr, nullptr, d0);
+    nh::launch_step_kernel(head_kernel<false>, grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st, act(DEC1B), n_ansatz,
+                           params + head_offset(), n_out, nullptr, nullptr, nullptr, nullptr, nullptr, d0);
     UNET_CUDA(u, cudaGetLastError());
     return NH_OK;
 }
@@ -1047,49 +1157,52 @@ int nh_unet_backward(nh_unet* u, const float* params, const float* n_ansatz, con
     UNET_CUDA(u, cudaMemsetAsync(loss, 0, sizeof(float), st));
     auto act = [&](int l) { return P<bf16>(u, u->act[l]); };
     auto pool = [&](int k) { return P<bf16>(u, u->pool_[k]); };
-    float* ga = P<float>(u, u->grad_a);
-    float* gb = P<float>(u, u->grad_b);
+    float* g = P<float>(u, u->grad);
     float* gskip[3] = {P<float>(u, u->grad_skip[0]), P<float>(u, u->grad_skip[1]), P<float>(u, u->grad_skip[2])};
-    float* gd1 = P<float>(u, u->gd1);
-    head_kernel<<<std::min(256, grid_for((int64_t)d0.nvox * d0.batch)), 256, 0, st>>>(
-        act(DEC1B), n_ansatz, params + head_offset(), nullptr, target, gd1, grad + head_offset(), loss, d0);
+    bf16 *gpa = P<bf16>(u, u->gp[0]), *gpb = P<bf16>(u, u->gp[1]);
+    auto gbias = [&](int l) { return grad + layer_offset(l) + 27LL * kConv[l].cin * kConv[l].cout; };
+    // layer l read by an upsampling to level `fine`, or by a pooling from level `fine` and a skip connection
+    auto up_bwd = [&](int l, int fine) {
+        const int C = kConv[l].cout;
+        nh::launch_step_kernel(up_bwd_kernel, group_grid((int64_t)u->lv[fine + 1].nvox * u->batch * (C / 8)), 256, 0, st, g,
+                               act(l), gpa, gbias(l), u->lv[fine], C);
+        return cudaGetLastError();
+    };
+    auto pool_bwd = [&](int l, int fine) {
+        const int C = kConv[l].cout;
+        nh::launch_step_kernel(pool_bwd_kernel, group_grid((int64_t)u->lv[fine].nvox * u->batch * (C / 8)), 256, 0, st, g,
+                               gskip[fine], act(l), gpa, gbias(l), u->lv[fine], C);
+        return cudaGetLastError();
+    };
+    nh::launch_step_kernel(head_kernel<true>, std::min(4 * 152, grid_for((int64_t)d0.nvox * d0.batch)), 256, 0, st,
+                           act(DEC1B), n_ansatz, params + head_offset(), nullptr, target, gpa, gbias(DEC1B),
+                           grad + head_offset(), loss, d0);
     UNET_CUDA(u, cudaGetLastError());
-    // decoder level 0: dec1b <- gd1, dec1a <- ga  (sources [up2 | e1])
-    UNET_CUDA(u, conv_bwd(u, DEC1B, 0, gd1, act(DEC1A), 16, nullptr, 0, false, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, cudaMemsetAsync(gskip[0], 0, (size_t)d0.nvox * d0.batch * 16 * sizeof(float), st));
-    UNET_CUDA(u, conv_bwd(u, DEC1A, 0, ga, act(DEC2B), 16, act(ENC1B), 16, true, gb, gskip[0], grad, true, st));
-    up_bwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 16), 256, 0, st>>>(gb, ga, u->lv[0], 16);  // -> g(dec2b)
-    UNET_CUDA(u, cudaGetLastError());
-    // decoder level 1
-    UNET_CUDA(u, conv_bwd(u, DEC2B, 1, ga, act(DEC2A), 16, nullptr, 0, false, gb, nullptr, grad, true, st));
-    UNET_CUDA(u, cudaMemsetAsync(gskip[1], 0, (size_t)u->lv[1].nvox * u->batch * 16 * sizeof(float), st));
-    UNET_CUDA(u, conv_bwd(u, DEC2A, 1, gb, act(DEC3B), 32, act(ENC2B), 16, true, ga, gskip[1], grad, true, st));
-    up_bwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 32), 256, 0, st>>>(ga, gb, u->lv[1], 32);  // -> g(dec3b)
-    UNET_CUDA(u, cudaGetLastError());
-    // decoder level 2
-    UNET_CUDA(u, conv_bwd(u, DEC3B, 2, gb, act(DEC3A), 32, nullptr, 0, false, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, cudaMemsetAsync(gskip[2], 0, (size_t)u->lv[2].nvox * u->batch * 32 * sizeof(float), st));
-    UNET_CUDA(u, conv_bwd(u, DEC3A, 2, ga, act(BOTB), 64, act(ENC3B), 32, true, gb, gskip[2], grad, true, st));
-    up_bwd_kernel<<<grid_for((int64_t)u->lv[3].nvox * u->batch * 64), 256, 0, st>>>(gb, ga, u->lv[2], 64);  // -> g(botb)
-    UNET_CUDA(u, cudaGetLastError());
+    // decoder: of each level the second convolution, then the first, whose sources are the upsampled level
+    // below and the encoder's skip connection
+    UNET_CUDA(u, conv_bwd(u, DEC1B, 0, gpa, act(DEC1A), 16, nullptr, 0, false, DEC1A, gpb, nullptr, nullptr, grad, st));
+    UNET_CUDA(u, conv_bwd(u, DEC1A, 0, gpb, act(DEC2B), 16, act(ENC1B), 16, true, -1, nullptr, g, gskip[0], grad, st));
+    UNET_CUDA(u, up_bwd(DEC2B, 0));
+    UNET_CUDA(u, conv_bwd(u, DEC2B, 1, gpa, act(DEC2A), 16, nullptr, 0, false, DEC2A, gpb, nullptr, nullptr, grad, st));
+    UNET_CUDA(u, conv_bwd(u, DEC2A, 1, gpb, act(DEC3B), 32, act(ENC2B), 16, true, -1, nullptr, g, gskip[1], grad, st));
+    UNET_CUDA(u, up_bwd(DEC3B, 1));
+    UNET_CUDA(u, conv_bwd(u, DEC3B, 2, gpa, act(DEC3A), 32, nullptr, 0, false, DEC3A, gpb, nullptr, nullptr, grad, st));
+    UNET_CUDA(u, conv_bwd(u, DEC3A, 2, gpb, act(BOTB), 64, act(ENC3B), 32, true, -1, nullptr, g, gskip[2], grad, st));
+    UNET_CUDA(u, up_bwd(BOTB, 2));
     // bottleneck
-    UNET_CUDA(u, conv_bwd(u, BOTB, 3, ga, act(BOTA), 64, nullptr, 0, false, gb, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, BOTA, 3, gb, pool(2), 32, nullptr, 0, false, ga, nullptr, grad, true, st));   // ga = g(pool2 out)
-    pool_bwd_kernel<<<grid_for((int64_t)u->lv[2].nvox * u->batch * 32), 256, 0, st>>>(ga, gskip[2], u->lv[2], 32);
-    UNET_CUDA(u, cudaGetLastError());
-    // encoder level 2 (e3 gradient complete in gskip[2])
-    UNET_CUDA(u, conv_bwd(u, ENC3B, 2, gskip[2], act(ENC3A), 32, nullptr, 0, false, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, ENC3A, 2, ga, pool(1), 16, nullptr, 0, false, gb, nullptr, grad, true, st));
-    pool_bwd_kernel<<<grid_for((int64_t)u->lv[1].nvox * u->batch * 16), 256, 0, st>>>(gb, gskip[1], u->lv[1], 16);
-    UNET_CUDA(u, cudaGetLastError());
-    // encoder level 1
-    UNET_CUDA(u, conv_bwd(u, ENC2B, 1, gskip[1], act(ENC2A), 16, nullptr, 0, false, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, ENC2A, 1, ga, pool(0), 16, nullptr, 0, false, gb, nullptr, grad, true, st));
-    pool_bwd_kernel<<<grid_for((int64_t)d0.nvox * d0.batch * 16), 256, 0, st>>>(gb, gskip[0], u->lv[0], 16);
-    UNET_CUDA(u, cudaGetLastError());
-    // encoder level 0 (the input needs no gradient)
-    UNET_CUDA(u, conv_bwd(u, ENC1B, 0, gskip[0], act(ENC1A), 16, nullptr, 0, false, ga, nullptr, grad, true, st));
-    UNET_CUDA(u, conv_bwd(u, ENC1A, 0, ga, P<bf16>(u, u->x), 16, nullptr, 0, false, nullptr, nullptr, grad, false, st));
+    UNET_CUDA(u, conv_bwd(u, BOTB, 3, gpa, act(BOTA), 64, nullptr, 0, false, BOTA, gpb, nullptr, nullptr, grad, st));
+    UNET_CUDA(u, conv_bwd(u, BOTA, 3, gpb, pool(2), 32, nullptr, 0, false, -1, nullptr, g, nullptr, grad, st));
+    // encoder: each level's output feeds the pooling and the skip connection
+    UNET_CUDA(u, pool_bwd(ENC3B, 2));
+    UNET_CUDA(u, conv_bwd(u, ENC3B, 2, gpa, act(ENC3A), 32, nullptr, 0, false, ENC3A, gpb, nullptr, nullptr, grad, st));
+    UNET_CUDA(u, conv_bwd(u, ENC3A, 2, gpb, pool(1), 16, nullptr, 0, false, -1, nullptr, g, nullptr, grad, st));
+    UNET_CUDA(u, pool_bwd(ENC2B, 1));
+    UNET_CUDA(u, conv_bwd(u, ENC2B, 1, gpa, act(ENC2A), 16, nullptr, 0, false, ENC2A, gpb, nullptr, nullptr, grad, st));
+    UNET_CUDA(u, conv_bwd(u, ENC2A, 1, gpb, pool(0), 16, nullptr, 0, false, -1, nullptr, g, nullptr, grad, st));
+    UNET_CUDA(u, pool_bwd(ENC1B, 0));
+    UNET_CUDA(u, conv_bwd(u, ENC1B, 0, gpa, act(ENC1A), 16, nullptr, 0, false, ENC1A, gpb, nullptr, nullptr, grad, st));
+    // (the input needs no gradient)
+    UNET_CUDA(u, conv_bwd(u, ENC1A, 0, gpb, P<bf16>(u, u->x), 16, nullptr, 0, false, -1, nullptr, nullptr, nullptr, grad, st));
     return NH_OK;
 }
 
@@ -1108,8 +1221,8 @@ int nh_unet_adam(float* params, const float* grad, float* m, float* v, int64_t c
     if (!params || !grad || !m || !v || count < 1 || step < 1) return unet_fail(nullptr, NH_EINVAL, "bad Adam arguments");
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-    adam_kernel<<<grid_for(count), 256, 0, static_cast<cudaStream_t>(stream)>>>(params, grad, m, v, count, lr, b1, b2,
-                                                                                 1e-8f, c1, c2);
+    nh::launch_step_kernel(adam_kernel, grid_for(count), 256, 0, static_cast<cudaStream_t>(stream), params, grad, m, v,
+                           count, lr, b1, b2, 1e-8f, c1, c2);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return unet_fail(nullptr, NH_ECUDA, std::string("adam: ") + cudaGetErrorString(e));
     return NH_OK;
