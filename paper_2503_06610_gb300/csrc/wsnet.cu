@@ -78,23 +78,31 @@ struct Dims {
 
 // ------------------------------------------------------------------ convolution on tcgen05: forward and data gradient
 //
-// One CTA (four warps) computes 8 x 16 output voxels of a z plane x NB output
-// channels per step and walks up a chunk of planes; each plane is the implicit
-// GEMM D[128][NB] = sum over the 27 taps of A_t[128][K] W_t^T.  Planes of the
-// input with a one-voxel halo in x and y (10 x 18 voxels) sit in a ring of four
-// shared-memory slots in the tensor core's no-swizzle K-major layout, 16-byte
-// channel groups of consecutive voxels next to each other: the eight voxels of
-// an x run are a core matrix, so the A operand of *every* tap is the same plane
-// read from a shifted start address (LBO = one channel-group plane, SBO = one
-// row of ten voxels), and a plane is copied once instead of once per tap.
-// (Copying each tap's rows took 339 us for a 16 -> 16 layer of 8 x 64 x 64 x 32
-// voxels, bound by the copies and a barrier per three taps.)  The weights of all
-// taps stay in shared memory for the CTA's life.  One thread issues a plane's 27
-// K/16 MMAs (kind::f16, BF16 x BF16 -> FP32, M = 128, N = NB, K = 16) into one of
-// two TMEM accumulators and commits them to its mbarrier; the copies of the plane
-// after next and the epilogue of the plane before run meanwhile.  Every mbarrier
-// wait is bounded: on expiry the kernel raises a.status, skips the epilogue,
-// waits for its copies and frees its TMEM.
+// One CTA (five warps) computes 8 x 16 voxels x NB output channels of a chunk of
+// z planes.  It walks along the *input* planes: a plane with a one-voxel halo in x
+// and y (10 x 18 voxels) is copied once into a ring of shared-memory slots, in
+// the tensor core's no-swizzle K-major layout with 16-byte channel groups of
+// consecutive voxels next to each other.  The eight voxels of an x run are a core
+// matrix, so the A operand of each of the nine (dy, dx) taps is the same plane
+// read from a shifted start address (LBO = one channel-group plane, SBO = one row
+// of ten voxels).  An input plane is a term of the three output planes next to it:
+// their accumulators are neighbours on a strip of 128 TMEM columns, and the three
+// dz taps' weights are stacked to 3 NB rows of B, so that one MMA (M = 128,
+// N = 3 NB, K = 16) serves all three.  At N = 16 an MMA is bound by reading A from
+// shared memory, whatever N is up to 48.  (16 -> 16 layer of 8 x 64 x 64 x 32
+// voxels, caches cold: 339 us with each tap's rows copied, 41 us with one MMA per
+// tap, 28 us so.)  Where the window of three runs past the strip's end it is
+// issued in two parts; the accumulator that enters the window is cleared by its
+// first MMA, and the two that lie outside the chunk are not read.
+// The weights of all taps stay in shared memory for the CTA's life.  The fifth
+// warp issues a plane's MMAs and commits them to an mbarrier; the other four copy
+// the planes to come and write the output plane that the previous input plane
+// completed meanwhile.  What bounds the kernel is the issuing warp's instructions
+// (predicating the MMAs off changes nothing, leaving out copies or epilogue
+// neither), so K is a template argument and the descriptors are constants added to
+// two bases: eight cells' forward pass 281 us with K at run time, 242 us so.
+// Every mbarrier wait is bounded: on expiry the kernel raises a.status, skips the
+// epilogue, waits for its copies and frees its TMEM.
 //
 // Forward: input = the layer's sources, D + bias, ReLU, BF16 rows.  Data gradient
 // (Flip): input = the pre-activation gradient, taps mirrored, transposed weights.
@@ -110,10 +118,11 @@ struct ConvTc {
     const bf16* src2;  // concatenated after src1 (c2 = 0: none)
     int c2;
     int up1;           // src1 is held at half the resolution and read nearest (upsampling)
-    const bf16* w;     // [27][n][c1 + c2]
+    const bf16* w;     // the weights' image (tc_weight_index)
     int n;             // output channels; blockIdx.y takes NB of them
     Dims d;
     int zc;            // planes per chunk
+    int ring;          // input planes held in shared memory, 2 ... kTcMaxRing
     const float* bias; // forward: [n]
     bf16* out;         // forward: [vox][n]
     const bf16* mask;  // data gradient: the source's activations [vox][n], or null
@@ -126,12 +135,35 @@ struct ConvTc {
 };
 
 constexpr int kTcM = 128;
-constexpr int kTcThreads = 128;
+constexpr int kTcCopy = 128;     // threads of the four warps that copy planes and run the epilogue
+constexpr int kTcThreads = 160;  // and a warp that issues the MMAs
 constexpr int kTcX = 8, kTcY = 16;                                // output voxels of a plane step
 constexpr int kTcHX = kTcX + 2, kTcHY = kTcY + 2, kTcHalo = kTcHX * kTcHY;
-constexpr int kTcRing = 4;
-inline size_t tc_smem(int K, int NB) { return (size_t)K * 2 * (kTcRing * kTcHalo + 27 * NB) + 64 + NB * sizeof(float); }
-constexpr size_t kTcMaxSmem = 227 * 1024;
+constexpr int kTcMaxRing = 5;      // input planes held: one in use, the others being copied
+constexpr uint32_t kTcCols = 128;  // TMEM columns of a CTA: a strip of 128 / NB accumulators
+// Ring, weights, voxel offsets, barriers, bias.  At least 46 KB, so that an SM takes at most the four CTAs whose
+// 512 columns it has.
+inline size_t tc_smem(int K, int NB, int ring)
+{
+    const size_t b = (size_t)K * 2 * (ring * kTcHalo + 27 * NB) + 2 * kTcHalo * sizeof(int) + 64 + NB * sizeof(float);
+    return std::max<size_t>(b, 46 * 1024);
+}
+constexpr size_t kTcMaxSmem = 227 * 1024, kTcSmSmem = 228 * 1024;  // of a block, of an SM
+
+// Output channels of a CTA: 32 where two such weight sets fit an SM, else 16 (more CTAs on the coarse levels, whose
+// wide layers have few voxels).
+__host__ __device__ constexpr int tc_nb(int n, int K) { return n % 32 == 0 && K <= 32 ? 32 : 16; }
+
+// Where w[tap][row][k] (n rows of K) stands in the image that the CTAs copy: per group of NB rows the B operands of
+// the nine (dy, dx) taps as they lie in shared memory, 3 NB rows each (dz tap 2, then 1, then 0, for the
+// output planes that an input plane is the last, second and first term of), rows of eight and 16-byte groups of k as the tensor core's core matrices.  A CTA's part
+// is contiguous, one bulk copy: copied and arranged by each CTA's threads, the weights took 92 us of the 366 us of
+// the fourteen layers' forward pass of eight cells of 64 x 64 x 32, most of it in layers of few CTAs.
+__device__ __forceinline__ int tc_weight_index(int n, int K, int tap, int row, int k)
+{
+    const int NB = tc_nb(n, K), r = (2 - tap / 9) * NB + row % NB;
+    return row / NB * (27 * NB * K) + ((tap % 9 * (3 * NB / 8) + r / 8) * (K / 8) + k / 8) * 64 + r % 8 * 8 + k % 8;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
@@ -210,22 +242,22 @@ __device__ __forceinline__ void unpack8(const uint4 y, float v[8])
     }
 }
 
-template <int NB, bool Flip>
-__global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
+template <int NB, bool Flip, int K>
+__global__ void __launch_bounds__(kTcThreads, NB == 32 && Flip ? 3 : 4) conv_tc_kernel(const ConvTc a)
 {
     extern __shared__ __align__(128) unsigned char tc_smem_raw[];
-    nh::step_kernel_enter();
-    const int K = a.c1 + a.c2, kb = K / 8;  // 16-byte channel groups
+    constexpr int kb = K / 8;  // 16-byte channel groups
     constexpr uint32_t kGroup = kTcHalo * 16;              // one channel group of a plane
-    const uint32_t plane_bytes = (uint32_t)kb * kGroup;
-    const uint32_t tap_bytes = (uint32_t)NB * K * 2;
-    const uint32_t ring = smem_u32(tc_smem_raw), wbase = ring + kTcRing * plane_bytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem_raw + kTcRing * plane_bytes + 27 * tap_bytes);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
+    constexpr uint32_t plane_bytes = (uint32_t)kb * kGroup;
+    constexpr uint32_t tap_bytes = 3u * NB * K * 2;  // of a (dy, dx) tap
+    const uint32_t ring = smem_u32(tc_smem_raw), wbase = ring + (uint32_t)a.ring * plane_bytes;
+    int* voxel = reinterpret_cast<int*>(tc_smem_raw + (uint32_t)a.ring * plane_bytes + 9 * tap_bytes);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(voxel + 2 * kTcHalo);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 5);
     float* bshared = reinterpret_cast<float*>(bars + 8);  // bias gradient of the CTA's voxels (with mask)
     if (Flip && threadIdx.x < NB) bshared[threadIdx.x] = 0.f;
-    constexpr uint32_t kCols = 2 * NB;  // two accumulators: 32 or 64 columns
-    static_assert(NB == 16 || NB == 32, "TMEM columns are allocated in powers of two, at least 32");
+    constexpr int kSlots = kTcCols / NB;
+    static_assert(NB == 16 || NB == 32, "3 NB is a valid N, and the strip holds the window of three and one being read");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const Dims d = a.d;
     const int tx = (d.nx + kTcX - 1) / kTcX, ty = (d.ny + kTcY - 1) / kTcY, tz = (d.nz + a.zc - 1) / a.zc;
@@ -239,54 +271,72 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
-                     "r"(kCols)
+                     "r"(kTcCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
+    // bars[0], [1]: the MMAs of an even or odd input plane are done; bars[2], [3]: its copies are; bars[4]: the weights are here
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&bars[0])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&bars[1])) : "memory");
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&bars[i])), "r"(i == 2 || i == 3 ? kTcCopy : 1)
+                         : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
 
     // a thread copies one channel group of every vstep-th voxel of a plane
-    const int cq = tid % kb, vfirst = tid / kb, vstep = kTcThreads / kb;
-    const bool loader = vfirst < vstep;
+    const int cq = tid % kb, vfirst = tid / kb, vstep = kTcCopy / kb;
+    const bool loader = tid < kTcCopy && vfirst < vstep;
     const bool from1 = cq * 8 < a.c1;
     const bool up = from1 && a.up1;
     const bf16* lsrc = from1 ? a.src1 + cq * 8 : a.src2 + (cq * 8 - a.c1);
     const int lc = from1 ? a.c1 : a.c2;
-    auto load_plane = [&](int z) {  // zero beyond the volume in z
-        if (loader) {
-            const bool zin = z >= 0 && z < d.nz;
-            const uint32_t dst = ring + (uint32_t)(z & (kTcRing - 1)) * plane_bytes + (uint32_t)cq * kGroup;
-            for (int v = vfirst; v < kTcHalo; v += vstep) {
-                const int hy = v / kTcHX, hx = v - hy * kTcHX;
-                int x = x0 - 1 + hx, y = y0 - 1 + hy;
-                x = x < 0 ? x + d.nx : (x >= d.nx ? x - d.nx : x);
-                y = y < 0 ? y + d.ny : (y >= d.ny ? y - d.ny : y);
-                const bool ok = zin && x < d.nx && y < d.ny;  // beyond a ragged tile's halo: unused, zero
-                const int s = up ? batch * (d.nvox >> 3) + (x >> 1) + (d.nx >> 1) * ((y >> 1) + (d.ny >> 1) * (z >> 1))
-                                 : batch * d.nvox + x + d.nx * (y + d.ny * z);
-                cp_async16(dst + (uint32_t)v * 16u, ok ? lsrc + (size_t)s * lc : lsrc, ok);
-            }
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    };
-    for (int i = tid; i < 27 * NB * kb; i += kTcThreads) {
-        const int q = i % kb, r = i / kb, n = r % NB, t = r / NB;
-        cp_async16(wbase + (uint32_t)t * tap_bytes + (uint32_t)(n >> 3) * (uint32_t)(kb * 128) + (uint32_t)q * 128u +
-                       (uint32_t)(n & 7) * 16u,
-                   a.w + ((size_t)t * a.n + n0 + n) * K + q * 8, true);
+    // where a plane's voxels lie in a z layer of the source, and in one of half the resolution
+    for (int v = tid; v < kTcHalo; v += kTcThreads) {
+        const int hy = v / kTcHX, hx = v - hy * kTcHX;
+        int x = x0 - 1 + hx, y = y0 - 1 + hy;
+        x = x < 0 ? x + d.nx : (x >= d.nx ? x - d.nx : x);
+        y = y < 0 ? y + d.ny : (y >= d.ny ? y - d.ny : y);
+        const bool ok = x < d.nx && y < d.ny;  // beyond a ragged tile's halo: unused, zero
+        voxel[v] = ok ? x + d.nx * y : -1;
+        voxel[kTcHalo + v] = ok ? (x >> 1) + (d.nx >> 1) * (y >> 1) : -1;
     }
-    for (int z = z0 - 1; z <= z0 + 1; ++z) load_plane(z);
-
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    nh::step_kernel_enter();  // nothing above reads or writes global memory
+    if (tid == kTcCopy) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(&bars[4])), "r"(9 * tap_bytes)
+                     : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(wbase),
+                     "l"(a.w + (size_t)blockIdx.y * (27 * NB * K)), "r"(9 * tap_bytes), "r"(smem_u32(&bars[4]))
+                     : "memory");
+    }
+    const int* lvox = voxel + (up ? kTcHalo : 0);
+    int lslot = 0;
+    // the input planes upwards from z0 - 1, for the mirrored taps of the data gradient downwards from z1: either way
+    // an output plane's terms come in the order of the taps
+    auto plane = [&](int w) { return Flip ? z1 - w : z0 - 1 + w; };
+    auto load_plane = [&](int w) {  // input plane w, zero beyond the volume in z; nothing beyond the chunk's
+        if (loader && w < z1 - z0 + 2) {
+            const int z = plane(w);
+            const bool zin = z >= 0 && z < d.nz;
+            const uint32_t dst = ring + (uint32_t)lslot * plane_bytes + (uint32_t)cq * kGroup;
+            const int first = up ? batch * (d.nvox >> 3) + (d.nx >> 1) * (d.ny >> 1) * (z >> 1) : batch * d.nvox + d.nx * d.ny * z;
+            for (int v = vfirst; v < kTcHalo; v += vstep) {
+                const int o = lvox[v];
+                const bool ok = zin && o >= 0;
+                cp_async16(dst + (uint32_t)v * 16u, ok ? lsrc + (size_t)(first + o) * lc : lsrc, ok);
+            }
+        }
+        if (++lslot == a.ring) lslot = 0;
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    const int steps = z1 - z0 + 2;  // input planes z0 - 1 ... z1
+    if (tid < kTcCopy)
+        for (int w = 0; w < a.ring - 1; ++w) load_plane(w);
 
-    constexpr uint32_t idesc = umma_idesc_bf16(kTcM, NB);
     // row r of the accumulator is voxel (x0 + r % 8, y0 + r / 8) of the plane
     const int row = warp * 32 + lane;
     const int vx = x0 + (row & 7), vy = y0 + (row >> 3);
@@ -294,8 +344,26 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
     float bsum[Flip ? NB : 1];  // bias gradient of this thread's voxels (with mask)
 #pragma unroll
     for (int i = 0; i < (Flip ? NB : 1); ++i) bsum[i] = 0.f;
-    auto epilogue = [&](int z) {
-        const uint32_t acc0 = tmem + (uint32_t)(((z - z0) & 1) * NB) + ((uint32_t)(warp * 32) << 16);
+    // the epilogue's operands, on their way while the tensor core works: the bias, or the next plane's ReLU mask
+    float bias[Flip ? 1 : NB];
+    uint4 mask[Flip ? NB / 8 : 1];
+    if constexpr (!Flip) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i) bias[i] = __ldg(a.bias + n0 + i);
+    }
+    auto load_mask = [&](int k) {
+        if constexpr (Flip)
+            if (a.mask != nullptr && inside && k < z1 - z0) {
+                const int z = plane(k + 1);
+                const size_t v = (size_t)batch * d.nvox + vx + (size_t)d.nx * (vy + (size_t)d.ny * z);
+#pragma unroll
+                for (int h = 0; h < NB / 8; ++h) mask[h] = __ldg(reinterpret_cast<const uint4*>(a.mask + v * a.n + n0) + h);
+            }
+    };
+    load_mask(0);
+    auto epilogue = [&](int k) {  // the k-th output plane
+        const int z = plane(k + 1);
+        const uint32_t acc0 = tmem + (uint32_t)((k + 2) % kSlots * NB) + ((uint32_t)(warp * 32) << 16);
         const size_t v = (size_t)batch * d.nvox + vx + (size_t)d.nx * (vy + (size_t)d.ny * z);
 #pragma unroll
         for (int c0 = 0; c0 < NB; c0 += 16) {
@@ -305,20 +373,18 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
             if constexpr (!Flip) {
                 uint32_t packed[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float b0 = __ldg(a.bias + n0 + c0 + 2 * i), b1 = __ldg(a.bias + n0 + c0 + 2 * i + 1);
-                    packed[i] = pack_bf16(fmaxf(acc[2 * i] + b0, 0.f), fmaxf(acc[2 * i + 1] + b1, 0.f));
-                }
+                for (int i = 0; i < 8; ++i)
+                    packed[i] = pack_bf16(fmaxf(acc[2 * i] + bias[c0 + 2 * i], 0.f),
+                                          fmaxf(acc[2 * i + 1] + bias[c0 + 2 * i + 1], 0.f));
                 uint4* dst = reinterpret_cast<uint4*>(a.out + v * a.n + n0 + c0);
                 dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                 dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
             } else if (a.mask != nullptr) {
-                const uint4* m = reinterpret_cast<const uint4*>(a.mask + v * a.n + n0 + c0);
                 uint4* dst = reinterpret_cast<uint4*>(a.gp + v * a.n + n0 + c0);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     float* g = acc + 8 * h;
-                    relu_mask(g, __ldg(m + h));
+                    relu_mask(g, mask[c0 / 8 + h]);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) bsum[c0 + 8 * h + i] += g[i];
                     dst[h] = pack8(g);
@@ -331,62 +397,90 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
                 for (int i = 0; i < 4; ++i) dst[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
             }
         }
+        load_mask(k + 1);
     };
 
     bool ok = true;
-    for (int z = z0; z < z1; ++z) {
-        const int k = z - z0;
-        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the copies, to the tensor core's view
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");  // the epilogue's TMEM reads
-        ok = __syncthreads_and(ok) != 0;
-        if (!ok) break;
-        if (tid == 0) {
+    if (warp == kTcCopy / 32) {
+        // The warp runs as one, its first lane's instructions taking effect: descriptors stay in uniform registers.
+        const uint32_t lead = lane == 0;
+        const uint64_t ad0 = umma_desc(0, kGroup, kTcHX * 16), bd0 = umma_desc(0, 128u, (uint32_t)kb * 128u);
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[4]), 0)) != 0;
+        // accumulators w, w + 1, w + 2 of the strip: output planes number w - 2, w - 1 and w of the chunk
+        for (int w = 0, slot = 0; w < steps && ok; ++w, slot = slot + 1 == a.ring ? 0 : slot + 1) {
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[2 + (w & 1)]), (w >> 1) & 1)) != 0;
+            if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            const uint64_t ad0 = umma_desc(0, kGroup, kTcHX * 16), bd0 = umma_desc(0, 128u, (uint32_t)kb * 128u);
-            const uint32_t acc0 = tmem + (uint32_t)((k & 1) * NB);
-            uint32_t acc = 0;
-            for (int dz = 0; dz < 3; ++dz) {
-                const int zp = Flip ? z + 1 - dz : z - 1 + dz;
-                const uint32_t pa = (ring + (uint32_t)(zp & (kTcRing - 1)) * plane_bytes) >> 4;
-#pragma unroll
-                for (int q = 0; q < 9; ++q) {
-                    const int off = Flip ? (2 - q / 3) * kTcHX + (2 - q % 3) : (q / 3) * kTcHX + q % 3;
-                    const uint32_t wa = (wbase + (uint32_t)(dz * 9 + q) * tap_bytes) >> 4;
-                    for (int j = 0; j < kb / 2; ++j) {
-                        const uint64_t ad = ad0 | (uint64_t)(pa + off + (uint32_t)j * (2 * kGroup >> 4));
-                        const uint64_t bd = bd0 | (uint64_t)(wa + (uint32_t)j * 16u);
-                        asm volatile(
-                            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc0),
-                            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                            : "memory");
-                        acc = 1;
-                    }
-                }
+            const uint32_t pa = (ring + (uint32_t)slot * plane_bytes) >> 4;
+            const int s = w % kSlots;
+            // rows o ... o + count - 1 of the stacked weights into the accumulators from slot t on
+            auto mma = [&](int q, int j, int o, int count, int t, uint32_t acc) {
+                const int off = Flip ? (2 - q / 3) * kTcHX + (2 - q % 3) : (q / 3) * kTcHX + q % 3;
+                const uint64_t ad = ad0 | (uint64_t)(pa + off + (uint32_t)j * (2 * kGroup >> 4));
+                const uint64_t bd = bd0 | (uint64_t)(((wbase + (uint32_t)q * tap_bytes) >> 4) +
+                                                     (uint32_t)o * (uint32_t)(NB * kb) + (uint32_t)j * 16u);
+                asm volatile(
+                    "{\n.reg .pred p, l;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 l, %5, 0;\n"
+                    "@l tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(t * NB)),
+                    "l"(ad), "l"(bd), "r"(umma_idesc_bf16(kTcM, count * NB)), "r"(acc), "r"(lead)
+                    : "memory");
+            };
+            const int head = min(3, kSlots - s);  // accumulators of the window before the strip's end
+            if (head == 1) {
+                mma(0, 0, 0, 1, s, 1);
+                mma(0, 0, 1, 1, 0, 1);
+            } else {
+                mma(0, 0, 0, 2, s, 1);
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                             smem_u32(&bars[k & 1]))
+            mma(0, 0, 2, 1, (s + 2) % kSlots, 0);
+            auto rest = [&](auto&& f) {
+#pragma unroll
+                for (int i = 1; i < 9 * (kb / 2); ++i) f(i / (kb / 2), i % (kb / 2));
+            };
+            if (head == 3)
+                rest([&](int q, int j) { mma(q, j, 0, 3, s, 1); });
+            else
+                rest([&](int q, int j) {
+                    mma(q, j, 0, head, s, 1);
+                    mma(q, j, head, 3 - head, 0, 1);
+                });
+            asm volatile("{\n.reg .pred l;\nsetp.ne.b32 l, %1, 0;\n"
+                         "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+                             smem_u32(&bars[w & 1])), "r"(lead)
                          : "memory");
+            __syncwarp();
         }
-        __syncwarp();
-        // the MMAs of plane z - 1 are done: their lowest input plane's slot takes plane z + 2
-        if (k > 0) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[(k - 1) & 1]), ((k - 1) >> 1) & 1)) != 0;
-        if (ok && z + 1 < z1) load_plane(z + 2);
-        if (ok && k > 0) {
+    } else {
+        for (int w = 0; w < steps && ok; ++w) {
+            if (a.ring == 5)
+                asm volatile("cp.async.wait_group 3;\n" ::: "memory");
+            else if (a.ring == 4)
+                asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+            else if (a.ring == 3)
+                asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+            else
+                asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the copies, to the tensor core's view
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");  // the epilogue's TMEM reads
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&bars[2 + (w & 1)])) : "memory");
+            // the MMAs of the plane before are done: its slot takes the next to come, and its lowest output is complete
+            if (w > 0) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[(w - 1) & 1]), ((w - 1) >> 1) & 1)) != 0;
+            if (ok) load_plane(w + a.ring - 1);
+            if (ok && w > 2) {
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                epilogue(w - 3);
+            }
+        }
+        if (ok) {
+            const int k = steps - 1;
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[k & 1]), (k >> 1) & 1)) != 0;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            epilogue(z - 1);
+            if (ok) epilogue(steps - 3);
         }
-    }
-    if (ok) {
-        const int k = z1 - 1 - z0;
-        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[k & 1]), (k >> 1) & 1)) != 0;
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        if (ok) epilogue(z1 - 1);
     }
     if (!ok && lane == 0) atomicExch(a.status, 1);
     if constexpr (Flip) {
-        if (a.mask != nullptr) {
+        if (a.mask != nullptr && tid < kTcCopy) {
             // halve the channels a lane holds as the lanes that add to it double: after the steps lane l has the
             // warp's sum of channel l mod NB (of NB 16, lanes l and l + 16 each half of it)
 #pragma unroll
@@ -407,49 +501,59 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const ConvTc a)
     if constexpr (Flip)
         if (a.mask != nullptr && tid < NB) atomicAdd(a.gb + n0 + tid, bshared[tid]);
     if (warp == 0) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTcCols) : "memory");
     }
 }
 
-// Launch over every plane tile of the level.  NB = 32 where two such weight
-// sets fit an SM (K <= 32), else 16: more CTAs on the coarse levels, whose wide
-// layers have few voxels.  Planes per chunk: the CTAs run in waves of as many as
-// an SM holds (shared memory, TMEM columns), and a chunk loads two planes beyond
-// its own; the split with the least waves x (planes + 2).  (8 planes of
-// 8 x 64 x 64 x 32 voxels made 1024 CTAs of which 912 are resident.)
-template <bool Flip>
+// Launch over every plane tile of the level.  Planes per chunk and of the ring: the
+// CTAs run in waves of as many as an SM holds (shared memory, TMEM columns,
+// registers), and a chunk loads two planes beyond its own; the pair with the least
+// waves x (planes + 2).  (8 x 64 x 64 x 32 voxels at K = 32: three planes held, three
+// CTAs an SM and two waves of 11 planes 66 us, two held, four an SM and one wave of
+// 16 planes 55 us, both with K at run time.)
+template <bool Flip, int K, int NB>
 cudaError_t launch_conv_tc(ConvTc a, cudaStream_t st)
 {
     static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<16, Flip>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTcMaxSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv_tc_kernel<32, Flip>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcMaxSmem);
+        const cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<NB, Flip, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)kTcMaxSmem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    const int K = a.c1 + a.c2;
-    const int NB = a.n % 32 == 0 && K <= 32 ? 32 : 16;
-    if (K % 16 || a.n % 16 || a.c1 % 8 || tc_smem(K, NB) > kTcMaxSmem) return cudaErrorInvalidValue;
+    if (a.n % NB || a.c1 % 8) return cudaErrorInvalidValue;
     const int cols = ((a.d.nx + kTcX - 1) / kTcX) * ((a.d.ny + kTcY - 1) / kTcY) * a.d.batch;
-    const int resident = 152 * std::min((int)(kTcMaxSmem / (tc_smem(K, NB) + 1024)), 512 / (2 * NB));
     int64_t best = -1;
-    for (int n = 1; n <= a.d.nz; ++n) {
-        const int zc = (a.d.nz + n - 1) / n;
-        const int64_t blocks = (int64_t)cols * ((a.d.nz + zc - 1) / zc) * (a.n / NB);
-        const int64_t cost = (blocks + resident - 1) / resident * (zc + 2);
-        if (best < 0 || cost < best) {
+    for (int ring = 2; ring <= kTcMaxRing && tc_smem(K, NB, ring) <= kTcMaxSmem; ++ring) {
+        const int per_sm = std::min((int)(kTcSmSmem / (tc_smem(K, NB, ring) + 1024)), NB == 32 && Flip ? 3 : 4);
+        for (int n = 1; n <= a.d.nz; ++n) {
+            const int zc = (a.d.nz + n - 1) / n;
+            const int64_t blocks = (int64_t)cols * ((a.d.nz + zc - 1) / zc) * (a.n / NB);
+            const int64_t cost = (blocks + 152 * per_sm - 1) / (152 * per_sm) * (zc + 2);
+            if (best >= 0 && (cost > best || (cost == best && ring == a.ring))) continue;
             best = cost;
             a.zc = zc;
+            a.ring = ring;
         }
     }
     const dim3 grid(cols * ((a.d.nz + a.zc - 1) / a.zc), a.n / NB);
-    if (NB == 32)
-        nh::launch_step_kernel(conv_tc_kernel<32, Flip>, grid, kTcThreads, tc_smem(K, NB), st, a);
-    else
-        nh::launch_step_kernel(conv_tc_kernel<16, Flip>, grid, kTcThreads, tc_smem(K, NB), st, a);
+    nh::launch_step_kernel(conv_tc_kernel<NB, Flip, K>, grid, kTcThreads, tc_smem(K, NB, a.ring), st, a);
     return cudaGetLastError();
+}
+
+// The depths K and widths that the network's layers have, forward and (Flip) backward.
+template <bool Flip>
+cudaError_t launch_conv_tc(const ConvTc& a, cudaStream_t st)
+{
+    const int K = a.c1 + a.c2, NB = tc_nb(a.n, K);
+    if (K == 16) return NB == 32 ? launch_conv_tc<Flip, 16, 32>(a, st) : launch_conv_tc<Flip, 16, 16>(a, st);
+    if (K == 32) return NB == 32 ? launch_conv_tc<Flip, 32, 32>(a, st) : launch_conv_tc<Flip, 32, 16>(a, st);
+    if (K == 64) return launch_conv_tc<Flip, 64, 16>(a, st);
+    if constexpr (!Flip) {  // concatenated sources
+        if (K == 48) return launch_conv_tc<Flip, 48, 16>(a, st);
+        if (K == 96) return launch_conv_tc<Flip, 96, 16>(a, st);
+    }
+    return cudaErrorInvalidValue;
 }
 
 // ------------------------------------------------------------------ convolution: weight gradient
@@ -474,9 +578,12 @@ struct ConvBwdW {
 // activations again for every tap made this 2291 us for a 16 -> 16 layer of
 // 8 x 64 x 64 x 32 voxels.  Warp w takes the nine taps of dz = w % 3 - 1 and half
 // w / 3 of the tile's voxels: per 16 voxels (two x runs of eight) one transposed
-// ldmatrix of the gradient is multiplied with nine of the shifted activations;
-// the 9 x 16 x 16 sums stay in registers (72 a thread) until the block's last
-// tile.  Rows are 32 bytes; their two 16-byte halves are swapped on every other
+// ldmatrix of the gradient is multiplied with nine of the shifted activations,
+// whose pairs of rows serve all three dy (five ldmatrix per dx and layer instead of
+// twelve); the 9 x 16 x 16 sums stay in registers (72 a thread) until the block's
+// last tile.  Two blocks an SM of 164 registers: 36 us for that layer with an
+// ldmatrix per tap and three blocks of 96 registers, with spills if those kept the
+// rows; with caches cold 58 us then and 45 us now.  Rows are 32 bytes; their two 16-byte halves are swapped on every other
 // group of four voxels of a run, so that the eight rows of an ldmatrix hit
 // distinct banks at any x shift.
 constexpr int kWTx = 8, kWTy = 8, kWTz = 4, kWVox = kWTx * kWTy * kWTz;
@@ -484,7 +591,8 @@ constexpr int kWHx = kWTx + 2, kWHy = kWTy + 2, kWHz = kWTz + 2, kWHalo = kWHx *
 constexpr int kWThreads = 192;
 constexpr int kWStage = (kWVox + kWHalo) * 32;  // bytes: gradient rows, then activation rows
 constexpr int kWSmem = 2 * kWStage;
-constexpr int kWBlocksPerSM = 3;
+constexpr int kWBlocksPerSM = 2;
+static_assert(kWHx * kWHy * 2 == kWThreads + 8 && 8 * kWHz <= kWThreads, "the halo's copies");
 
 __device__ __forceinline__ void ldm_x4_trans(uint32_t addr, uint32_t r[4])
 {
@@ -509,14 +617,31 @@ __global__ void __launch_bounds__(kWThreads, kWBlocksPerSM) conv_bwd_w_kernel(co
     const int tx = (d.nx + kWTx - 1) / kWTx, ty = (d.ny + kWTy - 1) / kWTy, tz = (d.nz + kWTz - 1) / kWTz;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    // copies of one tile into stage s; rows outside the volume (and the
-    // gradient of voxels beyond a ragged tile's end) are zero
-    auto load_tile = [&](int t, int s) {
-        const int x0 = (t % tx) * kWTx;
-        int r = t / tx;
-        const int y0 = (r % ty) * kWTy;
-        r /= ty;
-        const int z0 = (r % tz) * kWTz, batch = r / tz, vb = batch * d.nvox;
+    // tile t and its successors t + gridDim.x, ...: x, y, z, batch advance with carries
+    int t = blockIdx.x, bx = t % tx, by = t / tx % ty, bz = t / (tx * ty) % tz, bb = t / (tx * ty * tz);
+    const int G = gridDim.x, sx = G % tx, sy = G / tx % ty, sz = G / (tx * ty) % tz, sb = G / (tx * ty * tz);
+    // Copies of the current tile into stage s; rows outside the volume (and the gradient of voxels beyond a ragged
+    // tile's end) are zero.  A thread copies one half row of the halo's 10 x 10 columns in all its layers (the last
+    // eight of the 200 half rows go to 48 threads, a layer each), so that a column's wrapped address is found once.
+    const int h2 = kWThreads + (tid & 7);
+    auto load_halo = [&](uint32_t X, int h, int z0, int lo, int hi) {
+        const int c = h & 1, hy = (h >> 1) / kWHx, hx = (h >> 1) - hy * kWHx;
+        int x = bx * kWTx - 1 + hx, y = by * kWTy - 1 + hy;
+        x = x < 0 ? x + d.nx : (x >= d.nx ? x - d.nx : x);
+        y = y < 0 ? y + d.ny : (y >= d.ny ? y - d.ny : y);
+        const bool xyok = x < d.nx && y < d.ny;
+        const int shift = up ? 1 : 0, layer = (d.nx >> shift) * (d.ny >> shift);
+        const bf16* col = xs + (size_t)(bb * (up ? d.nvox >> 3 : d.nvox) + (x >> shift) + (d.nx >> shift) * (y >> shift)) * xc + 8 * c;
+        const uint32_t dst = X + (uint32_t)(h >> 1) * 32u + (uint32_t)((c ^ ((hx >> 2) & 1)) << 4);
+#pragma unroll
+        for (int hz = lo; hz < hi; ++hz) {
+            const int z = z0 - 1 + hz;
+            const bool ok = xyok && z >= 0 && z < d.nz;
+            cp_async16(dst + (uint32_t)hz * (kWHx * kWHy * 32), ok ? col + (size_t)(layer * (z >> shift)) * xc : xs, ok);
+        }
+    };
+    auto load_tile = [&](int s) {
+        const int x0 = bx * kWTx, y0 = by * kWTy, z0 = bz * kWTz, vb = bb * d.nvox;
         const uint32_t G = smem0 + (uint32_t)s * kWStage, X = G + kWVox * 32;
         for (int i = tid; i < kWVox * 2; i += kWThreads) {
             const int c = i & 1, v = i >> 1;
@@ -525,20 +650,16 @@ __global__ void __launch_bounds__(kWThreads, kWBlocksPerSM) conv_bwd_w_kernel(co
             const bf16* src = ok ? a.gp + (size_t)(vb + x + d.nx * (y + d.ny * z)) * a.cout + co0 + 8 * c : a.gp;
             cp_async16(G + v * 32 + ((c ^ ((v >> 2) & 1)) << 4), src, ok);
         }
-        for (int i = tid; i < kWHalo * 2; i += kWThreads) {
-            const int c = i & 1, v = i >> 1;
-            const int hx = v % kWHx, hy = (v / kWHx) % kWHy, hz = v / (kWHx * kWHy);
-            int x = x0 - 1 + hx, y = y0 - 1 + hy;
-            const int z = z0 - 1 + hz;
-            x = x < 0 ? x + d.nx : (x >= d.nx ? x - d.nx : x);
-            y = y < 0 ? y + d.ny : (y >= d.ny ? y - d.ny : y);
-            const bool ok = x < d.nx && y < d.ny && z >= 0 && z < d.nz;
-            const int sv = up ? batch * (d.nvox >> 3) + (x >> 1) + (d.nx >> 1) * ((y >> 1) + (d.ny >> 1) * (z >> 1))
-                              : vb + x + d.nx * (y + d.ny * z);
-            const bf16* src = ok ? xs + (size_t)sv * xc + 8 * c : xs;
-            cp_async16(X + v * 32 + ((c ^ ((hx >> 2) & 1)) << 4), src, ok);
-        }
+        load_halo(X, tid, z0, 0, kWHz);
+        if (tid < 8 * kWHz) load_halo(X, h2, z0, tid >> 3, (tid >> 3) + 1);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
+        bx += sx;
+        by += sy + (bx >= tx);
+        bx -= bx >= tx ? tx : 0;
+        bz += sz + (by >= ty);
+        by -= by >= ty ? ty : 0;
+        bb += sb + (bz >= tz);
+        bz -= bz >= tz ? tz : 0;
     };
 
     const int dz = warp % 3, half = warp / 3;
@@ -556,30 +677,47 @@ __global__ void __launch_bounds__(kWThreads, kWBlocksPerSM) conv_bwd_w_kernel(co
 #pragma unroll
         for (int h = 0; h < 2; ++h) acc[q][h][0] = acc[q][h][1] = acc[q][h][2] = acc[q][h][3] = 0.f;
 
-    int t = blockIdx.x;
-    if (t < a.tiles) load_tile(t, 0);
+    if (t < a.tiles) load_tile(0);
     for (int s = 0; t < a.tiles; t += gridDim.x, s ^= 1) {
         if (t + (int)gridDim.x < a.tiles) {
-            load_tile(t + gridDim.x, s ^ 1);
+            load_tile(s ^ 1);
             asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         }
         __syncthreads();
         const uint32_t G = smem0 + (uint32_t)s * kWStage, X = G + kWVox * 32;
-#pragma unroll 2
-        for (int k = 0; k < 8; ++k) {  // 16 voxels: rows y = 2 j, 2 j + 1 of layer z
-            const int z = 2 * half + (k >> 2), j = k & 3;
-            uint32_t fa[4];
-            ldm_x4_trans(G + laneA + (uint32_t)((z * kWTy + 2 * j) * kWTx * 32), fa);
-            const uint32_t xb = X + (uint32_t)(((z + dz) * kWHy + 2 * j) * (kWHx * 32));
 #pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                uint32_t fb[4];
-                ldm_x4_trans(xb + laneB[q % 3] + (uint32_t)(q / 3) * (kWHx * 32), fb);
-                mma16816(acc[q][0], fa, fb);
-                mma16816(acc[q][1], fa, fb + 2);
+        for (int dx = 0; dx < 3; ++dx) {
+            // a tile's sums by themselves: the tensor core's additions do not round to nearest, and a chain of them
+            // through all of a block's tiles is off by as many units in the last place
+            float part[3][2][4] = {};
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                const uint32_t xb = X + laneB[dx] + (uint32_t)((2 * half + z + dz) * kWHy * (kWHx * 32));
+                uint32_t fa[4][4];  // 16 voxels: rows y = 2 j, 2 j + 1
+#pragma unroll
+                for (int j = 0; j < 4; ++j) ldm_x4_trans(G + laneA + (uint32_t)(((2 * half + z) * kWTy + 2 * j) * kWTx * 32), fa[j]);
+                uint32_t lo[4], hi[4];  // halo rows 2 j, 2 j + 1 and the two above
+                ldm_x4_trans(xb, lo);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    ldm_x4_trans(xb + (uint32_t)((2 * j + 2) * (kWHx * 32)), hi);
+                    const uint32_t b0[2] = {lo[1], hi[0]}, b1[2] = {lo[3], hi[2]};
+                    mma16816(part[0][0], fa[j], lo);
+                    mma16816(part[0][1], fa[j], lo + 2);
+                    mma16816(part[1][0], fa[j], b0);
+                    mma16816(part[1][1], fa[j], b1);
+                    mma16816(part[2][0], fa[j], hi);
+                    mma16816(part[2][1], fa[j], hi + 2);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) lo[i] = hi[i];
+                }
             }
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[3 * q + dx][i >> 2][i & 3] += part[q][i >> 2][i & 3];
         }
         __syncthreads();
     }
@@ -746,27 +884,16 @@ __global__ void input_kernel(const float* __restrict__ n, const float* __restric
     }
 }
 
-// Head (1x1x1 conv 16 -> 3), residual on the ansatz, normalisation.  Train: the
-// loss mean |n - target|^2, the gradients of W_head and b_head, and the last
-// convolution's pre-activation gradient (ReLU mask of d1, BF16) and bias gradient.
-template <bool Train>
+// Head (1x1x1 conv 16 -> 3), residual on the ansatz, normalisation.
 __global__ void __launch_bounds__(256) head_kernel(const bf16* __restrict__ d1, const float* __restrict__ n_ans,
-                                                   const float* __restrict__ params_head, float* __restrict__ n_out,
-                                                   const float* __restrict__ target, bf16* __restrict__ gp,
-                                                   float* __restrict__ gb, float* __restrict__ g_head,
-                                                   float* __restrict__ loss, Dims d)
+                                                   const float* __restrict__ params_head, float* __restrict__ n_out, Dims d)
 {
     nh::step_kernel_enter();
-    constexpr int kW = kHeadOut * kHeadIn, kSums = kW + kHeadOut + 1 + kHeadIn;  // W, b, loss, bias of the last conv
+    constexpr int kW = kHeadOut * kHeadIn;
     __shared__ float sh[kW + kHeadOut];
-    __shared__ float red[kSums][8];
     for (int k = threadIdx.x; k < kW + kHeadOut; k += blockDim.x) sh[k] = params_head[k];
     __syncthreads();
     const int total = d.nvox * d.batch;
-    const float inv_total = 1.f / (float)total;
-    float gacc[Train ? kSums : 1];
-#pragma unroll
-    for (int k = 0; k < (Train ? kSums : 1); ++k) gacc[k] = 0.f;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < total; v += gridDim.x * blockDim.x) {
         const int b = v / d.nvox, r = v - b * d.nvox;
         const size_t o0 = (size_t)b * 3 * d.nvox + r;
@@ -783,61 +910,119 @@ __global__ void __launch_bounds__(256) head_kernel(const bf16* __restrict__ d1, 
             vv[o] = n_ans[o0 + (size_t)o * d.nvox] + s;
         }
         const float len = sqrtf(vv[0] * vv[0] + vv[1] * vv[1] + vv[2] * vv[2]);
-        const float nn[3] = {vv[0] / len, vv[1] / len, vv[2] / len};
-        if (n_out)
 #pragma unroll
-            for (int o = 0; o < 3; ++o) n_out[o0 + (size_t)o * d.nvox] = nn[o];
-        if constexpr (Train) {
-            float gn[3], dot = 0.f, l = 0.f;
-#pragma unroll
-            for (int o = 0; o < 3; ++o) {
-                const float diff = nn[o] - target[o0 + (size_t)o * d.nvox];
-                l += diff * diff;
-                gn[o] = 2.f * diff * inv_total;
-                dot += gn[o] * nn[o];
-            }
-            gacc[kW + kHeadOut] += l * inv_total;
-            float gd[3];
-#pragma unroll
-            for (int o = 0; o < 3; ++o) gd[o] = (gn[o] - dot * nn[o]) / len;  // d/dv of v/|v|
-            float g[kHeadIn];
-#pragma unroll
-            for (int c = 0; c < kHeadIn; ++c) {
-                float s = 0.f;
-#pragma unroll
-                for (int o = 0; o < 3; ++o) {
-                    s += sh[o * kHeadIn + c] * gd[o];
-                    gacc[o * kHeadIn + c] += gd[o] * h[c];
-                }
-                g[c] = h[c] > 0.f ? s : 0.f;
-                gacc[kW + kHeadOut + 1 + c] += g[c];
-            }
-#pragma unroll
-            for (int o = 0; o < 3; ++o) gacc[kW + o] += gd[o];
-            uint4* dst = reinterpret_cast<uint4*>(gp + (size_t)v * kHeadIn);
-            dst[0] = pack8(g);
-            dst[1] = pack8(g + 8);
-        }
+        for (int o = 0; o < 3; ++o)
+            if (n_out) n_out[o0 + (size_t)o * d.nvox] = vv[o] / len;
     }
-    if constexpr (Train) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+}
+
+// The head again with the loss mean |n - target|^2, the gradients of W_head and
+// b_head, and the last convolution's pre-activation gradient (ReLU mask of d1,
+// BF16) and bias gradient.  Two lanes share a voxel, eight channels each, and
+// pass on their halves of the three dot products: a lane keeps 36 running sums
+// where a thread per voxel kept 68, which held an SM to one block of 164
+// registers (58 us at 8 x 64 x 64 x 32 voxels, waiting for memory; now 35 us).
+__global__ void __launch_bounds__(256, 2) head_bwd_kernel(const bf16* __restrict__ d1, const float* __restrict__ n_ans,
+                                                          const float* __restrict__ params_head,
+                                                          const float* __restrict__ target, bf16* __restrict__ gp,
+                                                          float* __restrict__ gb, float* __restrict__ g_head,
+                                                          float* __restrict__ loss, Dims d)
+{
+    nh::step_kernel_enter();
+    constexpr int kW = kHeadOut * kHeadIn;
+    // a lane's sums: W[3][8], bias of its eight channels, b_head[3], loss (of both lanes of a voxel: halved)
+    constexpr int kSums = kHeadOut * 8 + 8 + kHeadOut + 1;
+    __shared__ float red[2][kSums][8];
+    const int half = threadIdx.x & 1;
+    float w[kHeadOut][8], b3[kHeadOut];
 #pragma unroll
-        for (int k = 0; k < kSums; ++k) {
-            float s = gacc[k];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) red[k][warp] = s;
+    for (int o = 0; o < kHeadOut; ++o) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) w[o][c] = params_head[o * kHeadIn + half * 8 + c];
+        b3[o] = params_head[kW + o];
+    }
+    const int total = d.nvox * d.batch;
+    const float inv_total = 1.f / (float)total;
+    float sum[kSums];
+#pragma unroll
+    for (int k = 0; k < kSums; ++k) sum[k] = 0.f;
+    const int stride = (gridDim.x * blockDim.x) >> 1;
+    // the voxel count (of 16 x 16 x 8 at least, in eights) and the stride are multiples of 16: a warp stays together
+    for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 1; v < total; v += stride) {
+        const int b = v / d.nvox, r = v - b * d.nvox;
+        const size_t o0 = (size_t)b * 3 * d.nvox + r;
+        float h[8];
+        unpack8(__ldg(reinterpret_cast<const uint4*>(d1 + (size_t)v * kHeadIn) + half), h);
+        float vv[3], tg[3];
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            vv[o] = __ldg(n_ans + o0 + (size_t)o * d.nvox);
+            tg[o] = __ldg(target + o0 + (size_t)o * d.nvox);
         }
-        __syncthreads();
-        for (int k = threadIdx.x; k < kSums; k += blockDim.x) {
-            float s = 0.f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[k][w];
-            if (k < kW + kHeadOut)
-                atomicAdd(&g_head[k], s);
-            else if (k == kW + kHeadOut)
-                atomicAdd(loss, s);
-            else
-                atomicAdd(&gb[k - (kW + kHeadOut + 1)], s);
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            // b + the sixteen products one after another, as the forward head adds them: where n_ansatz and the
+            // correction nearly cancel, another order would move n
+            float s = b3[o];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) s += w[o][c] * h[c];
+            s = __shfl_xor_sync(0xffffffffu, s, 1);  // of the upper lane: the lower one's sum
+#pragma unroll
+            for (int c = 0; c < 8; ++c) s += w[o][c] * h[c];
+            vv[o] += __shfl_sync(0xffffffffu, s, threadIdx.x | 1);
         }
+        const float len = sqrtf(vv[0] * vv[0] + vv[1] * vv[1] + vv[2] * vv[2]);
+        float gn[3], nn[3], dot = 0.f, l = 0.f;
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            nn[o] = vv[o] / len;
+            const float diff = nn[o] - tg[o];
+            l += diff * diff;
+            gn[o] = 2.f * diff * inv_total;
+            dot += gn[o] * nn[o];
+        }
+        sum[kSums - 1] += l * inv_total;
+        float g[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) g[c] = 0.f;
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            const float gd = (gn[o] - dot * nn[o]) / len;  // d/dv of v/|v|
+            sum[32 + o] += gd;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                g[c] += w[o][c] * gd;
+                sum[o * 8 + c] += gd * h[c];
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            g[c] = h[c] > 0.f ? g[c] : 0.f;
+            sum[24 + c] += g[c];
+        }
+        reinterpret_cast<uint4*>(gp + (size_t)v * kHeadIn)[half] = pack8(g);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < kSums; ++k) {
+        float s = sum[k];
+        for (int o = 16; o > 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane < 2) red[lane][k][warp] = s;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * kSums; i += blockDim.x) {
+        const int hh = i / kSums, k = i - hh * kSums;
+        if (hh == 1 && k >= 32) continue;  // both lanes have these
+        float s = 0.f;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += red[hh][k][q];
+        if (k < 24)
+            atomicAdd(&g_head[(k >> 3) * kHeadIn + hh * 8 + (k & 7)], s);
+        else if (k < 32)
+            atomicAdd(&gb[hh * 8 + k - 24], s);
+        else if (k < 35)
+            atomicAdd(&g_head[kW + k - 32], s);
+        else
+            atomicAdd(loss, s);
     }
 }
 
@@ -847,26 +1032,25 @@ __global__ void bf16_to_f32_kernel(const bf16* __restrict__ a, float* __restrict
         out[i] = __bfloat162float(a[i]);
 }
 
-// BF16 copies of all parameters, and of the convolution weights transposed,
-// wt[l][tap][ci][co] = w[l][tap][co][ci], in one launch (one per layer took 45 us).
+// BF16 weights of all convolutions as the forward pass's and the data gradient's
+// images, in one launch (one per layer took 45 us).
 struct ParamTable {
     int begin[kLayers + 1];  // first parameter of each layer, and of the head
     int cin[kLayers], cout[kLayers];
-    bf16* wt[kLayers];
+    bf16 *w[kLayers], *wt[kLayers];
 };
-__global__ void params_kernel(const float* __restrict__ p, bf16* __restrict__ w, const ParamTable t, int n)
+__global__ void params_kernel(const float* __restrict__ p, const ParamTable t)
 {
     nh::step_kernel_enter();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const bf16 v = __float2bfloat16_rn(p[i]);
-        w[i] = v;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < t.begin[kLayers]; i += gridDim.x * blockDim.x) {
         int l = 0;
-        while (l < kLayers && i >= t.begin[l + 1]) ++l;
-        if (l == kLayers) continue;
-        const int k = i - t.begin[l], cc = t.cin[l] * t.cout[l];
+        while (i >= t.begin[l + 1]) ++l;
+        const int cin = t.cin[l], cout = t.cout[l], k = i - t.begin[l], cc = cin * cout;
         if (k >= 27 * cc) continue;  // bias
-        const int tap = k / cc, r = k - tap * cc, co = r / t.cin[l], ci = r - co * t.cin[l];
-        t.wt[l][tap * cc + ci * t.cout[l] + co] = v;
+        const int tap = k / cc, r = k - tap * cc, co = r / cin, ci = r - co * cin;
+        const bf16 v = __float2bfloat16_rn(p[i]);
+        t.w[l][tc_weight_index(cout, cin, tap, co, ci)] = v;
+        t.wt[l][tc_weight_index(cin, cout, tap, ci, co)] = v;
     }
 }
 
@@ -902,7 +1086,7 @@ struct nh_unet {
     size_t ws_bytes = 0;
     size_t need = 0;
     // offsets into the workspace
-    size_t wbf, wt[kLayers], x, act[kLayers], pool_[3], grad, grad_skip[3], gp[2], status;
+    size_t w[kLayers], wt[kLayers], x, act[kLayers], pool_[3], grad, grad_skip[3], gp[2], status;
     std::string err;
 };
 
@@ -925,9 +1109,10 @@ void plan(nh_unet* u)
         off += al(b);
         return o;
     };
-    const int64_t P = total_params();
-    u->wbf = take(P * sizeof(bf16));
-    for (int l = 0; l < kLayers; ++l) u->wt[l] = take(27 * (size_t)kConv[l].cin * kConv[l].cout * sizeof(bf16));
+    for (int l = 0; l < kLayers; ++l) {
+        u->w[l] = take(27 * (size_t)kConv[l].cin * kConv[l].cout * sizeof(bf16));
+        u->wt[l] = take(27 * (size_t)kConv[l].cin * kConv[l].cout * sizeof(bf16));
+    }
     const size_t V0 = (size_t)u->lv[0].nvox * u->batch;
     u->x = take(V0 * kInCh * sizeof(bf16));
     const int level_of[kLayers] = {0, 0, 1, 1, 2, 2, 3, 3, 2, 2, 1, 1, 0, 0};
@@ -962,7 +1147,7 @@ cudaError_t conv_fwd(nh_unet* u, int l, int level, const bf16* s1, int c1, const
     a.src2 = s2;
     a.c2 = c2;
     a.up1 = up1;
-    a.w = P<bf16>(u, u->wbf) + layer_offset(l);
+    a.w = P<bf16>(u, u->w[l]);
     a.n = kConv[l].cout;
     a.bias = params + layer_offset(l) + 27LL * kConv[l].cin * kConv[l].cout;
     a.out = P<bf16>(u, u->act[l]);
@@ -1095,16 +1280,16 @@ int nh_unet_set_params(nh_unet* u, const float* params, void* stream)
 {
     if (!u || !u->ws || !params) return unet_fail(u, NH_EINVAL, "unbound network or NULL params");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int n = (int)total_params();
     ParamTable t;
     for (int l = 0; l < kLayers; ++l) {
         t.begin[l] = (int)layer_offset(l);
         t.cin[l] = kConv[l].cin;
         t.cout[l] = kConv[l].cout;
+        t.w[l] = P<bf16>(u, u->w[l]);
         t.wt[l] = P<bf16>(u, u->wt[l]);
     }
     t.begin[kLayers] = (int)head_offset();
-    nh::launch_step_kernel(params_kernel, grid_for(n), 256, 0, st, params, P<bf16>(u, u->wbf), t, n);
+    nh::launch_step_kernel(params_kernel, grid_for(head_offset()), 256, 0, st, params, t);
     UNET_CUDA(u, cudaGetLastError());
     return NH_OK;
 }
@@ -1140,8 +1325,8 @@ int nh_unet_forward(nh_unet* u, const float* params, const float* n_ansatz, cons
     UNET_CUDA(u, conv_fwd(u, DEC2B, 1, act(DEC2A), 16, nullptr, 0, false, params, st));
     UNET_CUDA(u, conv_fwd(u, DEC1A, 0, act(DEC2B), 16, act(ENC1B), 16, true, params, st));
     UNET_CUDA(u, conv_fwd(u, DEC1B, 0, act(DEC1A), 16, nullptr, 0, false, params, st));
-    nh::launch_step_kernel(head_kernel<false>, grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st, act(DEC1B), n_ansatz,
-                           params + head_offset(), n_out, nullptr, nullptr, nullptr, nullptr, nullptr, d0);
+    nh::launch_step_kernel(head_kernel, grid_for((int64_t)d0.nvox * d0.batch), 256, 0, st, act(DEC1B), n_ansatz,
+                           params + head_offset(), n_out, d0);
     UNET_CUDA(u, cudaGetLastError());
     return NH_OK;
 }
@@ -1174,8 +1359,8 @@ int nh_unet_backward(nh_unet* u, const float* params, const float* n_ansatz, con
                                gskip[fine], act(l), gpa, gbias(l), u->lv[fine], C);
         return cudaGetLastError();
     };
-    nh::launch_step_kernel(head_kernel<true>, std::min(4 * 152, grid_for((int64_t)d0.nvox * d0.batch)), 256, 0, st,
-                           act(DEC1B), n_ansatz, params + head_offset(), nullptr, target, gpa, gbias(DEC1B),
+    nh::launch_step_kernel(head_bwd_kernel, std::min(2 * 152, grid_for((int64_t)d0.nvox * d0.batch * 2)), 256, 0, st,
+                           act(DEC1B), n_ansatz, params + head_offset(), target, gpa, gbias(DEC1B),
                            grad + head_offset(), loss, d0);
     UNET_CUDA(u, cudaGetLastError());
     // decoder: of each level the second convolution, then the first, whose sources are the upsampled level
