@@ -859,6 +859,8 @@ namespace {
 
 struct BatchPlan {
     std::vector<nh_ctx*> ctxs;
+    nh_ctx* owner = nullptr;         // the batch's first channel, which counts launches and keeps times
+    std::vector<BatchPlan> groups;   // of channels that stay in L2 together (batch_groups); empty: none
     std::vector<int64_t> epochs;
     int variant = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -889,6 +891,40 @@ void drop_batch_plans(const nh_ctx* c)
         } else {
             ++it;
         }
+    }
+}
+
+// Groups of consecutive channels whose LB steps find each other's populations in
+// the 129 MB L2: two population buffers and the force, kGroupBytes together.  64
+// steps of 64 channels (7 M sites, FP32, dt_fd 16): all channels at once 12.9 ms, in
+// pairs of steps 11.7, groups of 60, 84 and 110 MB with their FD updates 11.7, 11.3
+// and 12.2, groups of 70, 84 and 100 MB for the LB steps alone 10.1, 10.2 and 10.9
+// (12 channels: 2.0 each, at once 2.6; dt_fd 4: 17.6 at once, 15.9).  Blocks of two
+// steps gain nothing (23.4 | 23.5).  Not where the channels take pairs of steps
+// (large ones).
+constexpr double kGroupBytes = 84e6;
+constexpr int kGroupMinSteps = 4;
+bool batch_pair_ok(const BatchPlan* b);
+void batch_groups(BatchPlan* b)
+{
+    double total = 0;
+    std::vector<double> bytes;
+    for (const nh_ctx* c : b->ctxs) {
+        const double reals = c->p.precision == NH_FP64 ? 8 : 4;
+        bytes.push_back((2 * 19 * (double)store_size(c->p) + 3 * reals) * (double)c->N);
+        total += bytes.back();
+    }
+    const int groups = (int)std::ceil(total / kGroupBytes);
+    if (groups < 2 || b->ctxs.size() < 2 || batch_pair_ok(b)) return;
+    double sum = 0;  // cut where the running sum passes an even share
+    for (size_t k = 0; k < b->ctxs.size(); ++k) {
+        if (b->groups.empty() || sum + 0.5 * bytes[k] > total * (double)b->groups.size() / groups) {
+            b->groups.emplace_back();
+            b->groups.back().owner = b->owner;
+            b->groups.back().variant = b->variant;
+        }
+        b->groups.back().ctxs.push_back(b->ctxs[k]);
+        sum += bytes[k];
     }
 }
 
@@ -931,6 +967,7 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
         plan = new (std::nothrow) BatchPlan();
         if (!plan) return fail(nullptr, NH_ENOMEM, "host allocation of the batch plan failed");
         plan->ctxs = key;
+        plan->owner = c0;
         plan->epochs = epochs;
         // ctxs[0]'s shape if it was set and fits every channel (the row-staged one runs single channels only),
         // else the default of the batch's channels taken as one domain
@@ -946,6 +983,7 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
         if (!fits(v)) v = 2;
         if (!fits(v)) v = 1;  // one site per thread fits every domain
         plan->variant = v;
+        batch_groups(plan);
     }
     *out = plan;
     return NH_OK;
@@ -974,6 +1012,7 @@ int batch_prepare_relax(nh_ctx* const* ctxs, int count, int64_t n_fd_steps, Batc
     if (r) return fail(nullptr, r, c0->err);
     static thread_local BatchPlan plan;
     plan.ctxs.assign(ctxs, ctxs + count);
+    plan.owner = c0;
     *out = &plan;
     return NH_OK;
 }
@@ -981,7 +1020,7 @@ int batch_prepare_relax(nh_ctx* const* ctxs, int count, int64_t n_fd_steps, Batc
 template <typename Real, typename Store>
 int batch_lb_typed(BatchPlan* b, bool write_macro, cudaStream_t st)
 {
-    nh_ctx* c0 = b->ctxs[0];
+    nh_ctx* c0 = b->owner;
     const int n = (int)b->ctxs.size();
     static thread_local LBBatch<Real, Store> batch;  // large parameter block, kept off the stack
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
@@ -1009,7 +1048,7 @@ int batch_enqueue_lb(BatchPlan* b, bool write_macro, cudaStream_t st)
 template <typename Real>
 int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
 {
-    nh_ctx* c0 = b->ctxs[0];
+    nh_ctx* c0 = b->owner;
     const int n = (int)b->ctxs.size();
     static thread_local FDBatch<Real> batch;
     // the fused kernels only when every channel runs on them (not the three-constant energy, lap_wide or
@@ -1091,19 +1130,19 @@ int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
     return NH_OK;
 }
 
+// Pairs where every channel would take them alone.  (Small channels are too few
+// tiles for the march of a pair: 8 to 24 of 32^2 x 16 to 96^2 x 32 sites took
+// 0.035-0.050 ns a site and step in pairs, 0.030 in single steps.)
 bool batch_pair_ok(const BatchPlan* b)
 {
-    double sites = 0;
-    for (const nh_ctx* c : b->ctxs) {
-        if (!pair_fits(c)) return false;
-        sites += c->N;
-    }
-    return lb_pair_pays(sites);
+    for (const nh_ctx* c : b->ctxs)
+        if (!pair_fits(c) || !lb_pair_pays((double)c->N)) return false;
+    return true;
 }
 
 int batch_enqueue_lb_pair(BatchPlan* b, bool write_macro, cudaStream_t st)
 {
-    nh_ctx* c0 = b->ctxs[0];
+    nh_ctx* c0 = b->owner;
     const int n = (int)b->ctxs.size();
     static thread_local LBBatch<float, float> batch;
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
@@ -1116,9 +1155,8 @@ int batch_enqueue_lb_pair(BatchPlan* b, bool write_macro, cudaStream_t st)
     return NH_OK;
 }
 
-// The next batched LB step, or two in one launch (as enqueue_next), and the
-// batched FD update when the step count reaches a multiple of dt_fd, for every
-// channel of the plan; left: steps up to the end of the call or block.
+// The next batched LB step, or two in one launch (as enqueue_next), for every
+// channel of the plan or group; left: steps up to the end of the call or block.
 int batch_next(BatchPlan* b, int64_t left, bool ends_call, cudaStream_t st, int64_t* done)
 {
     nh_ctx* c0 = b->ctxs[0];
@@ -1132,8 +1170,29 @@ int batch_next(BatchPlan* b, int64_t left, bool ends_call, cudaStream_t st, int6
         c->phase ^= *done & 1;
         c->step += *done;
     }
-    if (fd) return c0->p.precision == NH_FP64 ? batch_fd_typed<double>(b, st) : batch_fd_typed<float>(b, st);
     return NH_OK;
+}
+
+// The next steps (at most up to the end of a dt_fd block) of every channel: LB
+// steps group by group where there are enough for a group's populations to be read
+// from L2 often, else of all channels at once, then the FD update of all channels
+// (which small groups would leave short of blocks).
+int batch_block(BatchPlan* b, int64_t steps, bool ends_call, cudaStream_t st)
+{
+    auto run = [&](BatchPlan* g) {
+        int r = NH_OK;
+        for (int64_t left = steps, done = 0; left > 0 && r == NH_OK; left -= done)
+            r = batch_next(g, left, ends_call, st, &done);
+        return r;
+    };
+    int r = NH_OK;
+    if (b->groups.empty() || steps < kGroupMinSteps)
+        r = run(b);
+    else
+        for (size_t k = 0; k < b->groups.size() && r == NH_OK; ++k) r = run(&b->groups[k]);
+    const nh_ctx* c0 = b->ctxs[0];
+    if (r || c0->step % c0->p.dt_fd != 0) return r;
+    return c0->p.precision == NH_FP64 ? batch_fd_typed<double>(b, st) : batch_fd_typed<float>(b, st);
 }
 
 int batch_capture(BatchPlan* b, int parity)
@@ -1153,8 +1212,7 @@ int batch_capture(BatchPlan* b, int parity)
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     int r = e == cudaSuccess ? NH_OK : cuda_fail(c0, e, "cudaStreamBeginCapture");
     if (r == NH_OK) {
-        for (int64_t left = c0->p.dt_fd, done = 0; left > 0 && r == NH_OK; left -= done)
-            r = batch_next(b, left, false, cs, &done);
+        r = batch_block(b, c0->p.dt_fd, false, cs);
         b->graph_end[parity] = c0->cur;
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(cs, &g);
@@ -1752,10 +1810,10 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
             }
             left -= dt;
         } else {
-            int64_t done = 1;
-            r = batch_next(plan, left, true, st, &done);
+            const int64_t block = std::min<int64_t>(left, dt - c0->step % dt);
+            r = batch_block(plan, block, block == left, st);
             if (r) return fail(nullptr, r, "batch step: " + c0->err);
-            left -= done;
+            left -= block;
         }
     }
     close_segment(c0);
