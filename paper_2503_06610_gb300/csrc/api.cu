@@ -631,7 +631,8 @@ int enqueue_one_step(nh_ctx* c, bool last_of_call, cudaStream_t st, bool sums)
         int r = enqueue_lb(c, c->cur, true, st);
         if (r) return r;
         const size_t fbytes = 3 * (size_t)c->N * (c->p.precision == NH_FP64 ? sizeof(double) : sizeof(float));
-        NH_CUDA(c, cudaMemcpyAsync(c->ws + c->L.Fprev, c->ws + c->L.F, fbytes, cudaMemcpyDeviceToDevice, st));
+        NH_CUDA(c, launch_copy_region(c->ws + c->L.F, c->ws + c->L.Fprev, fbytes, st));
+        c->launches += 1;
         r = enqueue_fd_any(c, st);
         if (r) return r;
         r = enqueue_lb(c, c->cur, false, st, true);

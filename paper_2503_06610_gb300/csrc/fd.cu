@@ -1550,6 +1550,16 @@ __global__ void __launch_bounds__(256) relax_end_kernel(const FDBatch<Real> b, b
     }
 }
 
+// A region's copy as a kernel: a device-to-device copy in the stream would wait for the kernel before it and hold back
+// the one after it, which start with programmatic serialisation otherwise.
+__global__ void __launch_bounds__(256) copy_region_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t bytes)
+{
+    step_kernel_enter();
+    const size_t n = bytes / 16, t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (size_t i = t; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = src[i];
+    if (t < bytes % 16 / 4) reinterpret_cast<uint32_t*>(dst + n)[t] = reinterpret_cast<const uint32_t*>(src + n)[t];
+}
+
 template <typename Real>
 inline int fused_tiles(const FDChan<Real>& c)
 {
@@ -1672,6 +1682,13 @@ cudaError_t launch_relax_end(const FDBatch<Real>& b, bool copy, cudaStream_t st)
 {
     if (b.count < 1 || b.count > kMaxBatch) return cudaErrorInvalidValue;
     launch_step_kernel(relax_end_kernel<Real>, dim3(64, b.count), 256, 0, st, b, copy);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy_region(const void* src, void* dst, size_t bytes, cudaStream_t st)
+{
+    const int blocks = (int)std::min<size_t>((bytes / 16 + 255) / 256 + 1, 8 * 152);
+    launch_step_kernel(copy_region_kernel, blocks, 256, 0, st, static_cast<const uint4*>(src), static_cast<uint4*>(dst), bytes);
     return cudaGetLastError();
 }
 

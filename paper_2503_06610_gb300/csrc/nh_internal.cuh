@@ -277,6 +277,8 @@ cudaError_t launch_fd_fused_b(const FDChan<Real>& c, const Real* nin, Real* ncop
                               const BDiag* diag = nullptr);
 template <typename Real>
 cudaError_t launch_relax(const FDChan<Real>& c, const Real* nin, Real* nout, cudaStream_t s);  // A at u = 0 (u not read)
+// bytes (a multiple of 4) from one workspace region to another (256-byte aligned)
+cudaError_t launch_copy_region(const void* src, void* dst, size_t bytes, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_relax_end(const FDBatch<Real>& b, bool copy, cudaStream_t s);  // u = 0; copy: n <- nP
 template <typename Real>
