@@ -201,7 +201,8 @@ int nh_restore(nh_ctx* ctx, const double* n, const double* F, const double* u, c
                int64_t step, int on_device);
 
 /* Advance n_lb_steps LB steps (Sec. II.D): every step one fused LB
- * collide-and-stream launch; after each step whose count s is a multiple of
+ * collide-and-stream launch (FP32 stores of 7.5e5 sites or more, without
+ * obstacles: two steps per launch where no FD update lies between); after each step whose count s is a multiple of
  * dt_fd, the FD predictor-corrector on n with that step's u, then the LC
  * stress and force.  Asynchronous on stream (NULL = the context's stream).
  * Whole dt_fd blocks of at least 12 steps run from a CUDA graph unless timing is on. */
@@ -215,7 +216,9 @@ int nh_fd_update(nh_ctx* ctx, void* stream);
  * by n_lb_steps each.  Every pass (LB sweep, FD predict, correct, stress,
  * force) is one persistent launch per group of up to 64 channels: the grid
  * walks a work list of (channel, tile) pairs, and the channel descriptors
- * travel as kernel parameters.  Whole dt_fd blocks (of at least 12 steps) are replayed from a CUDA
+ * travel as kernel parameters.  The LB steps of a block of at least four
+ * steps run group by group of channels whose populations fit in L2 together
+ * (large FP32 channels take two steps per launch instead).  Whole dt_fd blocks (of at least 12 steps) are replayed from a CUDA
  * graph cached per list of contexts (dropped when a context is rebound,
  * re-tuned or destroyed).  All contexts must share precision, storage,
  * shifted and dt_fd, be on one device, have fields set and be at the same
@@ -374,7 +377,8 @@ int64_t nh_launch_count(const nh_ctx* ctx);
  * staged in shared memory by bulk asynchronous copies, the next row in flight
  * while a block collides the current one, four sites per thread (needs
  * nx % 128 == 0 and nx <= 256; with obstacles it runs as variant 0).  All variants compute the same arithmetic
- * and give bit-identical results.  Batches use variants 0 .. 5 (a batch of
+ * and give bit-identical results.  Steps
+ * taken two per launch (see nh_step) have a shape of their own.  Batches use variants 0 .. 5 (a batch of
  * channels set to 6 runs variant 2, or 1 with an odd nx among them).  NH_EINVAL if the variant does not fit
  * the domain.  Variant 6 bounds its waits on the copies: an expired wait is
  * reported by the next nh_diagnostics / nh_diagnostics_read as NH_ETIMEOUT
