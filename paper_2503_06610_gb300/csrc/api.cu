@@ -761,6 +761,20 @@ int store_field(nh_ctx* c, size_t off, double* dst, int64_t count, int on_device
                                      : launch_store<float>(c, src, dst, count, on_device, st);
 }
 
+// n, u and rho (those asked for) into device buffers.
+template <typename Real>
+int store_fields(nh_ctx* c, double* n, double* u, double* rho, cudaStream_t st)
+{
+    if (!n && !u && !rho) return NH_OK;
+    const int64_t N = c->N;
+    NH_CUDA(c, launch_store_fields(StoreFields<Real>{{c->at<const Real>(c->L.n), c->at<const Real>(c->L.u), c->at<const Real>(c->L.rho)},
+                                                     {n, u, rho},
+                                                     {n ? 3 * N : 0, u ? 3 * N : 0, rho ? N : 0}},
+                                   st));
+    c->launches += 1;
+    return NH_OK;
+}
+
 template <typename Store>
 int decode_all(nh_ctx* c, double* f, int on_device, cudaStream_t st)
 {
@@ -1613,9 +1627,14 @@ int nh_get_fields(nh_ctx* c, double* n, double* u, double* rho, int on_device)
     if ((r = set_device(c))) return r;
     cudaStream_t st = c->stream;
     if ((r = bounded_wait(c, st))) return r;
-    if ((r = store_field(c, c->L.n, n, 3 * (int64_t)c->N, on_device, st))) return r;
-    if ((r = store_field(c, c->L.u, u, 3 * (int64_t)c->N, on_device, st))) return r;
-    if ((r = store_field(c, c->L.rho, rho, (int64_t)c->N, on_device, st))) return r;
+    if (on_device) {
+        r = c->p.precision == NH_FP64 ? store_fields<double>(c, n, u, rho, st) : store_fields<float>(c, n, u, rho, st);
+        if (r) return r;
+    } else {
+        if ((r = store_field(c, c->L.n, n, 3 * (int64_t)c->N, on_device, st))) return r;
+        if ((r = store_field(c, c->L.u, u, 3 * (int64_t)c->N, on_device, st))) return r;
+        if ((r = store_field(c, c->L.rho, rho, (int64_t)c->N, on_device, st))) return r;
+    }
     NH_CUDA(c, cudaStreamSynchronize(st));
     return NH_OK;
 }

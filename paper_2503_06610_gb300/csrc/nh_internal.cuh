@@ -302,6 +302,15 @@ cudaError_t launch_frank3_p(const FDChan<Real>& c, bool from_predictor, cudaStre
 template <typename Real>
 cudaError_t launch_load_fields(const double* n, const double* u, const double* rho, Real* dn, Real* du, Real* drho,
                                int N, cudaStream_t s);
+// fields to double, count 0: none
+template <typename Real>
+struct StoreFields {
+    const Real* src[3];
+    double* dst[3];
+    int64_t count[3];
+};
+template <typename Real>
+cudaError_t launch_store_fields(const StoreFields<Real>& f, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_store_vec(const Real* src, double* dst, int64_t count, cudaStream_t s);
 template <typename Real, typename Store>
