@@ -198,6 +198,52 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return fma(a, b, c); }
 
+// e . v for a lattice vector with components in {-1, 0, 1} (constants once the
+// direction loop is unrolled): sums and differences only.
+template <typename Real>
+__device__ __forceinline__ Real edot(int X, int Y, int Z, Real vx, Real vy, Real vz)
+{
+    Real r = Real(0);
+    if (X != 0) r = X > 0 ? vx : -vx;
+    if (Y != 0) r = (X != 0) ? (Y > 0 ? r + vy : r - vy) : (Y > 0 ? vy : -vy);
+    if (Z != 0) r = (X != 0 || Y != 0) ? (Z > 0 ? r + vz : r - vz) : (Z > 0 ? vz : -vz);
+    return r;
+}
+
+// Relaxation of one site, direction pair by direction pair, from the streamed populations f, rho, u and the force:
+//   f^eq = w rho [3 eu + 4.5 eu^2 - 1.5 u.u] + w (rho - 1 | rho)
+//   S    = w [3 eF + 9 eu eF - 3 u.F]
+//   f*   = omc f + omega f^eq + cS S,  omc = 1 - omega, cS = 1 - omega / 2
+// base: rho - 1 for shifted populations, else rho.
+template <typename Real>
+__device__ __forceinline__ void relax_by_pairs(const Real (&f)[19], Real (&fo)[19], Real rho, Real base, Real ux, Real uy,
+                                               Real uz, Real Fx, Real Fy, Real Fz, Real omega, Real omc, Real cS)
+{
+    NH_D3Q19_TABLES
+    const Real uu15 = mul_rn(Real(1.5), fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux))));
+    const Real uF3 = mul_rn(Real(3), fma_rn(uz, Fz, fma_rn(uy, Fy, mul_rn(ux, Fx))));
+    // rest population (w = 1/3)
+    const Real w0 = Real(1) / Real(3);
+    fo[0] = fma_rn(omc, f[0], fma_rn(mul_rn(omega, w0), fma_rn(-rho, uu15, base), -mul_rn(mul_rn(cS, w0), uF3)));
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int i = 2 * k + 1;
+        const Real w = i < 7 ? Real(1) / Real(18) : Real(1) / Real(36);
+        const Real ow = mul_rn(omega, w);
+        const Real A = mul_rn(ow, rho);
+        const Real B = mul_rn(ow, base);
+        const Real C = mul_rn(cS, w);
+        const Real eu = edot(EX[i], EY[i], EZ[i], ux, uy, uz);
+        const Real eF = edot(EX[i], EY[i], EZ[i], Fx, Fy, Fz);
+        const Real X = fma_rn(mul_rn(Real(4.5), eu), eu, -uu15);
+        const Real Y = fma_rn(mul_rn(Real(9), eu), eF, -uF3);
+        const Real even = fma_rn(C, Y, fma_rn(A, X, B));
+        const Real odd = mul_rn(Real(3), fma_rn(A, eu, mul_rn(C, eF)));
+        fo[i] = fma_rn(omc, f[i], even) + odd;
+        fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
+    }
+}
+
 // Moments, equilibrium, Guo source and relaxation of one site s from its
 // streamed populations f (decoded values; raw 2^k-scaled ones for the 16-bit
 // stores, whose power-of-two factors inv_in and scale_out are folded in) and
@@ -211,9 +257,13 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
                                                 Real (&fo)[19], Real flx, Real fly, Real flz, float inv_in,
                                                 float scale_out, Real& psum, Real& pmax, int& pbad, float& amax)
 {
+    NH_D3Q19_TABLES
     constexpr bool kScaled = sizeof(Store) == 2;
     constexpr bool WriteMacro = Macro >= 1;
     constexpr bool Partials = Macro == 2;
+    // A 16-bit store rounds to 8 or 11 bits, so that a last bit of FP32 moves a population by a whole unit of the store:
+    // these keep the order that every result of theirs was computed with.
+    constexpr bool ByPairs = kScaled;
     const int N = c.g.N;
     // 2. moments: pair sums and differences of (e_i, -e_i)
     Real d[9];
@@ -223,10 +273,21 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
         sum += f[2 * k + 1] + f[2 * k + 2];
         d[k] = f[2 * k + 1] - f[2 * k + 2];
     }
-    // pairs: x, y, z, (x+y, x-y), (x+z, x-z), (y+z, y-z)
-    Real mx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
-    Real my = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
-    Real mz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
+    Real mx, my, mz;
+    if constexpr (ByPairs) {
+        mx = my = mz = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int i = 2 * k + 1;
+            if (EX[i] != 0) mx += EX[i] > 0 ? d[k] : -d[k];
+            if (EY[i] != 0) my += EY[i] > 0 ? d[k] : -d[k];
+            if (EZ[i] != 0) mz += EZ[i] > 0 ? d[k] : -d[k];
+        }
+    } else {  // pairs: x, y, z, (x+y, x-y), (x+z, x-z), (y+z, y-z)
+        mx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+        my = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+        mz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
+    }
     if (kScaled) {  // raw populations: scale the sums once
         sum = mul_rn(sum, Real(inv_in));
         mx = mul_rn(mx, Real(inv_in));
@@ -254,54 +315,55 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
         c.rho[s] = rho;
     }
 
-    // 3-4. equilibrium, Guo source and relaxation, per (e_i, -e_i) pair:
-    //   f^eq = w rho [3 eu + 4.5 eu^2 - 1.5 u.u] + w (rho - 1 | rho)
-    //   S    = w [3 eF + 9 eu eF - 3 u.F]
-    //   f*   = (1 - omega) f + omega f^eq + (1 - omega/2) S
-    // With g = 1.5 omega rho u + 3 (1 - omega/2) F and h = g + 1.5 omega rho u the two sums are
-    //   omega f^eq + (1 - omega/2) S = w [3 (e.u)(e.g) + T + e.h],  T = omega (rho - 1 | rho) - u.g
-    // so a pair costs one even and one odd part from three projections: 150
-    // operations a site instead of 215.  FP64 LB is bound by the FP64 pipe and
-    // the 16-bit stores by issue (times in the launch variants' table).
-    // With a 16-bit store the constants carry scale_out (and omc the raw
-    // input's inv_in), so fo[] leaves here already in encoded units.
-    const Real so = kScaled ? Real(scale_out) : Real(1);
-    const Real omega = mul_rn(c.omega, so);
-    const Real omc = mul_rn(Real(1) - c.omega, kScaled ? mul_rn(Real(inv_in), so) : Real(1));
-    const Real cS3 = mul_rn(Real(3), mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so));
-    const Real a15 = mul_rn(mul_rn(Real(1.5), omega), rho);
-    const Real gx = fma_rn(a15, ux, mul_rn(cS3, Fx));
-    const Real gy = fma_rn(a15, uy, mul_rn(cS3, Fy));
-    const Real gz = fma_rn(a15, uz, mul_rn(cS3, Fz));
-    constexpr Real w36 = Real(1) / Real(36), w12 = Real(1) / Real(12);
-    const Real hx = mul_rn(w36, fma_rn(a15, ux, gx));
-    const Real hy = mul_rn(w36, fma_rn(a15, uy, gy));
-    const Real hz = mul_rn(w36, fma_rn(a15, uz, gz));
-    const Real vx = mul_rn(w12, ux), vy = mul_rn(w12, uy), vz = mul_rn(w12, uz);
-    const Real ug = fma_rn(uz, gz, fma_rn(uy, gy, mul_rn(ux, gx)));
-    const Real T = fma_rn(mul_rn(w36, omega), Shifted ? sum : rho, -mul_rn(w36, ug));
-    fo[0] = fma_rn(Real(12), T, mul_rn(omc, f[0]));
-    const Real omc_half = mul_rn(Real(0.5), omc);
-    // axis pair (w = 1/18: twice the 1/36 parts), diagonal pair
-    auto axis = [&](int i, Real v, Real g, Real h) {
-        const Real even = fma_rn(v, g, T);
-        fo[i] = mul_rn(Real(2), fma_rn(omc_half, f[i], even) + h);
-        fo[i + 1] = mul_rn(Real(2), fma_rn(omc_half, f[i + 1], even) - h);
-    };
-    auto diagonal = [&](int i, Real v, Real g, Real h) {
-        const Real even = fma_rn(v, g, T);
-        fo[i] = fma_rn(omc, f[i], even + h);
-        fo[i + 1] = fma_rn(omc, f[i + 1], even - h);
-    };
-    axis(1, vx, gx, hx);
-    axis(3, vy, gy, hy);
-    axis(5, vz, gz, hz);
-    diagonal(7, vx + vy, gx + gy, hx + hy);
-    diagonal(9, vx - vy, gx - gy, hx - hy);
-    diagonal(11, vx + vz, gx + gz, hx + hz);
-    diagonal(13, vx - vz, gx - gz, hx - hz);
-    diagonal(15, vy + vz, gy + gz, hy + hz);
-    diagonal(17, vy - vz, gy - gz, hy - hz);
+    // 3-4. equilibrium, Guo source and relaxation.  With a 16-bit store the
+    // constants carry scale_out (and omc the raw input's inv_in), so fo[] leaves
+    // here already in encoded units.
+    if constexpr (ByPairs) {
+        const Real so = kScaled ? Real(scale_out) : Real(1);
+        relax_by_pairs(f, fo, rho, Shifted ? sum : rho, ux, uy, uz, Fx, Fy, Fz, mul_rn(c.omega, so),
+                       mul_rn(Real(1) - c.omega, kScaled ? mul_rn(Real(inv_in), so) : Real(1)),
+                       mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so));
+    } else {
+        // With g = 1.5 omega rho u + 3 (1 - omega/2) F and h = g + 1.5 omega rho u the two sums are
+        //   omega f^eq + (1 - omega/2) S = w [3 (e.u)(e.g) + T + e.h],  T = omega (rho - 1 | rho) - u.g
+        // so a pair costs one even and one odd part from three projections: 150
+        // operations a site instead of 215.  FP64 LB is bound by the FP64 pipe.
+        const Real omega = c.omega, omc = Real(1) - c.omega;
+        const Real cS3 = mul_rn(Real(3), fma_rn(Real(-0.5), c.omega, Real(1)));
+        const Real a15 = mul_rn(mul_rn(Real(1.5), omega), rho);
+        const Real gx = fma_rn(a15, ux, mul_rn(cS3, Fx));
+        const Real gy = fma_rn(a15, uy, mul_rn(cS3, Fy));
+        const Real gz = fma_rn(a15, uz, mul_rn(cS3, Fz));
+        constexpr Real w36 = Real(1) / Real(36), w12 = Real(1) / Real(12);
+        const Real hx = mul_rn(w36, fma_rn(a15, ux, gx));
+        const Real hy = mul_rn(w36, fma_rn(a15, uy, gy));
+        const Real hz = mul_rn(w36, fma_rn(a15, uz, gz));
+        const Real vx = mul_rn(w12, ux), vy = mul_rn(w12, uy), vz = mul_rn(w12, uz);
+        const Real ug = fma_rn(uz, gz, fma_rn(uy, gy, mul_rn(ux, gx)));
+        const Real T = fma_rn(mul_rn(w36, omega), Shifted ? sum : rho, -mul_rn(w36, ug));
+        fo[0] = fma_rn(Real(12), T, mul_rn(omc, f[0]));
+        const Real omc_half = mul_rn(Real(0.5), omc);
+        // axis pair (w = 1/18: twice the 1/36 parts), diagonal pair
+        auto axis = [&](int i, Real v, Real g, Real h) {
+            const Real even = fma_rn(v, g, T);
+            fo[i] = mul_rn(Real(2), fma_rn(omc_half, f[i], even) + h);
+            fo[i + 1] = mul_rn(Real(2), fma_rn(omc_half, f[i + 1], even) - h);
+        };
+        auto diagonal = [&](int i, Real v, Real g, Real h) {
+            const Real even = fma_rn(v, g, T);
+            fo[i] = fma_rn(omc, f[i], even + h);
+            fo[i + 1] = fma_rn(omc, f[i + 1], even - h);
+        };
+        axis(1, vx, gx, hx);
+        axis(3, vy, gy, hy);
+        axis(5, vz, gz, hz);
+        diagonal(7, vx + vy, gx + gy, hx + hy);
+        diagonal(9, vx - vy, gx - gy, hx - hy);
+        diagonal(11, vx + vz, gx + gz, hx + hz);
+        diagonal(13, vx - vz, gx - gz, hx - hz);
+        diagonal(15, vy + vz, gy + gz, hy + hz);
+        diagonal(17, vy - vz, gy - gz, hy - hz);
+    }
     if (Partials) {  // the sums nh_diagnostics forms from the stored state, site by site
         const Real u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
         Real fs = fo[0];
