@@ -872,15 +872,25 @@ namespace {
 
 // ------------------------------------------------------------ batched channels
 
+// A captured dt_FD block.  Channels that take pairs of steps and channels that take
+// single ones change buffers at different rates, so the block is kept with the
+// buffer every channel starts and ends in.
+struct BatchGraph {
+    cudaGraphExec_t exec = nullptr;
+    int64_t kernels = 0;
+    std::vector<int> start, end;
+};
+// Two kinds of channels, each in either of its buffers; other mixtures (channels that
+// stepped alone before) launch directly.
+constexpr size_t kBatchGraphs = 4;
+
 struct BatchPlan {
     std::vector<nh_ctx*> ctxs;
     nh_ctx* owner = nullptr;         // the batch's first channel, which counts launches and keeps times
     std::vector<BatchPlan> groups;   // of channels that stay in L2 together (batch_groups); empty: none
     std::vector<int64_t> epochs;
     int variant = 0;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    int64_t graph_kernels[2] = {0, 0};
-    int graph_end[2] = {0, 0};  // buffer a block that starts in buffer 0 / 1 ends in
+    std::vector<BatchGraph> graphs;
 };
 
 std::mutex g_batch_mu;
@@ -888,11 +898,8 @@ std::map<std::vector<nh_ctx*>, BatchPlan*> g_batch_plans;
 
 void batch_drop_graphs(BatchPlan* b)
 {
-    for (int k = 0; k < 2; ++k) {
-        if (b->graph[k]) cudaGraphExecDestroy(b->graph[k]);
-        b->graph[k] = nullptr;
-        b->graph_kernels[k] = 0;
-    }
+    for (BatchGraph& g : b->graphs) cudaGraphExecDestroy(g.exec);
+    b->graphs.clear();
 }
 
 void drop_batch_plans(const nh_ctx* c)
@@ -1210,16 +1217,17 @@ int batch_block(BatchPlan* b, int64_t steps, bool ends_call, cudaStream_t st)
     return c0->p.precision == NH_FP64 ? batch_fd_typed<double>(b, st) : batch_fd_typed<float>(b, st);
 }
 
-int batch_capture(BatchPlan* b, int parity)
+// Capture a whole dt_fd block that starts in the channels' present buffers.
+int batch_capture(BatchPlan* b)
 {
     nh_ctx* c0 = b->ctxs[0];
-    std::vector<int> cur, phase;
+    BatchGraph g;
+    std::vector<int> phase;
     std::vector<int64_t> step;
     for (nh_ctx* c : b->ctxs) {
-        cur.push_back(c->cur);
+        g.start.push_back(c->cur);
         phase.push_back(c->phase);
         step.push_back(c->step);
-        c->cur = parity;
         c->step = 0;
     }
     const int64_t saved_launches = c0->launches;
@@ -1228,28 +1236,40 @@ int batch_capture(BatchPlan* b, int parity)
     int r = e == cudaSuccess ? NH_OK : cuda_fail(c0, e, "cudaStreamBeginCapture");
     if (r == NH_OK) {
         r = batch_block(b, c0->p.dt_fd, false, cs);
-        b->graph_end[parity] = c0->cur;
-        cudaGraph_t g = nullptr;
-        e = cudaStreamEndCapture(cs, &g);
+        cudaGraph_t graph = nullptr;
+        e = cudaStreamEndCapture(cs, &graph);
         if (r == NH_OK && e != cudaSuccess) r = cuda_fail(c0, e, "cudaStreamEndCapture");
         if (r == NH_OK) {
-            cudaGraphExec_t ex = nullptr;
-            e = cudaGraphInstantiate(&ex, g, 0);
-            if (e != cudaSuccess)
-                r = cuda_fail(c0, e, "cudaGraphInstantiate");
-            else {
-                b->graph[parity] = ex;
-                b->graph_kernels[parity] = c0->launches - saved_launches;
-            }
+            e = cudaGraphInstantiate(&g.exec, graph, 0);
+            if (e != cudaSuccess) r = cuda_fail(c0, e, "cudaGraphInstantiate");
         }
-        if (g) cudaGraphDestroy(g);
+        if (graph) cudaGraphDestroy(graph);
     }
+    g.kernels = c0->launches - saved_launches;
     c0->launches = saved_launches;
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
-        b->ctxs[k]->cur = cur[k];
+        g.end.push_back(b->ctxs[k]->cur);
+        b->ctxs[k]->cur = g.start[k];
         b->ctxs[k]->phase = phase[k];
         b->ctxs[k]->step = step[k];
     }
+    if (r == NH_OK) b->graphs.push_back(std::move(g));
+    return r;
+}
+
+// The graph of a block that starts in the channels' present buffers, captured if
+// there is room for it; null in *out: launch the block directly.
+int batch_graph(BatchPlan* b, const BatchGraph** out)
+{
+    *out = nullptr;
+    for (const BatchGraph& g : b->graphs) {
+        bool same = true;
+        for (size_t k = 0; k < b->ctxs.size(); ++k) same = same && b->ctxs[k]->cur == g.start[k];
+        if (same) *out = &g;
+    }
+    if (*out || b->graphs.size() == kBatchGraphs) return NH_OK;
+    int r = batch_capture(b);
+    if (r == NH_OK) *out = &b->graphs.back();
     return r;
 }
 
@@ -1811,20 +1831,18 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
     const int dt = c0->p.dt_fd;
     int64_t left = n_lb_steps;
     while (left > 0) {
-        // (channels that stepped alone in pairs may sit in different buffers: direct launches then)
-        bool one_buffer = true;
-        for (nh_ctx* c : plan->ctxs) one_buffer = one_buffer && c->cur == c0->cur;
-        if (use_block_graph(c0) && one_buffer && c0->step % dt == 0 && left >= dt) {
-            const int parity = c0->cur;
-            if (!plan->graph[parity]) {
-                r = batch_capture(plan, parity);
-                if (r) return fail(nullptr, r, "batch graph capture: " + c0->err);
-            }
-            cudaError_t e = cudaGraphLaunch(plan->graph[parity], st);
+        const BatchGraph* graph = nullptr;
+        if (use_block_graph(c0) && c0->step % dt == 0 && left >= dt) {
+            r = batch_graph(plan, &graph);
+            if (r) return fail(nullptr, r, "batch graph capture: " + c0->err);
+        }
+        if (graph) {
+            cudaError_t e = cudaGraphLaunch(graph->exec, st);
             if (e != cudaSuccess) return fail(nullptr, NH_ECUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
-            c0->launches += plan->graph_kernels[parity];
-            for (nh_ctx* c : plan->ctxs) {
-                c->cur = plan->graph_end[parity];
+            c0->launches += graph->kernels;
+            for (size_t k = 0; k < plan->ctxs.size(); ++k) {
+                nh_ctx* c = plan->ctxs[k];
+                c->cur = graph->end[k];
                 c->phase ^= dt & 1;
                 c->step += dt;
             }
