@@ -884,12 +884,12 @@ struct BatchGraph {
 // stepped alone before) launch directly.
 constexpr size_t kBatchGraphs = 4;
 
+using Channels = std::vector<nh_ctx*>;
 struct BatchPlan {
-    std::vector<nh_ctx*> ctxs;
-    nh_ctx* owner = nullptr;         // the batch's first channel, which counts launches and keeps times
-    std::vector<BatchPlan> groups;   // of channels that stay in L2 together (batch_groups); empty: none
+    Channels ctxs;                  // the first one counts launches and keeps times
+    std::vector<Channels> groups;   // of channels that stay in L2 together (batch_groups); empty: none
     std::vector<int64_t> epochs;
-    int variant = 0;
+    int variant = 0;                // launch shape of the single steps
     std::vector<BatchGraph> graphs;
 };
 
@@ -926,7 +926,7 @@ void drop_batch_plans(const nh_ctx* c)
 // (large ones).
 constexpr double kGroupBytes = 84e6;
 constexpr int kGroupMinSteps = 4;
-bool batch_pair_ok(const BatchPlan* b);
+bool batch_pair_ok(const Channels& ctxs);
 void batch_groups(BatchPlan* b)
 {
     double total = 0;
@@ -937,15 +937,11 @@ void batch_groups(BatchPlan* b)
         total += bytes.back();
     }
     const int groups = (int)std::ceil(total / kGroupBytes);
-    if (groups < 2 || b->ctxs.size() < 2 || batch_pair_ok(b)) return;
+    if (groups < 2 || b->ctxs.size() < 2 || batch_pair_ok(b->ctxs)) return;
     double sum = 0;  // cut where the running sum passes an even share
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
-        if (b->groups.empty() || sum + 0.5 * bytes[k] > total * (double)b->groups.size() / groups) {
-            b->groups.emplace_back();
-            b->groups.back().owner = b->owner;
-            b->groups.back().variant = b->variant;
-        }
-        b->groups.back().ctxs.push_back(b->ctxs[k]);
+        if (b->groups.empty() || sum + 0.5 * bytes[k] > total * (double)b->groups.size() / groups) b->groups.emplace_back();
+        b->groups.back().push_back(b->ctxs[k]);
         sum += bytes[k];
     }
 }
@@ -989,7 +985,6 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
         plan = new (std::nothrow) BatchPlan();
         if (!plan) return fail(nullptr, NH_ENOMEM, "host allocation of the batch plan failed");
         plan->ctxs = key;
-        plan->owner = c0;
         plan->epochs = epochs;
         // ctxs[0]'s shape if it was set and fits every channel (the row-staged one runs single channels only),
         // else the default of the batch's channels taken as one domain
@@ -1034,20 +1029,19 @@ int batch_prepare_relax(nh_ctx* const* ctxs, int count, int64_t n_fd_steps, Batc
     if (r) return fail(nullptr, r, c0->err);
     static thread_local BatchPlan plan;
     plan.ctxs.assign(ctxs, ctxs + count);
-    plan.owner = c0;
     *out = &plan;
     return NH_OK;
 }
 
 template <typename Real, typename Store>
-int batch_lb_typed(BatchPlan* b, bool write_macro, cudaStream_t st)
+int batch_lb_typed(const BatchPlan* b, const Channels& ctxs, bool write_macro, cudaStream_t st)
 {
-    nh_ctx* c0 = b->owner;
-    const int n = (int)b->ctxs.size();
+    nh_ctx* c0 = b->ctxs[0];
+    const int n = (int)ctxs.size();
     static thread_local LBBatch<Real, Store> batch;  // large parameter block, kept off the stack
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
         batch.count = std::min(kMaxBatch, n - g0);
-        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<Real, Store>(b->ctxs[g0 + k], b->ctxs[g0 + k]->cur);
+        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<Real, Store>(ctxs[g0 + k], ctxs[g0 + k]->cur);
         const int grid = 8 * c0->sm_count;
         int r = timed(c0, NH_KCLASS_LB, st,
                       [&] { return launch_lb_batch(batch, c0->p.shifted != 0, write_macro, b->variant, grid, st); },
@@ -1057,20 +1051,21 @@ int batch_lb_typed(BatchPlan* b, bool write_macro, cudaStream_t st)
     return NH_OK;
 }
 
-int batch_enqueue_lb(BatchPlan* b, bool write_macro, cudaStream_t st)
+// One LB step of these channels of the batch, with the batch's launch shape.
+int batch_enqueue_lb(const BatchPlan* b, const Channels& ctxs, bool write_macro, cudaStream_t st)
 {
     switch (b->ctxs[0]->p.storage) {
-    case NH_STORE_F64: return batch_lb_typed<double, double>(b, write_macro, st);
-    case NH_STORE_F32: return batch_lb_typed<float, float>(b, write_macro, st);
-    case NH_STORE_F16S: return batch_lb_typed<float, __half>(b, write_macro, st);
-    default: return batch_lb_typed<float, __nv_bfloat16>(b, write_macro, st);
+    case NH_STORE_F64: return batch_lb_typed<double, double>(b, ctxs, write_macro, st);
+    case NH_STORE_F32: return batch_lb_typed<float, float>(b, ctxs, write_macro, st);
+    case NH_STORE_F16S: return batch_lb_typed<float, __half>(b, ctxs, write_macro, st);
+    default: return batch_lb_typed<float, __nv_bfloat16>(b, ctxs, write_macro, st);
     }
 }
 
 template <typename Real>
 int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
 {
-    nh_ctx* c0 = b->owner;
+    nh_ctx* c0 = b->ctxs[0];
     const int n = (int)b->ctxs.size();
     static thread_local FDBatch<Real> batch;
     // the fused kernels only when every channel runs on them (not the three-constant energy, lap_wide or
@@ -1155,21 +1150,21 @@ int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
 // Pairs where every channel would take them alone.  (Small channels are too few
 // tiles for the march of a pair: 8 to 24 of 32^2 x 16 to 96^2 x 32 sites took
 // 0.035-0.050 ns a site and step in pairs, 0.030 in single steps.)
-bool batch_pair_ok(const BatchPlan* b)
+bool batch_pair_ok(const Channels& ctxs)
 {
-    for (const nh_ctx* c : b->ctxs)
+    for (const nh_ctx* c : ctxs)
         if (!pair_fits(c) || !lb_pair_pays((double)c->N)) return false;
     return true;
 }
 
-int batch_enqueue_lb_pair(BatchPlan* b, bool write_macro, cudaStream_t st)
+int batch_enqueue_lb_pair(const BatchPlan* b, const Channels& ctxs, bool write_macro, cudaStream_t st)
 {
-    nh_ctx* c0 = b->owner;
-    const int n = (int)b->ctxs.size();
+    nh_ctx* c0 = b->ctxs[0];
+    const int n = (int)ctxs.size();
     static thread_local LBBatch<float, float> batch;
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
         batch.count = std::min(kMaxBatch, n - g0);
-        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<float, float>(b->ctxs[g0 + k], b->ctxs[g0 + k]->cur);
+        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<float, float>(ctxs[g0 + k], ctxs[g0 + k]->cur);
         int r = timed(c0, NH_KCLASS_LB, st,
                       [&] { return launch_lb_pair_batch(batch, c0->p.shifted != 0, write_macro, st); }, "lb_pair_batch");
         if (r) return r;
@@ -1177,17 +1172,18 @@ int batch_enqueue_lb_pair(BatchPlan* b, bool write_macro, cudaStream_t st)
     return NH_OK;
 }
 
-// The next batched LB step, or two in one launch (as enqueue_next), for every
-// channel of the plan or group; left: steps up to the end of the call or block.
-int batch_next(BatchPlan* b, int64_t left, bool ends_call, cudaStream_t st, int64_t* done)
+// The next batched LB step, or two in one launch (as enqueue_next), of these
+// channels of the batch (all of them, or a group); left: steps up to the end of the
+// call or block.
+int batch_next(const BatchPlan* b, const Channels& ctxs, int64_t left, bool ends_call, cudaStream_t st, int64_t* done)
 {
-    nh_ctx* c0 = b->ctxs[0];
+    const nh_ctx* c0 = ctxs[0];
     const int dt = c0->p.dt_fd;
-    *done = left >= 2 && (c0->step + 1) % dt != 0 && batch_pair_ok(b) ? 2 : 1;
+    *done = left >= 2 && (c0->step + 1) % dt != 0 && batch_pair_ok(ctxs) ? 2 : 1;
     const bool fd = (c0->step + *done) % dt == 0, macro = fd || (ends_call && left == *done);
-    int r = *done == 2 ? batch_enqueue_lb_pair(b, macro, st) : batch_enqueue_lb(b, macro, st);
+    int r = *done == 2 ? batch_enqueue_lb_pair(b, ctxs, macro, st) : batch_enqueue_lb(b, ctxs, macro, st);
     if (r) return r;
-    for (nh_ctx* c : b->ctxs) {
+    for (nh_ctx* c : ctxs) {
         c->cur ^= 1;
         c->phase ^= *done & 1;
         c->step += *done;
@@ -1195,23 +1191,26 @@ int batch_next(BatchPlan* b, int64_t left, bool ends_call, cudaStream_t st, int6
     return NH_OK;
 }
 
+// Whether this many steps run group by group: where there are enough for a group's
+// populations to be read from L2 often.
+bool batch_grouped(const BatchPlan* b, int64_t steps) { return !b->groups.empty() && steps >= kGroupMinSteps; }
+
 // The next steps (at most up to the end of a dt_fd block) of every channel: LB
-// steps group by group where there are enough for a group's populations to be read
-// from L2 often, else of all channels at once, then the FD update of all channels
-// (which small groups would leave short of blocks).
+// steps group by group or of all channels at once, then the FD update of all
+// channels (which small groups would leave short of blocks).
 int batch_block(BatchPlan* b, int64_t steps, bool ends_call, cudaStream_t st)
 {
-    auto run = [&](BatchPlan* g) {
+    auto run = [&](const Channels& ctxs) {
         int r = NH_OK;
         for (int64_t left = steps, done = 0; left > 0 && r == NH_OK; left -= done)
-            r = batch_next(g, left, ends_call, st, &done);
+            r = batch_next(b, ctxs, left, ends_call, st, &done);
         return r;
     };
     int r = NH_OK;
-    if (b->groups.empty() || steps < kGroupMinSteps)
-        r = run(b);
+    if (batch_grouped(b, steps))
+        for (size_t k = 0; k < b->groups.size() && r == NH_OK; ++k) r = run(b->groups[k]);
     else
-        for (size_t k = 0; k < b->groups.size() && r == NH_OK; ++k) r = run(&b->groups[k]);
+        r = run(b->ctxs);
     const nh_ctx* c0 = b->ctxs[0];
     if (r || c0->step % c0->p.dt_fd != 0) return r;
     return c0->p.precision == NH_FP64 ? batch_fd_typed<double>(b, st) : batch_fd_typed<float>(b, st);
@@ -1869,6 +1868,20 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
     const int saved_timing = c0->timing;
     c0->timing = 0;
     cudaEvent_t e0 = get_event(c0), e1 = get_event(c0);
+    // The launches as the blocks make them: by groups where the blocks go by groups, and of those the groups that
+    // take single steps (pairs have a shape of their own).
+    std::vector<Channels> sets;
+    if (batch_grouped(plan, c0->p.dt_fd))
+        for (const Channels& g : plan->groups)
+            if (!batch_pair_ok(g)) sets.push_back(g);
+    if (sets.empty()) sets.push_back(plan->ctxs);
+    // streams the current buffers into the others, no swap
+    auto trial = [&](int reps) {
+        int e = NH_OK;
+        for (const Channels& g : sets)
+            for (int k = 0; k < reps && e == NH_OK; ++k) e = batch_enqueue_lb(plan, g, false, st);
+        return e;
+    };
     float best_ms = 1e30f;
     int best = plan->variant;
     const int saved = plan->variant;
@@ -1877,10 +1890,10 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
         for (nh_ctx* c : plan->ctxs) ok = ok && lb_variant_valid(v, c->p.nx);
         if (!ok) continue;
         plan->variant = v;
-        r = batch_enqueue_lb(plan, false, st);  // streams the current buffers into the others, no swap
+        r = trial(1);
         if (r) break;
         cudaEventRecord(e0, st);
-        for (int k = 0; k < 5 && r == NH_OK; ++k) r = batch_enqueue_lb(plan, false, st);
+        r = trial(5);
         cudaEventRecord(e1, st);
         if (r) break;
         if (cudaEventSynchronize(e1) != cudaSuccess) {
