@@ -2162,7 +2162,7 @@ int nh_set_lb_variant(nh_ctx* c, int variant)
     if (!c) return fail(nullptr, NH_EINVAL, "ctx is NULL");
     if (!lb_variant_valid_for(variant, c->p.nx, (int)store_size(c->p)))
         return fail(c, NH_EINVAL, "LB variant not valid for this domain");
-    if (variant != c->lb_variant) drop_graphs(c);
+    if (variant != c->lb_variant || !c->lb_chosen) drop_graphs(c);  // a batch's plan asks for both
     c->lb_variant = variant;
     c->lb_chosen = true;
     return NH_OK;
@@ -2236,9 +2236,9 @@ int nh_autotune(nh_ctx* c, void* stream, int* chosen)
     c->free_events.push_back(e0);
     c->free_events.push_back(e1);
     c->timing = saved_timing;
+    if (best != saved_variant || !c->lb_chosen) drop_graphs(c);  // a batch's plan asks for both
     c->lb_variant = best;
     c->lb_chosen = true;
-    if (best != saved_variant) drop_graphs(c);
     if (chosen) *chosen = best;
     return r;
 }

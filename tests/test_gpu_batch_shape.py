@@ -59,3 +59,12 @@ def test_tuned_shape_is_launched_in_groups(nh, tmp_path):
     count, shapes = _launched(nh, batch, 8, tmp_path / "t.json")
     assert count == 16
     assert shapes == {SHAPES[chosen]}
+
+
+def test_shape_that_the_channel_has_already_is_set(nh, tmp_path):
+    """Four channels of 2^14 sites take a shape by their joint size; set, the first one's own."""
+    batch = [_channel(nh, (32, 32, 16), "f32") for _ in range(4)]
+    nh.batch_step(batch, 1)
+    assert _launched(nh, batch, 1, tmp_path / "a.json")[1] == {SHAPES[2]}
+    batch[0].set_lb_variant(3)
+    assert _launched(nh, batch, 1, tmp_path / "b.json")[1] == {SHAPES[3]}
