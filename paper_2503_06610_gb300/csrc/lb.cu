@@ -244,6 +244,51 @@ __device__ __forceinline__ void relax_by_pairs(const Real (&f)[19], Real (&fo)[1
     }
 }
 
+// The same for shifted populations in 144 operations a site instead of 215, and with rounding errors that
+// conserve mass and momentum.  With the momentum j = rho u, P = cS F, H = omega j + P (the momentum that the step
+// moves) and g = H + P, a direction of weight w takes
+//   omega f^eq + cS S = w [omega (rho - 1) - 1.5 u.g + 4.5 (e.u)(e.g) + 3 e.H],
+// one even and one odd part a pair.  The weights are not numbers of the type: sums of rounded w * x are off by the
+// same part of x at every site and step, which makes the errors of u grow with the number of steps.  So only the
+// diagonals take theirs from a rounded twelfth of H and a rounded 36th of S; the axes take the rest of H (4 axis +
+// 8 diagonal parts = H), the rest population the rest of S (1 + 6 * 2 + 12 parts, less what u.g gives back).
+// Error of u after 250 steps against the order by pairs, which has such a bias too, on the CPU in FP32: 0.05 at tau
+// 0.55, 0.03 at 0.7, 0.01 at 0.8, 0.04 at 1, 0.1 at 1.478, 0.7 at 2.5; FP64 (20 steps) 0.1 to 0.4.  One twelfth and one
+// 36th for all, without the rests: 2.9 at tau 0.7 and in FP64 5.0 at tau 1.478.
+template <typename Real>
+__device__ __forceinline__ void relax_conserving(const Real (&f)[19], Real (&fo)[19], Real drho, Real jx, Real jy, Real jz,
+                                                 Real ux, Real uy, Real uz, Real Fx, Real Fy, Real Fz, Real omega)
+{
+    const Real omc = Real(1) - omega, cS = fma_rn(Real(-0.5), omega, Real(1));
+    const Real Px = mul_rn(cS, Fx), Py = mul_rn(cS, Fy), Pz = mul_rn(cS, Fz);
+    const Real Hx = fma_rn(omega, jx, Px), Hy = fma_rn(omega, jy, Py), Hz = fma_rn(omega, jz, Pz);
+    const Real gx = Hx + Px, gy = Hy + Py, gz = Hz + Pz;
+    constexpr Real w12 = Real(1) / Real(12), w36 = Real(1) / Real(36);
+    const Real qx = mul_rn(w12, Hx), qy = mul_rn(w12, Hy), qz = mul_rn(w12, Hz);
+    const Real vx = mul_rn(Real(0.125), ux), vy = mul_rn(Real(0.125), uy), vz = mul_rn(Real(0.125), uz);
+    const Real ug8 = fma_rn(vz, gz, fma_rn(vy, gy, mul_rn(vx, gx)));
+    const Real S = fma_rn(omega, drho, mul_rn(Real(-12), ug8));
+    const Real T = mul_rn(w36, S);
+    fo[0] = fma_rn(omc, f[0], fma_rn(Real(-24), T, S));
+    auto pair = [&](int i, Real even, Real odd) {
+        fo[i] = fma_rn(omc, f[i], even) + odd;
+        fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
+    };
+    auto axis = [&](int i, Real v, Real g, Real H, Real q) {
+        pair(i, mul_rn(Real(2), fma_rn(v, g, T)), fma_rn(Real(-4), q, mul_rn(Real(0.5), H)));
+    };
+    auto diagonal = [&](int i, Real v, Real g, Real q) { pair(i, fma_rn(v, g, T), q); };
+    axis(1, vx, gx, Hx, qx);
+    axis(3, vy, gy, Hy, qy);
+    axis(5, vz, gz, Hz, qz);
+    diagonal(7, vx + vy, gx + gy, qx + qy);
+    diagonal(9, vx - vy, gx - gy, qx - qy);
+    diagonal(11, vx + vz, gx + gz, qx + qz);
+    diagonal(13, vx - vz, gx - gz, qx - qz);
+    diagonal(15, vy + vz, gy + gz, qy + qz);
+    diagonal(17, vy - vz, gy - gz, qy - qz);
+}
+
 // Moments, equilibrium, Guo source and relaxation of one site s from its
 // streamed populations f (decoded values; raw 2^k-scaled ones for the 16-bit
 // stores, whose power-of-two factors inv_in and scale_out are folded in) and
@@ -262,8 +307,9 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
     constexpr bool WriteMacro = Macro >= 1;
     constexpr bool Partials = Macro == 2;
     // A 16-bit store rounds to 8 or 11 bits, so that a last bit of FP32 moves a population by a whole unit of the store:
-    // these keep the order that every result of theirs was computed with.
-    constexpr bool ByPairs = kScaled;
+    // these keep the order that every result of theirs was computed with.  Unshifted populations, whose errors come
+    // from rounding f = w + ..., gain nothing from the other one (u up to 1.2 times as far off).
+    constexpr bool ByPairs = kScaled || !Shifted;
     const int N = c.g.N;
     // 2. moments: pair sums and differences of (e_i, -e_i)
     Real d[9];
@@ -305,9 +351,8 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
         Hy = fma_rn(rho, c.gy, c.Fu[N + s]);
         Hz = fma_rn(rho, c.gz, c.Fu[2 * N + s]);
     }
-    const Real ux = mul_rn(fma_rn(Real(0.5), Hx, mx), inv_rho);
-    const Real uy = mul_rn(fma_rn(Real(0.5), Hy, my), inv_rho);
-    const Real uz = mul_rn(fma_rn(Real(0.5), Hz, mz), inv_rho);
+    const Real jx = fma_rn(Real(0.5), Hx, mx), jy = fma_rn(Real(0.5), Hy, my), jz = fma_rn(Real(0.5), Hz, mz);
+    const Real ux = mul_rn(jx, inv_rho), uy = mul_rn(jy, inv_rho), uz = mul_rn(jz, inv_rho);
     if (WriteMacro) {
         c.u[s] = ux;
         c.u[N + s] = uy;
@@ -324,45 +369,7 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
                        mul_rn(Real(1) - c.omega, kScaled ? mul_rn(Real(inv_in), so) : Real(1)),
                        mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so));
     } else {
-        // With g = 1.5 omega rho u + 3 (1 - omega/2) F and h = g + 1.5 omega rho u the two sums are
-        //   omega f^eq + (1 - omega/2) S = w [3 (e.u)(e.g) + T + e.h],  T = omega (rho - 1 | rho) - u.g
-        // so a pair costs one even and one odd part from three projections: 150
-        // operations a site instead of 215.  FP64 LB is bound by the FP64 pipe.
-        const Real omega = c.omega, omc = Real(1) - c.omega;
-        const Real cS3 = mul_rn(Real(3), fma_rn(Real(-0.5), c.omega, Real(1)));
-        const Real a15 = mul_rn(mul_rn(Real(1.5), omega), rho);
-        const Real gx = fma_rn(a15, ux, mul_rn(cS3, Fx));
-        const Real gy = fma_rn(a15, uy, mul_rn(cS3, Fy));
-        const Real gz = fma_rn(a15, uz, mul_rn(cS3, Fz));
-        constexpr Real w36 = Real(1) / Real(36), w12 = Real(1) / Real(12);
-        const Real hx = mul_rn(w36, fma_rn(a15, ux, gx));
-        const Real hy = mul_rn(w36, fma_rn(a15, uy, gy));
-        const Real hz = mul_rn(w36, fma_rn(a15, uz, gz));
-        const Real vx = mul_rn(w12, ux), vy = mul_rn(w12, uy), vz = mul_rn(w12, uz);
-        const Real ug = fma_rn(uz, gz, fma_rn(uy, gy, mul_rn(ux, gx)));
-        const Real T = fma_rn(mul_rn(w36, omega), Shifted ? sum : rho, -mul_rn(w36, ug));
-        fo[0] = fma_rn(Real(12), T, mul_rn(omc, f[0]));
-        const Real omc_half = mul_rn(Real(0.5), omc);
-        // axis pair (w = 1/18: twice the 1/36 parts), diagonal pair
-        auto axis = [&](int i, Real v, Real g, Real h) {
-            const Real even = fma_rn(v, g, T);
-            fo[i] = mul_rn(Real(2), fma_rn(omc_half, f[i], even) + h);
-            fo[i + 1] = mul_rn(Real(2), fma_rn(omc_half, f[i + 1], even) - h);
-        };
-        auto diagonal = [&](int i, Real v, Real g, Real h) {
-            const Real even = fma_rn(v, g, T);
-            fo[i] = fma_rn(omc, f[i], even + h);
-            fo[i + 1] = fma_rn(omc, f[i + 1], even - h);
-        };
-        axis(1, vx, gx, hx);
-        axis(3, vy, gy, hy);
-        axis(5, vz, gz, hz);
-        diagonal(7, vx + vy, gx + gy, hx + hy);
-        diagonal(9, vx - vy, gx - gy, hx - hy);
-        diagonal(11, vx + vz, gx + gz, hx + hz);
-        diagonal(13, vx - vz, gx - gz, hx - hz);
-        diagonal(15, vy + vz, gy + gz, hy + hz);
-        diagonal(17, vy - vz, gy - gz, hy - hz);
+        relax_conserving(f, fo, sum, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz, c.omega);
     }
     if (Partials) {  // the sums nh_diagnostics forms from the stored state, site by site
         const Real u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));

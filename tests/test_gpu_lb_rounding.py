@@ -99,3 +99,41 @@ def test_16_bit_stores_round_as_by_pairs(storage, bits, dims):
     normal = np.abs(want) > 2.0 ** -10 * np.abs(want).max()  # F16S: above the store's subnormal range
     assert normal.mean() > 0.9
     assert np.array_equal(got[normal], want[normal])
+
+
+# sites per thread by size: odd rows, small blocks, two sites; pairs of steps collide with the same code
+@pytest.mark.parametrize("dims", [(33, 18, 9), (64, 64, 28)])
+@pytest.mark.parametrize("tau", [0.7, 1.1])
+def test_unshifted_fp32_rounds_as_by_pairs(dims, tau):
+    ch = channel("f32", False, dims, tau)
+    (want, wu, wrho), (got, u, rho) = step_by_pairs(ch, dims, False, tau)
+    assert np.array_equal(u.astype(R), wu) and np.array_equal(rho.astype(R), wrho)
+    assert np.array_equal(got.astype(R), want)
+
+
+# 7.5e5 sites and more: pairs of steps
+@pytest.mark.parametrize("dims", [(48, 40, 24), (160, 120, 40)])
+@pytest.mark.parametrize("tau", [0.55, 0.7, 0.8, 1.0, 1.1, 1.478])
+@pytest.mark.parametrize("walls", [True, False])
+def test_shifted_fp32_errors_do_not_grow_with_the_steps(dims, tau, walls):
+    """Velocity of 250 steps against FP64.  A step rounds u a few times, to 2^-24 of it each; errors that are not the
+    same at every site and step add as their root mean square, sqrt(250) * 2^-24 = 0.94e-6 for one a step, less what
+    viscosity takes away.  A bias of the weights by 2^-25 would give 250 / tau * 2^-25 = 7.5e-6 / tau."""
+    from paper_2503_06610_gb300 import nh
+    nx, ny, nz = dims
+    N = nx * ny * nz
+    n = np.zeros((3, N))
+    n[2] = 1.0  # uniform: no force from the director
+    x, y, z = np.meshgrid(np.arange(nx), np.arange(ny), np.arange(nz), indexing="ij")
+    kx, ky = 2 * np.pi / nx, 2 * np.pi / ny
+    prof = np.sin(np.pi * (z + 0.5) / nz) if walls else 1.0 + 0.3 * np.sin(2 * np.pi * z / nz)
+    u = 2e-3 * np.stack([(prof * f).transpose(2, 1, 0).ravel() for f in (1 + 0.3 * np.cos(ky * y), 0.6 + np.cos(kx * x + 1),
+                                                                         0.3 * np.cos(kx * x - ky * y))])
+    out = []
+    for precision, storage in (("fp64", "f64"), ("fp32", "f32")):
+        ch = nh.Channel(dict(nx=nx, ny=ny, nz=nz, walls_z=walls, anchoring="none", shifted=True, tau=tau, g=(2.0 ** -20, 0.0, 0.0),
+                             K=0.005, q0=0.0, W0=0.0, dt_fd=1000, precision=precision, storage=storage, **I.LESLIE_ALIGN_09))
+        ch.set_fields(n, u.astype(R).astype(np.float64))
+        ch.step(250)
+        out.append(np.asarray(ch.get_fields()[1]).ravel())
+    assert np.linalg.norm(out[1] - out[0]) < 250 ** 0.5 * 2.0 ** -24 * np.linalg.norm(out[0])
