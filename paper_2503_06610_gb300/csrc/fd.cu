@@ -1570,27 +1570,27 @@ inline int fused_tiles(const FDChan<Real>& c)
 template <typename Real>
 cudaError_t prepare_fused()
 {
-    static bool done = false;  // the attribute is per function; setting it twice is harmless
-    if (done) return cudaSuccess;
-    const int a = (int)fused_a_smem<Real>(), b = (int)fused_b_smem<Real>(), r = (int)relax_smem<Real>();
-    const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(fused_a_kernel<Real, false>, attr, a);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_a_kernel<Real, true>, attr, a);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_b_kernel<Real, false>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_b_kernel<Real, true>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_b_diag_kernel<Real>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 0, false>, attr, a);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 0, true>, attr, a);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 1, false>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 1, true>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, false>, attr, r);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, true>, attr, r);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 3, false>, attr, r);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 3, true>, attr, r);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(relax_kernel<Real, false>, attr, r);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(relax_kernel<Real, true>, attr, r);
-    if (e == cudaSuccess) done = true;
-    return e;
+    static OncePerDevice once;
+    return once_per_device(once, [] {
+        const int a = (int)fused_a_smem<Real>(), b = (int)fused_b_smem<Real>(), r = (int)relax_smem<Real>();
+        const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(fused_a_kernel<Real, false>, attr, a);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_a_kernel<Real, true>, attr, a);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_b_kernel<Real, false>, attr, b);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_b_kernel<Real, true>, attr, b);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_b_diag_kernel<Real>, attr, b);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 0, false>, attr, a);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 0, true>, attr, a);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 1, false>, attr, b);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 1, true>, attr, b);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, false>, attr, r);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 2, true>, attr, r);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 3, false>, attr, r);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_batch_kernel<Real, 3, true>, attr, r);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(relax_kernel<Real, false>, attr, r);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(relax_kernel<Real, true>, attr, r);
+        return e;
+    });
 }
 
 inline int blocks_for(int N) { return (N + 255) / 256; }

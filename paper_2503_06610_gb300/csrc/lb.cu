@@ -21,6 +21,7 @@
 // count), so that the diagnostics of that state need not read the
 // populations, u and rho again.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "nh_internal.cuh"
@@ -852,23 +853,25 @@ bool lb_rows_valid(int nx, int store_bytes)
 // grid), computed once per row length by lb_rows_prepare, outside any graph
 // capture.
 template <typename Real, typename Store, bool Shifted, int Macro>
-int& rows_resident(int nx)
+std::atomic<int>& rows_resident(int nx)
 {
-    static int resident[kRowMaxNx / (32 * kRowSPT) + 1] = {};
+    static std::atomic<int> resident[kRowMaxNx / (32 * kRowSPT) + 1];
     return resident[nx / (32 * kRowSPT)];
 }
 
 template <typename Real, typename Store, bool Shifted, int Macro>
 cudaError_t prepare_rows_one(int nx)
 {
-    int& resident = rows_resident<Real, Store, Shifted, Macro>(nx);
-    if (resident > 0) return cudaSuccess;
+    std::atomic<int>& resident = rows_resident<Real, Store, Shifted, Macro>(nx);
     auto kern = lb_rows_kernel<Real, Store, Shifted, Macro>;
     const size_t smem = lb_rows_smem(nx, (int)sizeof(Store));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)lb_rows_smem(kRowMaxNx, 2));
+    static OncePerDevice once;
+    cudaError_t e = once_per_device(once, [kern] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lb_rows_smem(kRowMaxNx, 2));
+    });
+    if (e != cudaSuccess || resident > 0) return e;
     int dev = 0, sms = 0, per_sm = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nx / kRowSPT, smem);
     if (e == cudaSuccess) resident = (per_sm > 0 ? per_sm : 1) * sms;
@@ -1160,16 +1163,16 @@ cudaError_t pair_attr()
 }
 cudaError_t prepare_pair()
 {
-    static bool done = false;  // the attribute is per function; setting it twice is harmless
-    if (done) return cudaSuccess;
-    cudaError_t e = pair_attr<true, 0>();
-    if (e == cudaSuccess) e = pair_attr<true, 1>();
-    if (e == cudaSuccess) e = pair_attr<true, 2>();
-    if (e == cudaSuccess) e = pair_attr<false, 0>();
-    if (e == cudaSuccess) e = pair_attr<false, 1>();
-    if (e == cudaSuccess) e = pair_attr<false, 2>();
-    done = e == cudaSuccess;
-    return e;
+    static OncePerDevice once;
+    return once_per_device(once, [] {
+        cudaError_t e = pair_attr<true, 0>();
+        if (e == cudaSuccess) e = pair_attr<true, 1>();
+        if (e == cudaSuccess) e = pair_attr<true, 2>();
+        if (e == cudaSuccess) e = pair_attr<false, 0>();
+        if (e == cudaSuccess) e = pair_attr<false, 1>();
+        if (e == cudaSuccess) e = pair_attr<false, 2>();
+        return e;
+    });
 }
 
 template <bool Shifted>

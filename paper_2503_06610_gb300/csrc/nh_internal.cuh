@@ -11,6 +11,7 @@
 #include <string>
 
 #include "../../include/nh.h"
+#include "once_per_device.h"
 
 namespace nh {
 
@@ -218,6 +219,15 @@ inline void launch_step_kernel(void (*kernel)(Params...), dim3 grid, int threads
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     (void)cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+// Opt-ins and other set-up of the current device, once.
+template <typename F>
+inline cudaError_t once_per_device(OncePerDevice& once, F&& set)
+{
+    int device = 0;
+    const cudaError_t e = cudaGetDevice(&device);
+    return e == cudaSuccess ? once(device, set) : e;
 }
 
 // ------------------------------------------------------------------ launchers (host)

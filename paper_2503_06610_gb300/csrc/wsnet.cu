@@ -514,13 +514,12 @@ __global__ void __launch_bounds__(kTcThreads, NB == 32 && Flip ? 3 : 4) conv_tc_
 template <bool Flip, int K, int NB>
 cudaError_t launch_conv_tc(ConvTc a, cudaStream_t st)
 {
-    static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<NB, Flip, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)kTcMaxSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static nh::OncePerDevice once;  // the opt-in to more than 48 KB of shared memory
+    const cudaError_t e = nh::once_per_device(once, [] {
+        return cudaFuncSetAttribute(conv_tc_kernel<NB, Flip, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kTcMaxSmem);
+    });
+    if (e != cudaSuccess) return e;
     if (a.n % NB || a.c1 % 8) return cudaErrorInvalidValue;
     const int cols = ((a.d.nx + kTcX - 1) / kTcX) * ((a.d.ny + kTcY - 1) / kTcY) * a.d.batch;
     int64_t best = -1;
@@ -1176,17 +1175,15 @@ cudaError_t conv_bwd(nh_unet* u, int l, int level, const bf16* gp, const bf16* s
     w.gw = grad + layer_offset(l);
     w.d = d;
     w.tiles = ((d.nx + kWTx - 1) / kWTx) * ((d.ny + kWTy - 1) / kWTy) * ((d.nz + kWTz - 1) / kWTz) * d.batch;
-    static bool attr_set = false;  // the opt-in to more than 48 KB of shared memory, once per process
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(conv_bwd_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static nh::OncePerDevice once;  // the opt-in to more than 48 KB of shared memory
+    cudaError_t e = nh::once_per_device(
+        once, [] { return cudaFuncSetAttribute(conv_bwd_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem); });
+    if (e != cudaSuccess) return e;
     // one wave of resident blocks over the channel pairs; each walks its share of the tiles
     const int pairs = (cin / 16) * (cout / 16);
     dim3 grid(std::min(w.tiles, std::max(1, kWBlocksPerSM * 152 / pairs)), pairs);
     nh::launch_step_kernel(conv_bwd_w_kernel, grid, kWThreads, kWSmem, st, w);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess || (gp_below == nullptr && dst1 == nullptr)) return e;
     ConvTc b{};
     b.src1 = gp;
