@@ -211,51 +211,18 @@ __device__ __forceinline__ Real edot(int X, int Y, int Z, Real vx, Real vy, Real
     return r;
 }
 
-// Relaxation of one site, direction pair by direction pair, from the streamed populations f, rho, u and the force:
-//   f^eq = w rho [3 eu + 4.5 eu^2 - 1.5 u.u] + w (rho - 1 | rho)
-//   S    = w [3 eF + 9 eu eF - 3 u.F]
-//   f*   = omc f + omega f^eq + cS S,  omc = 1 - omega, cS = 1 - omega / 2
-// base: rho - 1 for shifted populations, else rho.
-template <typename Real>
-__device__ __forceinline__ void relax_by_pairs(const Real (&f)[19], Real (&fo)[19], Real rho, Real base, Real ux, Real uy,
-                                               Real uz, Real Fx, Real Fy, Real Fz, Real omega, Real omc, Real cS)
-{
-    NH_D3Q19_TABLES
-    const Real uu15 = mul_rn(Real(1.5), fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux))));
-    const Real uF3 = mul_rn(Real(3), fma_rn(uz, Fz, fma_rn(uy, Fy, mul_rn(ux, Fx))));
-    // rest population (w = 1/3)
-    const Real w0 = Real(1) / Real(3);
-    fo[0] = fma_rn(omc, f[0], fma_rn(mul_rn(omega, w0), fma_rn(-rho, uu15, base), -mul_rn(mul_rn(cS, w0), uF3)));
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int i = 2 * k + 1;
-        const Real w = i < 7 ? Real(1) / Real(18) : Real(1) / Real(36);
-        const Real ow = mul_rn(omega, w);
-        const Real A = mul_rn(ow, rho);
-        const Real B = mul_rn(ow, base);
-        const Real C = mul_rn(cS, w);
-        const Real eu = edot(EX[i], EY[i], EZ[i], ux, uy, uz);
-        const Real eF = edot(EX[i], EY[i], EZ[i], Fx, Fy, Fz);
-        const Real X = fma_rn(mul_rn(Real(4.5), eu), eu, -uu15);
-        const Real Y = fma_rn(mul_rn(Real(9), eu), eF, -uF3);
-        const Real even = fma_rn(C, Y, fma_rn(A, X, B));
-        const Real odd = mul_rn(Real(3), fma_rn(A, eu, mul_rn(C, eF)));
-        fo[i] = fma_rn(omc, f[i], even) + odd;
-        fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
-    }
-}
-
-// The same for shifted populations in 144 operations a site instead of 215, and with rounding errors that
-// conserve mass and momentum.  With the momentum j = rho u, P = cS F, H = omega j + P (the momentum that the step
-// moves) and g = H + P, a direction of weight w takes
+// Relaxation of a site with shifted populations, cS = 1 - omega / 2: what lb_collide_site writes out by pairs, in 144
+// operations instead of 215 and with rounding errors that conserve mass and momentum.  With the momentum j = rho u,
+// P = cS F, H = omega j + P (the momentum that the step moves) and g = H + P, a direction of weight w takes
 //   omega f^eq + cS S = w [omega (rho - 1) - 1.5 u.g + 4.5 (e.u)(e.g) + 3 e.H],
-// one even and one odd part a pair.  The weights are not numbers of the type: sums of rounded w * x are off by the
-// same part of x at every site and step, which makes the errors of u grow with the number of steps.  So only the
-// diagonals take theirs from a rounded twelfth of H and a rounded 36th of S; the axes take the rest of H (4 axis +
-// 8 diagonal parts = H), the rest population the rest of S (1 + 6 * 2 + 12 parts, less what u.g gives back).
-// Error of u after 250 steps against the order by pairs, which has such a bias too, on the CPU in FP32: 0.05 at tau
-// 0.55, 0.03 at 0.7, 0.01 at 0.8, 0.04 at 1, 0.1 at 1.478, 0.7 at 2.5; FP64 (20 steps) 0.1 to 0.4.  One twelfth and one
-// 36th for all, without the rests: 2.9 at tau 0.7 and in FP64 5.0 at tau 1.478.
+// one even and one odd part a pair.  The weights are not numbers of the type: a rounded w puts every x in w x off by
+// the same factor at every site and step, and the errors of u grow with the number of steps.  So only the diagonals
+// take a rounded twelfth of H and, like the axes, a rounded 36th T of the even sum S; the axes take what is left of H
+// (four of their parts and eight of the diagonals' make H), the rest population what is left of S (24 T of it are the
+// others').
+// Error of u after 250 steps, that of the order by pairs (biased too) being 1, FP32 on the CPU: 0.05 at tau 0.55, 0.03
+// at 0.7, 0.01 at 0.8, 0.04 at 1, 0.1 at 1.478, 0.7 at 2.5; FP64, 20 steps, 0.1 to 0.4.  Rounded twelfths and 36ths for
+// all directions alike: 2.9 at tau 0.7, and in FP64 5.0 at tau 1.478.
 template <typename Real>
 __device__ __forceinline__ void relax_conserving(const Real (&f)[19], Real (&fo)[19], Real drho, Real jx, Real jy, Real jz,
                                                  Real ux, Real uy, Real uz, Real Fx, Real Fy, Real Fz, Real omega)
@@ -313,24 +280,25 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
     constexpr bool ByPairs = kScaled || !Shifted;
     const int N = c.g.N;
     // 2. moments: pair sums and differences of (e_i, -e_i)
-    Real d[9];
-    Real sum = f[0];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        sum += f[2 * k + 1] + f[2 * k + 2];
-        d[k] = f[2 * k + 1] - f[2 * k + 2];
-    }
-    Real mx, my, mz;
+    Real sum = f[0], mx = 0, my = 0, mz = 0;
     if constexpr (ByPairs) {
-        mx = my = mz = 0;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int i = 2 * k + 1;
-            if (EX[i] != 0) mx += EX[i] > 0 ? d[k] : -d[k];
-            if (EY[i] != 0) my += EY[i] > 0 ? d[k] : -d[k];
-            if (EZ[i] != 0) mz += EZ[i] > 0 ? d[k] : -d[k];
+            sum += f[i] + f[i + 1];
+            const Real d = f[i] - f[i + 1];
+            if (EX[i] != 0) mx += EX[i] > 0 ? d : -d;
+            if (EY[i] != 0) my += EY[i] > 0 ? d : -d;
+            if (EZ[i] != 0) mz += EZ[i] > 0 ? d : -d;
         }
-    } else {  // pairs: x, y, z, (x+y, x-y), (x+z, x-z), (y+z, y-z)
+    } else {
+        Real d[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            sum += f[2 * k + 1] + f[2 * k + 2];
+            d[k] = f[2 * k + 1] - f[2 * k + 2];
+        }
+        // pairs: x, y, z, (x+y, x-y), (x+z, x-z), (y+z, y-z)
         mx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
         my = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
         mz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
@@ -352,8 +320,9 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
         Hy = fma_rn(rho, c.gy, c.Fu[N + s]);
         Hz = fma_rn(rho, c.gz, c.Fu[2 * N + s]);
     }
-    const Real jx = fma_rn(Real(0.5), Hx, mx), jy = fma_rn(Real(0.5), Hy, my), jz = fma_rn(Real(0.5), Hz, mz);
-    const Real ux = mul_rn(jx, inv_rho), uy = mul_rn(jy, inv_rho), uz = mul_rn(jz, inv_rho);
+    const Real ux = mul_rn(fma_rn(Real(0.5), Hx, mx), inv_rho);
+    const Real uy = mul_rn(fma_rn(Real(0.5), Hy, my), inv_rho);
+    const Real uz = mul_rn(fma_rn(Real(0.5), Hz, mz), inv_rho);
     if (WriteMacro) {
         c.u[s] = ux;
         c.u[N + s] = uy;
@@ -361,19 +330,52 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
         c.rho[s] = rho;
     }
 
-    // 3-4. equilibrium, Guo source and relaxation.  With a 16-bit store the
-    // constants carry scale_out (and omc the raw input's inv_in), so fo[] leaves
-    // here already in encoded units.
+    // 3-4. equilibrium, Guo source and relaxation
+    Real u2;
     if constexpr (ByPairs) {
+        // per (e_i, -e_i) pair:
+        //   f^eq = w rho [3 eu + 4.5 eu^2 - 1.5 u.u] + w (rho - 1 | rho)
+        //   S    = w [3 eF + 9 eu eF - 3 u.F]
+        //   f*   = (1 - omega) f + omega f^eq + (1 - omega/2) S
+        // with a 16-bit store the constants carry scale_out (and omc the raw
+        // input's inv_in), so fo[] leaves here already in encoded units
         const Real so = kScaled ? Real(scale_out) : Real(1);
-        relax_by_pairs(f, fo, rho, Shifted ? sum : rho, ux, uy, uz, Fx, Fy, Fz, mul_rn(c.omega, so),
-                       mul_rn(Real(1) - c.omega, kScaled ? mul_rn(Real(inv_in), so) : Real(1)),
-                       mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so));
+        const Real omega = mul_rn(c.omega, so);
+        const Real omc = mul_rn(Real(1) - c.omega, kScaled ? mul_rn(Real(inv_in), so) : Real(1));
+        const Real cS = mul_rn(fma_rn(Real(-0.5), c.omega, Real(1)), so);
+        u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
+        const Real uu15 = mul_rn(Real(1.5), u2);
+        const Real uF3 = mul_rn(Real(3), fma_rn(uz, Fz, fma_rn(uy, Fy, mul_rn(ux, Fx))));
+        const Real base = Shifted ? sum : rho;
+        // rest population (w = 1/3)
+        {
+            const Real w = Real(1) / Real(3);
+            const Real t = fma_rn(-rho, uu15, base);
+            fo[0] = fma_rn(omc, f[0], fma_rn(mul_rn(omega, w), t, -mul_rn(mul_rn(cS, w), uF3)));
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int i = 2 * k + 1;
+            const Real w = i < 7 ? Real(1) / Real(18) : Real(1) / Real(36);
+            const Real ow = mul_rn(omega, w);
+            const Real A = mul_rn(ow, rho);
+            const Real B = mul_rn(ow, base);
+            const Real C = mul_rn(cS, w);
+            const Real eu = edot(EX[i], EY[i], EZ[i], ux, uy, uz);
+            const Real eF = edot(EX[i], EY[i], EZ[i], Fx, Fy, Fz);
+            const Real X = fma_rn(mul_rn(Real(4.5), eu), eu, -uu15);
+            const Real Y = fma_rn(mul_rn(Real(9), eu), eF, -uF3);
+            const Real even = fma_rn(C, Y, fma_rn(A, X, B));
+            const Real odd = mul_rn(Real(3), fma_rn(A, eu, mul_rn(C, eF)));
+            fo[i] = fma_rn(omc, f[i], even) + odd;
+            fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
+        }
     } else {
-        relax_conserving(f, fo, sum, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz, c.omega);
+        u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
+        relax_conserving(f, fo, sum, fma_rn(Real(0.5), Hx, mx), fma_rn(Real(0.5), Hy, my), fma_rn(Real(0.5), Hz, mz), ux, uy, uz,
+                         Fx, Fy, Fz, c.omega);
     }
     if (Partials) {  // the sums nh_diagnostics forms from the stored state, site by site
-        const Real u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
         Real fs = fo[0];
 #pragma unroll
         for (int i = 1; i < 19; ++i) fs += fo[i];
@@ -1266,11 +1268,11 @@ bool lb_variant_valid_for(int variant, int nx, int store_bytes)
 
 // The default shape of a channel (microseconds of 16 LB steps and an FD update,
 // two sites x 256 | one x 256 | two x 128 | one x 128 | four x 128 | rows):
-//   FP32 32x32x16: 62 | 50 | 51 | 45 | 64, 96x96x32: 137 | 143 | 132 | 137 | 137,
-//   256x256x64: 1825 | 1818 | 1820 | 1821 | 1837 (at the HBM limit);
-//   F16S 64x64x32: 115 | 127 | 115 | 126 | 108, 180x140x50: 554 | 599 | 539 | 645 | 485,
-//   256x256x16: 439 | 496 | 427 | 519 | 385 | 363, 256x256x64: 1598 | 1716 | 1514 | 1875 | 1370 | 1265,
-//   128x128x32: 243 | 275 | 245 | 294 | 216 | 237.
+//   FP32 32x32x16: 52 | 42 | 44 | 38 | 56, 96x96x32: 123 | 134 | 120 | 128 | 126,
+//   256x256x64, single steps: 1825 | 1818 | 1820 | 1821 | 1837 (at the HBM limit);
+//   F16S 64x64x32: 113 | 129 | 116 | 126 | 111, 180x140x50: 745 | 635 | 645 | 668 | 511,
+//   256x256x16: 597 | 531 | 513 | 546 | 413 | 397, 256x256x64: 2311 | 1854 | 1897 | 1884 | 1430 | 1302,
+//   128x128x32: 305 | 291 | 279 | 300 | 226 | 258.
 // So: small blocks of single sites while they do not fill the GPU (up to 2^15
 // sites), two sites x 128 otherwise; the 16-bit stores, bound by issue rather than
 // HBM, take the four-site shape from 10^5 sites, and the staged rows where a row
