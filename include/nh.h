@@ -216,11 +216,11 @@ int nh_fd_update(nh_ctx* ctx, void* stream);
  * by n_lb_steps each.  Every pass (LB sweep, FD predict, correct, stress,
  * force) is one persistent launch per group of up to 64 channels: the grid
  * walks a work list of (channel, tile) pairs, and the channel descriptors
- * travel as kernel parameters.  The LB steps of a block of at least four
- * steps run group by group of channels whose populations fit in L2 together
- * (large FP32 channels take two steps per launch instead).  Whole dt_fd blocks (of at least 12 steps) are replayed from a CUDA
- * graph cached per list of contexts (dropped when a context is rebound,
- * re-tuned or destroyed).  All contexts must share precision, storage,
+ * travel as kernel parameters.  With FP32 stores the LB steps of a block of at
+ * least four steps run group by group of channels whose populations fit in L2
+ * together (large channels take two steps per launch instead).  Whole dt_fd
+ * blocks (of at least 12 steps) are replayed from a CUDA graph cached per list
+ * of contexts (dropped when a context is rebound, re-tuned or destroyed).  All contexts must share precision, storage,
  * shifted and dt_fd, be on one device, have fields set and be at the same
  * step phase (step mod dt_fd and buffer parity), and not use paper_order,
  * lap_wide or n_from_rate; otherwise NH_EINVAL and nothing runs.  The FD

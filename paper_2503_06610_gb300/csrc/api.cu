@@ -923,7 +923,10 @@ void drop_batch_plans(const nh_ctx* c)
 // and 12.2, groups of 70, 84 and 100 MB for the LB steps alone 10.1, 10.2 and 10.9
 // (12 channels: 2.0 each, at once 2.6; dt_fd 4: 17.6 at once, 15.9).  Blocks of two
 // steps gain nothing (23.4 | 23.5).  Not where the channels take pairs of steps
-// (large ones).
+// (large ones), and only FP32 stores, whose single steps HBM bounds: the 16-bit ones
+// are bound by issue and FP64 by its pipe, where smaller launches only lose (16
+// channels of 96x96x32, dt_fd 16, us a step in groups | at once: F16S 116 | 110, BF16S
+// 119 | 115, FP64 1724 | 1629).
 constexpr double kGroupBytes = 84e6;
 constexpr int kGroupMinSteps = 4;
 bool batch_pair_ok(const Channels& ctxs);
@@ -937,7 +940,7 @@ void batch_groups(BatchPlan* b)
         total += bytes.back();
     }
     const int groups = (int)std::ceil(total / kGroupBytes);
-    if (groups < 2 || b->ctxs.size() < 2 || batch_pair_ok(b->ctxs)) return;
+    if (b->ctxs[0]->p.storage != NH_STORE_F32 || groups < 2 || b->ctxs.size() < 2 || batch_pair_ok(b->ctxs)) return;
     double sum = 0;  // cut where the running sum passes an even share
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
         if (b->groups.empty() || sum + 0.5 * bytes[k] > total * (double)b->groups.size() / groups) b->groups.emplace_back();

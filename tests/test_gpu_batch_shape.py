@@ -24,7 +24,7 @@ def nh():
 def _channel(nh, dims, storage):
     nx, ny, nz = dims
     ch = nh.Channel(dict(nx=nx, ny=ny, nz=nz, walls_z=True, anchoring="homeotropic", shifted=True, tau=0.8, g=(1e-5, 0.0, 0.0),
-                         K=0.005, q0=0.2, W0=0.0, dt_fd=9, precision="fp32", storage=storage, **I.LESLIE_ALIGN_09))
+                         K=0.005, q0=0.2, W0=0.0, dt_fd=9, precision="fp64" if storage == "f64" else "fp32", storage=storage, **I.LESLIE_ALIGN_09))
     ch.set_fields(I.tilted_director(nx, ny, nz, amplitude=0.5, seed=1))
     return ch
 
@@ -51,13 +51,13 @@ def _launched(nh, batch, steps, path):
 
 
 def test_tuned_shape_is_launched_in_groups(nh, tmp_path):
-    """1.2 M sites of 88 bytes: two groups."""
-    batch = [_channel(nh, (96, 96, 32), "f16s") for _ in range(4)]
+    """1.2 M sites of 164 bytes: three groups."""
+    batch = [_channel(nh, (96, 96, 32), "f32") for _ in range(4)]
     batch[0].set_lb_variant(1)
     nh.batch_step(batch, 1)
     chosen = nh.batch_autotune(batch)
     count, shapes = _launched(nh, batch, 8, tmp_path / "t.json")
-    assert count == 16
+    assert count == 24
     assert shapes == {SHAPES[chosen]}
 
 
@@ -68,3 +68,11 @@ def test_shape_that_the_channel_has_already_is_set(nh, tmp_path):
     assert _launched(nh, batch, 1, tmp_path / "a.json")[1] == {SHAPES[2]}
     batch[0].set_lb_variant(3)
     assert _launched(nh, batch, 1, tmp_path / "b.json")[1] == {SHAPES[3]}
+
+
+@pytest.mark.parametrize("storage", ["f16s", "bf16s", "f64"])
+def test_only_fp32_stores_step_in_groups(nh, tmp_path, storage):
+    """Steps that HBM does not bound gain nothing from smaller launches: one for all channels."""
+    batch = [_channel(nh, (96, 96, 32), storage) for _ in range(4)]
+    nh.batch_step(batch, 1)
+    assert _launched(nh, batch, 8, tmp_path / "t.json")[0] == 8
