@@ -234,7 +234,8 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
 
 /* Autotuner of the batched LB launch: times every launch shape valid for all
  * channels on the batch itself (the state is not advanced), keeps the fastest
- * for this list of contexts and returns it in *chosen.  Synchronises. */
+ * for this list of contexts (the one in use unless another takes 3 % less time)
+ * and returns it in *chosen.  Synchronises. */
 int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen);
 
 /* ------------------------------------------------------------------------

@@ -1885,9 +1885,10 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
             for (int k = 0; k < reps && e == NH_OK; ++k) e = batch_enqueue_lb(plan, g, false, st);
         return e;
     };
-    float best_ms = 1e30f;
-    int best = plan->variant;
+    float ms[kLBVariantCount];
+    std::fill(ms, ms + kLBVariantCount, 1e30f);
     const int saved = plan->variant;
+    int best = saved;
     for (int v = 0; v < kLBVariantCount && r == NH_OK; ++v) {
         bool ok = true;
         for (nh_ctx* c : plan->ctxs) ok = ok && lb_variant_valid(v, c->p.nx);
@@ -1903,12 +1904,13 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
             r = fail(nullptr, NH_ECUDA, "cudaEventSynchronize");
             break;
         }
-        float ms = 0.f;
-        if (cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms) {
-            best_ms = ms;
-            best = v;
-        }
+        if (cudaEventElapsedTime(&ms[v], e0, e1) != cudaSuccess) ms[v] = 1e30f;
+        if (ms[v] < ms[best]) best = v;
     }
+    // The trials leave out the launches that write u and rho (they would change the state), which four sites a thread
+    // slow down most: 16 channels of 96x96x32, FP32, in groups took 168 us a step at dt_fd 4 with two sites and 175
+    // with four, which the trials saw ahead by 1 to 2 %.
+    if (ms[best] > 0.97f * ms[saved]) best = saved;
     c0->free_events.push_back(e0);
     c0->free_events.push_back(e1);
     c0->timing = saved_timing;
