@@ -219,6 +219,8 @@ struct nh_ctx {
     bool use_graphs = true;
     int lb_variant = 0;
     bool lb_chosen = false;  // the launch shape was set or autotuned, not the default of lb_default_variant
+    bool pairs = false;      // two LB steps per launch (pair_ok), cut as `pair`
+    PairGrid pair{};
     int fd_variant = -1;     // 1: fused 2.5D FD kernels; 0: per-site kernels; -1: by precision (fd_fused)
     int sm_count = 152;
     int64_t epoch = 0;  // bumped whenever buffers or launch shapes change (invalidates batch plans)
@@ -500,18 +502,17 @@ int enqueue_lb(nh_ctx* c, int src, bool write_macro, cudaStream_t st, bool stale
 }
 
 // Two LB steps in one launch: FP32 populations, no obstacles, large enough.
-bool pair_fits(const nh_ctx* c) { return c->p.storage == NH_STORE_F32 && !c->has_solid && lb_pair_valid(geom(c)); }
-bool pair_ok(const nh_ctx* c) { return lb_pair_pays(c->N) && pair_fits(c); }
+bool pair_ok(const nh_ctx* c) { return c->pairs && !c->has_solid; }
 
 int enqueue_lb_pair(nh_ctx* c, bool write_macro, cudaStream_t st, bool sums)
 {
     auto a = lb_chan<float, float>(c, c->cur);
     if (write_macro && sums && fold_ok(c)) {
         c->lbp_step = c->step + 2;
-        c->lbp_blocks = lb_pair_blocks(a.g);
+        c->lbp_blocks = pair_blocks(c->pair);
         a.part = c->at<double>(c->L.lbpart);
     }
-    return timed(c, NH_KCLASS_LB, st, [&] { return launch_lb_pair(a, c->p.shifted != 0, write_macro, st); }, "lb_pair");
+    return timed(c, NH_KCLASS_LB, st, [&] { return launch_lb_pair(a, c->pair, c->p.shifted != 0, write_macro, st); }, "lb_pair");
 }
 
 // Per-site predictor and corrector; with the three-constant energy each is
@@ -884,9 +885,14 @@ struct BatchGraph {
 // stepped alone before) launch directly.
 constexpr size_t kBatchGraphs = 4;
 
-using Channels = std::vector<nh_ctx*>;
+// Channels whose LB steps are launched together.
+struct Channels {
+    std::vector<nh_ctx*> ctxs;
+    bool pairs = false;            // they take two steps per launch (channels_plan) ...
+    std::vector<PairGrid> split;   // ... cut so
+};
 struct BatchPlan {
-    Channels ctxs;                  // the first one counts launches and keeps times
+    Channels all;                   // the first one counts launches and keeps times
     std::vector<Channels> groups;   // of channels that stay in L2 together (batch_groups); empty: none
     std::vector<int64_t> epochs;
     int variant = 0;                // launch shape of the single steps
@@ -929,24 +935,40 @@ void drop_batch_plans(const nh_ctx* c)
 // 119 | 115, FP64 1724 | 1629).
 constexpr double kGroupBytes = 84e6;
 constexpr int kGroupMinSteps = 4;
-bool batch_pair_ok(const Channels& ctxs);
+
+// Pairs where every channel would take them alone.  (Small channels are too few
+// tiles for the march of a pair: 8 to 24 of 32^2 x 16 to 96^2 x 32 sites took
+// 0.035-0.050 ns a site and step in pairs, 0.030 in single steps.)
+void channels_plan(Channels* s)
+{
+    s->pairs = true;
+    for (const nh_ctx* c : s->ctxs) s->pairs = s->pairs && pair_ok(c);
+    if (!s->pairs) return;
+    s->split.resize(s->ctxs.size());
+    std::vector<PairDomain> d;
+    for (const nh_ctx* c : s->ctxs) d.push_back(PairDomain{c->p.nx, c->p.ny, c->p.nz});
+    for (size_t g0 = 0; g0 < d.size(); g0 += kMaxBatch)  // the channels of a launch together
+        pair_plan(&d[g0], (int)std::min<size_t>(kMaxBatch, d.size() - g0), &s->split[g0]);
+}
+
 void batch_groups(BatchPlan* b)
 {
     double total = 0;
     std::vector<double> bytes;
-    for (const nh_ctx* c : b->ctxs) {
+    for (const nh_ctx* c : b->all.ctxs) {
         const double reals = c->p.precision == NH_FP64 ? 8 : 4;
         bytes.push_back((2 * 19 * (double)store_size(c->p) + 3 * reals) * (double)c->N);
         total += bytes.back();
     }
     const int groups = (int)std::ceil(total / kGroupBytes);
-    if (b->ctxs[0]->p.storage != NH_STORE_F32 || groups < 2 || b->ctxs.size() < 2 || batch_pair_ok(b->ctxs)) return;
+    if (b->all.ctxs[0]->p.storage != NH_STORE_F32 || groups < 2 || b->all.ctxs.size() < 2 || b->all.pairs) return;
     double sum = 0;  // cut where the running sum passes an even share
-    for (size_t k = 0; k < b->ctxs.size(); ++k) {
+    for (size_t k = 0; k < b->all.ctxs.size(); ++k) {
         if (b->groups.empty() || sum + 0.5 * bytes[k] > total * (double)b->groups.size() / groups) b->groups.emplace_back();
-        b->groups.back().push_back(b->ctxs[k]);
+        b->groups.back().ctxs.push_back(b->all.ctxs[k]);
         sum += bytes[k];
     }
+    for (Channels& g : b->groups) channels_plan(&g);
 }
 
 // Validate a batch and find (or build) its plan.
@@ -987,7 +1009,7 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
     if (!plan) {
         plan = new (std::nothrow) BatchPlan();
         if (!plan) return fail(nullptr, NH_ENOMEM, "host allocation of the batch plan failed");
-        plan->ctxs = key;
+        plan->all.ctxs = key;
         plan->epochs = epochs;
         // ctxs[0]'s shape if it was set and fits every channel (the row-staged one runs single channels only),
         // else the default of the batch's channels taken as one domain
@@ -1003,6 +1025,7 @@ int batch_prepare(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, BatchPlan*
         if (!fits(v)) v = 2;
         if (!fits(v)) v = 1;  // one site per thread fits every domain
         plan->variant = v;
+        channels_plan(&plan->all);
         batch_groups(plan);
     }
     *out = plan;
@@ -1031,20 +1054,20 @@ int batch_prepare_relax(nh_ctx* const* ctxs, int count, int64_t n_fd_steps, Batc
     int r = set_device(c0);
     if (r) return fail(nullptr, r, c0->err);
     static thread_local BatchPlan plan;
-    plan.ctxs.assign(ctxs, ctxs + count);
+    plan.all.ctxs.assign(ctxs, ctxs + count);
     *out = &plan;
     return NH_OK;
 }
 
 template <typename Real, typename Store>
-int batch_lb_typed(const BatchPlan* b, const Channels& ctxs, bool write_macro, cudaStream_t st)
+int batch_lb_typed(const BatchPlan* b, const Channels& s, bool write_macro, cudaStream_t st)
 {
-    nh_ctx* c0 = b->ctxs[0];
-    const int n = (int)ctxs.size();
+    nh_ctx* c0 = b->all.ctxs[0];
+    const int n = (int)s.ctxs.size();
     static thread_local LBBatch<Real, Store> batch;  // large parameter block, kept off the stack
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
         batch.count = std::min(kMaxBatch, n - g0);
-        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<Real, Store>(ctxs[g0 + k], ctxs[g0 + k]->cur);
+        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<Real, Store>(s.ctxs[g0 + k], s.ctxs[g0 + k]->cur);
         const int grid = 8 * c0->sm_count;
         int r = timed(c0, NH_KCLASS_LB, st,
                       [&] { return launch_lb_batch(batch, c0->p.shifted != 0, write_macro, b->variant, grid, st); },
@@ -1055,26 +1078,26 @@ int batch_lb_typed(const BatchPlan* b, const Channels& ctxs, bool write_macro, c
 }
 
 // One LB step of these channels of the batch, with the batch's launch shape.
-int batch_enqueue_lb(const BatchPlan* b, const Channels& ctxs, bool write_macro, cudaStream_t st)
+int batch_enqueue_lb(const BatchPlan* b, const Channels& s, bool write_macro, cudaStream_t st)
 {
-    switch (b->ctxs[0]->p.storage) {
-    case NH_STORE_F64: return batch_lb_typed<double, double>(b, ctxs, write_macro, st);
-    case NH_STORE_F32: return batch_lb_typed<float, float>(b, ctxs, write_macro, st);
-    case NH_STORE_F16S: return batch_lb_typed<float, __half>(b, ctxs, write_macro, st);
-    default: return batch_lb_typed<float, __nv_bfloat16>(b, ctxs, write_macro, st);
+    switch (b->all.ctxs[0]->p.storage) {
+    case NH_STORE_F64: return batch_lb_typed<double, double>(b, s, write_macro, st);
+    case NH_STORE_F32: return batch_lb_typed<float, float>(b, s, write_macro, st);
+    case NH_STORE_F16S: return batch_lb_typed<float, __half>(b, s, write_macro, st);
+    default: return batch_lb_typed<float, __nv_bfloat16>(b, s, write_macro, st);
     }
 }
 
 template <typename Real>
 int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
 {
-    nh_ctx* c0 = b->ctxs[0];
-    const int n = (int)b->ctxs.size();
+    nh_ctx* c0 = b->all.ctxs[0];
+    const int n = (int)b->all.ctxs.size();
     static thread_local FDBatch<Real> batch;
     // the fused kernels only when every channel runs on them (not the three-constant energy, lap_wide or
     // n_from_rate, nor a channel set to the per-site kernels)
     bool fused = true, frank3 = false;
-    for (nh_ctx* c : b->ctxs) {
+    for (nh_ctx* c : b->all.ctxs) {
         fused = fused && fd_fused(c);
         frank3 = frank3 || c->p.frank3;
     }
@@ -1084,7 +1107,7 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
         for (int k = 0; k < 2; ++k) {
             for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
                 batch.count = std::min(kMaxBatch, n - g0);
-                for (int j = 0; j < batch.count; ++j) batch.ch[j] = fd_chan<Real>(b->ctxs[g0 + j]);
+                for (int j = 0; j < batch.count; ++j) batch.ch[j] = fd_chan<Real>(b->all.ctxs[g0 + j]);
                 const int grid = 8 * c0->sm_count;
                 int r = timed(c0, classes[k], st, [&] { return launch_fd_fused_batch(batch, fstages[k], grid, st); },
                               "fd_fused_batch");
@@ -1102,7 +1125,7 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
             const int kernel_stage = pass == 0 ? pre : stage;
             for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
                 batch.count = std::min(kMaxBatch, n - g0);
-                for (int k = 0; k < batch.count; ++k) batch.ch[k] = fd_chan<Real>(b->ctxs[g0 + k]);
+                for (int k = 0; k < batch.count; ++k) batch.ch[k] = fd_chan<Real>(b->all.ctxs[g0 + k]);
                 const int grid = 8 * c0->sm_count;
                 int r = timed(c0, classes[stage], st, [&] { return launch_fd_batch(batch, kernel_stage, grid, st); },
                               "fd_batch");
@@ -1119,13 +1142,13 @@ int batch_fd_typed(BatchPlan* b, cudaStream_t st, int stages = 4)
 template <typename Real>
 int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
 {
-    nh_ctx* c0 = b->ctxs[0];
-    const int n = (int)b->ctxs.size();
+    nh_ctx* c0 = b->all.ctxs[0];
+    const int n = (int)b->all.ctxs.size();
     static thread_local FDBatch<Real> batch;
     bool fused = true;
-    for (nh_ctx* c : b->ctxs) fused = fused && relax_fused_ok(c);
+    for (nh_ctx* c : b->all.ctxs) fused = fused && relax_fused_ok(c);
     if (!fused) {
-        for (nh_ctx* c : b->ctxs)
+        for (nh_ctx* c : b->all.ctxs)
             if (cudaMemsetAsync(c->ws + c->L.u, 0, 3 * (size_t)c->N * sizeof(Real), st) != cudaSuccess)
                 return fail(c0, NH_ECUDA, "clearing u");
         for (int64_t k = 0; k < steps; ++k) {
@@ -1137,7 +1160,7 @@ int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
     const int grid = 8 * c0->sm_count;
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {  // channels are independent: group by group
         batch.count = std::min(kMaxBatch, n - g0);
-        for (int j = 0; j < batch.count; ++j) batch.ch[j] = fd_chan<Real>(b->ctxs[g0 + j]);
+        for (int j = 0; j < batch.count; ++j) batch.ch[j] = fd_chan<Real>(b->all.ctxs[g0 + j]);
         for (int64_t k = 0; k < steps; ++k) {
             int r = timed(c0, NH_KCLASS_FD_PREDICT, st,
                           [&] { return launch_fd_fused_batch(batch, (k & 1) ? 3 : 2, grid, st); }, "relax_batch");
@@ -1150,26 +1173,16 @@ int batch_relax_typed(BatchPlan* b, int64_t steps, cudaStream_t st)
     return NH_OK;
 }
 
-// Pairs where every channel would take them alone.  (Small channels are too few
-// tiles for the march of a pair: 8 to 24 of 32^2 x 16 to 96^2 x 32 sites took
-// 0.035-0.050 ns a site and step in pairs, 0.030 in single steps.)
-bool batch_pair_ok(const Channels& ctxs)
+int batch_enqueue_lb_pair(const BatchPlan* b, const Channels& s, bool write_macro, cudaStream_t st)
 {
-    for (const nh_ctx* c : ctxs)
-        if (!pair_fits(c) || !lb_pair_pays((double)c->N)) return false;
-    return true;
-}
-
-int batch_enqueue_lb_pair(const BatchPlan* b, const Channels& ctxs, bool write_macro, cudaStream_t st)
-{
-    nh_ctx* c0 = b->ctxs[0];
-    const int n = (int)ctxs.size();
+    nh_ctx* c0 = b->all.ctxs[0];
+    const int n = (int)s.ctxs.size();
     static thread_local LBBatch<float, float> batch;
     for (int g0 = 0; g0 < n; g0 += kMaxBatch) {
         batch.count = std::min(kMaxBatch, n - g0);
-        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<float, float>(ctxs[g0 + k], ctxs[g0 + k]->cur);
+        for (int k = 0; k < batch.count; ++k) batch.ch[k] = lb_chan<float, float>(s.ctxs[g0 + k], s.ctxs[g0 + k]->cur);
         int r = timed(c0, NH_KCLASS_LB, st,
-                      [&] { return launch_lb_pair_batch(batch, c0->p.shifted != 0, write_macro, st); }, "lb_pair_batch");
+                      [&] { return launch_lb_pair_batch(batch, &s.split[g0], c0->p.shifted != 0, write_macro, st); }, "lb_pair_batch");
         if (r) return r;
     }
     return NH_OK;
@@ -1178,15 +1191,15 @@ int batch_enqueue_lb_pair(const BatchPlan* b, const Channels& ctxs, bool write_m
 // The next batched LB step, or two in one launch (as enqueue_next), of these
 // channels of the batch (all of them, or a group); left: steps up to the end of the
 // call or block.
-int batch_next(const BatchPlan* b, const Channels& ctxs, int64_t left, bool ends_call, cudaStream_t st, int64_t* done)
+int batch_next(const BatchPlan* b, const Channels& s, int64_t left, bool ends_call, cudaStream_t st, int64_t* done)
 {
-    const nh_ctx* c0 = ctxs[0];
+    const nh_ctx* c0 = s.ctxs[0];
     const int dt = c0->p.dt_fd;
-    *done = left >= 2 && (c0->step + 1) % dt != 0 && batch_pair_ok(ctxs) ? 2 : 1;
+    *done = left >= 2 && (c0->step + 1) % dt != 0 && s.pairs ? 2 : 1;
     const bool fd = (c0->step + *done) % dt == 0, macro = fd || (ends_call && left == *done);
-    int r = *done == 2 ? batch_enqueue_lb_pair(b, ctxs, macro, st) : batch_enqueue_lb(b, ctxs, macro, st);
+    int r = *done == 2 ? batch_enqueue_lb_pair(b, s, macro, st) : batch_enqueue_lb(b, s, macro, st);
     if (r) return r;
-    for (nh_ctx* c : ctxs) {
+    for (nh_ctx* c : s.ctxs) {
         c->cur ^= 1;
         c->phase ^= *done & 1;
         c->step += *done;
@@ -1203,18 +1216,18 @@ bool batch_grouped(const BatchPlan* b, int64_t steps) { return !b->groups.empty(
 // channels (which small groups would leave short of blocks).
 int batch_block(BatchPlan* b, int64_t steps, bool ends_call, cudaStream_t st)
 {
-    auto run = [&](const Channels& ctxs) {
+    auto run = [&](const Channels& s) {
         int r = NH_OK;
         for (int64_t left = steps, done = 0; left > 0 && r == NH_OK; left -= done)
-            r = batch_next(b, ctxs, left, ends_call, st, &done);
+            r = batch_next(b, s, left, ends_call, st, &done);
         return r;
     };
     int r = NH_OK;
     if (batch_grouped(b, steps))
         for (size_t k = 0; k < b->groups.size() && r == NH_OK; ++k) r = run(b->groups[k]);
     else
-        r = run(b->ctxs);
-    const nh_ctx* c0 = b->ctxs[0];
+        r = run(b->all);
+    const nh_ctx* c0 = b->all.ctxs[0];
     if (r || c0->step % c0->p.dt_fd != 0) return r;
     return c0->p.precision == NH_FP64 ? batch_fd_typed<double>(b, st) : batch_fd_typed<float>(b, st);
 }
@@ -1222,11 +1235,11 @@ int batch_block(BatchPlan* b, int64_t steps, bool ends_call, cudaStream_t st)
 // Capture a whole dt_fd block that starts in the channels' present buffers.
 int batch_capture(BatchPlan* b)
 {
-    nh_ctx* c0 = b->ctxs[0];
+    nh_ctx* c0 = b->all.ctxs[0];
     BatchGraph g;
     std::vector<int> phase;
     std::vector<int64_t> step;
-    for (nh_ctx* c : b->ctxs) {
+    for (nh_ctx* c : b->all.ctxs) {
         g.start.push_back(c->cur);
         phase.push_back(c->phase);
         step.push_back(c->step);
@@ -1249,11 +1262,11 @@ int batch_capture(BatchPlan* b)
     }
     g.kernels = c0->launches - saved_launches;
     c0->launches = saved_launches;
-    for (size_t k = 0; k < b->ctxs.size(); ++k) {
-        g.end.push_back(b->ctxs[k]->cur);
-        b->ctxs[k]->cur = g.start[k];
-        b->ctxs[k]->phase = phase[k];
-        b->ctxs[k]->step = step[k];
+    for (size_t k = 0; k < b->all.ctxs.size(); ++k) {
+        g.end.push_back(b->all.ctxs[k]->cur);
+        b->all.ctxs[k]->cur = g.start[k];
+        b->all.ctxs[k]->phase = phase[k];
+        b->all.ctxs[k]->step = step[k];
     }
     if (r == NH_OK) b->graphs.push_back(std::move(g));
     return r;
@@ -1266,7 +1279,7 @@ int batch_graph(BatchPlan* b, const BatchGraph** out)
     *out = nullptr;
     for (const BatchGraph& g : b->graphs) {
         bool same = true;
-        for (size_t k = 0; k < b->ctxs.size(); ++k) same = same && b->ctxs[k]->cur == g.start[k];
+        for (size_t k = 0; k < b->all.ctxs.size(); ++k) same = same && b->all.ctxs[k]->cur == g.start[k];
         if (same) *out = &g;
     }
     if (*out || b->graphs.size() == kBatchGraphs) return NH_OK;
@@ -1520,6 +1533,11 @@ int nh_create(const nh_params* p, void* cuda_stream, nh_ctx** out)
     c->p = *p;
     c->N = p->nx * p->ny * p->nz;
     c->lb_variant = lb_default_variant(p->nx, p->ny, p->nz, (int)store_size(*p));
+    if (p->storage == NH_STORE_F32) {
+        const PairDomain d{p->nx, p->ny, p->nz};
+        pair_plan(&d, 1, &c->pair);
+        c->pairs = pair_pays(d) && pair_offsets_fit(d) && pair_partials_fit(d, c->pair);
+    }
     // the three-constant correction, the wide Laplacian and N from the rate run on the per-site FD kernels
     if (p->frank3 || p->lap_wide || p->n_from_rate) c->fd_variant = 0;
     c->L = make_layout(*p);
@@ -1842,8 +1860,8 @@ int nh_batch_step(nh_ctx* const* ctxs, int count, int64_t n_lb_steps, void* stre
             cudaError_t e = cudaGraphLaunch(graph->exec, st);
             if (e != cudaSuccess) return fail(nullptr, NH_ECUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
             c0->launches += graph->kernels;
-            for (size_t k = 0; k < plan->ctxs.size(); ++k) {
-                nh_ctx* c = plan->ctxs[k];
+            for (size_t k = 0; k < plan->all.ctxs.size(); ++k) {
+                nh_ctx* c = plan->all.ctxs[k];
                 c->cur = graph->end[k];
                 c->phase ^= dt & 1;
                 c->step += dt;
@@ -1876,8 +1894,8 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
     std::vector<Channels> sets;
     if (batch_grouped(plan, c0->p.dt_fd))
         for (const Channels& g : plan->groups)
-            if (!batch_pair_ok(g)) sets.push_back(g);
-    if (sets.empty()) sets.push_back(plan->ctxs);
+            if (!g.pairs) sets.push_back(g);
+    if (sets.empty()) sets.push_back(plan->all);
     // streams the current buffers into the others, no swap
     auto trial = [&](int reps) {
         int e = NH_OK;
@@ -1891,7 +1909,7 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
     int best = saved;
     for (int v = 0; v < kLBVariantCount && r == NH_OK; ++v) {
         bool ok = true;
-        for (nh_ctx* c : plan->ctxs) ok = ok && lb_variant_valid(v, c->p.nx);
+        for (nh_ctx* c : plan->all.ctxs) ok = ok && lb_variant_valid(v, c->p.nx);
         if (!ok) continue;
         plan->variant = v;
         r = trial(1);
@@ -1951,7 +1969,7 @@ int nh_batch_relax(nh_ctx* const* ctxs, int count, int64_t n_fd_steps, void* str
     if (r) return r;
     nh_ctx* c0 = ctxs[0];
     cudaStream_t st = pick(c0, stream);
-    for (nh_ctx* c : plan->ctxs) {
+    for (nh_ctx* c : plan->all.ctxs) {
         c->lbp_step = -1;  // u is cleared
         c->bdp_step = -1;
     }

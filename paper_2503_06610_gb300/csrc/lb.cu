@@ -938,16 +938,8 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
 // copies of 160 bytes (276 us), two sites a thread on the paired FP32
 // instructions (200 us: half the instructions, but too few warps) and a fourth
 // slot that saves a barrier (193 us) were slower.
-constexpr int kPairTX = 32, kPairTY = 7;
-constexpr int kPairHX = kPairTX + 2, kPairHY = kPairTY + 2, kPairPts = kPairHX * kPairHY;
-constexpr int kPairThreads = (kPairPts + 31) / 32 * 32;
+constexpr int kPairThreads = pair_threads(kPairTY);
 constexpr int kPairSmem = 43 * kPairPts * (int)sizeof(float);
-constexpr int kPairPerSM = 2;
-
-struct PairGrid {
-    int tx, ty, rows, zc, chunks;  // tiles in x and y, rows of a tile, layers per chunk, chunks
-};
-__host__ __device__ __forceinline__ int pair_blocks(const PairGrid& p) { return p.tx * p.ty * p.chunks; }
 
 __device__ __forceinline__ float ld_byte(const float* base, unsigned off)
 {
@@ -1111,45 +1103,6 @@ __global__ void __launch_bounds__(kPairThreads, kPairPerSM) lb_pair_batch_kernel
     lb_pair_tile<Shifted, Macro>(b.ch[lo], pb.pg[lo], t - b.prefix[lo], b.prefix[lo + 1] - b.prefix[lo]);
 }
 
-// Rows of a tile and layers per chunk: the blocks run in waves of two per SM, and
-// a block takes (layers + 2) x (points of a layer); the split with the least sum
-// (256x256x64: 296 blocks of 7 rows and 64 layers).
-PairGrid pair_split(const Geom& g, int rows, int chunks)
-{
-    PairGrid p{(g.nx + kPairTX - 1) / kPairTX, (g.ny + rows - 1) / rows, rows, (g.nz + chunks - 1) / chunks, 0};
-    p.chunks = (g.nz + p.zc - 1) / p.zc;
-    return p;
-}
-PairGrid pair_grid(const Geom& g)
-{
-    constexpr int kSlots = kPairPerSM * 152;
-    PairGrid best = pair_split(g, kPairTY, 1);
-    long long cost = -1;
-    for (int rows = kPairTY; rows >= 4; --rows)
-        for (int n = 1; n <= g.nz && n <= 64; ++n) {
-            const PairGrid p = pair_split(g, rows, n);
-            const long long w = (long long)((pair_blocks(p) + kSlots - 1) / kSlots) * (p.zc + 2) * (rows + 2);
-            if (cost < 0 || w < cost) {
-                cost = w;
-                best = p;
-            }
-        }
-    return best;
-}
-
-// From 7.5e5 sites, where the two population buffers no longer stay in L2 (16 LB
-// steps and an FD update, single steps | pairs, us: 128x128x32 195 | 218,
-// 160x128x32 275 | 288, 128x128x48 337 | 323, 256x256x12 343 | 315, 180x140x32 355 |
-// 355, 151x117x45 407 | 349, 256x256x64 1815 | 1446).
-constexpr double kPairMinSites = 7.5e5;
-bool lb_pair_pays(double sites) { return sites >= kPairMinSites; }
-// 32-bit byte offsets within the populations; no more blocks than the diagnostics' partials have room for
-bool lb_pair_valid(const Geom& g)
-{
-    return 19.0 * 4.0 * g.N < 4294967296.0 && pair_blocks(pair_grid(g)) <= (g.N + 127) / 128;
-}
-int lb_pair_blocks(const Geom& g) { return pair_blocks(pair_grid(g)); }
-
 namespace {
 
 template <bool Shifted, int Macro>
@@ -1180,7 +1133,7 @@ cudaError_t prepare_pair()
 template <bool Shifted>
 void launch_pair(const LBChan<float, float>& c, const PairGrid& pg, int macro, cudaStream_t st)
 {
-    const int blocks = pair_blocks(pg), threads = (kPairHX * (pg.rows + 2) + 31) / 32 * 32;
+    const int blocks = pair_blocks(pg), threads = pair_threads(pg.rows);
     if (macro == 0)
         launch_step_kernel(lb_pair_kernel<Shifted, 0>, blocks, threads, kPairSmem, st, c, pg);
     else if (macro == 1)
@@ -1191,20 +1144,21 @@ void launch_pair(const LBChan<float, float>& c, const PairGrid& pg, int macro, c
 
 }  // namespace
 
-cudaError_t launch_lb_pair(const LBChan<float, float>& c, bool shifted, bool write_macro, cudaStream_t st)
+cudaError_t launch_lb_pair(const LBChan<float, float>& c, const PairGrid& pg, bool shifted, bool write_macro, cudaStream_t st)
 {
-    if (c.solid != nullptr || c.Fu != nullptr || !lb_pair_valid(c.g)) return cudaErrorInvalidValue;
+    if (c.solid != nullptr || c.Fu != nullptr || !pair_offsets_fit(pair_domain(c.g))) return cudaErrorInvalidValue;
+    if (c.part != nullptr && !pair_partials_fit(pair_domain(c.g), pg)) return cudaErrorInvalidValue;
     cudaError_t e = prepare_pair();
     if (e != cudaSuccess) return e;
     const int macro = write_macro ? (c.part != nullptr ? 2 : 1) : 0;
     if (shifted)
-        launch_pair<true>(c, pair_grid(c.g), macro, st);
+        launch_pair<true>(c, pg, macro, st);
     else
-        launch_pair<false>(c, pair_grid(c.g), macro, st);
+        launch_pair<false>(c, pg, macro, st);
     return cudaGetLastError();
 }
 
-cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, bool shifted, bool write_macro, cudaStream_t st)
+cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, const PairGrid* pg, bool shifted, bool write_macro, cudaStream_t st)
 {
     if (b.count < 1 || b.count > kMaxBatch) return cudaErrorInvalidValue;
     cudaError_t e = prepare_pair();
@@ -1212,11 +1166,12 @@ cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, bool shifted, bool wr
     PairGridBatch pb;
     b.prefix[0] = 0;
     for (int k = 0; k < b.count; ++k) {
-        if (b.ch[k].solid != nullptr || !lb_pair_valid(b.ch[k].g)) return cudaErrorInvalidValue;
-        pb.pg[k] = pair_split(b.ch[k].g, kPairTY, b.count >= 8 ? 1 : (b.ch[k].g.nz + 15) / 16);
+        if (b.ch[k].solid != nullptr || !pair_offsets_fit(pair_domain(b.ch[k].g)) || pg[k].rows != pg[0].rows)
+            return cudaErrorInvalidValue;
+        pb.pg[k] = pg[k];
         b.prefix[k + 1] = b.prefix[k] + pair_blocks(pb.pg[k]);
     }
-    auto go = [&](auto kernel) { launch_step_kernel(kernel, b.prefix[b.count], kPairThreads, kPairSmem, st, b, pb); };
+    auto go = [&](auto kernel) { launch_step_kernel(kernel, b.prefix[b.count], pair_threads(pg[0].rows), kPairSmem, st, b, pb); };
     if (shifted)
         write_macro ? go(lb_pair_batch_kernel<true, 1>) : go(lb_pair_batch_kernel<true, 0>);
     else

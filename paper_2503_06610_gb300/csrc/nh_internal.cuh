@@ -12,6 +12,7 @@
 
 #include "../../include/nh.h"
 #include "once_per_device.h"
+#include "pair_plan.h"
 
 namespace nh {
 
@@ -259,12 +260,11 @@ int lb_blocks(int variant, int N);  // thread blocks of one LB launch of that sh
 template <typename Real, typename Store>
 cudaError_t launch_lb(const LBChan<Real, Store>& c, bool shifted, bool write_macro, int variant, cudaStream_t s);
 
-// Two LB steps in one pass (FP32 stores, no obstacles, one force): fsrc -> fdst.
-bool lb_pair_valid(const Geom& g);
-bool lb_pair_pays(double sites);  // for a channel, or the channels of a batch together
-int lb_pair_blocks(const Geom& g);  // thread blocks (and diagnostics partials) of one such launch
-cudaError_t launch_lb_pair(const LBChan<float, float>& c, bool shifted, bool write_macro, cudaStream_t s);
-cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, bool shifted, bool write_macro, cudaStream_t s);
+// Two LB steps in one pass (FP32 stores, no obstacles, one force): fsrc -> fdst,
+// cut as pair_plan says; the channels of a batch have been planned together.
+inline PairDomain pair_domain(const Geom& g) { return PairDomain{g.nx, g.ny, g.nz}; }
+cudaError_t launch_lb_pair(const LBChan<float, float>& c, const PairGrid& pg, bool shifted, bool write_macro, cudaStream_t s);
+cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, const PairGrid* pg, bool shifted, bool write_macro, cudaStream_t s);
 
 // Batched LB sweep over b.count channels with a persistent grid of at most
 // `grid` blocks (fills b.prefix).
