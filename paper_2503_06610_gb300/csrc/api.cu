@@ -1536,7 +1536,7 @@ int nh_create(const nh_params* p, void* cuda_stream, nh_ctx** out)
     if (p->storage == NH_STORE_F32) {
         const PairDomain d{p->nx, p->ny, p->nz};
         pair_plan(&d, 1, &c->pair);
-        c->pairs = pair_pays(d) && pair_offsets_fit(d) && pair_partials_fit(d, c->pair);
+        c->pairs = pair_pays(d, c->pair) && pair_offsets_fit(d) && pair_partials_fit(d, c->pair);
     }
     // the three-constant correction, the wide Laplacian and N from the rate run on the per-site FD kernels
     if (p->frank3 || p->lap_wide || p->n_from_rate) c->fd_variant = 0;

@@ -914,7 +914,8 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
 //
 // At 164 bytes a site and step the FP32 sweep runs at the HBM limit, so a second
 // step has to come from on-chip data.  A block takes a tile of 32 x rows columns
-// (7 rows at most) and marches up its layers.  For every layer it computes the
+// (7 rows at most; other widths in narrow domains, pair_columns) and marches up
+// its layers.  For every layer it computes the
 // first step on the tile and a ring of one site around it, straight from global
 // memory, and keeps the post-collision populations in shared memory; the second
 // step of the layer below then pulls from there and writes global memory: 82
@@ -929,7 +930,7 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
 //
 // Bound by issue (110 M warp instructions a pass at 256x256x64, a quarter of them
 // 64-bit addresses) and by the two barriers a layer.  Two steps at 256x256x64:
-// 155 us, two single steps 200 us.  Seven rows leave 96 registers to each of two
+// 153 us, two single steps 201 us.  Seven rows leave 96 registers to each of two
 // blocks per SM, so that the prefetch does not spill; with eight rows (80
 // registers) it does (181 us), without it a layer waits for its loads (158 us).
 // All tiles march up together, so that what neighbours share is read from HBM
@@ -938,7 +939,7 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
 // copies of 160 bytes (276 us), two sites a thread on the paired FP32
 // instructions (200 us: half the instructions, but too few warps) and a fourth
 // slot that saves a barrier (193 us) were slower.
-constexpr int kPairThreads = pair_threads(kPairTY);
+constexpr int kPairThreads = pair_threads(kPairPts);
 constexpr int kPairSmem = 43 * kPairPts * (int)sizeof(float);
 
 __device__ __forceinline__ float ld_byte(const float* base, unsigned off)
@@ -950,7 +951,8 @@ __device__ __forceinline__ void st_byte(float* base, unsigned off, float v)
     *reinterpret_cast<float*>(reinterpret_cast<char*>(base) + off) = v;
 }
 
-template <bool Shifted, int Macro>
+// Cols: columns of a tile, 0 where only the plan knows them (narrow domains).
+template <bool Shifted, int Macro, int Cols>
 __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, const PairGrid& pg, int tile, int ntiles)
 {
     NH_D3Q19_TABLES
@@ -962,27 +964,15 @@ __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, cons
     float* down = flat + 18 * kPairPts;     // 2 slots x 5: e_z = -1
     const Geom& g = c.g;
     const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N;
-    const int t = tile / pg.tx, rows = pg.rows, nown = kPairTX * rows;
-    const int x0 = (tile - t * pg.tx) * kPairTX, y0 = (t % pg.ty) * rows;
+    const int cols = Cols > 0 ? Cols : pg.cols, hw = cols + 2;
+    const int t = tile / pg.tx, rows = pg.rows;
+    const int x0 = (tile - t * pg.tx) * cols, y0 = (t % pg.ty) * rows;
     const int zb = (t / pg.ty) * pg.zc, ze = min(zb + pg.zc, nz);
     const int tid = threadIdx.x;
-    const bool own = tid < nown, point = tid < kPairHX * (rows + 2);
-    int hx, hy;  // the thread's point in the tile with its ring: own points first, then two rows, then two columns
-    if (own) {
-        hx = 1 + tid % kPairTX;
-        hy = 1 + tid / kPairTX;
-    } else {
-        const int e = tid - nown;
-        if (e < 2 * kPairHX) {
-            hy = e < kPairHX ? 0 : rows + 1;
-            hx = e < kPairHX ? e : e - kPairHX;
-        } else {
-            const int j = e - 2 * kPairHX;
-            hy = min(1 + (j >> 1), rows);
-            hx = (j & 1) ? kPairHX - 1 : 0;
-        }
-    }
-    const int i1 = hx + kPairHX * hy;
+    const bool own = tid < cols * rows, point = tid < pair_points(cols, rows);
+    int hx, hy;  // the thread's point in the tile with its ring
+    pair_place(tid, cols, rows, &hx, &hy);
+    const int i1 = point ? hx + hw * hy : 0;
     const bool active = own && x0 + hx - 1 < nx && y0 + hy - 1 < ny;
     // wrapped coordinates of the point (a ragged tile's outer points repeat inner ones) and, in bytes, the
     // x and row parts of its neighbours' places in a plane
@@ -1044,7 +1034,7 @@ __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, cons
                                    up + s2 * (5 * kPairPts) + i1};
             if (!g.walls || (z > 0 && z < nz - 1)) {
 #pragma unroll
-                for (int i = 0; i < 19; ++i) h[i] = src[1 + EZ[i]][GI[i] * kPairPts - EX[i] - kPairHX * EY[i]];
+                for (int i = 0; i < 19; ++i) h[i] = src[1 + EZ[i]][GI[i] * kPairPts - EX[i] - hw * EY[i]];
             } else {  // half-way bounce-back: the site's own opposite populations
                 const float* low = down + (z & 1) * (5 * kPairPts) + i1;
                 const float* high = up + s1 * (5 * kPairPts) + i1;
@@ -1056,7 +1046,7 @@ __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, cons
                     else if (EZ[i] < 0 && z == nz - 1)
                         h[i] = high[back];
                     else
-                        h[i] = src[1 + EZ[i]][GI[i] * kPairPts - EX[i] - kPairHX * EY[i]];
+                        h[i] = src[1 + EZ[i]][GI[i] * kPairPts - EX[i] - hw * EY[i]];
                 }
             }
         }
@@ -1076,18 +1066,18 @@ __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, cons
     if constexpr (Macro == 2) lb_block_partials(psum, pmax, pbad, c.part, tile, ntiles);
 }
 
-template <bool Shifted, int Macro>
+template <bool Shifted, int Macro, int Cols>
 __global__ void __launch_bounds__(kPairThreads, kPairPerSM) lb_pair_kernel(const LBChan<float, float> c, const PairGrid pg)
 {
     step_kernel_enter();
-    lb_pair_tile<Shifted, Macro>(c, pg, blockIdx.x, gridDim.x);
+    lb_pair_tile<Shifted, Macro, Cols>(c, pg, blockIdx.x, gridDim.x);
 }
 
 // Batch: one tile of one channel per block.
 struct PairGridBatch {
     PairGrid pg[kMaxBatch];
 };
-template <bool Shifted, int Macro>
+template <bool Shifted, int Macro, int Cols>
 __global__ void __launch_bounds__(kPairThreads, kPairPerSM) lb_pair_batch_kernel(const LBBatch<float, float> b, const PairGridBatch pb)
 {
     step_kernel_enter();
@@ -1100,61 +1090,78 @@ __global__ void __launch_bounds__(kPairThreads, kPairPerSM) lb_pair_batch_kernel
         else
             hi = mid - 1;
     }
-    lb_pair_tile<Shifted, Macro>(b.ch[lo], pb.pg[lo], t - b.prefix[lo], b.prefix[lo + 1] - b.prefix[lo]);
+    lb_pair_tile<Shifted, Macro, Cols>(b.ch[lo], pb.pg[lo], t - b.prefix[lo], b.prefix[lo + 1] - b.prefix[lo]);
 }
 
 namespace {
 
-template <bool Shifted, int Macro>
+template <bool Shifted, int Macro, int Cols>
 cudaError_t pair_attr()
 {
-    cudaError_t e = cudaFuncSetAttribute(lb_pair_kernel<Shifted, Macro>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kPairSmem);
+    const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(lb_pair_kernel<Shifted, Macro, Cols>, attr, kPairSmem);
     if constexpr (Macro < 2)
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(lb_pair_batch_kernel<Shifted, Macro>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kPairSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(lb_pair_batch_kernel<Shifted, Macro, Cols>, attr, kPairSmem);
+    return e;
+}
+template <int Cols>
+cudaError_t pair_attrs()
+{
+    cudaError_t e = pair_attr<true, 0, Cols>();
+    if (e == cudaSuccess) e = pair_attr<true, 1, Cols>();
+    if (e == cudaSuccess) e = pair_attr<true, 2, Cols>();
+    if (e == cudaSuccess) e = pair_attr<false, 0, Cols>();
+    if (e == cudaSuccess) e = pair_attr<false, 1, Cols>();
+    if (e == cudaSuccess) e = pair_attr<false, 2, Cols>();
     return e;
 }
 cudaError_t prepare_pair()
 {
     static OncePerDevice once;
     return once_per_device(once, [] {
-        cudaError_t e = pair_attr<true, 0>();
-        if (e == cudaSuccess) e = pair_attr<true, 1>();
-        if (e == cudaSuccess) e = pair_attr<true, 2>();
-        if (e == cudaSuccess) e = pair_attr<false, 0>();
-        if (e == cudaSuccess) e = pair_attr<false, 1>();
-        if (e == cudaSuccess) e = pair_attr<false, 2>();
-        return e;
+        const cudaError_t e = pair_attrs<kPairTX>();
+        return e == cudaSuccess ? pair_attrs<0>() : e;
     });
 }
 
-template <bool Shifted>
+template <bool Shifted, int Cols>
 void launch_pair(const LBChan<float, float>& c, const PairGrid& pg, int macro, cudaStream_t st)
 {
-    const int blocks = pair_blocks(pg), threads = pair_threads(pg.rows);
+    const int blocks = pair_blocks(pg), threads = pair_threads(pair_points(pg.cols, pg.rows));
     if (macro == 0)
-        launch_step_kernel(lb_pair_kernel<Shifted, 0>, blocks, threads, kPairSmem, st, c, pg);
+        launch_step_kernel(lb_pair_kernel<Shifted, 0, Cols>, blocks, threads, kPairSmem, st, c, pg);
     else if (macro == 1)
-        launch_step_kernel(lb_pair_kernel<Shifted, 1>, blocks, threads, kPairSmem, st, c, pg);
+        launch_step_kernel(lb_pair_kernel<Shifted, 1, Cols>, blocks, threads, kPairSmem, st, c, pg);
     else
-        launch_step_kernel(lb_pair_kernel<Shifted, 2>, blocks, threads, kPairSmem, st, c, pg);
+        launch_step_kernel(lb_pair_kernel<Shifted, 2, Cols>, blocks, threads, kPairSmem, st, c, pg);
 }
+
+template <bool Shifted, int Cols>
+void launch_pair_batch(const LBBatch<float, float>& b, const PairGridBatch& pb, int threads, bool write_macro, cudaStream_t st)
+{
+    const int blocks = b.prefix[b.count];
+    if (write_macro)
+        launch_step_kernel(lb_pair_batch_kernel<Shifted, 1, Cols>, blocks, threads, kPairSmem, st, b, pb);
+    else
+        launch_step_kernel(lb_pair_batch_kernel<Shifted, 0, Cols>, blocks, threads, kPairSmem, st, b, pb);
+}
+
+bool pair_fits_block(const PairGrid& p) { return p.cols >= 1 && p.rows >= 1 && pair_points(p.cols, p.rows) <= kPairPts; }
 
 }  // namespace
 
 cudaError_t launch_lb_pair(const LBChan<float, float>& c, const PairGrid& pg, bool shifted, bool write_macro, cudaStream_t st)
 {
-    if (c.solid != nullptr || c.Fu != nullptr || !pair_offsets_fit(pair_domain(c.g))) return cudaErrorInvalidValue;
-    if (c.part != nullptr && !pair_partials_fit(pair_domain(c.g), pg)) return cudaErrorInvalidValue;
+    const PairDomain d = pair_domain(c.g);
+    if (c.solid != nullptr || c.Fu != nullptr || !pair_offsets_fit(d) || !pair_fits_block(pg)) return cudaErrorInvalidValue;
+    if (c.part != nullptr && !pair_partials_fit(d, pg)) return cudaErrorInvalidValue;
     cudaError_t e = prepare_pair();
     if (e != cudaSuccess) return e;
     const int macro = write_macro ? (c.part != nullptr ? 2 : 1) : 0;
-    if (shifted)
-        launch_pair<true>(c, pg, macro, st);
+    if (pg.cols == kPairTX)
+        shifted ? launch_pair<true, kPairTX>(c, pg, macro, st) : launch_pair<false, kPairTX>(c, pg, macro, st);
     else
-        launch_pair<false>(c, pg, macro, st);
+        shifted ? launch_pair<true, 0>(c, pg, macro, st) : launch_pair<false, 0>(c, pg, macro, st);
     return cudaGetLastError();
 }
 
@@ -1164,18 +1171,23 @@ cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, const PairGrid* pg, b
     cudaError_t e = prepare_pair();
     if (e != cudaSuccess) return e;
     PairGridBatch pb;
+    int threads = 0;
+    bool columns = true;  // of the width that the kernel has at compile time
     b.prefix[0] = 0;
     for (int k = 0; k < b.count; ++k) {
-        if (b.ch[k].solid != nullptr || !pair_offsets_fit(pair_domain(b.ch[k].g)) || pg[k].rows != pg[0].rows)
+        if (b.ch[k].solid != nullptr || !pair_offsets_fit(pair_domain(b.ch[k].g)) || !pair_fits_block(pg[k]))
             return cudaErrorInvalidValue;
         pb.pg[k] = pg[k];
-        b.prefix[k + 1] = b.prefix[k] + pair_blocks(pb.pg[k]);
+        b.prefix[k + 1] = b.prefix[k] + pair_blocks(pg[k]);
+        threads = std::max(threads, pair_threads(pair_points(pg[k].cols, pg[k].rows)));
+        columns = columns && pg[k].cols == kPairTX;
     }
-    auto go = [&](auto kernel) { launch_step_kernel(kernel, b.prefix[b.count], pair_threads(pg[0].rows), kPairSmem, st, b, pb); };
-    if (shifted)
-        write_macro ? go(lb_pair_batch_kernel<true, 1>) : go(lb_pair_batch_kernel<true, 0>);
+    if (columns)
+        shifted ? launch_pair_batch<true, kPairTX>(b, pb, threads, write_macro, st)
+                : launch_pair_batch<false, kPairTX>(b, pb, threads, write_macro, st);
     else
-        write_macro ? go(lb_pair_batch_kernel<false, 1>) : go(lb_pair_batch_kernel<false, 0>);
+        shifted ? launch_pair_batch<true, 0>(b, pb, threads, write_macro, st)
+                : launch_pair_batch<false, 0>(b, pb, threads, write_macro, st);
     return cudaGetLastError();
 }
 
