@@ -102,7 +102,7 @@ struct Dims {
 // neither), so K is a template argument and the descriptors are constants added to
 // two bases: eight cells' forward pass 281 us with K at run time, 242 us so.
 // Every mbarrier wait is bounded: on expiry the kernel raises a.status, skips the
-// epilogue, waits for its copies and frees its TMEM.
+// epilogue, waits (again with a limit) for its copies and MMAs and frees its TMEM.
 //
 // Forward: input = the layer's sources, D + bias, ReLU, BF16 rows.  Data gradient
 // (Flip): input = the pre-activation gradient, taps mirrored, transposed weights.
@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(kTcThreads, NB == 32 && Flip ? 3 : 4) conv_tc_
         const uint32_t lead = lane == 0;
         const uint64_t ad0 = umma_desc(0, kGroup, kTcHX * 16), bd0 = umma_desc(0, 128u, (uint32_t)kb * 128u);
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[4]), 0)) != 0;
+        int issued = 0;  // input planes whose MMAs are under way or done
         // accumulators w, w + 1, w + 2 of the strip: output planes number w - 2, w - 1 and w of the chunk
         for (int w = 0, slot = 0; w < steps && ok; ++w, slot = slot + 1 == a.ring ? 0 : slot + 1) {
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[2 + (w & 1)]), (w >> 1) & 1)) != 0;
@@ -449,6 +450,11 @@ __global__ void __launch_bounds__(kTcThreads, NB == 32 && Flip ? 3 : 4) conv_tc_
                              smem_u32(&bars[w & 1])), "r"(lead)
                          : "memory");
             __syncwarp();
+            issued = w + 1;
+        }
+        if (!ok) {  // nothing of this CTA's may be under way when it leaves: the weights' copy, the last plane's MMAs
+            mbar_wait(smem_u32(&bars[4]), 0);
+            if (issued > 0) mbar_wait(smem_u32(&bars[(issued - 1) & 1]), ((issued - 1) >> 1) & 1);
         }
     } else {
         for (int w = 0; w < steps && ok; ++w) {
