@@ -201,8 +201,9 @@ int nh_restore(nh_ctx* ctx, const double* n, const double* F, const double* u, c
                int64_t step, int on_device);
 
 /* Advance n_lb_steps LB steps (Sec. II.D): every step one fused LB
- * collide-and-stream launch (FP32 stores of 7.5e5 sites or more, without
- * obstacles: two steps per launch where no FD update lies between); after each step whose count s is a multiple of
+ * collide-and-stream launch (FP32 stores of 7.5e5 sites or more in three layers
+ * or more, without obstacles: two steps per launch where no FD update lies
+ * between); after each step whose count s is a multiple of
  * dt_fd, the FD predictor-corrector on n with that step's u, then the LC
  * stress and force.  Asynchronous on stream (NULL = the context's stream).
  * Whole dt_fd blocks of at least 12 steps run from a CUDA graph unless timing is on. */

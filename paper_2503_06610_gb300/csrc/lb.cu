@@ -239,8 +239,8 @@ __device__ __forceinline__ void relax_conserving(const Real (&f)[19], Real (&fo)
     const Real T = mul_rn(w36, S);
     fo[0] = fma_rn(omc, f[0], fma_rn(Real(-24), T, S));
     auto pair = [&](int i, Real even, Real odd) {
-        fo[i] = fma_rn(omc, f[i], even) + odd;
-        fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
+        fo[i] = fma_rn(omc, f[i], even + odd);
+        fo[i + 1] = fma_rn(omc, f[i + 1], even - odd);
     };
     auto axis = [&](int i, Real v, Real g, Real H, Real q) {
         pair(i, mul_rn(Real(2), fma_rn(v, g, T)), fma_rn(Real(-4), q, mul_rn(Real(0.5), H)));
@@ -371,9 +371,9 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
             fo[i + 1] = fma_rn(omc, f[i + 1], even) - odd;
         }
     } else {
-        u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
         relax_conserving(f, fo, sum, fma_rn(Real(0.5), Hx, mx), fma_rn(Real(0.5), Hy, my), fma_rn(Real(0.5), Hz, mz), ux, uy, uz,
                          Fx, Fy, Fz, c.omega);
+        u2 = fma_rn(uz, uz, fma_rn(uy, uy, mul_rn(ux, ux)));
     }
     if (Partials) {  // the sums nh_diagnostics forms from the stored state, site by site
         Real fs = fo[0];
@@ -1193,8 +1193,11 @@ cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, const PairGrid* pg, b
 
 // Batched sweep: a persistent grid walks the (channel, tile) work list of up to
 // kMaxBatch channels; tiles of channel k are [prefix[k], prefix[k+1]).
+// FP32, two sites a thread: 80 registers, three blocks of 256 threads an SM or six of
+// 128; with the 87 that the compiler takes by itself 64 steps of 64 uneven channels
+// take 12.2 ms, with 80 (eight bytes spilled) 11.9.
 template <typename Real, typename Store, bool Shifted, bool WriteMacro, int SPT, bool Solid = false>
-__global__ void __launch_bounds__(kLBThreads) lb_batch_kernel(const LBBatch<Real, Store> b)
+__global__ void __launch_bounds__(kLBThreads, sizeof(Store) == 4 && SPT == 2 ? 3 : 0) lb_batch_kernel(const LBBatch<Real, Store> b)
 {
     step_kernel_enter();
     const int total = b.prefix[b.count];
