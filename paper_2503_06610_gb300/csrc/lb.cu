@@ -211,17 +211,17 @@ __device__ __forceinline__ Real edot(int X, int Y, int Z, Real vx, Real vy, Real
     return r;
 }
 
-// Relaxation of a site with shifted populations, cS = 1 - omega / 2: what lb_collide_site writes out by pairs, in 144
+// Relaxation of a site with shifted populations, cS = 1 - omega / 2: what lb_collide_site writes out by pairs, in 135
 // operations instead of 215 and with rounding errors that conserve mass and momentum.  With the momentum j = rho u,
 // P = cS F, H = omega j + P (the momentum that the step moves) and g = H + P, a direction of weight w takes
 //   omega f^eq + cS S = w [omega (rho - 1) - 1.5 u.g + 4.5 (e.u)(e.g) + 3 e.H],
 // one even and one odd part a pair.  The weights are not numbers of the type: a rounded w puts every x in w x off by
 // the same factor at every site and step, and the errors of u grow with the number of steps.  So only the diagonals
 // take a rounded twelfth of H and, like the axes, a rounded 36th T of the even sum S; the axes take what is left of H
-// (four of their parts and eight of the diagonals' make H), the rest population what is left of S (24 T of it are the
-// others').
-// Error of u after 250 steps, that of the order by pairs (biased too) being 1, FP32 on the CPU: 0.05 at tau 0.55, 0.03
-// at 0.7, 0.01 at 0.8, 0.04 at 1, 0.1 at 1.478, 0.7 at 2.5; FP64, 20 steps, 0.1 to 0.4.  Rounded twelfths and 36ths for
+// (four diagonals and an axis make one: H / 2 less four of the rounded twelfths, exact in either type), the rest
+// population what is left of S (24 T of it are the others').
+// Error of u after 250 steps, that of the order by pairs (biased too) being 1, FP32 on the CPU: 0.05 at tau 0.55, 0.04
+// at 0.7, 0.01 at 0.8, 0.04 at 1, 0.1 at 1.478, 0.8 at 2.5; FP64, 20 steps, 0.1 to 0.4.  Rounded twelfths and 36ths for
 // all directions alike: 2.9 at tau 0.7, and in FP64 5.0 at tau 1.478.
 template <typename Real>
 __device__ __forceinline__ void relax_conserving(const Real (&f)[19], Real (&fo)[19], Real drho, Real jx, Real jy, Real jz,
@@ -231,30 +231,27 @@ __device__ __forceinline__ void relax_conserving(const Real (&f)[19], Real (&fo)
     const Real Px = mul_rn(cS, Fx), Py = mul_rn(cS, Fy), Pz = mul_rn(cS, Fz);
     const Real Hx = fma_rn(omega, jx, Px), Hy = fma_rn(omega, jy, Py), Hz = fma_rn(omega, jz, Pz);
     const Real gx = Hx + Px, gy = Hy + Py, gz = Hz + Pz;
-    constexpr Real w12 = Real(1) / Real(12), w36 = Real(1) / Real(36);
-    const Real qx = mul_rn(w12, Hx), qy = mul_rn(w12, Hy), qz = mul_rn(w12, Hz);
+    constexpr Real w36 = Real(1) / Real(36), w12 = Real(1) / Real(12), axis12 = Real(0.5) - Real(4) * w12;
     const Real vx = mul_rn(Real(0.125), ux), vy = mul_rn(Real(0.125), uy), vz = mul_rn(Real(0.125), uz);
     const Real ug8 = fma_rn(vz, gz, fma_rn(vy, gy, mul_rn(vx, gx)));
     const Real S = fma_rn(omega, drho, mul_rn(Real(-12), ug8));
     const Real T = mul_rn(w36, S);
     fo[0] = fma_rn(omc, f[0], fma_rn(Real(-24), T, S));
-    auto pair = [&](int i, Real even, Real odd) {
-        fo[i] = fma_rn(omc, f[i], even + odd);
-        fo[i + 1] = fma_rn(omc, f[i + 1], even - odd);
+    auto pair = [&](int i, Real w, Real H, Real even) {
+        fo[i] = fma_rn(omc, f[i], fma_rn(w, H, even));
+        fo[i + 1] = fma_rn(omc, f[i + 1], fma_rn(-w, H, even));
     };
-    auto axis = [&](int i, Real v, Real g, Real H, Real q) {
-        pair(i, mul_rn(Real(2), fma_rn(v, g, T)), fma_rn(Real(-4), q, mul_rn(Real(0.5), H)));
-    };
-    auto diagonal = [&](int i, Real v, Real g, Real q) { pair(i, fma_rn(v, g, T), q); };
-    axis(1, vx, gx, Hx, qx);
-    axis(3, vy, gy, Hy, qy);
-    axis(5, vz, gz, Hz, qz);
-    diagonal(7, vx + vy, gx + gy, qx + qy);
-    diagonal(9, vx - vy, gx - gy, qx - qy);
-    diagonal(11, vx + vz, gx + gz, qx + qz);
-    diagonal(13, vx - vz, gx - gz, qx - qz);
-    diagonal(15, vy + vz, gy + gz, qy + qz);
-    diagonal(17, vy - vz, gy - gz, qy - qz);
+    auto axis = [&](int i, Real v, Real g, Real H) { pair(i, axis12, H, mul_rn(Real(2), fma_rn(v, g, T))); };
+    auto diagonal = [&](int i, Real v, Real g, Real H) { pair(i, w12, H, fma_rn(v, g, T)); };
+    axis(1, vx, gx, Hx);
+    axis(3, vy, gy, Hy);
+    axis(5, vz, gz, Hz);
+    diagonal(7, vx + vy, gx + gy, Hx + Hy);
+    diagonal(9, vx - vy, gx - gy, Hx - Hy);
+    diagonal(11, vx + vz, gx + gz, Hx + Hz);
+    diagonal(13, vx - vz, gx - gz, Hx - Hz);
+    diagonal(15, vy + vz, gy + gz, Hy + Hz);
+    diagonal(17, vy - vz, gy - gz, Hy - Hz);
 }
 
 // Moments, equilibrium, Guo source and relaxation of one site s from its
@@ -263,9 +260,11 @@ __device__ __forceinline__ void relax_conserving(const Real (&f)[19], Real (&fo)
 // its liquid-crystal force F_lc = (flx, fly, flz) (the body force rho g is added here), into
 // fo; u and rho written when Macro >= 1, the diagnostics partials accumulated
 // when Macro == 2, the largest |fo| (encoded units) into amax for the 16-bit
-// scale controller.  Every launch shape calls this for every site, and its
-// rounding order is explicit, so all shapes give bit-identical results.
-template <typename Real, typename Store, bool Shifted, int Macro>
+// scale controller.  Stale: c.Fu, if set, is the force that shifts u instead (the
+// printed loop order; never set in batches and pairs).  Every launch shape calls
+// this for every site, and its rounding order is explicit, so all shapes give
+// bit-identical results.
+template <typename Real, typename Store, bool Shifted, int Macro, bool Stale>
 __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, int s, const Real (&f)[19],
                                                 Real (&fo)[19], Real flx, Real fly, Real flz, float inv_in,
                                                 float scale_out, Real& psum, Real& pmax, int& pbad, float& amax)
@@ -315,7 +314,7 @@ __device__ __forceinline__ void lb_collide_site(const LBChan<Real, Store>& c, in
     const Real Fz = fma_rn(rho, c.gz, flz);
     const Real inv_rho = Real(1) / rho;
     Real Hx = Fx, Hy = Fy, Hz = Fz;  // force whose half shifts u
-    if (c.Fu != nullptr) {
+    if (Stale && c.Fu != nullptr) {
         Hx = fma_rn(rho, c.gx, c.Fu[s]);
         Hy = fma_rn(rho, c.gy, c.Fu[N + s]);
         Hz = fma_rn(rho, c.gz, c.Fu[2 * N + s]);
@@ -438,6 +437,9 @@ __device__ __forceinline__ void lb_block_partials(Real m, Real mx, int bad, doub
 template <typename Real, typename Store, bool Shifted, int Macro, int SPT, bool Solid = false, bool OneTile = false>
 __device__ __forceinline__ void lb_tile(const LBChan<Real, Store>& c, int tile, int ntiles)
 {
+    // batches have no stale force; without the test FP32 takes 79 registers instead of 86 (six blocks of 128 threads an
+    // SM instead of five), while the other stores' kernels that write u and rho take more (16-bit 128 -> 162)
+    constexpr bool kStale = OneTile || sizeof(Store) != 4;
     static_assert(!Solid || SPT == 1, "obstacles use one site per thread");
     NH_D3Q19_TABLES
     constexpr bool kScaled = sizeof(Store) == 2;
@@ -562,7 +564,7 @@ __device__ __forceinline__ void lb_tile(const LBChan<Real, Store>& c, int tile, 
         for (int j = 0; j < SPT; ++j) {
             if (solid_here) break;
             const int s = s0 + j;
-            lb_collide_site<Real, Store, Shifted, Macro>(c, s, f[j], fo[j], c.F[s], c.F[N + s], c.F[2 * N + s], inv_in,
+            lb_collide_site<Real, Store, Shifted, Macro, kStale>(c, s, f[j], fo[j], c.F[s], c.F[N + s], c.F[2 * N + s], inv_in,
                                                         scale_out, psum, pmax, pbad, amax);
         }
         if (kScaled) amax /= scale_out;  // back to population units for the controller
@@ -821,7 +823,7 @@ __global__ void __launch_bounds__(kRowMaxNx / kRowSPT, kRowMinBlocks) lb_rows_ke
             const float fx = j == 0 ? fl[0].x : (j == 1 ? fl[0].y : (j == 2 ? fl[0].z : fl[0].w));
             const float fy = j == 0 ? fl[1].x : (j == 1 ? fl[1].y : (j == 2 ? fl[1].z : fl[1].w));
             const float fz = j == 0 ? fl[2].x : (j == 1 ? fl[2].y : (j == 2 ? fl[2].z : fl[2].w));
-            lb_collide_site<Real, Store, Shifted, Macro>(c, s0 + j, f[j], fo[j], fx, fy, fz, inv_in, scale_out, psum,
+            lb_collide_site<Real, Store, Shifted, Macro, true>(c, s0 + j, f[j], fo[j], fx, fy, fz, inv_in, scale_out, psum,
                                                         pmax, pbad, amax);
         }
 #pragma unroll
@@ -1016,7 +1018,7 @@ __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, cons
     for (int p = zb - 1; p <= ze; ++p) {
         if (point && exists(p)) {
             float fo[19];
-            lb_collide_site<float, float, Shifted, 0>(c, 0, f, fo, F[0], F[1], F[2], 1.f, 1.f, none, none, inone, none);
+            lb_collide_site<float, float, Shifted, 0, true>(c, 0, f, fo, F[0], F[1], F[2], 1.f, 1.f, none, none, inone, none);
             float* dst[3] = {down + (p & 1) * (5 * kPairPts) + i1, flat + (p & 1) * (9 * kPairPts) + i1,
                              up + su * (5 * kPairPts) + i1};
 #pragma unroll
@@ -1053,7 +1055,7 @@ __device__ __forceinline__ void lb_pair_tile(const LBChan<float, float>& c, cons
         __syncthreads();  // the slots of planes p - 2 (up) and p - 1 (the others) may be overwritten
         if (second) {
             float ho[19];
-            lb_collide_site<float, float, Shifted, Macro>(c, (int)(here >> 2) + plane * z, h, ho, Fz[0], Fz[1], Fz[2], 1.f,
+            lb_collide_site<float, float, Shifted, Macro, true>(c, (int)(here >> 2) + plane * z, h, ho, Fz[0], Fz[1], Fz[2], 1.f,
                                                           1.f, psum, pmax, pbad, none);
             float* fz = c.fdst + (size_t)plane * z;
 #pragma unroll
@@ -1193,11 +1195,8 @@ cudaError_t launch_lb_pair_batch(LBBatch<float, float>& b, const PairGrid* pg, b
 
 // Batched sweep: a persistent grid walks the (channel, tile) work list of up to
 // kMaxBatch channels; tiles of channel k are [prefix[k], prefix[k+1]).
-// FP32, two sites a thread: 80 registers, three blocks of 256 threads an SM or six of
-// 128; with the 87 that the compiler takes by itself 64 steps of 64 uneven channels
-// take 12.2 ms, with 80 (eight bytes spilled) 11.9.
 template <typename Real, typename Store, bool Shifted, bool WriteMacro, int SPT, bool Solid = false>
-__global__ void __launch_bounds__(kLBThreads, sizeof(Store) == 4 && SPT == 2 ? 3 : 0) lb_batch_kernel(const LBBatch<Real, Store> b)
+__global__ void __launch_bounds__(kLBThreads) lb_batch_kernel(const LBBatch<Real, Store> b)
 {
     step_kernel_enter();
     const int total = b.prefix[b.count];
