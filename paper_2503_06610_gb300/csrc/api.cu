@@ -927,7 +927,8 @@ void drop_batch_plans(const nh_ctx* c)
 // steps of 64 channels (7 M sites, FP32, dt_fd 16): all channels at once 12.9 ms, in
 // pairs of steps 11.7, groups of 60, 84 and 110 MB with their FD updates 11.7, 11.3
 // and 12.2, groups of 70, 84 and 100 MB for the LB steps alone 10.1, 10.2 and 10.9
-// (12 channels: 2.0 each, at once 2.6; dt_fd 4: 17.6 at once, 15.9).  Blocks of two
+// (12 channels: 2.0 each, at once 2.6; dt_fd 4: 17.6 at once, 15.9; the groups of 84 MB
+// with the present collision: 9.2 and, at dt_fd 4, 14.7).  Blocks of two
 // steps gain nothing (23.4 | 23.5).  Not where the channels take pairs of steps
 // (large ones), and only FP32 stores, whose single steps HBM bounds: the 16-bit ones
 // are bound by issue and FP64 by its pipe, where smaller launches only lose (16
@@ -1925,9 +1926,9 @@ int nh_batch_autotune(nh_ctx* const* ctxs, int count, void* stream, int* chosen)
         if (cudaEventElapsedTime(&ms[v], e0, e1) != cudaSuccess) ms[v] = 1e30f;
         if (ms[v] < ms[best]) best = v;
     }
-    // The trials leave out the launches that write u and rho (they would change the state), which four sites a thread
-    // slow down most: 16 channels of 96x96x32, FP32, in groups took 168 us a step at dt_fd 4 with two sites and 175
-    // with four, which the trials saw ahead by 1 to 2 %.
+    // The trials leave out the launches that write u and rho (they would change the state), where the shapes differ
+    // too: four sites a thread, ahead by 1 to 2 % in them, took 175 us a step of 16 channels of 96x96x32 at dt_fd 4
+    // where two took 169 (FP32, in groups).
     if (ms[best] > 0.97f * ms[saved]) best = saved;
     c0->free_events.push_back(e0);
     c0->free_events.push_back(e1);

@@ -930,9 +930,9 @@ cudaError_t launch_lb_rows(const LBChan<Real, Store>& c, cudaStream_t st)
 // lb_collide_site, and the force is the same in both (it changes only in FD
 // updates): bit-identical to two single steps.
 //
-// Bound by issue (110 M warp instructions a pass at 256x256x64, a quarter of them
+// Bound by issue (113 M warp instructions a pass at 256x256x64, a quarter of them
 // 64-bit addresses) and by the two barriers a layer.  Two steps at 256x256x64:
-// 153 us, two single steps 201 us.  Seven rows leave 96 registers to each of two
+// 148 us, two single steps 201 us.  Seven rows leave 96 registers to each of two
 // blocks per SM, so that the prefetch does not spill; with eight rows (80
 // registers) it does (181 us), without it a layer waits for its loads (158 us).
 // All tiles march up together, so that what neighbours share is read from HBM

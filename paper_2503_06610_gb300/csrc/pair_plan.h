@@ -60,9 +60,9 @@ inline PairGrid pair_split(const PairDomain& d, int cols, int rows, int layers)
 // kernel then knows its strides only at run time; tiles of 11 to 16 columns read so
 // many more sectors than they need that they were slower than tiles of 32:
 // 1024x512x8 221 us a pair of steps instead of 159.)  Two steps, tiles of 32 columns |
-// these | single steps, us: 9x330x260 93 | 32 | 38, 33x1000x100 214 | 128 | 162,
-// 33x38x600 56 | 35 | 37, 48x640x128 181 | 145 | 189, 65x200x64 51 | 40 | 41,
-// 131x97x60 43 (11 columns) | 37 (27).
+// these | single steps, us: 9x330x260 93 | 32 | 38, 33x1000x100 214 | 126 | 160,
+// 33x38x600 56 | 34 | 36, 48x640x128 181 | 142 | 189, 65x200x64 51 | 39 | 41; of
+// 131x97x60 in tiles of 11 columns | 27 | single steps 43 | 36 | 38.
 inline int pair_columns(const PairDomain& d)
 {
     auto points = [&](int cols) {
@@ -83,8 +83,8 @@ inline int pair_columns(const PairDomain& d)
 // a block takes (layers + 2) x (points of a layer); the split with the least sum
 // (256x256x64: 296 blocks of 7 rows and 64 layers).  The channels of a launch share
 // the layers and fill the waves together.  A pair of steps of eight channels of
-// 128x128x48: 258 us in two waves of whole columns, 277 us with the split that each
-// takes alone; of 64x64x200: 282 us, whole columns 495 us; two of 151x117x45: 82 us,
+// 128x128x48: 250 us in two waves of whole columns, 277 us with the split that each
+// takes alone; of 64x64x200: 270 us, whole columns 495 us; two of 151x117x45: 79 us,
 // in chunks of 15 layers 89 us.
 inline void pair_plan(const PairDomain* d, int count, PairGrid* out)
 {
@@ -127,12 +127,12 @@ inline bool pair_partials_fit(const PairDomain& d, const PairGrid& p)
 }
 
 // From 7.5e5 sites, where the two population buffers no longer stay in L2 (16 LB
-// steps and an FD update, single steps | pairs, us: 128x128x32 195 | 218,
-// 160x128x32 275 | 288, 128x128x48 337 | 323, 256x256x12 343 | 315, 180x140x32 355 |
-// 355, 151x117x45 407 | 349, 256x256x64 1815 | 1446), and up to 2.5 points of the
+// steps and an FD update, single steps | pairs, us: 128x128x32 191 | 212,
+// 160x128x32 271 | 279, 128x128x48 329 | 315, 256x256x12 335 | 306, 180x140x32 353 |
+// 343, 151x117x45 394 | 335, 256x256x64 1798 | 1388), and up to 2.5 points of the
 // first step a site, rings and the layers at the ends of a march included
-// (256x256x64: 1.4; two steps, single | pair, us: 1024x512x3, 2.3 points, 78 | 71,
-// 1024x1024x2, 2.75 points, 102 | 104, 2048x2048x1, 4.1 points, 201 | 243).
+// (256x256x64: 1.4; two steps, single | pair, us: 1024x512x3, 2.3 points, 78 | 70,
+// 1024x1024x2, 2.75 points, 102 | 104, 2048x2048x1, 4.1 points, 201 | 242).
 constexpr double kPairMinSites = 7.5e5, kPairMaxPoints = 2.5;
 inline bool pair_pays(const PairDomain& d, const PairGrid& p)
 {
